@@ -59,8 +59,8 @@ __global__ void k_list_genes(const uint32_t* __restrict__ flag, const uint32_t* 
   }
 }
 
-// Sorts gene genes[x]'s vector by k-mer id into keys[off[x] ..): key = id <<
-// 32 | multiplicity.  n_pad = next_pow2(length) <= kSmem: in shared memory;
+// Sorts gene genes[x]'s vector by k-mer (by the start of its posting list)
+// into keys[off[x] ..): key = start << 32 | multiplicity.  n_pad = next_pow2(length) <= kSmem: in shared memory;
 // longer vectors use `spill` (a global copy padded to its power of two).
 constexpr uint32_t kSortThreads = 1024, kSortSmem = 16384;
 
@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(kSortThreads)
     const uint32_t n_pad = pdg::next_pow2(n);
     unsigned long long* a = n_pad <= kSortSmem ? sk : spill + spill_off[x];
     for (uint32_t i = threadIdx.x; i < n_pad; i += blockDim.x)
-      a[i] = i < n ? ((unsigned long long)P.mv_id[m0 + i] << 32) | P.mv_cnt[m0 + i] : ~0ull;
+      a[i] = i < n ? ((unsigned long long)P.mv[m0 + i].x << 32) | P.mv[m0 + i].y : ~0ull;
     __syncthreads();
     pdg::block_bitonic_sort(a, n_pad);
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) keys[off[x] + i] = a[i];
@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(256)
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
       const uint32_t La = P.La[ga], Lb = P.La[gb];
+      if (ga == gb) s = La;  // the vectors leave out the gene's own k-mers
       if (s_out) s_out[i] = s;
       if (den_out) den_out[i] = La + Lb - s;
     }

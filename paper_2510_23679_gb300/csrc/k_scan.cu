@@ -118,8 +118,8 @@ __global__ void k_store_total(const unsigned long long* total, Out* dst) {
 
 // Exclusive scan of in(0..n-1) into out[i * stride] (and out[n * stride] =
 // total if write_last; *total_dst = total if not null).
-template <typename In, typename Out>
-cudaError_t scan_impl(Launcher* L, In in, uint64_t n, Out* out, int write_last, Out* total_dst, void* temp,
+template <typename In, typename Out, typename Total = Out>
+cudaError_t scan_impl(Launcher* L, In in, uint64_t n, Out* out, int write_last, Total* total_dst, void* temp,
                       cudaStream_t s, uint32_t stride = 1) {
   uint64_t nb = (n + kTile - 1) / kTile;
   if (nb == 0) nb = 1;
@@ -137,7 +137,7 @@ cudaError_t scan_impl(Launcher* L, In in, uint64_t n, Out* out, int write_last, 
   if ((e = launch_end(L, "scan_down")) != cudaSuccess) return e;
   if (total_dst) {
     if ((e = launch_begin(L, "scan_total")) != cudaSuccess) return e;
-    k_store_total<Out><<<1, 1, 0, s>>>(total, total_dst);
+    k_store_total<Total><<<1, 1, 0, s>>>(total, total_dst);
     if ((e = launch_end(L, "scan_total")) != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -154,17 +154,22 @@ size_t scan_temp_bytes(uint64_t n) {
 cudaError_t scan_dict_blocks(Launcher* L, uint32_t* dict, uint64_t n_blocks, uint32_t* total, void* temp,
                              cudaStream_t s) {
   // in() reads words 1..7 of a block, out writes its word 0: no overlap
-  return scan_impl<DictIn, uint32_t>(L, DictIn{dict}, n_blocks, dict, 0, total, temp, s, 8u);
+  return scan_impl<DictIn, uint32_t, uint32_t>(L, DictIn{dict}, n_blocks, dict, 0, total, temp, s, 8u);
 }
 
 cudaError_t scan_u32(Launcher* L, const uint32_t* in, uint64_t n, uint32_t* out_excl_np1, void* temp,
                      cudaStream_t s) {
-  return scan_impl<U32In, uint32_t>(L, U32In{in}, n, out_excl_np1, 1, nullptr, temp, s);
+  return scan_impl<U32In, uint32_t, uint32_t>(L, U32In{in}, n, out_excl_np1, 1, nullptr, temp, s);
 }
 
 cudaError_t scan_u32_to_u64(Launcher* L, const uint32_t* in, uint64_t n, unsigned long long* out_excl_np1,
                             void* temp, cudaStream_t s) {
-  return scan_impl<U32In, unsigned long long>(L, U32In{in}, n, out_excl_np1, 1, nullptr, temp, s);
+  return scan_impl<U32In, unsigned long long, unsigned long long>(L, U32In{in}, n, out_excl_np1, 1, nullptr, temp, s);
+}
+
+cudaError_t scan_u32_total(Launcher* L, const uint32_t* in, uint64_t n, uint32_t* out_excl_np1,
+                           unsigned long long* total, void* temp, cudaStream_t s) {
+  return scan_impl<U32In, uint32_t, unsigned long long>(L, U32In{in}, n, out_excl_np1, 1, total, temp, s);
 }
 
 }  // namespace pdg

@@ -181,13 +181,14 @@ __device__ __forceinline__ uint32_t lower_bound_post(const uint32_t* __restrict_
   return lo;
 }
 
-// Exact multiplicity of k-mer id in gene g, for a saturated packed count.
-// A multiplicity vector is stored in hash order, so this is a linear scan
-// (rare: only counts at the cap of the packed field come here).
-__device__ __forceinline__ uint32_t mv_count_of(const ProfilesView& P, uint32_t g, uint32_t id) {
+// Exact multiplicity in gene g of the k-mer whose posting list starts at
+// `start`, for a saturated packed count.  A multiplicity vector is unordered,
+// so this is a linear scan (rare: only counts at the cap of the packed field
+// come here).
+__device__ __forceinline__ uint32_t mv_count_of(const ProfilesView& P, uint32_t g, uint32_t start) {
   const uint32_t off = P.win_off[g], n = P.mv_n[g];
   for (uint32_t e = 0; e < n; ++e)
-    if (P.mv_id[off + e] == id) return P.mv_cnt[off + e];
+    if (P.mv[off + e].x == start) return P.mv[off + e].y;
   return 0u;
 }
 
@@ -255,6 +256,9 @@ constexpr uint32_t kWarpWalkMinAvg = 16;
 // taken: below a few L2 sizes the merge-path walk's runs of postings keep
 // hitting the sectors they have already brought in.
 constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
+// Length field of a vector entry's z (the top bit marks lists holding another
+// gene of the same genome).
+constexpr uint32_t kListLength = 0x7FFFFFFFu;
 // Target genomes from which a query's Best Hits are ranked through per-genome
 // positions rather than pairwise.
 constexpr uint32_t kRankByGenomeMin = 64;
@@ -302,7 +306,6 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
       own1 = (uint32_t)P.genome_ptr[gg + 1];
       if (Q.tgt_end) tend = Q.tgt_end[gg];
       col = gg - Q.col_genome0;
-      if (Q.symbest) key_lo = (unsigned long long)own1 << P.cnt_bits;  // first posting past a's genome
     }
   } else {
     uint32_t tlo, thi;
@@ -336,10 +339,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
   }
   // the query's own vector (its dataset's, or the external query arrays)
   const bool ext = P.q_win_off != nullptr;
-  const uint32_t* __restrict__ q_mv_id = ext ? P.q_mv_id : P.mv_id;
-  const uint16_t* __restrict__ q_mv_cnt = ext ? P.q_mv_cnt : P.mv_cnt;
-  const uint32_t* __restrict__ q_mv_post = ext ? P.q_mv_post : P.mv_post;
-  const uint32_t* __restrict__ q_mv_plen = ext ? P.q_mv_plen : P.mv_plen;
+  const uint4* __restrict__ q_mv = ext ? P.q_mv : P.mv;
   const uint32_t m0 = (ext ? P.q_win_off : P.win_off)[a], E = (ext ? P.q_mv_n : P.mv_n)[a];
   const uint32_t La_a = (ext ? P.q_La : P.La)[a];
   const uint32_t cnt_mask = (1u << P.cnt_bits) - 1u;
@@ -350,6 +350,18 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
     sh->overflow = (kPacked && La_a >= cnt_mask) ? 1u : 0u;
   }
   __syncthreads();
+  // The part [lo, lo + len) of a vector entry's posting list that holds the
+  // query's targets.
+  auto narrow = [&](const uint4& v, uint32_t& lo, uint32_t& len) {
+    if (!Q.all_pairs) {
+      const uint32_t end = lo + len;
+      lo = lower_bound_post(P.post, lo, end, key_lo);
+      len = lower_bound_post(P.post, lo, end, key_hi) - lo;
+    } else if (Q.symbest) {  // the genomes after the query's own
+      lo += v.w;
+      len -= v.w;
+    }
+  };
   unsigned long long walked = 0;
   const uint32_t lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t kWarps = kThreads / 32;
@@ -361,7 +373,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
     // per-posting range tests.  `e` is the query's chunk entry of the k-mer.
     auto accumulate = [&](uint32_t p, uint32_t ca, uint32_t e) {
       uint32_t cb = p & cnt_mask;
-      if (cb == P.cnt_cap && ca > cb) cb = mv_count_of(P, p >> P.cnt_bits, q_mv_id[m0 + c0 + e]);
+      if (cb == P.cnt_cap && ca > cb) cb = mv_count_of(P, p >> P.cnt_bits, q_mv[m0 + c0 + e].x);
       const uint32_t key = kPacked ? (p & ~cnt_mask) : (p >> P.cnt_bits);
       if (!acc.add(mask, key, min(ca, cb), ca, cb)) sh->overflow = 1;
     };
@@ -370,25 +382,19 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
       // ranges (the restricted forms narrow lists to a target genome) are
       // dropped, so the staged list starts strictly increase, as the walk's
       // k-mer lookup needs.
-      uint32_t lo_loc[kItems], len_loc[kItems];
+      uint32_t lo_loc[kItems], len_loc[kItems], cnt_loc[kItems];
       uint32_t my_sum = 0, my_n = 0;
 #pragma unroll
       for (uint32_t r = 0; r < kItems; ++r) {
         const uint32_t e = tid * kItems + r;
         uint32_t lo = 0, len = 0;
+        cnt_loc[r] = 0;
         if (e < n_in) {
-          lo = q_mv_post[m0 + c0 + e];
-          const uint32_t plen = q_mv_plen[m0 + c0 + e];
-          uint32_t hi = lo + plen;
-          if (!ext && plen == 1u) {
-            hi = lo;  // the list holds only the query's own posting: never a target
-          } else if (!Q.all_pairs) {
-            lo = lower_bound_post(P.post, lo, hi, key_lo);
-            hi = lower_bound_post(P.post, lo, hi, key_hi);
-          } else if (Q.symbest) {
-            lo = lower_bound_post(P.post, lo, hi, key_lo);  // the genomes after the query's own
-          }
-          len = hi - lo;
+          const uint4 v = q_mv[m0 + c0 + e];
+          lo = v.x;
+          cnt_loc[r] = v.y;
+          len = v.z & kListLength;
+          narrow(v, lo, len);
         }
         lo_loc[r] = lo;
         len_loc[r] = len;
@@ -403,7 +409,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         const uint32_t e = tid * kItems + r;
         if (len_loc[r]) {
           c_post[slot] = lo_loc[r];
-          c_cnt[slot] = q_mv_cnt[m0 + c0 + e];
+          c_cnt[slot] = (uint16_t)cnt_loc[r];
           c_ent[slot] = (uint16_t)e;
           c_off[slot] = run;
           ++slot;
@@ -461,17 +467,12 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         const uint32_t e = tid * kItems + r;
         uint32_t len = 0;
         if (e < n_in) {
-          uint32_t lo = q_mv_post[m0 + c0 + e];
-          uint32_t hi = lo + q_mv_plen[m0 + c0 + e];
-          if (!Q.all_pairs) {
-            lo = lower_bound_post(P.post, lo, hi, key_lo);
-            hi = lower_bound_post(P.post, lo, hi, key_hi);
-          } else if (Q.symbest) {
-            lo = lower_bound_post(P.post, lo, hi, key_lo);  // the genomes after the query's own
-          }
+          const uint4 v = q_mv[m0 + c0 + e];
+          uint32_t lo = v.x;
+          len = v.z & kListLength;
+          narrow(v, lo, len);
           c_post[e] = lo;
-          c_cnt[e] = q_mv_cnt[m0 + c0 + e];
-          len = hi - lo;
+          c_cnt[e] = (uint16_t)v.y;
         }
         len_loc[r] = len;
         my_sum += len;

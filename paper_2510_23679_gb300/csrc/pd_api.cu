@@ -318,164 +318,154 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
       return fail(c, PD_ERR_BUDGET, "segments x 20^k exceed the dictionary limit (" +
                                         std::to_string(kMaxDictCodes >> 30) + " Gi codes)");
   }
-  const uint64_t n_dict = pdg::dict_blocks(n_seg * n_codes);
-  const size_t G1 = std::max<uint32_t>(n_genes, 1);
   pdg::Launcher* L = &c->L;
-
-  // ---- inputs on the device
-  Buf d_res, d_gene_ptr, d_mid, d_long, d_long_off, d_long_scratch, tmp, d_counts, minhash, d_code_base;
-  const uint8_t* res_dev = residues;
-  const int64_t* gp_devp = gene_ptr;
-  if (n_res > 0 && !is_device_ptr(residues)) {
-    ALLOC(d_res, n_res);
-    CK(cudaMemcpyAsync(d_res.p, residues, n_res, cudaMemcpyHostToDevice, c->stream));
-    res_dev = d_res.as<uint8_t>();
-  }
-  if (!gp_dev) {
-    ALLOC(d_gene_ptr, sizeof(int64_t) * (n_genes + 1));
-    CK(cudaMemcpyAsync(d_gene_ptr.p, gene_ptr, sizeof(int64_t) * (n_genes + 1), cudaMemcpyHostToDevice,
-                       c->stream));
-    gp_devp = d_gene_ptr.as<int64_t>();
-  }
-  ALLOC(P->genome_ptr, sizeof(int32_t) * (n_genomes + 1));
-  ALLOC(P->La, sizeof(uint32_t) * G1);
-  ALLOC(P->win_off, sizeof(uint32_t) * (n_genes + 1));
-  ALLOC(P->gene_genome, sizeof(uint16_t) * G1);
-  ALLOC(P->ginfo, sizeof(uint32_t) * G1);
-  CK(cudaMemcpyAsync(P->genome_ptr.p, genome_ptr, sizeof(int32_t) * (n_genomes + 1), cudaMemcpyDefault, c->stream));
-
-  // ---- window counts, window offsets and the gene classes, on the device
-  Buf d_win64, d_gtmp, d_wcount;
-  ALLOC(d_mid, sizeof(uint32_t) * G1);
-  ALLOC(d_long, sizeof(uint32_t) * G1);
-  ALLOC(d_long_off, sizeof(unsigned long long) * G1);
-  ALLOC(d_win64, sizeof(unsigned long long) * (n_genes + 1));
-  ALLOC(d_gtmp, pdg::scan_temp_bytes(n_genes + 1) + 64);
-  ALLOC(d_wcount, 4 * sizeof(unsigned long long));  // [n_mid, n_long] (u32), long_total (u64)
-  CK(cudaMemsetAsync(d_wcount.p, 0, 4 * sizeof(unsigned long long), c->stream));
-  unsigned long long* wcount64 = d_wcount.as<unsigned long long>();
-  if (n_genes)
-    CK(pdg::run_gene_windows(L, gp_devp, n_genes, n_res, gene_src ? 0 : 1, k, P->La.as<uint32_t>(),
-                             d_mid.as<uint32_t>(), d_long.as<uint32_t>(), d_long_off.as<unsigned long long>(),
-                             (uint32_t*)wcount64, wcount64 + 1, c->d_err, c->stream));
-  CK(pdg::scan_u32_to_u64(L, P->La.as<uint32_t>(), n_genes, d_win64.as<unsigned long long>(), d_gtmp.p, c->stream));
-  CK(pdg::run_narrow_u64(L, d_win64.as<unsigned long long>(), n_genes + 1, P->win_off.as<uint32_t>(), c->stream));
-  if (early_genomes)
-    CK(pdg::run_gene_info(L, P->genome_ptr.as<int32_t>(), n_genomes, P->La.as<uint32_t>(),
-                          P->gene_genome.as<uint16_t>(), P->ginfo.as<uint32_t>(), c->stream));
-
-  if (genome_seg) {
-    ALLOC(d_code_base, sizeof(unsigned long long) * n_genomes);
-    CK(cudaMemcpyAsync(d_code_base.p, code_base.data(), sizeof(unsigned long long) * n_genomes,
-                       cudaMemcpyHostToDevice, c->stream));
-  }
-
-  // ---- dictionary: present codes in rank blocks, then the blocks' rank bases
-  ALLOC(P->dict, 8 * sizeof(uint32_t) * n_dict);
-  CK(cudaMemsetAsync(P->dict.p, 0, 8 * sizeof(uint32_t) * n_dict, c->stream));
-  if (n_genes)
-    CK(pdg::run_encode_mark(L, res_dev, gp_devp, n_genes, k, P->dict.as<uint32_t>(),
-                            P->gene_genome.as<uint16_t>(), d_code_base.as<unsigned long long>(), gene_src,
-                            alphabet, n_res, c->d_err, c->stream));
-  const uint32_t kOrderShift = 16;  // 65536 min-hash buckets
-  const uint64_t n_order_b = (uint64_t)1 << (32 - kOrderShift);
-  ALLOC(tmp, pdg::scan_temp_bytes(std::max<uint64_t>(std::max<uint64_t>(n_dict, n_order_b), 24577)) + 64);
-  ALLOC(d_counts, 4 * sizeof(uint32_t));  // [0] = D, [1] = max posting
-  CK(cudaMemsetAsync(d_counts.p, 0, 4 * sizeof(uint32_t), c->stream));
-  CK(pdg::scan_dict_blocks(L, P->dict.as<uint32_t>(), n_dict, d_counts.as<uint32_t>(), tmp.p, c->stream));
-  // one synchronisation: the dictionary size, the window total, the gene
-  // classes and any error found in the offsets or the letters
-  unsigned long long* hb = c->h_build;
-  CK(cudaMemcpyAsync(hb, d_counts.p, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(hb + 2, d_win64.as<unsigned long long>() + n_genes, sizeof(unsigned long long),
-                     cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(hb + 3, wcount64, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
-  pd_status st = check_dev_err(c);  // synchronizes
-  if (st != PD_OK) return st;
-  const uint64_t D = (uint32_t)hb[0];
-  const uint64_t W = hb[2];
-  const uint32_t n_mid = (uint32_t)hb[3], n_long = (uint32_t)(hb[3] >> 32);
-  const uint64_t long_total = hb[4];
-  if (W > 0xFFFFFFF0ull) return fail(c, PD_ERR_ARG, "more than 2^32 k-mer windows in the dataset");
-  if (!early_genomes) {
-    if ((st = check_genomes()) != PD_OK) return st;
-    CK(pdg::run_gene_info(L, P->genome_ptr.as<int32_t>(), n_genomes, P->La.as<uint32_t>(),
-                          P->gene_genome.as<uint16_t>(), P->ginfo.as<uint32_t>(), c->stream));
-  }
-  P->h_genome_ptr = hgn;
-  const size_t W1 = std::max<uint64_t>(W, 1);
-
-  // ---- multiplicity vectors (and one index record per entry)
   // gene field wide enough to keep the all-ones id unused (see the packed
-  // accumulator slots of k_summin.cu)
+  // accumulator slots of k_summin.cu and the sort records of k_index.cu)
   const uint32_t gene_bits = bits_for(n_genes);
   const uint32_t cnt_bits = 32 - gene_bits;
   const uint32_t cnt_cap = std::min<uint32_t>((1u << cnt_bits) - 1u, 65535u);
-  Buf mvrec;
-  ALLOC(P->mv_id, sizeof(uint32_t) * W1);
-  ALLOC(P->mv_cnt, sizeof(uint16_t) * W1);
-  ALLOC(P->mv_n, sizeof(uint32_t) * G1);
-  ALLOC(minhash, sizeof(uint32_t) * G1);
-  ALLOC(mvrec, sizeof(unsigned long long) * W1);
-  if (n_long) ALLOC(d_long_scratch, sizeof(unsigned long long) * long_total);
-  pdg::MvOut M;
-  M.mv_id = P->mv_id.as<uint32_t>();
-  M.mv_cnt = P->mv_cnt.as<uint16_t>();
-  M.mv_n = P->mv_n.as<uint32_t>();
-  M.rec = mvrec.as<unsigned long long>();
-  M.minhash = minhash.as<uint32_t>();
-  M.cnt_bits = cnt_bits;
-  M.cnt_cap = cnt_cap;
-  M.err = c->d_err;
-  M.gene_genome = P->gene_genome.as<uint16_t>();
-  M.genome_code_base = d_code_base.as<unsigned long long>();
-  M.gene_src = gene_src;
-  M.alpha = alphabet;
-  M.length_buckets = length_buckets;
-  M.frozen = 0;
-  if (n_genes)
-    CK(pdg::run_mv_build(L, res_dev, gp_devp, P->win_off.as<uint32_t>(), n_genes, k, P->dict.as<uint32_t>(), M,
-                         d_mid.as<uint32_t>(), n_mid, d_long.as<uint32_t>(), n_long,
-                         d_long_scratch.as<unsigned long long>(), d_long_off.as<unsigned long long>(), c->stream));
+  pdg::SortKey K = pdg::sort_key(n_seg * n_codes, gene_bits);
 
-  // ---- inverted index: stable radix sort of the index records by k-mer id
-  // (records arrive in gene order, so every posting list ends up gene-sorted)
-  Buf recs, rcounts, rtmp;
-  ALLOC(recs, sizeof(unsigned long long) * W1);
-  ALLOC(rcounts, sizeof(uint32_t) * pdg::radix_counts_words(W));
-  ALLOC(rtmp, pdg::scan_temp_bytes(pdg::radix_counts_words(W)) + 64);
-  ALLOC(P->post_ptr, sizeof(uint32_t) * (D + 1));
-  ALLOC(P->post, sizeof(uint32_t) * W1);
-  CK(cudaMemsetAsync(P->post_ptr.p, 0, sizeof(uint32_t) * (D + 1), c->stream));
-  if (W && D)
-    CK(pdg::run_index_sort(L, mvrec.as<unsigned long long>(), recs.as<unsigned long long>(), W, bits_for((uint32_t)D),
-                           rcounts.as<uint32_t>(), rtmp.p, D, P->post.as<uint32_t>(), P->post_ptr.as<uint32_t>(),
-                           c->stream));
-  ALLOC(P->mv_post, sizeof(uint32_t) * W1);
-  ALLOC(P->mv_plen, sizeof(uint32_t) * W1);
-  if (n_genes && D)
-    CK(pdg::run_mv_post(L, P->win_off.as<uint32_t>(), P->mv_n.as<uint32_t>(), P->mv_id.as<uint32_t>(), n_genes,
-                        P->post_ptr.as<uint32_t>(), P->mv_post.as<uint32_t>(), P->mv_plen.as<uint32_t>(),
-                        d_counts.as<uint32_t>() + 1, (unsigned long long*)(d_counts.as<uint32_t>() + 2),
-                        c->stream));
+  // ---- per-gene arrays, inputs on the device
+  Carve cg;
+  const size_t o_genome_ptr = cg.add(sizeof(int32_t) * (n_genomes + 1)), o_La = cg.add(sizeof(uint32_t) * n_genes),
+               o_win_off = cg.add(sizeof(uint32_t) * (n_genes + 1)), o_mv_n = cg.add(sizeof(uint32_t) * n_genes),
+               o_gene_genome = cg.add(sizeof(uint16_t) * n_genes), o_ginfo = cg.add(sizeof(uint32_t) * n_genes),
+               o_order = cg.add(sizeof(uint32_t) * n_genes);
+  ALLOC(P->genes, cg.bytes);
+  int32_t* d_genome_ptr = piece<int32_t>(P->genes, o_genome_ptr);
+  uint32_t *d_La = piece<uint32_t>(P->genes, o_La), *d_win_off = piece<uint32_t>(P->genes, o_win_off),
+           *d_mv_n = piece<uint32_t>(P->genes, o_mv_n), *d_ginfo = piece<uint32_t>(P->genes, o_ginfo),
+           *d_order = piece<uint32_t>(P->genes, o_order);
+  uint16_t* d_gene_genome = piece<uint16_t>(P->genes, o_gene_genome);
+  const bool copy_res = n_res > 0 && !is_device_ptr(residues);
+  Carve ct;
+  // zeroed words first: [0] windows, [1..4] postings and ids (so far, before the slice), [5] join, [6] longest
+  // list, [7] records of the slice; then the order's counts
+  const size_t o_words = ct.add(8 * sizeof(unsigned long long)),
+               o_ocount = ct.add(sizeof(uint32_t) * (2 * pdg::kOrderBuckets + 1)), zeroed = ct.bytes,
+               o_minhash = ct.add(sizeof(uint32_t) * n_genes), o_cursor = ct.add(sizeof(uint32_t) * n_genes),
+               o_start = ct.add(sizeof(unsigned long long) * pdg::kDigitStarts),
+               o_scan = ct.add(pdg::scan_temp_bytes(std::max<uint64_t>((uint64_t)n_genes + 1, pdg::kOrderBuckets)) + 64),
+               o_gene_ptr = ct.add(gp_dev ? 0 : sizeof(int64_t) * (n_genes + 1)),
+               o_code_base = ct.add(genome_seg ? sizeof(unsigned long long) * n_genomes : 0),
+               o_res = ct.add(copy_res ? n_res : 0);
+  Buf tmp1, tmp2;
+  ALLOC(tmp1, ct.bytes);
+  unsigned long long* words = piece<unsigned long long>(tmp1, o_words);
+  uint32_t* minhash = piece<uint32_t>(tmp1, o_minhash);
+  void* scan_tmp = piece<void>(tmp1, o_scan);
+  const uint8_t* res_dev = residues;
+  const int64_t* gp_devp = gene_ptr;
+  if (copy_res) {
+    CK(cudaMemcpyAsync(piece<uint8_t>(tmp1, o_res), residues, n_res, cudaMemcpyHostToDevice, c->stream));
+    res_dev = piece<uint8_t>(tmp1, o_res);
+  }
+  if (!gp_dev) {
+    CK(cudaMemcpyAsync(piece<int64_t>(tmp1, o_gene_ptr), gene_ptr, sizeof(int64_t) * (n_genes + 1),
+                       cudaMemcpyHostToDevice, c->stream));
+    gp_devp = piece<int64_t>(tmp1, o_gene_ptr);
+  }
+  CK(cudaMemsetAsync(words, 0, zeroed, c->stream));
+  CK(cudaMemsetAsync(minhash, 0xFF, sizeof(uint32_t) * std::max<uint32_t>(n_genes, 1), c->stream));
+  CK(cudaMemcpyAsync(d_genome_ptr, genome_ptr, sizeof(int32_t) * (n_genomes + 1), cudaMemcpyDefault, c->stream));
+
+  // ---- offsets and letters checked, window offsets, genes' genomes
+  if (n_genes)
+    CK(pdg::run_gene_windows(L, gp_devp, n_genes, n_res, gene_src ? 0 : 1, k, d_La, c->d_err, c->stream));
+  CK(pdg::scan_u32_total(L, d_La, n_genes, d_win_off, words, scan_tmp, c->stream));
+  if (n_genes)
+    CK(pdg::run_check_letters(L, res_dev, n_res, gp_devp, gene_src, n_genes, alphabet, c->d_err, c->stream));
+  if (early_genomes)
+    CK(pdg::run_gene_info(L, d_genome_ptr, n_genomes, d_La, d_gene_genome, d_ginfo, c->stream));
+  unsigned long long* d_code_base = nullptr;
+  if (genome_seg) {
+    d_code_base = piece<unsigned long long>(tmp1, o_code_base);
+    CK(cudaMemcpyAsync(d_code_base, code_base.data(), sizeof(unsigned long long) * n_genomes, cudaMemcpyHostToDevice,
+                       c->stream));
+  }
+  // one synchronisation: the window total and any error found so far
+  unsigned long long* hb = c->h_build;
+  CK(cudaMemcpyAsync(hb, words, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+  pd_status st = check_dev_err(c);  // synchronizes
+  if (st != PD_OK) return st;
+  const uint64_t W = hb[0];
+  if (W > 0xFFFFFFF0ull) return fail(c, PD_ERR_ARG, "more than 2^32 k-mer windows in the dataset");
+  if (!early_genomes) {
+    if ((st = check_genomes()) != PD_OK) return st;
+    CK(pdg::run_gene_info(L, d_genome_ptr, n_genomes, d_La, d_gene_genome, d_ginfo, c->stream));
+  }
+  P->h_genome_ptr = hgn;
+
+  // ---- vectors, postings, and one record buffer that ends up holding the
+  // posting-list starts and the codes (at most one of each per window)
+  const bool wide_codes = n_seg * n_codes > (1ull << 32);
+  Carve cw;
+  const size_t o_mv = cw.add(sizeof(uint4) * W), o_post = cw.add(sizeof(uint32_t) * W),
+               o_lists = cw.add(2 * sizeof(uint32_t) * (W + 1)), o_code_hi = cw.add(wide_codes ? W : 0);
+  ALLOC(P->windows, cw.bytes);
+  uint4* d_mv = piece<uint4>(P->windows, o_mv);
+  uint32_t *d_post = piece<uint32_t>(P->windows, o_post), *d_post_ptr = piece<uint32_t>(P->windows, o_lists);
+  uint32_t* d_code_lo = d_post_ptr + (W + 1);
+  uint8_t* d_code_hi = wide_codes ? piece<uint8_t>(P->windows, o_code_hi) : nullptr;
+  if (W == 0) {
+    CK(cudaMemsetAsync(d_post_ptr, 0, sizeof(uint32_t), c->stream));
+    if (n_genes) CK(cudaMemsetAsync(d_mv_n, 0, sizeof(uint32_t) * n_genes, c->stream));
+  } else {
+    const pdg::SortScratch X = pdg::sort_scratch(K, W);
+    const uint32_t n_dtiles = pdg::dedupe_tiles(W);
+    Carve cs;
+    const size_t o_tile_gene = cs.add(sizeof(uint32_t) * (pdg::sort_tiles(W) + 1)),
+                 o_tile_e = cs.add(sizeof(uint32_t) * (n_dtiles + 1)), o_tile_id = cs.add(sizeof(uint32_t) * (n_dtiles + 1)),
+                 o_scratch = cs.add(X.bytes), o_rec = cs.add(sizeof(unsigned long long) * W);
+    ALLOC(tmp2, cs.bytes);
+    uint8_t* scratch = piece<uint8_t>(tmp2, o_scratch);
+    uint32_t *tile_e = piece<uint32_t>(tmp2, o_tile_e), *tile_id = piece<uint32_t>(tmp2, o_tile_id);
+    pdg::WindowSource S{res_dev, gp_devp, gene_src, d_win_off, piece<uint32_t>(tmp2, o_tile_gene), d_gene_genome,
+                        d_code_base, k, alphabet, W};
+    CK(pdg::run_tile_genes(L, d_win_off, n_genes, W, piece<uint32_t>(tmp2, o_tile_gene), c->stream));
+    // two record buffers, one of which ends up holding lists and codes
+    unsigned long long *rec = piece<unsigned long long>(tmp2, o_rec), *other = (unsigned long long*)d_post_ptr;
+    const bool odd = K.passes & 1u;
+    unsigned long long* start = piece<unsigned long long>(tmp1, o_start);
+    uint32_t* cursor = piece<uint32_t>(tmp1, o_cursor);
+    CK(cudaMemcpyAsync(cursor, d_win_off, sizeof(uint32_t) * n_genes, cudaMemcpyDeviceToDevice, c->stream));
+    Buf slice_rec;
+    for (K.slice = 0; K.slice < K.n_slices; ++K.slice) {
+      CK(cudaMemsetAsync(scratch, 0, X.bytes, c->stream));
+      CK(pdg::run_code_hist(L, S, K, scratch, X, start, words + 7, K.slice ? nullptr : minhash, c->stream));
+      uint64_t n = W;
+      if (K.n_slices > 1) {
+        CK(cudaMemcpyAsync(hb, words + 7, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+        CK(cudaStreamSynchronize(c->stream));
+        n = hb[0];
+        if (n == 0) continue;
+        // the memory above holds what the slices before left: records of their own
+        ALLOC(slice_rec, 2 * sizeof(unsigned long long) * n);
+        rec = slice_rec.as<unsigned long long>();
+        other = rec + n;
+      }
+      unsigned long long* sorted = nullptr;
+      CK(pdg::run_sort(L, S, K, n, scratch, X, start, odd ? rec : other, odd ? other : rec, &sorted, c->d_err,
+                       c->stream));
+      CK(pdg::run_dedupe(L, sorted, n, K, scratch, X, cnt_bits, cnt_cap, words + 1, d_post, d_post_ptr, d_code_lo,
+                         d_code_hi, tile_e, tile_id, c->d_err, c->stream));
+      CK(pdg::run_lists(L, sorted, n, K, tile_e, tile_id, d_post, d_post_ptr, d_code_lo, d_code_hi, cnt_bits, cnt_cap,
+                        d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5, c->stream));
+    }
+    if (K.n_slices > 1) CK(cudaStreamSynchronize(c->stream));  // the last slice's records end here
+    CK(pdg::run_vector_lengths(L, cursor, d_win_off, n_genes, d_mv_n, c->stream));
+  }
 
   // ---- all-pairs query order: min-hash buckets
-  Buf ocount;
-  ALLOC(P->order, sizeof(uint32_t) * G1);
-  ALLOC(ocount, sizeof(uint32_t) * (2 * n_order_b + 1));
-  CK(cudaMemsetAsync(ocount.p, 0, sizeof(uint32_t) * n_order_b, c->stream));
   if (n_genes)
-    CK(pdg::run_order(L, minhash.as<uint32_t>(), n_genes, kOrderShift, ocount.as<uint32_t>(),
-                      P->order.as<uint32_t>(), tmp.p, c->stream));
-
-  uint32_t* hb32 = (uint32_t*)c->h_build;  // [0] = E, [2..5] = d_counts
-  CK(cudaMemcpyAsync(hb32, P->post_ptr.as<uint32_t>() + D, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(hb32 + 2, d_counts.p, 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
+    CK(pdg::run_order(L, minhash, d_La, n_genes, length_buckets, piece<uint32_t>(tmp1, o_ocount), d_order, scan_tmp,
+                      c->stream));
+  CK(cudaMemcpyAsync(hb, words, 7 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
   st = check_dev_err(c);  // synchronizes; temporaries are released after this
   if (st != PD_OK) return st;
-  const uint64_t E = hb32[0];
-  const uint32_t max_posting = hb32[3];
-  const uint64_t n_join = ((const unsigned long long*)c->h_build)[2];  // d_counts words 2-3
+  const uint64_t E = hb[1], D = hb[2], n_join = hb[5];
+  const uint32_t max_posting = (uint32_t)hb[6];
 
   pdg::ProfilesView& v = P->view;
   v.k = k;
@@ -488,21 +478,18 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   v.cnt_cap = cnt_cap;
   v.max_posting = max_posting;
   v.n_join = n_join;
-  v.win_off = P->win_off.as<uint32_t>();
-  v.mv_n = P->mv_n.as<uint32_t>();
-  v.mv_id = P->mv_id.as<uint32_t>();
-  v.mv_cnt = P->mv_cnt.as<uint16_t>();
-  v.mv_post = P->mv_post.as<uint32_t>();
-  v.mv_plen = P->mv_plen.as<uint32_t>();
-  v.La = P->La.as<uint32_t>();
-  v.gene_genome = P->gene_genome.as<uint16_t>();
-  v.ginfo = P->ginfo.as<uint32_t>();
-  v.genome_ptr = P->genome_ptr.as<int32_t>();
-  v.dict = P->dict.as<uint32_t>();
-  v.n_dict_blocks = n_dict;
-  v.post_ptr = P->post_ptr.as<uint32_t>();
-  v.post = P->post.as<uint32_t>();
-  v.order = P->order.as<uint32_t>();
+  v.win_off = d_win_off;
+  v.mv_n = d_mv_n;
+  v.mv = d_mv;
+  v.La = d_La;
+  v.gene_genome = d_gene_genome;
+  v.ginfo = d_ginfo;
+  v.genome_ptr = d_genome_ptr;
+  v.code_lo = d_code_lo;
+  v.code_hi = d_code_hi;
+  v.post_ptr = d_post_ptr;
+  v.post = d_post;
+  v.order = d_order;
   pd_profiles_info& in = P->info;
   in.k = k;
   in.n_genes = n_genes;
@@ -514,9 +501,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   in.n_join = n_join;
   in.count_bits = cnt_bits;
   in.alphabet = alphabet;
-  in.device_bytes = P->genome_ptr.n + P->La.n + P->win_off.n + P->mv_n.n + P->mv_id.n + P->mv_cnt.n +
-                    P->mv_post.n + P->mv_plen.n + P->gene_genome.n + P->ginfo.n + P->dict.n +
-                    P->post_ptr.n + P->post.n + P->order.n;
+  in.device_bytes = P->genes.n + P->windows.n;
   *out = guard.release();
   return PD_OK;
 }
@@ -600,28 +585,32 @@ PD_API pd_status pd_profiles_copy_mv(pd_ctx* c, const pd_profiles* P, int64_t* m
     CK(cudaSetDevice(c->device));
     const pdg::ProfilesView& v = P->view;
     pdg::Launcher* L = &c->L;
-    Buf ptr, tmp, code_of_id, d_codes, d_counts, pad_off, pad;
+    Buf ptr, tmp, n_of, fill, d_codes, d_counts, pad_off, pad;
     ALLOC(ptr, sizeof(unsigned long long) * (v.n_genes + 1));
+    ALLOC(n_of, sizeof(uint32_t) * std::max<uint32_t>(v.n_genes, 1));
     ALLOC(tmp, pdg::scan_temp_bytes(v.n_genes + 1) + 64);
-    CK(pdg::scan_u32_to_u64(L, v.mv_n, v.n_genes, ptr.as<unsigned long long>(), tmp.p, c->stream));
+    CK(cudaMemsetAsync(n_of.p, 0, sizeof(uint32_t) * std::max<uint32_t>(v.n_genes, 1), c->stream));
+    if (v.n_entries) CK(pdg::run_export_mv_count(L, v, n_of.as<uint32_t>(), c->stream));
+    CK(pdg::scan_u32_to_u64(L, n_of.as<uint32_t>(), v.n_genes, ptr.as<unsigned long long>(), tmp.p, c->stream));
     if ((codes || counts) && v.n_genes) {
       // per-gene power-of-two scratch for the sort by code
       std::vector<uint32_t> n(v.n_genes);
-      CK(cudaMemcpyAsync(n.data(), v.mv_n, sizeof(uint32_t) * v.n_genes, cudaMemcpyDeviceToHost, c->stream));
+      CK(cudaMemcpyAsync(n.data(), n_of.p, sizeof(uint32_t) * v.n_genes, cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
       std::vector<unsigned long long> off(v.n_genes + 1, 0);
       for (uint32_t g = 0; g < v.n_genes; ++g) off[g + 1] = off[g] + (n[g] ? pdg::next_pow2(n[g]) : 0);
       ALLOC(pad_off, sizeof(unsigned long long) * (v.n_genes + 1));
       ALLOC(pad, sizeof(unsigned long long) * std::max<unsigned long long>(off[v.n_genes], 1));
+      ALLOC(fill, sizeof(uint32_t) * v.n_genes);
       CK(cudaMemcpyAsync(pad_off.p, off.data(), sizeof(unsigned long long) * (v.n_genes + 1), cudaMemcpyHostToDevice,
                          c->stream));
-      ALLOC(code_of_id, sizeof(unsigned long long) * std::max<uint64_t>(v.n_distinct, 1));
-      CK(pdg::run_select_codes(L, v.dict, v.n_dict_blocks, code_of_id.as<unsigned long long>(), c->stream));
+      CK(cudaMemsetAsync(pad.p, 0xFF, sizeof(unsigned long long) * off[v.n_genes], c->stream));
+      CK(cudaMemsetAsync(fill.p, 0, sizeof(uint32_t) * v.n_genes, c->stream));
       ALLOC(d_codes, sizeof(unsigned long long) * std::max<uint64_t>(v.n_entries, 1));
       ALLOC(d_counts, sizeof(uint32_t) * std::max<uint64_t>(v.n_entries, 1));
-      CK(pdg::run_export_mv(L, v, ptr.as<unsigned long long>(), pad_off.as<unsigned long long>(),
-                            pad.as<unsigned long long>(), code_of_id.as<unsigned long long>(),
-                            d_codes.as<unsigned long long>(), d_counts.as<uint32_t>(), c->stream));
+      CK(pdg::run_export_mv(L, v, ptr.as<unsigned long long>(), pad_off.as<unsigned long long>(), fill.as<uint32_t>(),
+                            pad.as<unsigned long long>(), d_codes.as<unsigned long long>(), d_counts.as<uint32_t>(),
+                            c->stream));
       CK(cudaStreamSynchronize(c->stream));  // host offsets must outlive the copy
     }
     pd_status st;
@@ -654,7 +643,7 @@ PD_API pd_status pd_profiles_copy_index(pd_ctx* c, const pd_profiles* P, int64_t
     }
     if (codes) {
       ALLOC(code_of_id, sizeof(unsigned long long) * std::max<uint64_t>(v.n_distinct, 1));
-      CK(pdg::run_select_codes(L, v.dict, v.n_dict_blocks, code_of_id.as<unsigned long long>(), c->stream));
+      CK(pdg::run_export_codes(L, v, code_of_id.as<unsigned long long>(), c->stream));
     }
     if (genes) ALLOC(d_genes, sizeof(int32_t) * std::max<uint64_t>(v.n_entries, 1));
     if (counts) ALLOC(d_counts, sizeof(uint32_t) * std::max<uint64_t>(v.n_entries, 1));
@@ -774,14 +763,29 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
   return fail(c, PD_ERR_INTERNAL, "Best Hit output did not converge");
 }
 
+pd_status pdh::build_dictionary(pd_ctx* c, pd_profiles* P) {
+  pdg::ProfilesView& v = P->view;
+  const uint64_t n_dict = pdg::dict_blocks(pow_u64((uint64_t)P->info.alphabet, v.k));
+  Buf tmp;
+  ALLOC(P->dict, 8 * sizeof(uint32_t) * n_dict);
+  ALLOC(tmp, pdg::scan_temp_bytes(n_dict) + 64);
+  CK(cudaMemsetAsync(P->dict.p, 0, 8 * sizeof(uint32_t) * n_dict, c->stream));
+  if (v.n_distinct)
+    CK(pdg::run_dict_mark(&c->L, v.code_lo, v.code_hi, v.n_distinct, P->dict.as<uint32_t>(), c->stream));
+  uint32_t* total = (uint32_t*)((unsigned char*)tmp.p + pdg::scan_temp_bytes(n_dict));
+  CK(pdg::scan_dict_blocks(&c->L, P->dict.as<uint32_t>(), n_dict, total, tmp.p, c->stream));
+  CK(cudaStreamSynchronize(c->stream));  // the scan's scratch ends here
+  v.dict = P->dict.as<uint32_t>();
+  v.n_dict_blocks = n_dict;
+  P->info.device_bytes += P->dict.n;
+  return PD_OK;
+}
+
 pdg::ProfilesView pdh::external_view(const pd_profiles* P, const QueryProfiles& Qp) {
   pdg::ProfilesView v = P->view;
   v.q_win_off = Qp.win_off.as<uint32_t>();
   v.q_mv_n = Qp.mv_n.as<uint32_t>();
-  v.q_mv_id = Qp.mv_id.as<uint32_t>();
-  v.q_mv_cnt = Qp.mv_cnt.as<uint16_t>();
-  v.q_mv_post = Qp.mv_post.as<uint32_t>();
-  v.q_mv_plen = Qp.mv_plen.as<uint32_t>();
+  v.q_mv = Qp.mv.as<uint4>();
   v.q_La = Qp.La.as<uint32_t>();
   return v;
 }
@@ -816,16 +820,12 @@ pd_status pdh::query_profiles_impl(pd_ctx* c, const pd_profiles* P, const uint8_
   win_off[n_genes] = (uint32_t)W;
   const size_t G1 = std::max<uint32_t>(n_genes, 1), W1 = std::max<uint64_t>(W, 1);
   Qp->n_genes = n_genes;
-  Buf d_gp, d_mid, d_long, d_long_off, d_long_scratch, dummy;
+  Buf d_gp, d_mid, d_long, d_long_off, d_long_scratch;
   ALLOC(d_gp, sizeof(int64_t) * (n_genes + 1));
   ALLOC(Qp->win_off, sizeof(uint32_t) * (n_genes + 1));
   ALLOC(Qp->La, sizeof(uint32_t) * G1);
   ALLOC(Qp->mv_n, sizeof(uint32_t) * G1);
-  ALLOC(Qp->mv_id, sizeof(uint32_t) * W1);
-  ALLOC(Qp->mv_cnt, sizeof(uint16_t) * W1);
-  ALLOC(Qp->mv_post, sizeof(uint32_t) * W1);
-  ALLOC(Qp->mv_plen, sizeof(uint32_t) * W1);
-  ALLOC(dummy, 16);
+  ALLOC(Qp->mv, sizeof(uint4) * W1);
   CK(cudaMemcpyAsync(d_gp.p, gene_ptr, sizeof(int64_t) * (n_genes + 1), cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(Qp->win_off.p, win_off.data(), sizeof(uint32_t) * (n_genes + 1), cudaMemcpyHostToDevice,
                      c->stream));
@@ -842,29 +842,12 @@ pd_status pdh::query_profiles_impl(pd_ctx* c, const pd_profiles* P, const uint8_
     CK(cudaMemcpyAsync(d_long_off.p, lng_off.data(), sizeof(unsigned long long) * lng_off.size(),
                        cudaMemcpyHostToDevice, c->stream));
   }
-  pdg::MvOut M{};
-  M.mv_id = Qp->mv_id.as<uint32_t>();
-  M.mv_cnt = Qp->mv_cnt.as<uint16_t>();
-  M.mv_n = Qp->mv_n.as<uint32_t>();
-  M.rec = nullptr;
-  M.minhash = nullptr;
-  M.cnt_bits = v.cnt_bits;
-  M.cnt_cap = v.cnt_cap;
-  M.err = c->d_err;
-  M.gene_genome = nullptr;
-  M.genome_code_base = nullptr;
-  M.gene_src = nullptr;
-  M.alpha = P->info.alphabet;
-  M.length_buckets = 0;
-  M.frozen = 1;
+  const pdg::MvOut M{Qp->mv.as<uint4>(), Qp->mv_n.as<uint32_t>(), v.post_ptr, c->d_err, P->info.alphabet};
   if (n_genes) {
     CK(pdg::run_mv_build(L, residues_dev, d_gp.as<int64_t>(), Qp->win_off.as<uint32_t>(), n_genes, k, v.dict, M,
                          d_mid.as<uint32_t>(), (uint32_t)mid.size(), d_long.as<uint32_t>(),
                          (uint32_t)lng.size(), d_long_scratch.as<unsigned long long>(),
                          d_long_off.as<unsigned long long>(), c->stream));
-    CK(pdg::run_mv_post(L, Qp->win_off.as<uint32_t>(), Qp->mv_n.as<uint32_t>(), Qp->mv_id.as<uint32_t>(), n_genes,
-                        v.post_ptr, Qp->mv_post.as<uint32_t>(), Qp->mv_plen.as<uint32_t>(), dummy.as<uint32_t>(),
-                        nullptr, c->stream));
   }
   return check_dev_err(c);  // synchronizes: the host offsets and temporaries end here
 }

@@ -148,6 +148,21 @@ struct Buf {
   }
 };
 
+// Pieces of one allocation (256-byte aligned): reserve them all, allocate the
+// total, then take each piece's address.
+struct Carve {
+  size_t bytes = 0;
+  size_t add(size_t n) {
+    const size_t at = bytes;
+    bytes += (std::max<size_t>(n, 1) + 255) & ~(size_t)255;
+    return at;
+  }
+};
+template <typename T>
+T* piece(const Buf& b, size_t at) {
+  return (T*)((unsigned char*)b.p + at);
+}
+
 #define ALLOC(buf, bytes)                                                                        \
   do {                                                                                           \
     if (!(buf).alloc(c, (bytes))) return fail(c, PD_ERR_OOM, "device allocation of " +           \
@@ -210,8 +225,9 @@ struct pd_profiles {
   pd_ctx* ctx = nullptr;
   pdg::ProfilesView view{};
   pd_profiles_info info{};
-  Buf genome_ptr, La, win_off, mv_n, mv_id, mv_cnt, mv_post, mv_plen, gene_genome, ginfo, dict, post_ptr,
-      post, order;
+  Buf genes;    // per-gene and per-genome arrays
+  Buf windows;  // vectors, postings, posting-list starts and codes
+  Buf dict;     // dictionary, when outside queries need it
   std::vector<int32_t> h_genome_ptr;
 };
 
@@ -245,17 +261,19 @@ struct pd_bbh_set {
 // into its index, while La counts every window.
 struct QueryProfiles {
   uint32_t n_genes = 0;
-  Buf win_off, mv_n, mv_id, mv_cnt, mv_post, mv_plen, La;
+  Buf win_off, mv_n, mv, La;
 };
 
 // ------------------------------------------------------------------ internal entry points (pd_api.cu)
 namespace pdh {
 
 // Profiles of n_genes genes (residues on the device, gene_ptr on the host from
-// 0) against the dictionary and index of P; windows with letters outside the
+// 0) against the dictionary (build_dictionary) and index of P; windows with letters outside the
 // alphabet must have been rejected by the caller.
 pd_status query_profiles_impl(pd_ctx* c, const pd_profiles* P, const uint8_t* residues_dev, const int64_t* gene_ptr,
                               uint32_t n_genes, QueryProfiles* out);
+// Gives P the dictionary that outside queries look their k-mers up in.
+pd_status build_dictionary(pd_ctx* c, pd_profiles* P);
 // P's view with the external query arrays of Qp.
 pdg::ProfilesView external_view(const pd_profiles* P, const QueryProfiles& Qp);
 // run_hits on an explicit view (external queries).

@@ -5,15 +5,30 @@
 //
 //   gene g (global id, 0..G-1) has La[g] = max(0, |g|-k+1) k-mer windows.
 //   win_off[G+1]   uint32  exclusive prefix of La: window range of each gene.
-//   mv_n[G]        uint32  distinct k-mers of the gene (E_g <= La[g]).
-//   mv_id[W]       uint32  dense k-mer id, gene g at win_off[g] .. +mv_n[g]
-//                          (the multiplicity vector of Algorithm 1, stored in
-//                          the gene's window range: "padded CSR"; the entries
-//                          of one gene are unordered).
-//   mv_cnt[W]      uint16  multiplicity of that k-mer in the gene.
-//   mv_post[W],    uint32  posting range of that k-mer (copied from post_ptr so
-//   mv_plen[W]             a query reads its list bounds with its own vector).
+//   post_ptr[D+1]  uint32  inverted index: postings of id w (k-mers numbered by
+//   post[E]        uint32  ascending code) are post[post_ptr[w] .. post_ptr[w+1]),
+//                          ascending by gene, each packed as (gene << cnt_bits)
+//                          | min(count, cnt_cap) with cnt_bits = 32 -
+//                          bits(G).  A count equal to cnt_cap is saturated;
+//                          the exact value is in the gene's vector.
+//   code_lo[D]     uint32  code of each id (with code_hi[D], its bits above 32,
+//                          when the codes need more).
+//   mv_n[G]        uint32  k-mers of the gene that another gene has too.
+//   mv[W]          uint4   the gene's multiplicity vector (Algorithm 1) over
+//                          those k-mers, at win_off[g] .. +mv_n[g] (the entries
+//                          of one gene are unordered).  x: start of the k-mer's
+//                          posting list; y: its multiplicity in the gene; z: the
+//                          list's length, with the top bit set if it holds
+//                          another gene of the same genome; w: offset in the
+//                          list of the first gene past the gene's genome.  A
+//                          k-mer of one gene only is left out, since no other
+//                          gene can share it (unless its count is saturated).
 //   gene_genome[G] uint16  genome of each gene; ginfo[G] = La | genome << 16.
+//   order[G]       uint32  all-pairs query order: genes grouped by a hash of
+//                          their min-hash (minimum of a hash of their k-mers),
+//                          so likely homologs run together.
+// Outside queries (genes profiled against a dataset they are not part of) also
+// need
 //   dict[8 * ceil(20^k / 224)] uint32  the dictionary, one bit per possible
 //                          k-mer code in rank blocks of 32 bytes (one DRAM
 //                          sector): block b covers codes 224b .. 224b+223,
@@ -23,15 +38,6 @@
 //                          present code is word 0 plus the set bits before it
 //                          in its block (ascending in code order), read with
 //                          one sector per lookup.
-//   post_ptr[D+1]  uint32  inverted index: postings of id w are
-//   post[E]        uint32  post[post_ptr[w] .. post_ptr[w+1]), ascending by
-//                          gene, each packed as (gene << cnt_bits) | min(count,
-//                          cnt_cap) with cnt_bits = 32 - bits(G-1).  A count
-//                          equal to cnt_cap is saturated; the exact value is
-//                          in the gene's multiplicity vector.
-//   order[G]       uint32  all-pairs query order: genes grouped by the top bits
-//                          of their min-hash (minimum of a hash of their k-mer
-//                          ids), so likely homologs run together.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -79,7 +85,12 @@ __device__ __forceinline__ uint32_t dict_rank(const uint32_t* __restrict__ dict,
   }
   return r;
 }
-constexpr int kAlphabetSize = 20;
+
+// Code of id i.
+__device__ __forceinline__ unsigned long long code_at(const uint32_t* __restrict__ lo, const uint8_t* __restrict__ hi,
+                                                      uint64_t i) {
+  return (unsigned long long)lo[i] | (hi ? (unsigned long long)hi[i] << 32 : 0ull);
+}
 
 // ---------------------------------------------------------------- errors
 // Device error block: kernels record the first error code and a detail value
@@ -184,17 +195,16 @@ struct ProfilesView {
   uint32_t cnt_bits, cnt_cap, max_posting;
   uint64_t n_join;              // postings the all-against-all walk visits (sum over entries of list length)
   const uint32_t* win_off;      // [G+1] window range of each gene
-  const uint32_t* mv_n;         // [G]   distinct k-mers of each gene
-  const uint32_t* mv_id;        // [W]   multiplicity vectors: dense ids
-  const uint16_t* mv_cnt;       // [W]   multiplicities
-  const uint32_t* mv_post;      // [W]   posting-list start of each entry's id
-  const uint32_t* mv_plen;      // [W]   posting-list length of each entry's id
+  const uint32_t* mv_n;         // [G]   entries of each gene's vector
+  const uint4* mv;              // [W]   multiplicity vectors
   const uint32_t* La;           // [G]   windows per gene
   const uint16_t* gene_genome;  // [G]   genome of each gene
   const uint32_t* ginfo;        // [G]   La | genome << 16
   const int32_t* genome_ptr;    // [n+1] device copy
-  const uint32_t* dict;         // [8 * n_dict_blocks] dictionary rank blocks
+  const uint32_t* dict;         // [8 * n_dict_blocks] dictionary rank blocks (null unless built)
   uint64_t n_dict_blocks;
+  const uint32_t* code_lo;      // [D]   code of each id ...
+  const uint8_t* code_hi;       // [D]   ... its bits above 32 (null if none has any)
   const uint32_t* post_ptr;     // [D+1]
   const uint32_t* post;         // [E]   packed postings
   const uint32_t* order;        // [G]   all-pairs query order (min-hash buckets)
@@ -204,10 +214,7 @@ struct ProfilesView {
   // query's own numbering) while targets stay this dataset's genes.
   const uint32_t* q_win_off;
   const uint32_t* q_mv_n;
-  const uint32_t* q_mv_id;
-  const uint16_t* q_mv_cnt;
-  const uint32_t* q_mv_post;
-  const uint32_t* q_mv_plen;
+  const uint4* q_mv;
   const uint32_t* q_La;
 };
 
@@ -321,43 +328,93 @@ cudaError_t scan_u32(Launcher* L, const uint32_t* in, uint64_t n, uint32_t* out_
                      cudaStream_t s);
 cudaError_t scan_u32_to_u64(Launcher* L, const uint32_t* in, uint64_t n, unsigned long long* out_excl_np1,
                             void* temp, cudaStream_t s);
+// The same with the prefix in 32 bits and the 64-bit sum of all at *total.
+cudaError_t scan_u32_total(Launcher* L, const uint32_t* in, uint64_t n, uint32_t* out_excl_np1,
+                           unsigned long long* total, void* temp, cudaStream_t s);
 
-// profiles (k_profiles.cu)
+// profiles and index of a dataset (k_index.cu)
 // Gene offsets -> window counts on the device.  Checks every gene (offsets
 // from 0, non-decreasing, ending at n_res unless check_end is 0; at most
 // PD_MAX_WINDOWS windows), recording PD_ERR_ARG / PD_ERR_GENE_TOO_LONG with
-// the gene as detail (such a gene gets La 0); lists the genes whose vector
-// table exceeds the small (mid) and the large (long) shared-memory build, with
-// a scratch offset for each long gene.  counts: [n_mid, n_long] (uint32) and
-// long_total (uint64, after them, 8-byte aligned).
+// the gene as detail (such a gene gets La 0).
 cudaError_t run_gene_windows(Launcher* L, const int64_t* gene_ptr, uint32_t n_genes, uint64_t n_res, int check_end,
-                             int k, uint32_t* La, uint32_t* mid_list, uint32_t* long_list,
-                             unsigned long long* long_off, uint32_t* counts, unsigned long long* long_total,
-                             DevErr* err, cudaStream_t s);
-// u64 -> u32 copy of n values.
-cudaError_t run_narrow_u64(Launcher* L, const unsigned long long* in, uint64_t n, uint32_t* out, cudaStream_t s);
-// n_res bounds the residues of every gene read through gene_ptr (genes read
-// through gene_src are trusted).
-cudaError_t run_encode_mark(Launcher* L, const uint8_t* res, const int64_t* gene_ptr, uint32_t n_genes, int k,
-                            uint32_t* dict, const uint16_t* gene_genome,
-                            const unsigned long long* genome_code_base, const int64_t* gene_src, int alpha,
-                            uint64_t n_res, DevErr* err, cudaStream_t s);
-// Outputs of the multiplicity-vector build.
-struct MvOut {
-  uint32_t* mv_id;
-  uint16_t* mv_cnt;
-  uint32_t* mv_n;
-  unsigned long long* rec;  // [W] (id << 32) | packed posting; all-ones in unused slots
-  uint32_t* minhash;
-  uint32_t cnt_bits, cnt_cap;
-  DevErr* err;
-  const uint16_t* gene_genome;                 // genome of each gene
+                             int k, uint32_t* La, DevErr* err, cudaStream_t s);
+// PD_ERR_ALPHABET (detail: the position) for a byte outside the alphabet: all
+// n_res bytes, or with gene_src the genes' bytes.
+cudaError_t run_check_letters(Launcher* L, const uint8_t* res, uint64_t n_res, const int64_t* gene_ptr,
+                              const int64_t* gene_src, uint32_t n_genes, int alpha, DevErr* err, cudaStream_t s);
+// Windows of a dataset in gene order.
+struct WindowSource {
+  const uint8_t* res;
+  const int64_t* gene_ptr;
+  const int64_t* gene_src;     // per gene: first residue, or null (gene_ptr[g])
+  const uint32_t* win_off;
+  const uint32_t* tile_gene;   // gene of the first window of each sort tile
+  const uint16_t* gene_genome;
   const unsigned long long* genome_code_base;  // per genome: segment * 20^k, or null (one segment)
-  const int64_t* gene_src;                     // per gene: first residue, or null (gene_ptr[g])
-  int alpha;                                   // alphabet size: 20 or 4
-  int length_buckets;                          // query order: length buckets first (1) or min-hash only (0)
-  int frozen;                                  // 1: the dictionary is another dataset's; windows
-                                               // whose code it lacks are left out of the vector
+  int k, alpha;
+  uint64_t n_windows;
+};
+// A sort record: code << gene_bits | gene.  Codes that do not fit beside the
+// gene are sorted in slices of equal high bits (code >> code_bits == slice).
+constexpr uint32_t kMaxSortPasses = 4;
+struct SortKey {
+  uint32_t gene_bits, total_bits, code_bits, n_slices;  // total_bits: of a whole code
+  uint32_t passes, width, last_mask;  // digits: width bits each, the last one's mask
+  unsigned long long slice;
+};
+SortKey sort_key(uint64_t n_codes, uint32_t gene_bits);
+// Byte offsets into the zeroed scratch of one slice.
+struct SortScratch {
+  size_t tickets, hist, dedupe, pass[kMaxSortPasses], bytes;
+  bool wide;
+};
+SortScratch sort_scratch(const SortKey& K, uint64_t n);
+uint32_t sort_tiles(uint64_t n);    // tiles of the sort (tile_gene holds one more entry)
+uint32_t dedupe_tiles(uint64_t n);  // tiles of the dedupe pass (tile_e and tile_id hold one more entry)
+constexpr size_t kDigitStarts = (size_t)kMaxSortPasses * 512;
+cudaError_t run_tile_genes(Launcher* L, const uint32_t* win_off, uint32_t n_genes, uint64_t n_windows,
+                           uint32_t* tile_gene, cudaStream_t s);
+// Digit starts of every pass, the records of the slice (*total) and, if not
+// null, the min-hashes (set to all ones before).
+cudaError_t run_code_hist(Launcher* L, const WindowSource& S, const SortKey& K, uint8_t* scratch, const SortScratch& X,
+                          unsigned long long* digit_start, unsigned long long* total, uint32_t* minhash,
+                          cudaStream_t s);
+// The slice's n records sorted by code, equal codes by gene: in a after an odd
+// number of passes, else in b.
+cudaError_t run_sort(Launcher* L, const WindowSource& S, const SortKey& K, uint64_t n, uint8_t* scratch,
+                     const SortScratch& X, const unsigned long long* digit_start, unsigned long long* a,
+                     unsigned long long* b, unsigned long long** sorted, DevErr* err, cudaStream_t s);
+// Sorted records -> post, post_ptr, code_lo / code_hi and the postings and ids
+// before each tile; totals: [4] words, the postings and ids so far first.
+cudaError_t run_dedupe(Launcher* L, const unsigned long long* rec, uint64_t n, const SortKey& K, uint8_t* scratch,
+                       const SortScratch& X, uint32_t cnt_bits, uint32_t cnt_cap, unsigned long long* totals,
+                       uint32_t* post, uint32_t* post_ptr, uint32_t* code_lo, uint8_t* code_hi, uint32_t* tile_e,
+                       uint32_t* tile_id, DevErr* err, cudaStream_t s);
+// Vector entries of the slice's postings; cursor: the next free place of each
+// gene's vector (its first window before the first slice).  The longest list
+// and the sum of squared list lengths (the postings an all-against-all walk
+// visits) are added to *max_list and *join.
+cudaError_t run_lists(Launcher* L, const unsigned long long* rec, uint64_t n, const SortKey& K, const uint32_t* tile_e,
+                      const uint32_t* tile_id, const uint32_t* post, const uint32_t* post_ptr, const uint32_t* code_lo,
+                      const uint8_t* code_hi, uint32_t cnt_bits, uint32_t cnt_cap, const int32_t* genome_ptr,
+                      uint32_t n_genomes, uint32_t n_genes, uint32_t* cursor, uint4* mv, uint32_t* max_list,
+                      unsigned long long* join, cudaStream_t s);
+cudaError_t run_vector_lengths(Launcher* L, const uint32_t* cursor, const uint32_t* win_off, uint32_t n_genes,
+                               uint32_t* mv_n, cudaStream_t s);
+
+// profiles (k_profiles.cu)
+// The bits of all codes of an index in a zeroed dictionary.
+cudaError_t run_dict_mark(Launcher* L, const uint32_t* code_lo, const uint8_t* code_hi, uint64_t n, uint32_t* dict,
+                          cudaStream_t s);
+// Vectors of genes from outside the dataset that dict and post_ptr belong to;
+// k-mers it lacks are left out.
+struct MvOut {
+  uint4* mv;
+  uint32_t* mv_n;
+  const uint32_t* post_ptr;
+  DevErr* err;
+  int alpha;  // alphabet size: 20 or 4
 };
 // Table slots used for a gene with La windows (genes above 16384 slots use
 // global scratch of that many 64-bit slots, listed in long_genes).
@@ -366,31 +423,20 @@ cudaError_t run_mv_build(Launcher* L, const uint8_t* res, const int64_t* gene_pt
                          uint32_t n_genes, int k, const uint32_t* dict, const MvOut& M, const uint32_t* mid_genes, uint32_t n_mid, const uint32_t* long_genes,
                          uint32_t n_long, unsigned long long* long_scratch, const unsigned long long* long_scratch_off,
                          cudaStream_t s);
-// Stable LSD radix sort of the n index records in `a` (ping-pong with `b`) by
-// the low key_bits bits of their high word, then postings and id offsets:
-// post[0..E) and post_ptr[0..n_ids] (post_ptr[n_ids] = E).  `counts` holds
-// radix_counts_words(n) words; scan_tmp serves a scan of that many.
-size_t radix_counts_words(uint64_t n);
-cudaError_t run_index_sort(Launcher* L, unsigned long long* a, unsigned long long* b, uint64_t n, uint32_t key_bits,
-                           uint32_t* counts, void* scan_tmp, uint64_t n_ids, uint32_t* post, uint32_t* post_ptr,
-                           cudaStream_t s);
-// Posting range of every multiplicity-vector entry; also the longest list and
-// (join not null) the sum of the entries' list lengths.
-cudaError_t run_mv_post(Launcher* L, const uint32_t* win_off, const uint32_t* mv_n, const uint32_t* mv_id,
-                        uint32_t n_genes, const uint32_t* post_ptr, uint32_t* mv_post, uint32_t* mv_plen,
-                        uint32_t* max_posting, unsigned long long* join, cudaStream_t s);
-// count must hold 2 * 2^(32-shift) + 1 words (counts, then their prefix sum).
-cudaError_t run_order(Launcher* L, const uint32_t* minhash, uint32_t n_genes, uint32_t shift, uint32_t* count,
-                      uint32_t* order, void* scan_tmp, cudaStream_t s);
+// count must hold 2 * kOrderBuckets + 1 words (zeroed counts, then their prefix sum).
+constexpr uint32_t kOrderBuckets = 65536;
+cudaError_t run_order(Launcher* L, const uint32_t* minhash, const uint32_t* La, uint32_t n_genes, int length_buckets,
+                      uint32_t* count, uint32_t* order, void* scan_tmp, cudaStream_t s);
 cudaError_t run_gene_info(Launcher* L, const int32_t* genome_ptr, uint32_t n_genomes, const uint32_t* La,
                           uint16_t* gene_genome, uint32_t* ginfo, cudaStream_t s);
-cudaError_t run_select_codes(Launcher* L, const uint32_t* dict, uint64_t n_blocks, unsigned long long* code_of_id,
-                             cudaStream_t s);
-// pad_off: n_genes+1 offsets of power-of-two padded per-gene scratch regions in pad.
+cudaError_t run_export_codes(Launcher* L, const ProfilesView& P, unsigned long long* codes, cudaStream_t s);
+// Distinct k-mers per gene (n zeroed before).
+cudaError_t run_export_mv_count(Launcher* L, const ProfilesView& P, uint32_t* n, cudaStream_t s);
+// pad_off: n_genes+1 offsets of power-of-two padded per-gene scratch regions in
+// pad (all ones before); fill: zeroed, one word per gene.
 cudaError_t run_export_mv(Launcher* L, const ProfilesView& P, const unsigned long long* mv_ptr,
-                          const unsigned long long* pad_off, unsigned long long* pad,
-                          const unsigned long long* code_of_id, unsigned long long* codes, uint32_t* counts,
-                          cudaStream_t s);
+                          const unsigned long long* pad_off, uint32_t* fill, unsigned long long* pad,
+                          unsigned long long* codes, uint32_t* counts, cudaStream_t s);
 cudaError_t run_export_index(Launcher* L, const ProfilesView& P, int32_t* genes, uint32_t* counts,
                              cudaStream_t s);
 

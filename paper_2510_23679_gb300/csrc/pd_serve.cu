@@ -264,7 +264,9 @@ pd_status build_level_on(pd_ctx* c, int k, const uint8_t* res, const std::vector
                                      g1 - g0, k, nullptr, &P);
   if (st != PD_OK) return st;
   L->P.reset(P);
-  return PD_OK;
+  st = build_dictionary(c, P);
+  if (st != PD_OK) L->P.reset();
+  return st;
 }
 
 pd_status build_level(pd_index* I, uint32_t g0, uint32_t g1, Level* L) {
