@@ -115,9 +115,10 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
   Carve cv_mem{scratch};
   const uint32_t rows = std::max<uint32_t>(nA, 1);
   const uint32_t targets = std::max<uint32_t>(ta1 - ta0, 2);
-  unsigned long long* counters = cv_mem.take<unsigned long long>(4);
+  unsigned long long* counters = cv_mem.take<unsigned long long>(5);
   unsigned long long* row_off = cv_mem.take<unsigned long long>(rows);
   uint32_t* row_len = cv_mem.take<uint32_t>(rows);
+  uint32_t* def0 = cv_mem.take<uint32_t>(rows);
   uint32_t* def1 = cv_mem.take<uint32_t>(rows);
   uint32_t* def2 = cv_mem.take<uint32_t>(rows);
   uint32_t* out_b = cv_mem.take<uint32_t>(PD_NOALLOC_MAX_HITS);
@@ -130,7 +131,7 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
   B.vals = cv_mem.take<uint32_t>((size_t)B.cap * kGlobalTierBlocks);
   B.used = cv_mem.take<uint32_t>((size_t)B.cap * kGlobalTierBlocks);
   B.out = cv_mem.take<unsigned long long>((size_t)B.out_cap * kGlobalTierBlocks);
-  if (!counters || !row_off || !row_len || !def1 || !def2 || !out_b || !out_s || !scan_tmp || !B.keys || !B.vals ||
+  if (!counters || !row_off || !row_len || !def0 || !def1 || !def2 || !out_b || !out_s || !scan_tmp || !B.keys || !B.vals ||
       !B.used || !B.out)
     return ctx_fail(ctx, PD_ERR_INTERNAL, "pd_best_hits_noalloc: scratch layout exceeds the array");
 
@@ -153,12 +154,15 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
   O.walked = counters + 1;
   O.n_def1 = (uint32_t*)(counters + 2);
   O.n_def2 = (uint32_t*)(counters + 3);
+  O.n_def0 = (uint32_t*)(counters + 4);
+  O.ticket = O.n_def0 + 1;
+  O.def0 = def0;
   O.row_off = row_off;
   O.row_len = row_len;
   O.def1 = def1;
   O.def2 = def2;
   unsigned long long h[4] = {0, 0, 0, 0};
-  if ((e = cudaMemsetAsync(counters, 0, 4 * sizeof(unsigned long long), st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
+  if ((e = cudaMemsetAsync(counters, 0, 5 * sizeof(unsigned long long), st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
   if ((e = cudaMemsetAsync(row_len, 0, sizeof(uint32_t) * rows, st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
   if (nA) {
     if ((e = run_summin_tiers(L, *P, Q, O, cv.d_err, false, st)) != cudaSuccess)

@@ -235,6 +235,94 @@ __device__ __forceinline__ void sym_update(const QuerySet& Q, unsigned long long
   }
 }
 
+// Length field of a vector entry's z (the top bit marks lists holding another
+// gene of the same genome).
+constexpr uint32_t kListLength = 0x7FFFFFFFu;
+
+// A query gene, its output row and its targets.
+struct Query {
+  uint32_t a, row;
+  uint32_t own0, own1;  // all-pairs forms: genes that are no targets (its own genome)
+  uint32_t tend;        // ... and those from here on
+  uint32_t t0, t1;      // other forms: the target genes
+  uint32_t col, self;   // column of the reverse maxima; a gene that is no target
+  const uint32_t* mask; // target genomes (null: every other)
+};
+
+__device__ __forceinline__ bool wanted(const Query& q, uint32_t genome) {
+  return !q.mask || ((q.mask[genome >> 5] >> (genome & 31u)) & 1u);
+}
+
+// False if the query is another shard's.
+__device__ __forceinline__ bool load_query(uint32_t qi, const ProfilesView& P, const QuerySet& Q, Query* q) {
+  q->own0 = q->own1 = q->t0 = q->t1 = q->col = 0;
+  q->tend = q->self = kEmpty;
+  q->mask = nullptr;
+  if (Q.all_pairs) {
+    const uint32_t a = Q.order ? Q.order[qi] : Q.q0 + qi;
+    if (Q.n_shards && a % Q.n_shards != Q.shard) return false;
+    q->a = q->row = a;
+    if (Q.q_genome) {  // external query: no own genome among the targets
+      const uint32_t x = Q.q_genome[a];
+      q->own0 = q->own1 = kEmpty;
+      if (Q.tgt_end) q->tend = Q.tgt_end[x];
+      q->col = x;
+    } else {
+      const uint32_t gg = P.gene_genome[a];
+      q->own0 = (uint32_t)P.genome_ptr[gg];
+      q->own1 = (uint32_t)P.genome_ptr[gg + 1];
+      if (Q.tgt_end) q->tend = Q.tgt_end[gg];
+      if (Q.tgt_mask) q->mask = Q.tgt_mask + (size_t)gg * Q.mask_words;
+      q->col = gg - Q.col_genome0;
+    }
+    return true;
+  }
+  q->row = qi;
+  if (Q.q_gene) {
+    q->a = Q.q_gene[qi];
+    q->t0 = Q.q_t0[qi];
+    q->t1 = Q.q_t1[qi];
+  } else if (Q.paralog) {
+    q->a = q->self = Q.q0 + qi;
+    const uint32_t gg = P.gene_genome[q->a];
+    q->t0 = (uint32_t)P.genome_ptr[gg];
+    q->t1 = (uint32_t)P.genome_ptr[gg + 1];
+  } else if (qi < Q.nA) {
+    q->a = Q.qa0 + qi;
+    q->t0 = Q.ta0;
+    q->t1 = Q.ta1;
+  } else {
+    q->a = Q.qb0 + (qi - Q.nA);
+    q->t0 = Q.tb0;
+    q->t1 = Q.tb1;
+  }
+  return true;
+}
+
+// The part [lo, lo + len) of a vector entry's posting list that holds the
+// query's targets.
+__device__ __forceinline__ void narrow_list(const ProfilesView& P, const QuerySet& Q, const Query& q, const uint4& v,
+                                            uint32_t* lo, uint32_t* len) {
+  *lo = v.x;
+  *len = v.z & kListLength;
+  if (Q.symbest) {  // the genomes after the query's own
+    *lo += v.w;
+    *len -= v.w;
+  } else if (Q.paralog) {  // its own genome: the entry says whether another gene of it is there, and where it ends
+    const uint32_t end = v.x + v.w;
+    if (v.z == *len) {
+      *len = 0;
+    } else {
+      *lo = lower_bound_post(P.post, v.x, end, (unsigned long long)q.t0 << P.cnt_bits);
+      *len = end - *lo;
+    }
+  } else if (!Q.all_pairs) {
+    const uint32_t end = v.x + *len;
+    *lo = lower_bound_post(P.post, v.x, end, (unsigned long long)q.t0 << P.cnt_bits);
+    *len = lower_bound_post(P.post, *lo, end, (unsigned long long)q.t1 << P.cnt_bits) - *lo;
+  }
+}
+
 template <int kThreads>
 struct Chunk {
   static constexpr uint32_t kSize = 2 * kThreads;  // query k-mers staged per round
@@ -256,9 +344,16 @@ constexpr uint32_t kWarpWalkMinAvg = 16;
 // taken: below a few L2 sizes the merge-path walk's runs of postings keep
 // hitting the sectors they have already brought in.
 constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
-// Length field of a vector entry's z (the top bit marks lists holding another
-// gene of the same genome).
-constexpr uint32_t kListLength = 0x7FFFFFFFu;
+// The warp tier pays when there are queries for several per resident warp
+// (3648 of them: with one genome pair's 3000 queries the launch takes 0.17
+// against 0.11 ms, with 4800 0.12 against 0.09), and either a query meets few
+// targets (lists of fewer than 8 postings on average, or one target range:
+// 39k queries of 23 genomes 0.33 against 0.50 ms, paralogs of 180k genes 1.0
+// against 1.8) or its lists are long and the index far larger than L2 (200
+// genomes x 4000 genes: 26 against 27 ms).  Between them (50 x 3000) a query
+// meets several hundred chance targets, more of which overflow the warp's
+// table, and the block tier is the faster one (3.2 against 3.4 ms).
+constexpr uint32_t kWarpTierMinQueries = 16384, kWarpTierMaxAvg = 8;
 // Target genomes from which a query's Best Hits are ranked through per-genome
 // positions rather than pairwise.
 constexpr uint32_t kRankByGenomeMin = 64;
@@ -288,55 +383,11 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
   uint16_t* c_ent = c_cnt + Chunk<kThreads>::kSize;  // chunk entry of each staged k-mer
   unsigned long long* out = tb.out;
   const uint32_t mask = tb.cap - 1u;
-  // ---- query gene, its output row and its targets
-  uint32_t a, row, own0 = 0, own1 = 0, tend = 0xFFFFFFFFu, col = 0, self = kEmpty;
-  unsigned long long key_lo = 0, key_hi = 0;
-  if (Q.all_pairs) {
-    a = Q.order ? Q.order[qi] : Q.q0 + qi;
-    if (Q.n_shards && a % Q.n_shards != Q.shard) return;  // another shard's query (uniform over the block)
-    row = a;
-    if (Q.q_genome) {  // external query: no own genome among the targets
-      const uint32_t x = Q.q_genome[a];
-      own0 = own1 = kEmpty;
-      if (Q.tgt_end) tend = Q.tgt_end[x];
-      col = x;
-    } else {
-      const uint32_t gg = P.gene_genome[a];
-      own0 = (uint32_t)P.genome_ptr[gg];
-      own1 = (uint32_t)P.genome_ptr[gg + 1];
-      if (Q.tgt_end) tend = Q.tgt_end[gg];
-      col = gg - Q.col_genome0;
-    }
-  } else {
-    uint32_t tlo, thi;
-    if (Q.q_gene) {
-      a = Q.q_gene[qi];
-      tlo = Q.q_t0[qi];
-      thi = Q.q_t1[qi];
-    } else if (Q.paralog) {
-      a = Q.q0 + qi;
-      const uint32_t gg = P.gene_genome[a];
-      tlo = (uint32_t)P.genome_ptr[gg];
-      thi = (uint32_t)P.genome_ptr[gg + 1];
-      self = a;
-    } else if (qi < Q.nA) {
-      a = Q.qa0 + qi;
-      tlo = Q.ta0;
-      thi = Q.ta1;
-    } else {
-      a = Q.qb0 + (qi - Q.nA);
-      tlo = Q.tb0;
-      thi = Q.tb1;
-    }
-    row = qi;
-    key_lo = (unsigned long long)tlo << P.cnt_bits;
-    key_hi = (unsigned long long)thi << P.cnt_bits;
-  }
+  Query q;
+  if (!load_query(qi, P, Q, &q)) return;  // another shard's query (uniform over the block)
+  const uint32_t a = q.a, row = q.row, own0 = q.own0, own1 = q.own1, tend = q.tend, col = q.col, self = q.self;
   // one target range that fits the table: direct slots instead of hashing
-  if (!Q.all_pairs) {
-    const uint32_t tlo = (uint32_t)(key_lo >> P.cnt_bits), thi = (uint32_t)(key_hi >> P.cnt_bits);
-    if (thi > tlo && thi - tlo <= tb.cap) acc.dense_lo = tlo;
-  }
+  if (!Q.all_pairs && q.t1 > q.t0 && q.t1 - q.t0 <= tb.cap) acc.dense_lo = q.t0;
   // the query's own vector (its dataset's, or the external query arrays)
   const bool ext = P.q_win_off != nullptr;
   const uint4* __restrict__ q_mv = ext ? P.q_mv : P.mv;
@@ -350,18 +401,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
     sh->overflow = (kPacked && La_a >= cnt_mask) ? 1u : 0u;
   }
   __syncthreads();
-  // The part [lo, lo + len) of a vector entry's posting list that holds the
-  // query's targets.
-  auto narrow = [&](const uint4& v, uint32_t& lo, uint32_t& len) {
-    if (!Q.all_pairs) {
-      const uint32_t end = lo + len;
-      lo = lower_bound_post(P.post, lo, end, key_lo);
-      len = lower_bound_post(P.post, lo, end, key_hi) - lo;
-    } else if (Q.symbest) {  // the genomes after the query's own
-      lo += v.w;
-      len -= v.w;
-    }
-  };
+  auto narrow = [&](const uint4& v, uint32_t& lo, uint32_t& len) { narrow_list(P, Q, q, v, &lo, &len); };
   unsigned long long walked = 0;
   const uint32_t lane = tid & 31u, warp = tid >> 5;
   constexpr uint32_t kWarps = kThreads / 32;
@@ -391,9 +431,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         cnt_loc[r] = 0;
         if (e < n_in) {
           const uint4 v = q_mv[m0 + c0 + e];
-          lo = v.x;
           cnt_loc[r] = v.y;
-          len = v.z & kListLength;
           narrow(v, lo, len);
         }
         lo_loc[r] = lo;
@@ -468,8 +506,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         uint32_t len = 0;
         if (e < n_in) {
           const uint4 v = q_mv[m0 + c0 + e];
-          uint32_t lo = v.x;
-          len = v.z & kListLength;
+          uint32_t lo;
           narrow(v, lo, len);
           c_post[e] = lo;
           c_cnt[e] = (uint16_t)v.y;
@@ -578,6 +615,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         acc.get(tb.used[u], &b, &s);
         if ((Q.all_pairs && ((b >= own0 && b < own1) || b >= tend)) || b == self) continue;  // not a target
         const uint32_t gi = P.ginfo[b];
+        if (!wanted(q, gi >> 16)) continue;
         if (kFilter && !filter_pass(Q, P.k, La_a, gi & 0xFFFFu, acc.vpa[tb.used[u]], acc.vpb[tb.used[u]])) continue;
         const uint32_t den = La_a + (gi & 0xFFFFu) - s;
         best_update(&best[Q.all_pairs ? (gi >> 16) : 0u], s, den);
@@ -591,7 +629,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         acc.get(h, &b, &s);
         const uint32_t gi = P.ginfo[b];
         const unsigned long long bv = best[Q.all_pairs ? (gi >> 16) : 0u];
-        if (!(Q.all_pairs && ((b >= own0 && b < own1) || b >= tend)) && b != self &&
+        if (!(Q.all_pairs && ((b >= own0 && b < own1) || b >= tend)) && b != self && wanted(q, gi >> 16) &&
             (!kFilter || filter_pass(Q, P.k, La_a, gi & 0xFFFFu, acc.vpa[h], acc.vpb[h])) &&
             ratio_equal(s, La_a + (gi & 0xFFFFu) - s, (uint32_t)(bv >> 32), (uint32_t)bv)) {
           // s <= La <= 65535 and the genome < 65536: (b, genome, s) in one word
@@ -677,6 +715,296 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
     }
   }
   __syncthreads();
+}
+
+// ---- warp tier: one warp per query
+// Most queries meet a few hundred targets, so a whole block spends more on its
+// block-wide scans, table scans and barriers than on the postings.  Here one
+// warp owns a query and a small table, and nothing waits for another warp:
+//   * entries of the query's vector are staged 32 at a time in a ring;
+//     groups of kGroup lanes take lists in turn, four postings a lane (one
+//     16-byte load) at a step, a step's loads in flight while the postings of
+//     the step before are accumulated;
+//   * a posting looks at the two slots of its home bucket and adds to the one
+//     that holds its gene; the others (first postings of a gene, the few whose
+//     bucket is full) are put aside, and handled 32 together: probing, claiming
+//     a slot and listing it;
+//   * the Best Hit passes run over the listed slots only: the maxima of each
+//     target genome, then the hits at the maximum counted per genome, whose
+//     running sum is each genome's first position in the row.
+// A query that lists more than kWUsed slots, or whose vector is longer than
+// kWEntries, goes to the next tier.
+constexpr uint32_t kWSlots = 1024, kWUsed = 832, kWEntries = 2048, kWPend = 160, kWRing = 64;
+constexpr int kWThreads = 128, kWWarps = kWThreads / 32;
+// Target genomes up to which the warp tier runs (10 bytes each per warp).
+constexpr uint32_t kWMaxGenomes = 512;
+constexpr uint16_t kWHit = 0x8000u;  // mark of a listed slot that is a Best Hit
+static_assert(kWSlots <= 0x8000u, "slot and mark share 16 bits");
+static_assert(kWEntries <= 0x10000u && kWUsed < 0x10000u, "16-bit entries and counts");
+__host__ __device__ constexpr size_t warp_tier_bytes(uint32_t n_best) {
+  return ((size_t)kWSlots * 4 + kWRing * 12 + (size_t)n_best * 8 + (size_t)kWPend * 4 + 8 + (size_t)kWUsed * 2 +
+          ((size_t)n_best + 1) * 2 + 15) & ~(size_t)15;
+}
+
+template <int kGroup>
+__global__ void __launch_bounds__(kWThreads, 6)
+    k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  unsigned char* mine = smem + (size_t)warp * warp_tier_bytes(n_best);
+  uint32_t* tab = (uint32_t*)mine;
+  unsigned long long* best = (unsigned long long*)(tab + kWSlots);
+  uint2* ring = (uint2*)(best + n_best);            // first and past-the-end posting
+  uint32_t* ring_ce = (uint32_t*)(ring + kWRing);   // count | entry << 16
+  uint32_t* n_pend = ring_ce + kWRing;
+  uint32_t* pend = n_pend + 2;
+  uint16_t* used = (uint16_t*)(pend + kWPend);
+  uint16_t* hcnt = used + kWUsed;
+  for (uint32_t h = lane; h < kWSlots; h += 32) tab[h] = kEmpty;
+  if (lane == 0) *n_pend = 0;
+  __syncwarp();
+  constexpr uint32_t kAll = 0xFFFFFFFFu;
+  const uint32_t cmask = (1u << P.cnt_bits) - 1u, hi = ~cmask, cap = P.cnt_cap;
+  const uint32_t below = (1u << lane) - 1u;
+  constexpr uint32_t kFirst = kGroup == 1 ? 0xFFFFFFFFu : kGroup == 2 ? 0x55555555u : 0x11111111u;  // a lane of each group
+  const uint32_t groups_below = kFirst & ((1u << (lane / kGroup * kGroup)) - 1u), part = (lane % kGroup) * 4u;
+  const bool ext = P.q_win_off != nullptr;
+  const uint4* __restrict__ q_mv = ext ? P.q_mv : P.mv;
+  const uint32_t* __restrict__ post = P.post;
+  static_assert(kWSlots == 2u << 9, "512 buckets of two slots");
+  auto home = [](uint32_t key) { return ((key * 0x9E3779B1u) >> 22) & ~1u; };
+  unsigned long long walked = 0;
+  for (;;) {
+    uint32_t qi = 0;
+    if (lane == 0) qi = atomicAdd(ticket, 1u);
+    qi = __shfl_sync(kAll, qi, 0);
+    if (qi >= Q.n_queries) break;
+    Query q;
+    if (!load_query(qi, P, Q, &q)) continue;
+    const uint32_t m0 = (ext ? P.q_win_off : P.win_off)[q.a], E = (ext ? P.q_mv_n : P.mv_n)[q.a];
+    const uint32_t La_a = (ext ? P.q_La : P.La)[q.a];
+    // a packed slot holds s <= La_a
+    bool overflow = E > kWEntries || La_a >= cmask;
+    uint32_t n_used = 0;
+    // Adds the postings put aside (words gene | min of the counts) in [from, to).
+    auto flush = [&](uint32_t from, uint32_t to) {
+      uint32_t claimed = kEmpty;
+      bool lost = false;
+      if (from + lane < to) {
+        const uint32_t w = pend[from + lane], key = w & hi;
+        uint32_t h = home(key), probe = 0;
+        for (; probe < kMaxProbe; ++probe) {
+          uint32_t k = *((volatile uint32_t*)&tab[h]);
+          if (k == kEmpty) {
+            k = atomicCAS(&tab[h], kEmpty, w);
+            if (k == kEmpty) {
+              claimed = h;
+              break;
+            }
+          }
+          if ((k & hi) == key) {
+            atomicAdd(&tab[h], w & cmask);
+            break;
+          }
+          h = (h + 1u) & (kWSlots - 1u);
+        }
+        lost = probe == kMaxProbe;
+      }
+      const uint32_t c = __ballot_sync(kAll, claimed != kEmpty);
+      const uint32_t at = n_used + (uint32_t)__popc(c & below);
+      if (claimed != kEmpty && at < kWUsed) used[at] = (uint16_t)claimed;
+      n_used += (uint32_t)__popc(c);
+      if (__any_sync(kAll, lost) || n_used > kWUsed) overflow = true;
+      if (lane == 0) *n_pend = from;
+      __syncwarp();
+    };
+    // ---- walk.  Ring: entries [taken, staged) wait; c0: the next ones of the vector.
+    uint32_t staged = 0, taken = 0, c0 = 0;
+    uint32_t at = 0, first = 0, end = 0, ce = 0;  // the group's list: next posting (a multiple of 4), bounds, count
+    uint4 nv = make_uint4(0, 0, 0, 0);
+    if (!overflow && lane < E) nv = q_mv[m0 + lane];
+    auto stage = [&]() {  // 32 entries more, without those that have no targets
+      uint32_t lo = 0, len = 0;
+      if (c0 + lane < E) narrow_list(P, Q, q, nv, &lo, &len);
+      const uint32_t some = __ballot_sync(kAll, len != 0u);
+      if (len) {
+        const uint32_t x = (staged + (uint32_t)__popc(some & below)) & (kWRing - 1u);
+        ring[x] = make_uint2(lo, lo + len);
+        ring_ce[x] = nv.y | (c0 + lane) << 16;
+      }
+      staged += (uint32_t)__popc(some);
+      walked += len;
+      c0 += 32u;
+      if (c0 + lane < E) nv = q_mv[m0 + c0 + lane];
+      __syncwarp();
+    };
+    // Next step's postings (kEmpty where the lane has none) and their list's count.
+    auto next = [&](uint4& p, uint32_t& c) {
+      const uint32_t want = __ballot_sync(kAll, at >= end) & kFirst;
+      if (at >= end) {
+        const uint32_t x = taken + (uint32_t)__popc(want & groups_below);
+        if (x < staged) {
+          const uint2 t = ring[x & (kWRing - 1u)];
+          ce = ring_ce[x & (kWRing - 1u)];
+          first = t.x;
+          end = t.y;
+          at = t.x & ~3u;
+        } else {
+          at = end = 0;
+        }
+      }
+      taken = min(staged, taken + (uint32_t)__popc(want));
+      const uint32_t i = at + part;
+      p = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
+      if (i < end) {
+        p = *reinterpret_cast<const uint4*>(post + i);
+        if (i < first || i + 4u > end) {
+          if (i < first) p.x = kEmpty;
+          if (i + 1u < first || i + 1u >= end) p.y = kEmpty;
+          if (i + 2u < first || i + 2u >= end) p.z = kEmpty;
+          if (i + 3u >= end) p.w = kEmpty;
+        }
+      }
+      c = ce;
+      at += 4u * kGroup;
+    };
+    auto add = [&](const uint4& p, uint32_t c) {
+      uint32_t w[4] = {p.x, p.y, p.z, p.w};
+      const uint32_t ca = c & 0xFFFFu;
+      unsigned long long k[4];
+      uint32_t h[4], m[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        h[j] = home(w[j] & hi);
+        k[j] = *reinterpret_cast<volatile unsigned long long*>(&tab[h[j]]);
+        m[j] = min(ca, w[j] & cmask);
+      }
+      if (ca > cap) {  // counts that do not fit a posting
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (w[j] != kEmpty && (w[j] & cmask) == cap)
+            m[j] = min(ca, mv_count_of(P, w[j] >> P.cnt_bits, q_mv[m0 + (c >> 16)].x));
+      }
+      uint32_t miss = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t key = w[j] & hi;
+        const bool f0 = (((uint32_t)k[j] ^ key) & hi) == 0u, f1 = (((uint32_t)(k[j] >> 32) ^ key) & hi) == 0u;
+        if (w[j] != kEmpty) {
+          if (f0 || f1) atomicAdd(&tab[h[j] + (f0 ? 0u : 1u)], m[j]);
+          else miss |= 1u << j;
+        }
+      }
+      if (miss) {
+        uint32_t x = atomicAdd(n_pend, (uint32_t)__popc(miss));
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((miss >> j) & 1u) pend[x++] = (w[j] & hi) | m[j];
+      }
+      __syncwarp();
+      for (uint32_t n = *(volatile uint32_t*)n_pend; n >= 32u; n -= 32u) flush(n - 32u, n);
+    };
+    if (!overflow && E) {
+      stage();
+      while (staged == 0 && c0 < E) stage();
+      uint4 p, pn;
+      uint32_t c, cn;
+      next(p, c);
+      while (!overflow) {
+        while (staged - taken <= 32u && c0 < E) stage();
+        const bool more = taken < staged || __any_sync(kAll, at < end);
+        if (more) next(pn, cn);
+        add(p, c);
+        if (!more) break;
+        p = pn;
+        c = cn;
+      }
+      __syncwarp();
+      const uint32_t n = *(volatile uint32_t*)n_pend;
+      __syncwarp();
+      if (n) flush(0, n);
+    }
+    if (overflow) {
+      for (uint32_t h = lane; h < kWSlots; h += 32) tab[h] = kEmpty;
+      if (lane == 0) {
+        *n_pend = 0;
+        T.def_list[atomicAdd(T.def_count, 1u)] = qi;
+        O.row_off[q.row] = 0;
+        O.row_len[q.row] = 0;
+      }
+      __syncwarp();
+      continue;
+    }
+    // ---- per target genome: the maximum ratio, then the entries at it
+    for (uint32_t j = lane; j <= n_best; j += 32) {
+      if (j < n_best) best[j] = 0ull;
+      hcnt[j] = 0u;
+    }
+    __syncwarp();
+    auto is_target = [&](uint32_t b) {
+      return !(Q.all_pairs && ((b >= q.own0 && b < q.own1) || b >= q.tend)) && b != q.self;
+    };
+    for (uint32_t u = lane; u < n_used; u += 32) {
+      const uint32_t k = tab[used[u]], b = k >> P.cnt_bits, s = k & cmask;
+      if (!is_target(b)) continue;
+      const uint32_t gi = P.ginfo[b], den = La_a + (gi & 0xFFFFu) - s;
+      if (!wanted(q, gi >> 16)) continue;
+      if (Q.symbest) sym_update(Q, &Q.symbest[(size_t)q.col * P.n_genes + b], b, q.a, s, den);
+      if (Q.colbest) best_update(&Q.colbest[(size_t)b * Q.col_stride + q.col], s, den);
+      best_update(&best[Q.all_pairs ? (gi >> 16) : 0u], s, den);
+    }
+    __syncwarp();
+    for (uint32_t u = lane; u < n_used; u += 32) {
+      const uint32_t h = used[u], k = tab[h], b = k >> P.cnt_bits, s = k & cmask;
+      if (!is_target(b)) continue;
+      const uint32_t gi = P.ginfo[b], g = Q.all_pairs ? (gi >> 16) : 0u;
+      const unsigned long long bv = best[g];
+      if (wanted(q, gi >> 16) && ratio_equal(s, La_a + (gi & 0xFFFFu) - s, (uint32_t)(bv >> 32), (uint32_t)bv)) {
+        // 16-bit counts, two to a word
+        atomicAdd((uint32_t*)((uintptr_t)&hcnt[g] & ~(uintptr_t)3), ((uintptr_t)&hcnt[g] & 2u) ? 0x10000u : 1u);
+        used[u] = (uint16_t)(h | kWHit);
+      }
+    }
+    __syncwarp();
+    // ---- first position of each genome's hits in the row
+    uint32_t n_out = 0;
+    for (uint32_t j0 = 0; j0 <= n_best; j0 += 32) {
+      const uint32_t c = j0 + lane < n_best ? hcnt[j0 + lane] : 0u;
+      const uint32_t inc = warp_inclusive_scan(c);
+      if (j0 + lane <= n_best) hcnt[j0 + lane] = (uint16_t)(n_out + inc - c);
+      n_out += __shfl_sync(kAll, inc, 31);
+    }
+    unsigned long long base = 0;
+    if (lane == 0) {
+      base = atomicAdd(O.cursor, (unsigned long long)n_out);
+      O.row_off[q.row] = base;
+      O.row_len[q.row] = n_out;
+    }
+    base = __shfl_sync(kAll, base, 0);
+    __syncwarp();
+    const bool fits = base + n_out <= O.out_cap;
+    for (uint32_t u = lane; u < n_used; u += 32) {
+      const uint32_t w = used[u];
+      if (!(w & kWHit) || !fits) continue;
+      const uint32_t k = tab[w & (kWSlots - 1u)], b = k >> P.cnt_bits;
+      const uint32_t g = Q.all_pairs ? (P.ginfo[b] >> 16) : 0u;
+      uint32_t rank = hcnt[g];
+      if (hcnt[g + 1] - rank > 1u)  // tied hits of one genome: by gene
+        for (uint32_t x = 0; x < n_used; ++x) {
+          if (!(used[x] & kWHit)) continue;
+          const uint32_t y = tab[used[x] & (kWSlots - 1u)] >> P.cnt_bits;
+          rank += y < b && (!Q.all_pairs || (P.ginfo[y] >> 16) == g) ? 1u : 0u;
+        }
+      O.out_b[base + rank] = b;
+      O.out_s[base + rank] = k & cmask;
+    }
+    __syncwarp();
+    for (uint32_t u = lane; u < n_used; u += 32) tab[used[u] & (kWSlots - 1u)] = kEmpty;
+    __syncwarp();
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) walked += __shfl_xor_sync(kAll, walked, o);
+  if (lane == 0 && walked) atomicAdd(O.walked, walked);
 }
 
 // ---- shared-memory tiers: [table][chunk | (used list, hits)][best]
@@ -842,6 +1170,29 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   TierIO t1{nullptr, nullptr, O.def1, O.n_def1};
   TierIO t2{O.def1, O.n_def1, O.def2, O.n_def2};
   cudaError_t e;
+  // Where one warp per query pays (see kWarpTier*); tier 1 takes what it defers.
+  const bool long_lists = P.n_join >= (uint64_t)kWarpWalkMinAvg * P.n_entries &&
+                          P.n_entries * 4ull >= kWarpWalkMinIndexBytes;
+  const bool short_rows = !Q.all_pairs || P.n_join < (uint64_t)kWarpTierMaxAvg * P.n_entries;
+  if (!emit_all && Q.walk == PD_WALK_AUTO && n_best <= kWMaxGenomes && Q.n_queries >= kWarpTierMinQueries &&
+      (long_lists || short_rows)) {
+    auto kernel = long_lists ? k_summin_warp<2> : k_summin_warp<1>;
+    const size_t smem = kWWarps * warp_tier_bytes(n_best);
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+      return e;
+    int per_sm = 1, dev = 0, n_sm = 152;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWThreads, smem);
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>((Q.n_queries + kWWarps - 1) / kWWarps,
+                                                                   (uint32_t)n_sm * std::max(per_sm, 1)));
+    TierIO t0{nullptr, nullptr, O.def0, O.n_def0};
+    if ((e = launch_begin(L, "summin_warp")) != cudaSuccess) return e;
+    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best);
+    if ((e = launch_end(L, "summin_warp")) != cudaSuccess) return e;
+    t1.in_list = O.def0;
+    t1.in_count = O.n_def0;
+  }
   // tier 1: several resident blocks per SM, each looping over queries
   if (emit_all)
     e = launch_smem(k_summin_smem<kT1Threads, kT1MinBlocks, kT1Cap, kT1OutEmit, true, true, false, kT1Used>, L, "summin_pairs",

@@ -689,8 +689,9 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
   else
     cap = (uint64_t)nq * 4 + 4096;
   if (emit_all) cap = (uint64_t)nq * 64 + 4096;
-  Buf counters, def1, def2;
-  ALLOC(counters, 4 * sizeof(unsigned long long));
+  Buf counters, def0, def1, def2;
+  ALLOC(counters, 5 * sizeof(unsigned long long));
+  ALLOC(def0, sizeof(uint32_t) * std::max<uint32_t>(nq, 1));
   ALLOC(H->row_off, sizeof(unsigned long long) * std::max<uint32_t>(n_rows, 1));
   ALLOC(H->row_len, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1));
   ALLOC(def1, sizeof(uint32_t) * std::max<uint32_t>(nq, 1));
@@ -698,7 +699,7 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
   for (int attempt = 0; attempt < 3; ++attempt) {
     ALLOC(H->out_b, sizeof(uint32_t) * cap);
     ALLOC(H->out_s, sizeof(uint32_t) * cap);
-    CK(cudaMemsetAsync(counters.p, 0, 4 * sizeof(unsigned long long), c->stream));
+    CK(cudaMemsetAsync(counters.p, 0, 5 * sizeof(unsigned long long), c->stream));
     CK(cudaMemsetAsync(H->row_len.p, 0, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1), c->stream));
     if (Q.symbest) {  // a rerun starts the reverse maxima and their tie list afresh
       CK(cudaMemsetAsync(Q.symbest, 0, sizeof(unsigned long long) * v.n_genes * v.n_genomes, c->stream));
@@ -713,6 +714,9 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
     O.walked = cnt + 1;
     O.n_def1 = (uint32_t*)(cnt + 2);
     O.n_def2 = (uint32_t*)(cnt + 3);
+    O.n_def0 = (uint32_t*)(cnt + 4);
+    O.ticket = O.n_def0 + 1;
+    O.def0 = def0.as<uint32_t>();
     O.row_off = H->row_off.as<unsigned long long>();
     O.row_len = H->row_len.as<uint32_t>();
     O.def1 = def1.as<uint32_t>();

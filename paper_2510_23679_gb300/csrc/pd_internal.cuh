@@ -262,6 +262,10 @@ struct QuerySet {
   const uint32_t* q_gene;
   const uint32_t* q_t0;
   const uint32_t* q_t1;
+  // Target genomes of each query genome (all-pairs form; null = every other):
+  // bit t of the words from tgt_mask[genome * mask_words].
+  const uint32_t* tgt_mask;
+  uint32_t mask_words;
   // External queries (with the q_* arrays of the view): the genome of each
   // query gene among the queries' own genomes; it has no own-genome targets,
   // tgt_end and the colbest column are indexed by it.
@@ -283,7 +287,10 @@ struct HitsOut {
   unsigned long long* cursor;        // append cursor (keeps counting past cap)
   unsigned long long* row_off;       // per output row
   uint32_t* row_len;                 // per output row
-  uint32_t* def1;                    // queries deferred by tier 1 ...
+  uint32_t* ticket;                  // next query of the warp tier
+  uint32_t* def0;                    // queries deferred by the warp tier ...
+  uint32_t* n_def0;
+  uint32_t* def1;                    // ... by tier 1 ...
   uint32_t* n_def1;
   uint32_t* def2;                    // ... and by tier 2
   uint32_t* n_def2;
