@@ -56,31 +56,34 @@ struct ChunkJob {
 // Row lengths of a chunk's Best Hits into batch row order.
 __global__ void k_rows_len(const ChunkJob* __restrict__ jobs, uint32_t n_jobs, const uint32_t* __restrict__ row_len,
                            uint32_t* __restrict__ batch_len) {
-  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) {
-    const ChunkJob J = jobs[j];
-    for (uint32_t r = threadIdx.x; r < J.nA + J.nB; r += blockDim.x) batch_len[J.row0 + r] = row_len[J.a0 + r];
-  }
+  const uint32_t parts = gridDim.x / n_jobs;  // blocks of each job
+  const ChunkJob J = jobs[blockIdx.x / parts];
+  for (uint32_t r = (blockIdx.x % parts) * blockDim.x + threadIdx.x; r < J.nA + J.nB; r += parts * blockDim.x)
+    batch_len[J.row0 + r] = row_len[J.a0 + r];
 }
 
-// Best Hit rows of a chunk into the batch CSR, one warp per row; columns
-// become indices inside the partner genome.
+// Best Hit rows of a chunk into the batch CSR, eight lanes per row (rows of
+// one genome pair hold about one hit); columns become indices inside the
+// partner genome.  A few jobs of many rows must fill the chip, so every job
+// gets several blocks (0.05 against 1.5 ms for 16 jobs of 6500 rows with one
+// block each).
+constexpr uint32_t kFillLanes = 8;
 __global__ void k_rows_fill(const ChunkJob* __restrict__ jobs, uint32_t n_jobs,
                             const unsigned long long* __restrict__ row_off, const uint32_t* __restrict__ row_len,
                             const uint32_t* __restrict__ hit_b, const uint32_t* __restrict__ hit_s,
                             const unsigned long long* __restrict__ batch_ptr, int32_t* __restrict__ cols,
                             uint32_t* __restrict__ s) {
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) {
-    const ChunkJob J = jobs[j];
-    for (uint32_t r = warp; r < J.nA + J.nB; r += n_warps) {
-      const uint32_t g = J.a0 + r;
-      const uint32_t partner0 = r < J.nA ? J.b0 : J.a0;
-      const unsigned long long src = row_off[g], dst = batch_ptr[J.row0 + r];
-      const uint32_t len = row_len[g];
-      for (uint32_t i = lane; i < len; i += 32) {
-        cols[dst + i] = (int32_t)(hit_b[src + i] - partner0);
-        s[dst + i] = hit_s[src + i];
-      }
+  const uint32_t parts = gridDim.x / n_jobs;
+  const ChunkJob J = jobs[blockIdx.x / parts];
+  const uint32_t sub = threadIdx.x % kFillLanes, rows = blockDim.x / kFillLanes;
+  for (uint32_t r = (blockIdx.x % parts) * rows + threadIdx.x / kFillLanes; r < J.nA + J.nB; r += parts * rows) {
+    const uint32_t g = J.a0 + r, len = row_len[g];
+    if (len == 0) continue;
+    const uint32_t partner0 = r < J.nA ? J.b0 : J.a0;
+    const unsigned long long src = row_off[g], dst = batch_ptr[J.row0 + r];
+    for (uint32_t i = sub; i < len; i += kFillLanes) {
+      cols[dst + i] = (int32_t)(hit_b[src + i] - partner0);
+      s[dst + i] = hit_s[src + i];
     }
   }
 }
@@ -301,7 +304,7 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
     CK(cudaMemcpyAsync(C->d_jobs.p, C->jobs.data(), sizeof(ChunkJob) * C->jobs.size(), cudaMemcpyHostToDevice,
                        c->stream));
     const uint32_t nj = (uint32_t)C->jobs.size();
-    PD_KLAUNCH("batch_rows_len", (k_rows_len<<<grid_of(nj, 1, 152u * 16u), 256, 0, c->stream>>>(
+    PD_KLAUNCH("batch_rows_len", (k_rows_len<<<nj * std::max(1u, 152u * 8u / nj), 256, 0, c->stream>>>(
                                       C->d_jobs.as<ChunkJob>(), nj, C->hits.row_len.as<uint32_t>(),
                                       row_len.as<uint32_t>())));
     PD_KLAUNCH("batch_bbh_runs", (k_bbh_runs<<<grid_of(nj, 128, 152u * 4u), 128, 0, c->stream>>>(
@@ -330,7 +333,7 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
   for (auto& C : chunks) {
     const uint32_t nj = (uint32_t)C->jobs.size();
     PD_KLAUNCH("batch_rows_fill",
-               (k_rows_fill<<<grid_of(nj, 1, 152u * 16u), 256, 0, c->stream>>>(
+               (k_rows_fill<<<nj * std::max(1u, 152u * 8u / nj), 256, 0, c->stream>>>(
                    C->d_jobs.as<ChunkJob>(), nj, C->hits.row_off.as<unsigned long long>(),
                    C->hits.row_len.as<uint32_t>(), C->hits.out_b.as<uint32_t>(), C->hits.out_s.as<uint32_t>(),
                    B->row_ptr.as<unsigned long long>(), B->cols.as<int32_t>(), B->s.as<uint32_t>())));
@@ -377,62 +380,124 @@ __device__ __forceinline__ uint32_t job_of_row(const PairJob* __restrict__ jobs,
   return lo;
 }
 
+// Rows of pairs hold about one hit each: eight lanes share a row.
+constexpr uint32_t kRowLanes = 8;
+
 // Rows into the batch CSR (columns made local to the partner genome).
 __global__ void k_pairs_rows_fill(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
                                   const unsigned long long* __restrict__ row_off, const uint32_t* __restrict__ row_len,
                                   const uint32_t* __restrict__ hit_b, const uint32_t* __restrict__ hit_s,
                                   const unsigned long long* __restrict__ batch_ptr, int32_t* __restrict__ cols,
                                   uint32_t* __restrict__ s) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += warps) {
+  const uint32_t sub = threadIdx.x % kRowLanes;
+  const uint32_t stride = gridDim.x * blockDim.x / kRowLanes;
+  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) / kRowLanes; r < n_rows; r += stride) {
+    const uint32_t len = row_len[r];
+    if (len == 0) continue;
     const PairJob J = jobs[job_of_row(jobs, n_jobs, r)];
     const uint32_t partner0 = r < J.row0 + J.nA ? J.B0 : J.A0;
     const unsigned long long src = row_off[r], dst = batch_ptr[r];
-    for (uint32_t i = lane; i < row_len[r]; i += 32) {
+    for (uint32_t i = sub; i < len; i += kRowLanes) {
       cols[dst + i] = (int32_t)(hit_b[src + i] - partner0);
       s[dst + i] = hit_s[src + i];
     }
   }
 }
 
-// Mutual check, warp per row of an A genome: b's own row lists a?
+// Mutual check, eight lanes per row of an A genome: b's own row lists a?
 __global__ void k_pairs_bbh(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
                             const unsigned long long* __restrict__ row_off, const uint32_t* __restrict__ row_len,
                             const uint32_t* __restrict__ hit_b, const uint32_t* __restrict__ start,
                             uint32_t* __restrict__ cnt, int32_t* __restrict__ pa, int32_t* __restrict__ pb) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < n_rows; r += warps) {
-    const PairJob J = jobs[job_of_row(jobs, n_jobs, r)];
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % kRowLanes, group = lane - sub;
+  const uint32_t mates = ((1u << kRowLanes) - 1u) << group;
+  const uint32_t stride = gridDim.x * blockDim.x / kRowLanes;
+  for (uint32_t r = (blockIdx.x * blockDim.x + threadIdx.x) / kRowLanes; r < n_rows; r += stride) {
     uint32_t n = 0;
-    if (r < J.row0 + J.nA) {
-      const uint32_t a = J.A0 + (r - J.row0);
-      const unsigned long long off = row_off[r];
-      const uint32_t len = row_len[r];
-      uint32_t pos = start ? start[r] : 0u;
-      for (uint32_t e0 = 0; e0 < len; e0 += 32) {
-        const uint32_t e = e0 + lane;
-        bool f = false;
-        uint32_t b = 0;
-        if (e < len) {
-          b = hit_b[off + e];
-          const uint32_t rb = J.row0 + J.nA + (b - J.B0);
-          f = row_has(hit_b, row_off[rb], row_len[rb], a);
+    const uint32_t len = row_len[r];
+    if (len) {
+      const PairJob J = jobs[job_of_row(jobs, n_jobs, r)];
+      if (r < J.row0 + J.nA) {
+        const uint32_t a = J.A0 + (r - J.row0);
+        const unsigned long long off = row_off[r];
+        uint32_t pos = start ? start[r] : 0u;
+        for (uint32_t e0 = 0; e0 < len; e0 += kRowLanes) {
+          const uint32_t e = e0 + sub;
+          bool f = false;
+          uint32_t b = 0;
+          if (e < len) {
+            b = hit_b[off + e];
+            const uint32_t rb = J.row0 + J.nA + (b - J.B0);
+            f = row_has(hit_b, row_off[rb], row_len[rb], a);
+          }
+          const uint32_t m = __ballot_sync(mates, f) >> group;
+          if (start && f) {
+            const uint32_t at = pos + (uint32_t)__popc(m & ((1u << sub) - 1u));
+            pa[at] = (int32_t)(a - J.A0);
+            pb[at] = (int32_t)(b - J.B0);
+          }
+          pos += (uint32_t)__popc(m);
+          n += (uint32_t)__popc(m);
         }
-        const uint32_t m = __ballot_sync(0xffffffffu, f);
-        if (start && f) {
-          const uint32_t at = pos + (uint32_t)__popc(m & ((1u << lane) - 1u));
-          pa[at] = (int32_t)(a - J.A0);
-          pb[at] = (int32_t)(b - J.B0);
-        }
-        pos += (uint32_t)__popc(m);
-        n += (uint32_t)__popc(m);
       }
     }
-    if (!start && lane == 0) cnt[r] = n;
+    if (!start && sub == 0) cnt[r] = n;
   }
 }
+
+// Query genes and their target ranges, row by row (listed form).
+__global__ void k_pairs_queries(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
+                                uint32_t* __restrict__ gene, uint32_t* __restrict__ t0, uint32_t* __restrict__ t1) {
+  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n_rows; r += gridDim.x * blockDim.x) {
+    const PairJob J = jobs[job_of_row(jobs, n_jobs, r)];
+    const uint32_t i = r - J.row0;
+    const bool of_a = i < J.nA;
+    gene[r] = of_a ? J.A0 + i : J.B0 + (i - J.nA);
+    t0[r] = of_a ? J.B0 : J.A0;
+    t1[r] = t0[r] + (of_a ? J.nB : J.nA);
+  }
+}
+
+// Genes of the listed genomes (first gene, genes, first place), one after the other.
+struct GenomeSpan {
+  uint32_t gene0, n, at;
+};
+__global__ void k_span_genes(const GenomeSpan* __restrict__ spans, uint32_t n_spans, uint32_t* __restrict__ genes) {
+  for (uint32_t x = blockIdx.x; x < n_spans; x += gridDim.x)
+    for (uint32_t i = threadIdx.x; i < spans[x].n; i += blockDim.x) genes[spans[x].at + i] = spans[x].gene0 + i;
+}
+
+// Row r of the batch is the part of its gene's row (over several target
+// genomes, ascending) that lies in its partner genome.
+__global__ void k_pairs_slices(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
+                               const unsigned long long* __restrict__ gene_off, const uint32_t* __restrict__ gene_len,
+                               const uint32_t* __restrict__ hit_b, unsigned long long* __restrict__ row_off,
+                               uint32_t* __restrict__ row_len) {
+  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < n_rows; r += gridDim.x * blockDim.x) {
+    const PairJob J = jobs[job_of_row(jobs, n_jobs, r)];
+    const uint32_t i = r - J.row0;
+    const bool of_a = i < J.nA;
+    const uint32_t g = of_a ? J.A0 + i : J.B0 + (i - J.nA);
+    const uint32_t t0 = of_a ? J.B0 : J.A0, t1 = t0 + (of_a ? J.nB : J.nA);
+    const unsigned long long off = gene_off[g];
+    const int32_t* row = (const int32_t*)hit_b + off;
+    const uint32_t lo = lower_bound_i32(row, gene_len[g], (int32_t)t0);
+    row_off[r] = off + lo;
+    row_len[r] = lower_bound_i32(row + lo, gene_len[g] - lo, (int32_t)t1);
+  }
+}
+
+// First BBH pair of each job: what the rows before its first hold.
+__global__ void k_pairs_job_ptr(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
+                                const uint32_t* __restrict__ start, unsigned long long* __restrict__ job_ptr) {
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j <= n_jobs; j += gridDim.x * blockDim.x)
+    job_ptr[j] = start[j < n_jobs ? jobs[j].row0 : n_rows];
+}
+
+// Postings that a gene's whole walk visits in the time of one listed query
+// (its genome's range searched in every list): 843 M postings for 180 k genes
+// take 5.0 ms, 1.8 M listed queries on the same dataset 20.9 ms.
+constexpr uint64_t kPostingsPerQuery = 2000;
 
 pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint32_t n_jobs, pd_batch** out) {
   if (n_jobs && !jobs) return fail(c, PD_ERR_ARG, "null jobs");
@@ -441,90 +506,126 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   const auto& gp = P->h_genome_ptr;
   const uint32_t n_genomes = P->view.n_genomes;
   std::vector<PairJob> pj(n_jobs);
-  std::vector<uint32_t> qg, qt0, qt1;
   uint32_t row = 0;
   for (uint32_t j = 0; j < n_jobs; ++j) {
     const uint32_t A = jobs[2 * j], B = jobs[2 * j + 1];
     if (A >= n_genomes || B >= n_genomes || A == B)
       return fail(c, PD_ERR_ARG, "job " + std::to_string(j) + " needs two distinct genome indices < n_genomes");
-    PairJob J{row, (uint32_t)(gp[A + 1] - gp[A]), (uint32_t)(gp[B + 1] - gp[B]), (uint32_t)gp[A], (uint32_t)gp[B]};
-    pj[j] = J;
-    for (uint32_t i = 0; i < J.nA; ++i) {
-      qg.push_back(J.A0 + i);
-      qt0.push_back((uint32_t)gp[B]);
-      qt1.push_back((uint32_t)gp[B + 1]);
-    }
-    for (uint32_t i = 0; i < J.nB; ++i) {
-      qg.push_back(J.B0 + i);
-      qt0.push_back((uint32_t)gp[A]);
-      qt1.push_back((uint32_t)gp[A + 1]);
-    }
-    row += J.nA + J.nB;
+    pj[j] = PairJob{row, (uint32_t)(gp[A + 1] - gp[A]), (uint32_t)(gp[B + 1] - gp[B]), (uint32_t)gp[A], (uint32_t)gp[B]};
+    row += pj[j].nA + pj[j].nB;
   }
   const uint32_t n_q = row;
   std::unique_ptr<pd_batch> Bt(new pd_batch());
   Bt->ctx = c;
-  Buf d_jobs, d_qg, d_t0, d_t1, tmp, cnt, start;
+  Buf d_jobs, d_qg, d_t0, d_t1, d_mask, d_spans, d_off, d_len, tmp, cnt, start;
   ALLOC(d_jobs, sizeof(PairJob) * std::max<uint32_t>(n_jobs, 1));
-  ALLOC(d_qg, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
-  ALLOC(d_t0, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
-  ALLOC(d_t1, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
   ALLOC(Bt->row_ptr, sizeof(unsigned long long) * (n_q + 1));
   ALLOC(Bt->job_ptr, sizeof(unsigned long long) * (n_jobs + 1));
   ALLOC(tmp, pdg::scan_temp_bytes(n_q + 1) + 64);
   ALLOC(cnt, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
   ALLOC(start, sizeof(uint32_t) * (n_q + 1));
   if (n_jobs) CK(cudaMemcpyAsync(d_jobs.p, pj.data(), sizeof(PairJob) * n_jobs, cudaMemcpyHostToDevice, c->stream));
-  if (n_q) {
-    CK(cudaMemcpyAsync(d_qg.p, qg.data(), sizeof(uint32_t) * n_q, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(d_t0.p, qt0.data(), sizeof(uint32_t) * n_q, cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(d_t1.p, qt1.data(), sizeof(uint32_t) * n_q, cudaMemcpyHostToDevice, c->stream));
+
+  // Genomes with several partners are better walked once for all of them: the
+  // queries are then the genes of the genomes named, each against the genomes
+  // its own is paired with, and the jobs' rows are slices of theirs.
+  const uint32_t words = (n_genomes + 31) / 32;
+  std::vector<uint32_t> mask((size_t)n_genomes * words, 0);
+  uint64_t n_named = 0, n_directed = 0;  // genes of the genomes named; rows of the distinct ordered pairs
+  std::vector<GenomeSpan> spans;
+  for (uint32_t j = 0; j < n_jobs; ++j)
+    for (int way = 0; way < 2; ++way) {
+      const uint32_t a = jobs[2 * j + way], b = jobs[2 * j + 1 - way];
+      uint32_t& w = mask[(size_t)a * words + b / 32];
+      if (!((w >> (b & 31)) & 1u)) n_directed += (uint64_t)(gp[a + 1] - gp[a]);
+      w |= 1u << (b & 31);
+    }
+  for (uint32_t g = 0; g < n_genomes; ++g) {
+    bool any = false;
+    for (uint32_t w = 0; w < words; ++w) any = any || mask[(size_t)g * words + w] != 0;
+    const uint32_t n = (uint32_t)(gp[g + 1] - gp[g]);
+    if (!any || n == 0) continue;
+    spans.push_back(GenomeSpan{(uint32_t)gp[g], n, (uint32_t)n_named});
+    n_named += n;
   }
-  // one sum-min / Best Hit launch sequence over every query of every job
+  const uint64_t walk = P->view.n_genes ? P->view.n_join / P->view.n_genes : 0;  // postings of one gene's walk
+  const bool grouped = n_q && kPostingsPerQuery * n_q >= n_named * walk;
   pd_hits H;
   H.ctx = c;
   pdg::QuerySet Q{};
-  Q.all_pairs = 0;
-  Q.n_queries = n_q;
-  Q.q_gene = d_qg.as<uint32_t>();
-  Q.q_t0 = d_t0.as<uint32_t>();
-  Q.q_t1 = d_t1.as<uint32_t>();
-  pd_status st = run_hits(c, P, Q, false, &H, 1);
-  if (st != PD_OK) return st;
+  pd_status st = PD_OK;
+  if (grouped) {
+    const uint32_t n_named32 = (uint32_t)n_named;
+    ALLOC(d_spans, sizeof(GenomeSpan) * spans.size());
+    ALLOC(d_mask, sizeof(uint32_t) * mask.size());
+    ALLOC(d_qg, sizeof(uint32_t) * n_named);
+    CK(cudaMemcpyAsync(d_spans.p, spans.data(), sizeof(GenomeSpan) * spans.size(), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(d_mask.p, mask.data(), sizeof(uint32_t) * mask.size(), cudaMemcpyHostToDevice, c->stream));
+    PD_KLAUNCH("pairs_genes", (k_span_genes<<<grid_of(spans.size(), 1, 152u * 8u), 256, 0, c->stream>>>(
+                                  d_spans.as<GenomeSpan>(), (uint32_t)spans.size(), d_qg.as<uint32_t>())));
+    Q.all_pairs = 1;
+    Q.order = d_qg.as<uint32_t>();
+    Q.n_queries = n_named32;
+    Q.tgt_mask = d_mask.as<uint32_t>();
+    Q.mask_words = words;
+    H.all_pairs = 1;
+    st = run_hits(c, P, Q, false, &H, (uint32_t)((n_directed + n_named - 1) / n_named));
+    if (st != PD_OK) return st;
+    ALLOC(d_off, sizeof(unsigned long long) * n_q);
+    ALLOC(d_len, sizeof(uint32_t) * n_q);
+    PD_KLAUNCH("pairs_slices", (k_pairs_slices<<<grid_of(n_q, 256, 152u * 16u), 256, 0, c->stream>>>(
+                                   d_jobs.as<PairJob>(), n_jobs, n_q, H.row_off.as<unsigned long long>(),
+                                   H.row_len.as<uint32_t>(), H.out_b.as<uint32_t>(), d_off.as<unsigned long long>(),
+                                   d_len.as<uint32_t>())));
+    H.row_off = std::move(d_off);
+    H.row_len = std::move(d_len);
+  } else {
+    // one sum-min / Best Hit launch sequence over every query of every job
+    ALLOC(d_qg, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
+    ALLOC(d_t0, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
+    ALLOC(d_t1, sizeof(uint32_t) * std::max<uint32_t>(n_q, 1));
+    if (n_q)
+      PD_KLAUNCH("pairs_queries", (k_pairs_queries<<<grid_of(n_q, 256, 152u * 16u), 256, 0, c->stream>>>(
+                                      d_jobs.as<PairJob>(), n_jobs, n_q, d_qg.as<uint32_t>(), d_t0.as<uint32_t>(),
+                                      d_t1.as<uint32_t>())));
+    Q.all_pairs = 0;
+    Q.n_queries = n_q;
+    Q.q_gene = d_qg.as<uint32_t>();
+    Q.q_t0 = d_t0.as<uint32_t>();
+    Q.q_t1 = d_t1.as<uint32_t>();
+    st = run_hits(c, P, Q, false, &H, 1);
+    if (st != PD_OK) return st;
+  }
   CK(pdg::scan_u32_to_u64(&c->L, H.row_len.as<uint32_t>(), n_q, Bt->row_ptr.as<unsigned long long>(), tmp.p,
                           c->stream));
   if (n_q)
-    PD_KLAUNCH("pairs_bbh_count", (k_pairs_bbh<<<grid_of((uint64_t)n_q * 32, 256, 152u * 16u), 256, 0, c->stream>>>(
+    PD_KLAUNCH("pairs_bbh_count", (k_pairs_bbh<<<grid_of((uint64_t)n_q * kRowLanes, 256, 152u * 16u), 256, 0, c->stream>>>(
                                        d_jobs.as<PairJob>(), n_jobs, n_q, H.row_off.as<unsigned long long>(),
                                        H.row_len.as<uint32_t>(), H.out_b.as<uint32_t>(), nullptr,
                                        cnt.as<uint32_t>(), nullptr, nullptr)));
   CK(pdg::scan_u32(&c->L, cnt.as<uint32_t>(), n_q, start.as<uint32_t>(), tmp.p, c->stream));
+  PD_KLAUNCH("pairs_job_ptr", (k_pairs_job_ptr<<<grid_of((uint64_t)n_jobs + 1, 128, 152u * 4u), 128, 0, c->stream>>>(
+                                  d_jobs.as<PairJob>(), n_jobs, n_q, start.as<uint32_t>(),
+                                  Bt->job_ptr.as<unsigned long long>())));
   unsigned long long n_hits = 0;
   uint32_t n_bbh = 0;
-  std::vector<uint32_t> h_start(n_q + 1);
   CK(cudaMemcpyAsync(&n_hits, Bt->row_ptr.as<unsigned long long>() + n_q, sizeof(n_hits), cudaMemcpyDeviceToHost,
                      c->stream));
-  CK(cudaMemcpyAsync(h_start.data(), start.p, sizeof(uint32_t) * (n_q + 1), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaMemcpyAsync(&n_bbh, start.as<uint32_t>() + n_q, sizeof(n_bbh), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  n_bbh = h_start[n_q];
-  std::vector<unsigned long long> job_ptr(n_jobs + 1);
-  for (uint32_t j = 0; j < n_jobs; ++j) job_ptr[j] = h_start[pj[j].row0];
-  job_ptr[n_jobs] = n_bbh;
-  CK(cudaMemcpyAsync(Bt->job_ptr.p, job_ptr.data(), sizeof(unsigned long long) * (n_jobs + 1),
-                     cudaMemcpyHostToDevice, c->stream));
   ALLOC(Bt->cols, sizeof(int32_t) * std::max<unsigned long long>(n_hits, 1));
   ALLOC(Bt->s, sizeof(uint32_t) * std::max<unsigned long long>(n_hits, 1));
   ALLOC(Bt->a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
   ALLOC(Bt->b, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
   if (n_q) {
     PD_KLAUNCH("pairs_rows_fill",
-               (k_pairs_rows_fill<<<grid_of((uint64_t)n_q * 32, 256, 152u * 16u), 256, 0, c->stream>>>(
+               (k_pairs_rows_fill<<<grid_of((uint64_t)n_q * kRowLanes, 256, 152u * 16u), 256, 0, c->stream>>>(
                    d_jobs.as<PairJob>(), n_jobs, n_q, H.row_off.as<unsigned long long>(), H.row_len.as<uint32_t>(),
                    H.out_b.as<uint32_t>(), H.out_s.as<uint32_t>(), Bt->row_ptr.as<unsigned long long>(),
                    Bt->cols.as<int32_t>(), Bt->s.as<uint32_t>())));
     if (n_bbh)
       PD_KLAUNCH("pairs_bbh_write",
-                 (k_pairs_bbh<<<grid_of((uint64_t)n_q * 32, 256, 152u * 16u), 256, 0, c->stream>>>(
+                 (k_pairs_bbh<<<grid_of((uint64_t)n_q * kRowLanes, 256, 152u * 16u), 256, 0, c->stream>>>(
                      d_jobs.as<PairJob>(), n_jobs, n_q, H.row_off.as<unsigned long long>(), H.row_len.as<uint32_t>(),
                      H.out_b.as<uint32_t>(), start.as<uint32_t>(), nullptr, Bt->a.as<int32_t>(),
                      Bt->b.as<int32_t>())));
