@@ -352,7 +352,9 @@ constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
 // against 1.8) or its lists are long and the index far larger than L2 (200
 // genomes x 4000 genes: 26 against 27 ms).  Between them (50 x 3000) a query
 // meets several hundred chance targets, more of which overflow the warp's
-// table, and the block tier is the faster one (3.2 against 3.4 ms).
+// table, and the block tier is the faster one (3.2 against 3.4 ms); so do
+// queries from outside the dataset, whose lists are whole (16k queries of a
+// served tick 0.25 ms more).
 constexpr uint32_t kWarpTierMinQueries = 16384, kWarpTierMaxAvg = 8;
 // Target genomes from which a query's Best Hits are ranked through per-genome
 // positions rather than pairwise.
@@ -1174,8 +1176,8 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   const bool long_lists = P.n_join >= (uint64_t)kWarpWalkMinAvg * P.n_entries &&
                           P.n_entries * 4ull >= kWarpWalkMinIndexBytes;
   const bool short_rows = !Q.all_pairs || P.n_join < (uint64_t)kWarpTierMaxAvg * P.n_entries;
-  if (!emit_all && Q.walk == PD_WALK_AUTO && n_best <= kWMaxGenomes && Q.n_queries >= kWarpTierMinQueries &&
-      (long_lists || short_rows)) {
+  if (!emit_all && !P.q_win_off && Q.walk == PD_WALK_AUTO && n_best <= kWMaxGenomes &&
+      Q.n_queries >= kWarpTierMinQueries && (long_lists || short_rows)) {
     auto kernel = long_lists ? k_summin_warp<2> : k_summin_warp<1>;
     const size_t smem = kWWarps * warp_tier_bytes(n_best);
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
