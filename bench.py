@@ -787,8 +787,8 @@ def main():
                "achieved": enc_bytes / (enc_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
                "frac": enc_bytes / (enc_ms / 1e3) / 1e9 / peak, "sort_passes": passes}
 
-    # ---- the merge form of Eq. (5) (pd_summin_list: two sorted vectors
-    # walked side by side, one warp per pair) on this step's BBH pairs, once
+    # ---- the pair form of Eq. (5) (pd_summin_list: the two vectors joined on
+    # their k-mers) on this step's BBH pairs, once
     merge_form = None
     if n_bbh:
         a_d, b_d = torch.empty(n_bbh, dtype=torch.int32, device=dev), torch.empty(n_bbh, dtype=torch.int32, device=dev)
@@ -802,8 +802,7 @@ def main():
             torch.cuda.synchronize()
         m_ms = e0.elapsed_time(e1)
         merge_form = {"pairs": n_bbh, "ms": m_ms, "pairs_per_s": n_bbh / (m_ms / 1e3),
-                      "what": "sum-min and sum-max of every BBH pair of the step by the two-pointer merge of their "
-                              "sorted multiplicity vectors (the vectors of the genes involved sorted first)"}
+                      "what": "sum-min and sum-max of every BBH pair of the step by joining the two multiplicity vectors"}
         del a_d, b_d, s_d, den_d
 
     # ---- end to end through the C ABI from pinned host buffers: inputs

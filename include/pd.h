@@ -221,10 +221,11 @@ pd_status pd_ctx_set_symmetric(pd_ctx* ctx, int enable);
  * posting lists are read either by the merge-path walk (each thread a run of
  * consecutive postings, batches of four) or by the warp-cooperative walk
  * (each warp 32 consecutive postings per round; suits long lists).
- * PD_WALK_AUTO (the default) takes the warp walk when the build's join
- * (pd_profiles_info.n_join) is at least 16 postings per vector entry and the
- * postings take at least 512 MB (smaller indexes stay close enough to L2
- * for the merge-path walk).
+ * PD_WALK_AUTO (the default) gives each query to one warp where that pays
+ * (many queries that meet few targets, or very long lists), else to one block
+ * with the warp walk when the build's join (pd_profiles_info.n_join) is at
+ * least 16 postings per vector entry and the postings take at least 512 MB
+ * (smaller indexes stay close enough to L2 for the merge-path walk).
  * Applies to every later Best Hit call on the context.  Errors: PD_ERR_ARG
  * (null context, unknown mode). */
 #define PD_WALK_AUTO 0u
@@ -351,15 +352,14 @@ pd_status pd_families(pd_ctx* ctx, const pd_bbh_set* bbh, uint32_t n_genes, int3
 
 /* ---------------------------------------------------------------- sum-min */
 
-/* Sum-min of listed gene pairs by the paper's own form: the two
- * multiplicity vectors, sorted by k-mer, walked side by side (the similarity
- * of Algorithm 2; Eq. (5)).  Pair i is (a[i], b[i]), global gene ids of this
+/* Sum-min of listed gene pairs: the two multiplicity vectors joined on their
+ * k-mers (the similarity of Algorithm 2; Eq. (5)).  Pair i is (a[i], b[i]), global gene ids of this
  * dataset (any genomes, a gene with itself allowed).  s[i] receives sum-min,
  * den[i] the Eq. (5) denominator sum-max = La + Lb - s; GJ = s / den (0/0 for
  * two genes without windows).  a, b, s, den are host or device pointers (n
- * entries each; s or den NULL to skip).  One warp merges one pair, so the
- * call suits known pairs (the similarity of BBH pairs, a candidate list); the
- * all-against-all search is pd_best_hits_all.  Errors: PD_ERR_ARG (a gene id
+ * entries each; s or den NULL to skip).  The call suits known pairs (the
+ * similarity of BBH pairs, a candidate list); the all-against-all search is
+ * pd_best_hits_all.  Errors: PD_ERR_ARG (a gene id
  * not below n_genes), PD_ERR_OOM, PD_ERR_CUDA. */
 pd_status pd_summin_list(pd_ctx* ctx, const pd_profiles* prof, const uint32_t* a, const uint32_t* b, uint64_t n,
                          uint32_t* s, uint32_t* den);

@@ -609,8 +609,8 @@ def pd_summin_pairs(ctx: Ctx, prof: Profiles, gi: int, gj: int):
 
 
 def pd_summin_list(ctx: Ctx, prof: Profiles, a, b, s=None, den=None):
-    """Sum-min and sum-max (Eq. (5)) of the gene pairs (a[i], b[i]) by merging
-    their sorted multiplicity vectors.  a, b: uint32 global gene ids (host
+    """Sum-min and sum-max (Eq. (5)) of the gene pairs (a[i], b[i]) by joining
+    their multiplicity vectors.  a, b: uint32 global gene ids (host
     arrays or device tensors).  Without output buffers returns host arrays
     (s uint32, den uint32); with them (host or device, n entries) returns None."""
     n = int(a.shape[0])
