@@ -72,11 +72,13 @@ constexpr uint32_t kMaxProbe = 64;
 // and linear probing.
 template <bool kPacked, bool kFilter = false>
 struct Acc {
-  static_assert(!(kPacked && kFilter), "filtered queries use the split layout");
   uint32_t* keys;  // packed: slot words
   uint32_t* vals;  // split only
-  uint32_t* vpa;   // filtered only: sum of mult_a over the shared k-mers (Eq. (7) numerator, a -> b)
-  uint32_t* vpb;   // filtered only: sum of mult_b over the shared k-mers (b -> a)
+  // filtered only: the sums of mult_a and of mult_b over the shared k-mers (Eq.
+  // (7) numerators, a -> b and b -> a); packed: both in vpa, mult_b's above
+  // 16 bits (each is at most its gene's windows, below 2^16)
+  uint32_t* vpa;
+  uint32_t* vpb;
   uint32_t cnt_bits;
   uint32_t hash_shift;  // 32 - log2(cap)
   // Target genes [dense_lo, dense_lo + cap) of a query whose targets fit the
@@ -108,13 +110,14 @@ struct Acc {
       if (kPacked) {
         if ((k & hi) == key) {
           atomicAdd(&keys[h], m);
+          if (kFilter) atomicAdd(&vpa[h], ca | cb << 16);
           return true;
         }
         if (k == kEmpty) {
           const uint32_t prev = atomicCAS(&keys[h], kEmpty, key | m);
-          if (prev == kEmpty) return true;
-          if ((prev & hi) == key) {
-            atomicAdd(&keys[h], m);
+          if (prev == kEmpty || (prev & hi) == key) {
+            if (prev != kEmpty) atomicAdd(&keys[h], m);
+            if (kFilter) atomicAdd(&vpa[h], ca | cb << 16);
             return true;
           }
         }
@@ -146,12 +149,16 @@ struct Acc {
       *s = vals[h];
     }
   }
+  __device__ __forceinline__ void sums(uint32_t h, uint32_t* pa, uint32_t* pb) const {
+    *pa = kPacked ? vpa[h] & 0xFFFFu : vpa[h];
+    *pb = kPacked ? vpa[h] >> 16 : vpb[h];
+  }
   __device__ __forceinline__ void clear(uint32_t h) const {
     keys[h] = kEmpty;
     if (!kPacked) vals[h] = 0;
     if (kFilter) {
       vpa[h] = 0;
-      vpb[h] = 0;
+      if (!kPacked) vpb[h] = 0;
     }
   }
 };
@@ -618,7 +625,11 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         if ((Q.all_pairs && ((b >= own0 && b < own1) || b >= tend)) || b == self) continue;  // not a target
         const uint32_t gi = P.ginfo[b];
         if (!wanted(q, gi >> 16)) continue;
-        if (kFilter && !filter_pass(Q, P.k, La_a, gi & 0xFFFFu, acc.vpa[tb.used[u]], acc.vpb[tb.used[u]])) continue;
+        if (kFilter) {
+          uint32_t pa, pb;
+          acc.sums(tb.used[u], &pa, &pb);
+          if (!filter_pass(Q, P.k, La_a, gi & 0xFFFFu, pa, pb)) continue;
+        }
         const uint32_t den = La_a + (gi & 0xFFFFu) - s;
         best_update(&best[Q.all_pairs ? (gi >> 16) : 0u], s, den);
         if (Q.colbest) best_update(&Q.colbest[(size_t)b * Q.col_stride + col], s, den);
@@ -631,8 +642,10 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         acc.get(h, &b, &s);
         const uint32_t gi = P.ginfo[b];
         const unsigned long long bv = best[Q.all_pairs ? (gi >> 16) : 0u];
+        uint32_t pa = 0, pb = 0;
+        if (kFilter) acc.sums(h, &pa, &pb);
         if (!(Q.all_pairs && ((b >= own0 && b < own1) || b >= tend)) && b != self && wanted(q, gi >> 16) &&
-            (!kFilter || filter_pass(Q, P.k, La_a, gi & 0xFFFFu, acc.vpa[h], acc.vpb[h])) &&
+            (!kFilter || filter_pass(Q, P.k, La_a, gi & 0xFFFFu, pa, pb)) &&
             ratio_equal(s, La_a + (gi & 0xFFFFu) - s, (uint32_t)(bv >> 32), (uint32_t)bv)) {
           // s <= La <= 65535 and the genome < 65536: (b, genome, s) in one word
           const uint32_t g = Q.all_pairs ? (gi >> 16) : 0u;
@@ -1016,7 +1029,7 @@ struct SmemTier {
   static_assert(kCap % kThreads == 0, "table must split evenly over the block");
   static_assert(kCap <= 65536, "slot indices are 16-bit");
   static_assert(kUsedCap <= kCap && kUsedCap % 8 == 0, "occupied-slot list");
-  static constexpr size_t kTable = (size_t)kCap * (kPacked ? 4 : (kFilter ? 16 : 8));
+  static constexpr size_t kTable = (size_t)kCap * (kPacked ? (kFilter ? 8 : 4) : (kFilter ? 16 : 8));
   static constexpr size_t kUsed = (size_t)kUsedCap * 2;
   static constexpr size_t kAfterWalk = kUsed + (size_t)kOutCap * 8;
   static constexpr size_t kUnion = Chunk<kThreads>::kBytes > kAfterWalk ? Chunk<kThreads>::kBytes : kAfterWalk;
@@ -1034,8 +1047,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_summin_smem(ProfilesVi
   Table<uint16_t> tb;
   tb.keys = (uint32_t*)smem;
   tb.vals = kPacked ? nullptr : tb.keys + kCap;
-  tb.vpa = kFilter ? tb.vals + kCap : nullptr;
-  tb.vpb = kFilter ? tb.vpa + kCap : nullptr;
+  tb.vpa = kFilter ? (kPacked ? tb.keys : tb.vals) + kCap : nullptr;
+  tb.vpb = kFilter && !kPacked ? tb.vpa + kCap : nullptr;
   tb.cap = kCap;
   tb.out_cap = kOutCap;
   tb.used_cap = kUsedCap;
@@ -1051,7 +1064,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_summin_smem(ProfilesVi
     if (!kPacked) tb.vals[h] = 0;
     if (kFilter) {
       tb.vpa[h] = 0;
-      tb.vpb[h] = 0;
+      if (!kPacked) tb.vpb[h] = 0;
     }
   }
   __syncthreads();
@@ -1134,8 +1147,14 @@ using T2E = SmemTier<kT2Threads, kT2Cap, kT2OutEmit, false>;
 static_assert(T1F::bytes(PD_MAX_GENOMES) <= 227 * 1024, "tier 1 shared memory");
 static_assert(T2::bytes(PD_MAX_GENOMES) <= 227 * 1024, "tier 2 shared memory");
 static_assert(T2E::bytes(1) <= 227 * 1024, "tier 2 (emit-all, one target genome) shared memory");
-// Filtered queries (Eqs. (6)-(7)): split 4096-slot table with the two
-// directional sums; what does not fit goes straight to the global tier.
+// Filtered queries (Eqs. (6)-(7)): packed 4096-slot table, the two directional
+// sums in one more word a slot (five blocks per SM: 60 k queries of 30 genomes
+// 1.7 ms, against 2.1 for the split table's two blocks); what does not fit goes
+// to a split table of as many slots, then straight to the global tier.
+constexpr int kF1MinBlocks = 5;
+constexpr uint32_t kF1Cap = 4096, kF1Used = 2560, kF1Out = 448;
+using TF1 = SmemTier<256, kF1Cap, kF1Out, true, true, kF1Used>;
+static_assert(TF1::bytes(PD_MAX_GENOMES) <= 227 * 1024, "filtered tier shared memory");
 constexpr int kFThreads = 256, kFMinBlocks = 2;
 constexpr uint32_t kFCap = 4096, kFOut = 512;
 using TF = SmemTier<kFThreads, kFCap, kFOut, false, true>;
@@ -1165,7 +1184,11 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   const uint32_t n_best = Q.all_pairs ? P.n_genomes : 1u;
   if (Q.filter) {
     if (emit_all) return cudaErrorInvalidValue;
-    TierIO tf{nullptr, nullptr, O.def2, O.n_def2};
+    TierIO tf1{nullptr, nullptr, O.def0, O.n_def0}, tf{O.def0, O.n_def0, O.def2, O.n_def2};
+    const cudaError_t e1 =
+        launch_smem(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used>, L, "summin_bh_f1", 256,
+                    TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s);
+    if (e1 != cudaSuccess) return e1;
     return launch_smem(k_summin_smem<kFThreads, kFMinBlocks, kFCap, kFOut, false, false, true>, L, "summin_bh_f",
                        kFThreads, TF::bytes(n_best), Q.n_queries, P, Q, O, tf, err, s);
   }
