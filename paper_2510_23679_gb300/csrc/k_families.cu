@@ -151,7 +151,7 @@ PD_API pd_status pd_families(pd_ctx* c, const pd_bbh_set* S, uint32_t n_genes, i
                              uint32_t* n_families) {
   if (!c || !S) return PD_ERR_ARG;
   try {
-    return components_impl(c, S->a.as<int32_t>(), S->b.as<int32_t>(), S->n, n_genes, family, n_families);
+    return components_impl(c, S->first(), S->second(), S->n, n_genes, family, n_families);
   } catch (const std::bad_alloc&) {
     return fail(c, PD_ERR_OOM, "host allocation failed");
   } catch (...) {

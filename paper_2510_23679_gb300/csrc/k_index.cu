@@ -29,10 +29,8 @@
 //
 // Each sort pass reads and writes every record once: a tile's digit counts
 // are combined with those of the tiles before it by decoupled look-back
-// (Merrill and Garland, "Single-pass Parallel Prefix Scan with Decoupled
-// Look-back", 2016; Adinets and Merrill, "Onesweep", 2022), with tiles
-// numbered by a ticket so that every tile waited for is already running.  A
-// wait that runs out raises PD_ERR_INTERNAL and its tile writes nothing.
+// (Adinets and Merrill, "Onesweep", 2022).  A wait that runs out raises
+// PD_ERR_INTERNAL and its tile writes nothing.
 //
 // Measured at 200 genomes x 4000 genes, k = 7 (264 M windows): 17.5 ms for the
 // whole build against 23.4 ms for a dictionary of all codes (marked and looked
@@ -94,27 +92,38 @@ __global__ void __launch_bounds__(256)
 }
 
 // ---------------------------------------------------------------- windows
-// Window counts of the genes.  A gene whose offsets are malformed, or reach
-// past the residues, is reported and gets no windows, so nothing after this
-// kernel reads outside the residues.
+// Window counts and genomes of the genes.  A gene whose offsets are malformed,
+// or reach past the residues, is reported and gets no windows, so nothing after
+// this kernel reads outside the residues.  The genome is the last that begins at
+// or before the gene (genome offsets not checked yet only misplace it).
 __global__ void k_gene_windows(const int64_t* __restrict__ gene_ptr, uint32_t n_genes, uint64_t n_res, int check_end,
-                               int k, uint32_t* __restrict__ La, DevErr* err) {
+                               int k, const int32_t* __restrict__ genome_ptr, uint32_t n_genomes,
+                               uint32_t* __restrict__ La, uint16_t* __restrict__ gene_genome,
+                               uint32_t* __restrict__ ginfo, uint32_t* __restrict__ minhash, DevErr* err) {
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x) {
     const int64_t r0 = gene_ptr[g], r1 = gene_ptr[g + 1];
     const bool bad = r1 < r0 || r0 < 0 || (g == 0 && r0 != 0) ||
                      (check_end && ((uint64_t)r1 > n_res || (g + 1 == n_genes && (uint64_t)r1 != n_res)));
+    uint64_t w = 0;
     if (bad) {
       raise_error(err, PD_ERR_ARG, g);
-      La[g] = 0;
-      continue;
+    } else {
+      const int64_t len = r1 - r0;
+      w = len >= k ? (uint64_t)(len - k + 1) : 0;
+      if (w > PD_MAX_WINDOWS) {
+        raise_error(err, PD_ERR_GENE_TOO_LONG, g);
+        w = 0;
+      }
     }
-    const int64_t len = r1 - r0;
-    uint64_t w = len >= k ? (uint64_t)(len - k + 1) : 0;
-    if (w > PD_MAX_WINDOWS) {
-      raise_error(err, PD_ERR_GENE_TOO_LONG, g);
-      w = 0;
+    uint32_t lo = 0, hi = n_genomes;
+    while (hi - lo > 1u) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (genome_ptr[mid] <= (int32_t)g) lo = mid; else hi = mid;
     }
     La[g] = (uint32_t)w;
+    gene_genome[g] = (uint16_t)lo;
+    ginfo[g] = (uint32_t)w | (lo << 16);
+    minhash[g] = kEmpty;
   }
 }
 
@@ -126,14 +135,16 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kItems = 15;
 constexpr uint32_t kTile = kThreads * kItems;
 constexpr int kSortBlocks = 2;  // resident blocks per SM
-constexpr int kMaxBins = 512;   // digits of at most 9 bits
+constexpr int kMaxBins = kSortBins;  // digits of at most 9 bits
 
 // Gene of the first window of every tile; tile_gene[n_tiles] = the last gene.
+// Also the first free place of every gene's vector.
 __global__ void k_tile_genes(const uint32_t* __restrict__ win_off, uint32_t n_genes, uint32_t n_tiles,
-                             uint32_t* __restrict__ tile_gene) {
+                             uint32_t* __restrict__ tile_gene, uint32_t* __restrict__ cursor) {
   if (blockIdx.x == 0 && threadIdx.x == 0) tile_gene[n_tiles] = n_genes - 1u;
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x) {
     const uint64_t w0 = win_off[g], w1 = win_off[g + 1];
+    cursor[g] = (uint32_t)w0;
     for (uint64_t t = (w0 + kTile - 1) / kTile; t * kTile < w1; ++t) tile_gene[t] = g;
   }
 }
@@ -256,99 +267,6 @@ __global__ void __launch_bounds__(kThreads)
     if (cnt[d]) atomicAdd(&hist[d], cnt[d]);
 }
 
-// Digit counts -> digit starts, one block per pass; total[0] = records.
-__global__ void __launch_bounds__(kMaxBins)
-    k_digit_starts(uint32_t* hist, u64* __restrict__ start, u64* __restrict__ total) {
-  __shared__ u64 tmp[kMaxBins];
-  const uint32_t d = threadIdx.x, p = blockIdx.x;
-  const u64 v = hist[p * kMaxBins + d];
-  tmp[d] = v;
-  __syncthreads();
-  for (uint32_t o = 1; o < kMaxBins; o <<= 1) {
-    const u64 x = d >= o ? tmp[d - o] : 0ull;
-    __syncthreads();
-    tmp[d] += x;
-    __syncthreads();
-  }
-  start[p * kMaxBins + d] = tmp[d] - v;
-  if (p == 0 && d == kMaxBins - 1) *total = tmp[d];
-}
-
-// ---------------------------------------------------------------- look-back
-// Status words: two flag bits above the value, written and read whole.  32-bit
-// words (sums below 2^30) for all but the largest inputs: the sort passes write
-// and read one per tile and digit, about 2% of their traffic.
-template <typename T>
-struct Status {
-  static constexpr T kAggregate = (T)1 << (sizeof(T) * 8 - 2);
-  static constexpr T kInclusive = (T)2 << (sizeof(T) * 8 - 2);
-  static constexpr T kValue = kAggregate - 1;
-};
-constexpr uint32_t kMaxPolls = 1u << 21;
-
-// Sum over the tiles before `tile` of one column of statuses (status[t *
-// stride]), walked back until an inclusive sum; four predecessors are read at
-// a time.  False if a wait ran out.
-template <typename T>
-__device__ __forceinline__ bool look_back(const volatile T* status, uint32_t tile, uint32_t stride, T* sum,
-                                          const DevErr* err) {
-  T s = 0;
-  uint32_t polls = 0;
-  int64_t t = (int64_t)tile - 1;
-  while (t >= 0) {
-    T v[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = t - j >= 0 ? status[(uint64_t)(t - j) * stride] : (T)0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (v[j] & Status<T>::kInclusive) {
-        *sum = s + (v[j] & Status<T>::kValue);
-        return true;
-      }
-      if (!(v[j] & Status<T>::kAggregate)) break;
-      s += v[j] & Status<T>::kValue;
-      --t;
-    }
-    if (++polls > 64u) {
-      __nanosleep(100);
-      if (polls > kMaxPolls || ((polls & 255u) == 0 && *(volatile const int*)&err->code)) return false;
-    }
-  }
-  *sum = s;
-  return true;
-}
-
-// The same for one column by a whole warp, 32 predecessors at a time.
-__device__ __forceinline__ bool look_back_warp(const volatile u64* status, uint32_t tile, u64* sum, const DevErr* err) {
-  using S = Status<u64>;
-  const uint32_t lane = threadIdx.x & 31u;
-  u64 s = 0;
-  uint32_t polls = 0;
-  for (int64_t t = (int64_t)tile - 1; t >= 0;) {
-    const int64_t mine = t - lane;
-    const u64 v = mine >= 0 ? status[mine] : S::kInclusive;
-    const uint32_t inc = __ballot_sync(0xffffffffu, (v & S::kInclusive) != 0ull);
-    const uint32_t set = __ballot_sync(0xffffffffu, (v & (S::kInclusive | S::kAggregate)) != 0ull);
-    // the lanes up to the first inclusive sum, or up to the first one missing
-    const uint32_t n = inc ? (uint32_t)__ffs((int)inc) : 32u;
-    const uint32_t ready = set == 0xffffffffu ? 32u : (uint32_t)__ffs((int)~set) - 1u;
-    const uint32_t take = min(n, ready);
-    u64 x = lane < take ? v & S::kValue : 0ull;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    s += x;
-    t -= take;
-    if (inc && n <= ready) break;
-    if (take < 32u && ++polls > 64u) {
-      __nanosleep(100);
-      const bool failed = (polls & 255u) == 0 && *(volatile const int*)&err->code;
-      if (polls > kMaxPolls || __any_sync(0xffffffffu, failed)) return false;
-    }
-  }
-  *sum = s;
-  return true;
-}
-
 // ---------------------------------------------------------------- sort pass
 template <int kBits>
 struct PassShared {
@@ -360,14 +278,27 @@ struct PassShared {
   int failed;
 };
 
+// Takes a tile.  The first one also scans the digit counts into gbase (the
+// digits' starts), so that the running sums over the tiles are output positions.
 template <int kBits>
-__device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, uint32_t* ticket) {
+__device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, const uint32_t* __restrict__ hist, uint32_t* ticket) {
   for (uint32_t x = threadIdx.x; x < (kWarps << kBits) / 2; x += kThreads) ((uint32_t*)&sh.wcnt[0][0])[x] = 0;
   if (threadIdx.x == 0) {
     sh.tile = atomicAdd(ticket, 1u);
     sh.failed = 0;
   }
   __syncthreads();
+  if (sh.tile == 0) {
+    uint32_t carry = 0;
+    for (uint32_t d0 = 0; d0 < (1u << kBits); d0 += kThreads) {
+      const uint32_t d = d0 + threadIdx.x;
+      uint32_t n;
+      const uint32_t ex = block_exclusive_scan(d < (1u << kBits) ? hist[d] : 0u, sh.warp_tmp, &n);
+      if (d < (1u << kBits)) sh.gbase[d] = carry + ex;
+      carry += n;
+    }
+    __syncthreads();
+  }
 }
 
 // Stable counting step of one tile.  xr: the thread's records, striped within
@@ -375,9 +306,8 @@ __device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, uint32_t* tick
 // Ranks within the warp come from the lanes holding the same digit (the AND
 // over the digit's bits of each bit's ballot or its complement).
 template <int kBits, typename T>
-__device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid_mask, uint32_t shift,
-                                               const u64* __restrict__ digit_start, T* status, u64* __restrict__ out,
-                                               PassShared<kBits>& sh, u64* stage, DevErr* err) {
+__device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid_mask, uint32_t shift, T* status,
+                                               u64* __restrict__ out, PassShared<kBits>& sh, u64* stage, DevErr* err) {
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   constexpr uint32_t bins = 1u << kBits, dmask = bins - 1u;
   constexpr int kOwn = (int)((bins + kThreads - 1) / kThreads);  // digits kOwn * t .. of thread t
@@ -417,9 +347,9 @@ __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid
         run += c;
       }
       tot[j] = run;
-      // the first tile's sums are inclusive at once
-      volatile T* st = status + (uint64_t)sh.tile * bins + d;
-      *st = (sh.tile == 0 ? Status<T>::kInclusive : Status<T>::kAggregate) | run;
+      // the first tile's sums are inclusive at once: the digit's start is known
+      *(volatile T*)(status + (uint64_t)sh.tile * bins + d) =
+          sh.tile == 0 ? Status<T>::kInclusive | (T)(sh.gbase[d] + run) : Status<T>::kAggregate | (T)run;
     }
     sum += tot[j];
   }
@@ -444,7 +374,9 @@ __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid
     const uint32_t d = kOwn * threadIdx.x + (uint32_t)j;
     if (d < bins) {
       T before = 0;
-      if (sh.tile != 0) {
+      if (sh.tile == 0) {
+        before = (T)sh.gbase[d];
+      } else {
         if (!look_back<T>(status + d, sh.tile, bins, &before, err)) {
           raise_error(err, PD_ERR_INTERNAL, sh.tile);
           sh.failed = 1;
@@ -453,7 +385,7 @@ __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid
           *st = Status<T>::kInclusive | (before + tot[j]);
         }
       }
-      sh.gbase[d] = digit_start[d] + before - sh.tbase[d];
+      sh.gbase[d] = (u64)before - sh.tbase[d];
     }
   }
   __syncthreads();
@@ -466,13 +398,13 @@ __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid
 
 template <int kBits, typename T, typename Code>
 __global__ void __launch_bounds__(kThreads, kSortBlocks)
-    k_sort_windows(WindowSource S, SortKey K, const u64* __restrict__ digit_start, T* status, uint32_t* ticket,
+    k_sort_windows(WindowSource S, SortKey K, const uint32_t* __restrict__ hist, T* status, uint32_t* ticket,
                    u64* __restrict__ out, DevErr* err) {
   extern __shared__ u64 stage[];
   __shared__ PassShared<kBits> sh;
   __shared__ uint8_t lut[256];
   init_code_table(lut, S.alpha);
-  begin_tile<kBits>(sh, ticket);
+  begin_tile<kBits>(sh, hist, ticket);
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint32_t at = threadIdx.x * kItems;
   // the all-ones word is no record: the gene field never holds all ones
@@ -491,16 +423,16 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
     valid |= xr[r] != ~0ull ? 1u << r : 0u;
   }
   __syncthreads();
-  rank_and_write<kBits, T>(xr, valid, K.gene_bits, digit_start, status, out, sh, stage, err);
+  rank_and_write<kBits, T>(xr, valid, K.gene_bits, status, out, sh, stage, err);
 }
 
 template <int kBits, typename T>
 __global__ void __launch_bounds__(kThreads, kSortBlocks)
-    k_sort_records(const u64* __restrict__ in, uint64_t n, uint32_t shift, const u64* __restrict__ digit_start,
+    k_sort_records(const u64* __restrict__ in, uint64_t n, uint32_t shift, const uint32_t* __restrict__ hist,
                    T* status, uint32_t* ticket, u64* __restrict__ out, DevErr* err) {
   extern __shared__ u64 stage[];
   __shared__ PassShared<kBits> sh;
-  begin_tile<kBits>(sh, ticket);
+  begin_tile<kBits>(sh, hist, ticket);
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint64_t t0 = (uint64_t)sh.tile * kTile + warp * 32u * kItems;
   u64 xr[kItems];
@@ -511,7 +443,7 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
     xr[r] = i < n ? in[i] : 0ull;
     valid |= i < n ? 1u << r : 0u;
   }
-  rank_and_write<kBits, T>(xr, valid, shift, digit_start, status, out, sh, stage, err);
+  rank_and_write<kBits, T>(xr, valid, shift, status, out, sh, stage, err);
 }
 
 // ---------------------------------------------------------------- dedupe
@@ -840,13 +772,6 @@ __global__ void __launch_bounds__(kDThreads, 3)
   }
 }
 
-// Entries of each gene's vector: what its cursor passed.
-__global__ void k_vector_lengths(const uint32_t* __restrict__ cursor, const uint32_t* __restrict__ win_off,
-                                 uint32_t n_genes, uint32_t* __restrict__ mv_n) {
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x)
-    mv_n[g] = cursor[g] - win_off[g];
-}
-
 unsigned grid_for(uint64_t items, unsigned per_block, unsigned cap) {
   return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>((items + per_block - 1) / per_block, cap));
 }
@@ -879,15 +804,14 @@ cudaError_t with_bits(uint32_t bits, F f) {
 
 template <typename T>
 cudaError_t sort_passes(Launcher* L, const WindowSource& S, const SortKey& K, uint64_t n, uint8_t* scratch,
-                        const SortScratch& X, const u64* digit_start, u64* a, u64* b, u64** sorted, DevErr* err,
-                        cudaStream_t s) {
+                        const SortScratch& X, u64* a, u64* b, u64** sorted, DevErr* err, cudaStream_t s) {
   const size_t smem = (size_t)kTile * sizeof(u64);
   uint32_t* ticket = (uint32_t*)(scratch + X.tickets);
   u64 *src = a, *dst = a;
   for (uint32_t p = 0; p < K.passes; ++p) {
     const uint32_t shift = K.gene_bits + p * K.width;
     T* status = (T*)(scratch + X.pass[p]);
-    const u64* start = digit_start + p * kMaxBins;
+    const uint32_t* hist = (const uint32_t*)(scratch + X.hist) + p * kMaxBins;
     const cudaError_t e = with_bits(pass_bits(K, p), [&](auto w) -> cudaError_t {
       constexpr int kBits = decltype(w)::value;
       cudaError_t e1;
@@ -896,14 +820,14 @@ cudaError_t sort_passes(Launcher* L, const WindowSource& S, const SortKey& K, ui
         auto kernel = K.total_bits <= 32 ? k_sort_windows<kBits, T, uint32_t> : k_sort_windows<kBits, T, u64>;
         if ((e1 = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
           return e1;
-        PD_LAUNCH(L, "sort_windows", kernel<<<sort_tiles(S.n_windows), kThreads, smem, s>>>(S, K, start, status,
+        PD_LAUNCH(L, "sort_windows", kernel<<<sort_tiles(S.n_windows), kThreads, smem, s>>>(S, K, hist, status,
                                                                                             ticket + p, dst, err));
       } else {
         if ((e1 = cudaFuncSetAttribute(k_sort_records<kBits, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem)) != cudaSuccess)
           return e1;
         PD_LAUNCH(L, "sort_records", k_sort_records<kBits, T><<<sort_tiles(n), kThreads, smem, s>>>(
-                                         src, n, shift, start, status, ticket + p, dst, err));
+                                         src, n, shift, hist, status, ticket + p, dst, err));
       }
       return cudaSuccess;
     });
@@ -955,9 +879,11 @@ SortScratch sort_scratch(const SortKey& K, uint64_t n) {
 }
 
 cudaError_t run_gene_windows(Launcher* L, const int64_t* gene_ptr, uint32_t n_genes, uint64_t n_res, int check_end,
-                             int k, uint32_t* La, DevErr* err, cudaStream_t s) {
+                             int k, const int32_t* genome_ptr, uint32_t n_genomes, uint32_t* La, uint16_t* gene_genome,
+                             uint32_t* ginfo, uint32_t* minhash, DevErr* err, cudaStream_t s) {
   PD_LAUNCH(L, "gene_windows", k_gene_windows<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(
-                                   gene_ptr, n_genes, n_res, check_end, k, La, err));
+                                   gene_ptr, n_genes, n_res, check_end, k, genome_ptr, n_genomes, La, gene_genome,
+                                   ginfo, minhash, err));
   return cudaSuccess;
 }
 
@@ -973,9 +899,9 @@ cudaError_t run_check_letters(Launcher* L, const uint8_t* res, uint64_t n_res, c
 }
 
 cudaError_t run_tile_genes(Launcher* L, const uint32_t* win_off, uint32_t n_genes, uint64_t n_windows,
-                           uint32_t* tile_gene, cudaStream_t s) {
+                           uint32_t* tile_gene, uint32_t* cursor, cudaStream_t s) {
   PD_LAUNCH(L, "tile_genes", k_tile_genes<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(
-                                 win_off, n_genes, sort_tiles(n_windows), tile_gene));
+                                 win_off, n_genes, sort_tiles(n_windows), tile_gene, cursor));
   return cudaSuccess;
 }
 
@@ -994,20 +920,18 @@ void launch_code_hist(const WindowSource& S, const SortKey& K, uint32_t n_tiles,
 }  // namespace
 
 cudaError_t run_code_hist(Launcher* L, const WindowSource& S, const SortKey& K, uint8_t* scratch,
-                          const SortScratch& X, u64* digit_start, u64* total, uint32_t* minhash, cudaStream_t s) {
+                          const SortScratch& X, uint32_t* minhash, cudaStream_t s) {
   const uint32_t n_tiles = sort_tiles(S.n_windows);
   uint32_t* hist = (uint32_t*)(scratch + X.hist);
   PD_LAUNCH(L, "code_hist", (K.total_bits <= 32 ? launch_code_hist<uint32_t>(S, K, n_tiles, hist, minhash, s)
                                                 : launch_code_hist<u64>(S, K, n_tiles, hist, minhash, s)));
-  PD_LAUNCH(L, "digit_starts", k_digit_starts<<<K.passes, kMaxBins, 0, s>>>(hist, digit_start, total));
   return cudaSuccess;
 }
 
 cudaError_t run_sort(Launcher* L, const WindowSource& S, const SortKey& K, uint64_t n, uint8_t* scratch,
-                     const SortScratch& X, const u64* digit_start, u64* a, u64* b, u64** sorted, DevErr* err,
-                     cudaStream_t s) {
-  return X.wide ? sort_passes<u64>(L, S, K, n, scratch, X, digit_start, a, b, sorted, err, s)
-                : sort_passes<uint32_t>(L, S, K, n, scratch, X, digit_start, a, b, sorted, err, s);
+                     const SortScratch& X, u64* a, u64* b, u64** sorted, DevErr* err, cudaStream_t s) {
+  return X.wide ? sort_passes<u64>(L, S, K, n, scratch, X, a, b, sorted, err, s)
+                : sort_passes<uint32_t>(L, S, K, n, scratch, X, a, b, sorted, err, s);
 }
 
 cudaError_t run_dedupe(Launcher* L, const u64* rec, uint64_t n, const SortKey& K, uint8_t* scratch,
@@ -1042,13 +966,6 @@ cudaError_t run_lists(Launcher* L, const u64* rec, uint64_t n, const SortKey& K,
   PD_LAUNCH(L, "lists", k_lists<<<std::min(nt, 152u * 3u), kDThreads, smem, s>>>(
                             tile_e, tile_id, nt, rec, n, K, code_lo, code_hi, post, post_ptr, cnt_bits, cnt_cap,
                             genome_ptr, n_genomes, n_genes, table_bits, cursor, mv, max_list, join));
-  return cudaSuccess;
-}
-
-cudaError_t run_vector_lengths(Launcher* L, const uint32_t* cursor, const uint32_t* win_off, uint32_t n_genes,
-                               uint32_t* mv_n, cudaStream_t s) {
-  PD_LAUNCH(L, "vector_lengths",
-            k_vector_lengths<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(cursor, win_off, n_genes, mv_n));
   return cudaSuccess;
 }
 

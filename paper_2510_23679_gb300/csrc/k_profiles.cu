@@ -162,10 +162,15 @@ __device__ __forceinline__ uint32_t order_bucket(uint32_t minhash, uint32_t La, 
   return (lb << 14) | (h >> 18);
 }
 
+// Also the length of every gene's vector: what its cursor passed.
 __global__ void k_order_count(const uint32_t* __restrict__ minhash, const uint32_t* __restrict__ La, uint32_t n_genes,
-                              int length_buckets, uint32_t* __restrict__ count) {
-  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x)
+                              int length_buckets, const uint32_t* __restrict__ cursor,
+                              const uint32_t* __restrict__ win_off, uint32_t* __restrict__ mv_n,
+                              uint32_t* __restrict__ count) {
+  for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x) {
     atomicAdd(&count[order_bucket(minhash[g], La[g], length_buckets)], 1u);
+    mv_n[g] = cursor[g] - win_off[g];
+  }
 }
 
 __global__ void k_order_scatter(const uint32_t* __restrict__ minhash, const uint32_t* __restrict__ La,
@@ -173,17 +178,6 @@ __global__ void k_order_scatter(const uint32_t* __restrict__ minhash, const uint
                                 uint32_t* __restrict__ order) {
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x)
     order[atomicAdd(&cursor[order_bucket(minhash[g], La[g], length_buckets)], 1u)] = g;
-}
-
-// ------------------------------------------------------------ small helpers
-__global__ void k_gene_info(const int32_t* __restrict__ genome_ptr, uint32_t n_genomes,
-                            const uint32_t* __restrict__ La, uint16_t* __restrict__ gene_genome,
-                            uint32_t* __restrict__ ginfo) {
-  for (uint32_t i = blockIdx.x; i < n_genomes; i += gridDim.x)
-    for (int32_t g = genome_ptr[i] + (int32_t)threadIdx.x; g < genome_ptr[i + 1]; g += blockDim.x) {
-      gene_genome[g] = (uint16_t)i;
-      ginfo[g] = La[g] | (i << 16);
-    }
 }
 
 // ------------------------------------------------------------ export
@@ -327,21 +321,14 @@ cudaError_t run_mv_build(Launcher* L, const uint8_t* res, const int64_t* gene_pt
 uint32_t mv_build_table_cap(uint32_t La) { return mv_table_cap(La); }
 
 cudaError_t run_order(Launcher* L, const uint32_t* minhash, const uint32_t* La, uint32_t n_genes, int length_buckets,
-                      uint32_t* count, uint32_t* order, void* scan_tmp, cudaStream_t s) {
-  PD_LAUNCH(L, "order_count", k_order_count<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(minhash, La, n_genes,
-                                                                                            length_buckets, count));
+                      const uint32_t* cursor, const uint32_t* win_off, uint32_t* mv_n, uint32_t* count,
+                      uint32_t* order, void* scan_tmp, cudaStream_t s) {
+  PD_LAUNCH(L, "order_count", k_order_count<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(
+                                  minhash, La, n_genes, length_buckets, cursor, win_off, mv_n, count));
   cudaError_t e = scan_u32(L, count, kOrderBuckets, count + kOrderBuckets, scan_tmp, s);  // n + 1 prefix entries
   if (e != cudaSuccess) return e;
   PD_LAUNCH(L, "order_scatter", k_order_scatter<<<grid_for(n_genes, 256, 152u * 8u), 256, 0, s>>>(
                                     minhash, La, n_genes, length_buckets, count + kOrderBuckets, order));
-  return cudaSuccess;
-}
-
-cudaError_t run_gene_info(Launcher* L, const int32_t* genome_ptr, uint32_t n_genomes, const uint32_t* La,
-                          uint16_t* gene_genome, uint32_t* ginfo, cudaStream_t s) {
-  PD_LAUNCH(L, "gene_info",
-            k_gene_info<<<grid_for(n_genomes, 1, 152u * 8u), 256, 0, s>>>(genome_ptr, n_genomes, La, gene_genome,
-                                                                         ginfo));
   return cudaSuccess;
 }
 

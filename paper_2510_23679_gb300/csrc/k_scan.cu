@@ -1,16 +1,18 @@
-// k_scan.cu -- device-wide exclusive prefix sums (reduce, spine, down-sweep).
+// k_scan.cu -- device-wide exclusive prefix sums in one launch.
 //
-// Used for: rank bases of the k-mer dictionary blocks (dense ids), posting-list offsets
-// from per-id counts, and Best Hit / BBH row offsets.  Three launches: each
-// tile of kTile elements is reduced, the tile sums are scanned by one block,
-// and each tile is rescanned with its offset.  Loads are striped over the
-// block (coalesced); partial sums are 64-bit.
+// Used for window offsets, rank bases of the k-mer dictionary blocks, query
+// order buckets, and Best Hit / BBH row offsets.  A tile of kTile elements is
+// one block; tiles get the sum of those before them by decoupled look-back (see
+// pd_internal.cuh), so a scan is one launch and one memset of its status words
+// (nothing but the launch for a single tile) where reduce, spine and down-sweep
+// were three.  Loads are striped over each warp's run (coalesced); sums are
+// 64-bit.
 #include "pd_internal.cuh"
 
 namespace pdg {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256, kWarps = kThreads / 32;
 constexpr int kItems = 16;
 constexpr uint64_t kTile = (uint64_t)kThreads * kItems;
 
@@ -22,27 +24,6 @@ __device__ __forceinline__ unsigned long long warp_incl_u64(unsigned long long v
     if (lane >= (uint32_t)o) v += y;
   }
   return v;
-}
-
-// Exclusive scan over the block; returns the prefix and writes the total.
-__device__ __forceinline__ unsigned long long block_excl_u64(unsigned long long v, unsigned long long* tmp,
-                                                             unsigned long long* total) {
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  constexpr uint32_t n_warps = kThreads / 32;
-  unsigned long long inc = warp_incl_u64(v);
-  if (lane == 31) tmp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    unsigned long long w = (lane < n_warps) ? tmp[lane] : 0ull;
-    unsigned long long wi = warp_incl_u64(w);
-    if (lane < n_warps) tmp[lane] = wi - w;
-    if (lane == n_warps - 1) tmp[n_warps] = wi;
-  }
-  __syncthreads();
-  unsigned long long r = tmp[warp] + inc - v;
-  *total = tmp[n_warps];
-  __syncthreads();
-  return r;
 }
 
 // Set bits of dictionary block i (its words 1..7; word 0 receives the scan).
@@ -61,86 +42,80 @@ struct U32In {
   __device__ __forceinline__ unsigned long long operator()(uint64_t i) const { return a[i]; }
 };
 
-template <typename In>
-__global__ void __launch_bounds__(kThreads) k_scan_reduce(In in, uint64_t n, unsigned long long* partial) {
-  __shared__ unsigned long long tmp[kThreads / 32 + 1];
-  const uint64_t base = (uint64_t)blockIdx.x * kTile;
-  unsigned long long sum = 0;
-#pragma unroll 4
+// out[i * stride] = sum of in(0..i-1); out[n * stride] = the total if
+// write_last; *total_dst = the total if not null.  In and out may be the same
+// array (a tile's inputs are read before its outputs are written).
+template <typename In, typename Out, typename Total>
+__global__ void __launch_bounds__(kThreads)
+    k_scan(In in, uint64_t n, Out* out, int write_last, Total* total_dst, uint32_t stride,
+           unsigned long long* status, uint32_t* ticket, DevErr* err) {
+  using S = Status<unsigned long long>;
+  __shared__ unsigned long long wsum[kWarps + 1], s_before;
+  __shared__ uint32_t s_tile;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) s_tile = gridDim.x > 1 ? atomicAdd(ticket, 1u) : 0u;
+  __syncthreads();
+  const uint32_t tile = s_tile;
+  const uint64_t base = (uint64_t)tile * kTile + (uint64_t)warp * (32 * kItems) + lane;
+  unsigned long long v[kItems], run = 0;
+#pragma unroll
+  for (int r = 0; r < kItems; ++r) v[r] = base + r * 32 < n ? in(base + r * 32) : 0ull;
+#pragma unroll
   for (int r = 0; r < kItems; ++r) {
-    uint64_t i = base + (uint64_t)r * kThreads + threadIdx.x;
-    if (i < n) sum += in(i);
+    const unsigned long long inc = warp_incl_u64(v[r]);
+    const unsigned long long sum = __shfl_sync(0xffffffffu, inc, 31);
+    v[r] = run + inc - v[r];
+    run += sum;
   }
-  unsigned long long total;
-  block_excl_u64(sum, tmp, &total);
-  if (threadIdx.x == 0) partial[blockIdx.x] = total;
-}
-
-// One block scans the tile sums in place (exclusive) and stores the total.
-__global__ void __launch_bounds__(kThreads) k_scan_spine(unsigned long long* partial, uint64_t nb,
-                                                         unsigned long long* total_out) {
-  __shared__ unsigned long long tmp[kThreads / 32 + 1];
-  unsigned long long carry = 0;
-  for (uint64_t c = 0; c < nb; c += kThreads) {
-    uint64_t i = c + threadIdx.x;
-    unsigned long long v = (i < nb) ? partial[i] : 0ull;
-    unsigned long long tot;
-    unsigned long long ex = block_excl_u64(v, tmp, &tot);
-    if (i < nb) partial[i] = carry + ex;
-    carry += tot;
+  if (lane == 31) wsum[warp] = run;
+  __syncthreads();
+  if (warp == 0) {
+    const unsigned long long w = lane < kWarps ? wsum[lane] : 0ull;
+    const unsigned long long inc = warp_incl_u64(w);
+    const unsigned long long all = __shfl_sync(0xffffffffu, inc, 31);
+    unsigned long long before = 0;
+    if (gridDim.x > 1) {
+      volatile unsigned long long* st = status;
+      if (tile == 0) {
+        if (lane == 0) st[0] = S::kInclusive | all;
+      } else {
+        if (lane == 0) st[tile] = S::kAggregate | all;
+        if (!look_back_warp(st, tile, &before, err)) {  // reported; offsets stay in range
+          if (lane == 0) raise_error(err, PD_ERR_INTERNAL, tile);
+          before = 0;
+        }
+        if (lane == 0) st[tile] = S::kInclusive | (before + all);
+      }
+    }
+    __syncwarp();
+    if (lane < kWarps) wsum[lane] = inc - w;
+    if (lane == 0) {
+      s_before = before;
+      if (tile == gridDim.x - 1) {
+        if (write_last) out[n * stride] = (Out)(before + all);
+        if (total_dst) *total_dst = (Total)(before + all);
+      }
+    }
   }
-  if (threadIdx.x == 0) *total_out = carry;
+  __syncthreads();
+  const unsigned long long off = s_before + wsum[warp];
+#pragma unroll
+  for (int r = 0; r < kItems; ++r)
+    if (base + r * 32 < n) out[(base + r * 32) * stride] = (Out)(off + v[r]);
 }
 
-template <typename In, typename Out>
-__global__ void __launch_bounds__(kThreads) k_scan_down(In in, uint64_t n, const unsigned long long* partial,
-                                                        const unsigned long long* total, Out* out,
-                                                        int write_last, uint32_t stride) {
-  __shared__ unsigned long long tmp[kThreads / 32 + 1];
-  const uint64_t base = (uint64_t)blockIdx.x * kTile;
-  unsigned long long carry = partial[blockIdx.x];
-  for (int r = 0; r < kItems; ++r) {
-    uint64_t i = base + (uint64_t)r * kThreads + threadIdx.x;
-    if (base + (uint64_t)r * kThreads >= n) break;  // uniform across the block
-    unsigned long long v = (i < n) ? in(i) : 0ull;
-    unsigned long long tot;
-    unsigned long long ex = block_excl_u64(v, tmp, &tot);
-    if (i < n) out[i * stride] = (Out)(carry + ex);
-    carry += tot;
-  }
-  if (write_last && blockIdx.x == 0 && threadIdx.x == 0) out[n * stride] = (Out)(*total);
-}
-
-template <typename Out>
-__global__ void k_store_total(const unsigned long long* total, Out* dst) {
-  *dst = (Out)(*total);
-}
-
-// Exclusive scan of in(0..n-1) into out[i * stride] (and out[n * stride] =
-// total if write_last; *total_dst = total if not null).
 template <typename In, typename Out, typename Total = Out>
 cudaError_t scan_impl(Launcher* L, In in, uint64_t n, Out* out, int write_last, Total* total_dst, void* temp,
                       cudaStream_t s, uint32_t stride = 1) {
   uint64_t nb = (n + kTile - 1) / kTile;
   if (nb == 0) nb = 1;
-  unsigned long long* partial = (unsigned long long*)temp;
-  unsigned long long* total = partial + nb;
+  unsigned long long* status = (unsigned long long*)temp;
   cudaError_t e;
-  if ((e = launch_begin(L, "scan_reduce")) != cudaSuccess) return e;
-  k_scan_reduce<In><<<(unsigned)nb, kThreads, 0, s>>>(in, n, partial);
-  if ((e = launch_end(L, "scan_reduce")) != cudaSuccess) return e;
-  if ((e = launch_begin(L, "scan_spine")) != cudaSuccess) return e;
-  k_scan_spine<<<1, kThreads, 0, s>>>(partial, nb, total);
-  if ((e = launch_end(L, "scan_spine")) != cudaSuccess) return e;
-  if ((e = launch_begin(L, "scan_down")) != cudaSuccess) return e;
-  k_scan_down<In, Out><<<(unsigned)nb, kThreads, 0, s>>>(in, n, partial, total, out, write_last, stride);
-  if ((e = launch_end(L, "scan_down")) != cudaSuccess) return e;
-  if (total_dst) {
-    if ((e = launch_begin(L, "scan_total")) != cudaSuccess) return e;
-    k_store_total<Total><<<1, 1, 0, s>>>(total, total_dst);
-    if ((e = launch_end(L, "scan_total")) != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  if (nb > 1 && (e = cudaMemsetAsync(temp, 0, (nb + 1) * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+  if ((e = launch_begin(L, "scan")) != cudaSuccess) return e;
+  k_scan<In, Out, Total><<<(unsigned)nb, kThreads, 0, s>>>(in, n, out, write_last, total_dst, stride, status,
+                                                          (uint32_t*)(status + nb), launch_err(L));
+  return launch_end(L, "scan");
 }
 
 }  // namespace

@@ -13,6 +13,8 @@
 // (the stored maxima and the ties that equal them, ascending) followed by its
 // forward Best Hits in the genomes after its own -- ascending overall, since
 // genes are numbered genome by genome.
+#include <algorithm>
+
 #include "pd_internal.cuh"
 
 namespace pdg {
@@ -25,13 +27,16 @@ __device__ __forceinline__ void unpack(unsigned long long w, uint32_t* s, uint32
 }
 
 // One thread per gene: stored maxima of the genomes before its own (the
-// maxima are genome-major, so neighbouring threads read neighbouring words).
-__global__ void __launch_bounds__(256) k_sym_count(SymRows R, uint32_t* __restrict__ stored) {
+// maxima are genome-major, so neighbouring threads read neighbouring words),
+// and the length of its row (tiecnt null: no ties).
+__global__ void __launch_bounds__(256) k_sym_count(SymRows R, const uint32_t* __restrict__ tiecnt,
+                                                   uint32_t* __restrict__ stored, uint32_t* __restrict__ total) {
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < R.n_genes; b += gridDim.x * blockDim.x) {
     const uint32_t gb = R.gene_genome[b];
     uint32_t n = 0;
     for (uint32_t g = 0; g < gb; ++g) n += R.symbest[(size_t)g * R.n_genes + b] != 0ull ? 1u : 0u;
     stored[b] = n;
+    total[b] = n + (tiecnt ? tiecnt[b] : 0u) + R.fwd_len[b];
   }
 }
 
@@ -52,7 +57,8 @@ __device__ __forceinline__ bool first_insert(unsigned long long* keys, unsigned 
 // One thread per tie (b << 32 | a, s): valid when its ratio equals the final
 // stored maximum of (b, genome of a), it is not the stored pair itself, and
 // it is the first record of the pair (a query that a tier hands to the next
-// after its Best Hit passes records its ties again).
+// after its Best Hit passes records its ties again).  Genes with valid ties are
+// listed.
 __global__ void k_sym_ties(SymRows R, uint32_t* __restrict__ tiecnt, uint8_t* __restrict__ tie_ok) {
   for (unsigned long long t = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; t < R.n_ties;
        t += (unsigned long long)gridDim.x * blockDim.x) {
@@ -64,14 +70,8 @@ __global__ void k_sym_ties(SymRows R, uint32_t* __restrict__ tiecnt, uint8_t* __
     const bool ok = w != 0ull && ma != a && ratio_equal(s, R.La[a] + R.La[b] - s, ms, md) &&
                     first_insert(R.tie_set, R.tie_set_mask, r);
     tie_ok[t] = ok ? 1 : 0;
-    if (ok) atomicAdd(&tiecnt[b], 1u);
+    if (ok && atomicAdd(&tiecnt[b], 1u) == 0u) R.tie_gene[atomicAdd(R.n_tie_genes, 1u)] = b;
   }
-}
-
-__global__ void k_sym_total(SymRows R, const uint32_t* __restrict__ stored, const uint32_t* __restrict__ tiecnt,
-                            uint32_t* __restrict__ total) {
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < R.n_genes; b += gridDim.x * blockDim.x)
-    total[b] = stored[b] + tiecnt[b] + R.fwd_len[b];
 }
 
 // One thread per gene: the stored maxima in genome order.
@@ -95,13 +95,18 @@ __global__ void __launch_bounds__(256)
 
 // The same through shared memory, for datasets of at most kRevTileGenomes
 // genomes: a block reads the maxima of 32 consecutive genes genome by genome
-// (coalesced) into a tile, then one warp per gene writes its row part
-// (coalesced).  Genes are numbered genome by genome, so the tile's last gene
-// has the largest genome of the 32.
+// (coalesced) into a tile, then one warp per gene writes its reverse part and,
+// if asked to, its forward part (coalesced), leaving room for its ties between.  Genes
+// are numbered genome by genome, so the tile's last gene has the largest genome
+// of the 32.
 constexpr uint32_t kRevTileGenomes = 372;  // 372 x 33 x 8 bytes < 96 KB of shared memory
+// Up to this many genomes (16 KB of tile) a launch writes the forward parts too
+// (50 genomes: 43 against 56 us); past it the tile leaves few blocks per SM to
+// copy with, and they get a launch of their own (200: 0.83 against 1.07 ms).
+constexpr uint32_t kRowTileGenomes = 62;
 __global__ void __launch_bounds__(256)
-    k_sym_write_rev_tile(SymRows R, const unsigned long long* __restrict__ row_ptr, uint32_t* __restrict__ out_b,
-                         uint32_t* __restrict__ out_s) {
+    k_sym_write_tile(SymRows R, const uint32_t* __restrict__ tiecnt, const unsigned long long* __restrict__ row_ptr,
+                     int forward, uint32_t* __restrict__ out_b, uint32_t* __restrict__ out_s) {
   extern __shared__ unsigned long long tile[];  // [genome][33]
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   for (uint32_t b0 = blockIdx.x * 32u; b0 < R.n_genes; b0 += gridDim.x * 32u) {
@@ -126,13 +131,21 @@ __global__ void __launch_bounds__(256)
         }
         at += __popc(m);
       }
+      if (!forward) continue;
+      if (tiecnt) at += tiecnt[b];
+      const unsigned long long fo = R.fwd_off[b];
+      const uint32_t fl = R.fwd_len[b];
+      for (uint32_t e = lane; e < fl; e += 32) {
+        out_b[at + e] = R.fwd_b[fo + e];
+        out_s[at + e] = R.fwd_s[fo + e];
+      }
     }
     __syncthreads();
   }
 }
 
 // One warp per gene: the forward part, after the stored maxima and room for
-// the gene's ties.
+// the gene's ties (tiecnt null: none).
 __global__ void __launch_bounds__(256)
     k_sym_write(SymRows R, const uint32_t* __restrict__ stored, const uint32_t* __restrict__ tiecnt,
                 const unsigned long long* __restrict__ row_ptr, uint32_t* __restrict__ out_b,
@@ -141,7 +154,7 @@ __global__ void __launch_bounds__(256)
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < R.n_genes; b += warps) {
     const unsigned long long base = row_ptr[b];
-    const unsigned long long fwd = base + stored[b] + tiecnt[b];
+    const unsigned long long fwd = base + stored[b] + (tiecnt ? tiecnt[b] : 0u);
     const unsigned long long fo = R.fwd_off[b];
     const uint32_t fl = R.fwd_len[b];
     for (uint32_t e = lane; e < fl; e += 32) {
@@ -166,27 +179,67 @@ __global__ void k_sym_put_ties(SymRows R, const uint8_t* __restrict__ tie_ok, co
   }
 }
 
-// One thread per gene with ties: insertion sort of its reverse part by gene
-// id (ties are exact equalities of two ratios, so such parts are rare).
-__global__ void k_sym_sort_ties(uint32_t n_genes, const uint32_t* __restrict__ stored,
-                                const uint32_t* __restrict__ tiecnt, const unsigned long long* __restrict__ row_ptr,
-                                uint32_t* __restrict__ out_b, uint32_t* __restrict__ out_s) {
-  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < n_genes; b += gridDim.x * blockDim.x) {
-    if (tiecnt[b] == 0) continue;
-    const uint32_t n = stored[b] + tiecnt[b];
+// One warp per gene with ties: its reverse part sorted by gene id.  The stored
+// maxima are ascending already, so an entry's place is its index among them
+// plus the ties below it, a tie's the stored below it (bisection) plus the ties
+// below it.  The part is read before it is written, at most kTieLanes entries a
+// lane; a longer part falls back to an insertion sort by one lane.
+constexpr uint32_t kTieLanes = 16;
+__global__ void __launch_bounds__(256)
+    k_sym_sort_ties(SymRows R, const uint32_t* __restrict__ stored, const uint32_t* __restrict__ tiecnt,
+                    const unsigned long long* __restrict__ row_ptr, uint32_t* __restrict__ out_b,
+                    uint32_t* __restrict__ out_s) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t n_listed = *R.n_tie_genes;
+  for (uint32_t x0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; x0 < n_listed; x0 += warps) {
+    const uint32_t b = R.tie_gene[x0];
+    const uint32_t ns = stored[b], nt = tiecnt[b], n = ns + nt;
     uint32_t* kb = out_b + row_ptr[b];
     uint32_t* ks = out_s + row_ptr[b];
-    for (uint32_t i = 1; i < n; ++i) {
-      const uint32_t x = kb[i], y = ks[i];
-      uint32_t j = i;
-      while (j > 0 && kb[j - 1] > x) {
-        kb[j] = kb[j - 1];
-        ks[j] = ks[j - 1];
-        --j;
+    if (n <= 32u * kTieLanes) {
+      uint32_t x[kTieLanes], y[kTieLanes], at[kTieLanes];
+#pragma unroll
+      for (uint32_t j = 0; j < kTieLanes; ++j) {
+        const uint32_t i = j * 32u + lane;
+        x[j] = y[j] = at[j] = 0;
+        if (i < n) {
+          x[j] = kb[i];
+          y[j] = ks[i];
+          uint32_t rank = i;  // a stored entry's index among the stored
+          if (i >= ns) {
+            uint32_t lo = 0, hi = ns;
+            while (lo < hi) {
+              const uint32_t mid = (lo + hi) >> 1;
+              if (kb[mid] < x[j]) lo = mid + 1; else hi = mid;
+            }
+            rank = lo;
+          }
+          for (uint32_t t = 0; t < nt; ++t) rank += kb[ns + t] < x[j] ? 1u : 0u;
+          at[j] = rank;
+        }
       }
-      kb[j] = x;
-      ks[j] = y;
+      __syncwarp();
+#pragma unroll
+      for (uint32_t j = 0; j < kTieLanes; ++j)
+        if (j * 32u + lane < n) {
+          kb[at[j]] = x[j];
+          ks[at[j]] = y[j];
+        }
+    } else if (lane == 0) {
+      for (uint32_t i = 1; i < n; ++i) {
+        const uint32_t x = kb[i], y = ks[i];
+        uint32_t j = i;
+        while (j > 0 && kb[j - 1] > x) {
+          kb[j] = kb[j - 1];
+          ks[j] = ks[j - 1];
+          --j;
+        }
+        kb[j] = x;
+        ks[j] = y;
+      }
     }
+    __syncwarp();
   }
 }
 
@@ -251,47 +304,50 @@ unsigned grid_of(uint64_t items, unsigned per_block, unsigned cap) {
 
 cudaError_t run_sym_count(Launcher* L, const SymRows& R, uint32_t* stored, uint32_t* tiecnt, uint8_t* tie_ok,
                           uint32_t* total, cudaStream_t s) {
-  cudaError_t e = launch_begin(L, "sym_count");
-  if (e != cudaSuccess) return e;
-  k_sym_count<<<grid_of((uint64_t)R.n_genes, 256, 152u * 16u), 256, 0, s>>>(R, stored);
-  if ((e = launch_end(L, "sym_count")) != cudaSuccess) return e;
+  cudaError_t e;
   if (R.n_ties) {
     if ((e = launch_begin(L, "sym_ties")) != cudaSuccess) return e;
     k_sym_ties<<<grid_of(R.n_ties, 256, 152u * 16u), 256, 0, s>>>(R, tiecnt, tie_ok);
     if ((e = launch_end(L, "sym_ties")) != cudaSuccess) return e;
   }
-  if ((e = launch_begin(L, "sym_total")) != cudaSuccess) return e;
-  k_sym_total<<<grid_of(R.n_genes, 256, 152u * 16u), 256, 0, s>>>(R, stored, tiecnt, total);
-  return launch_end(L, "sym_total");
+  if ((e = launch_begin(L, "sym_count")) != cudaSuccess) return e;
+  k_sym_count<<<grid_of((uint64_t)R.n_genes, 256, 152u * 16u), 256, 0, s>>>(R, R.n_ties ? tiecnt : nullptr, stored,
+                                                                            total);
+  return launch_end(L, "sym_count");
 }
 
 cudaError_t run_sym_write(Launcher* L, const SymRows& R, const uint32_t* stored, const uint32_t* tiecnt,
                           const uint8_t* tie_ok, const unsigned long long* row_ptr, uint32_t* tie_fill,
                           uint32_t* out_b, uint32_t* out_s, cudaStream_t s) {
-  cudaError_t e = launch_begin(L, "sym_write_rev");
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
+  const uint32_t* ties = R.n_ties ? tiecnt : nullptr;
+  const bool whole = R.n_genomes <= kRowTileGenomes;
+  if ((e = launch_begin(L, "sym_write_rev")) != cudaSuccess) return e;
   if (R.n_genomes <= kRevTileGenomes) {
     const size_t smem = (size_t)R.n_genomes * 33u * sizeof(unsigned long long);
-    if ((e = cudaFuncSetAttribute(k_sym_write_rev_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+    if ((e = cudaFuncSetAttribute(k_sym_write_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
         cudaSuccess)
       return e;
-    k_sym_write_rev_tile<<<grid_of((uint64_t)R.n_genes, 32, 152u * 8u), 256, smem, s>>>(R, row_ptr, out_b, out_s);
+    k_sym_write_tile<<<grid_of((uint64_t)R.n_genes, 32, 152u * 8u), 256, smem, s>>>(R, ties, row_ptr, whole, out_b,
+                                                                                    out_s);
   } else {
     k_sym_write_rev<<<grid_of((uint64_t)R.n_genes, 256, 152u * 16u), 256, 0, s>>>(R, row_ptr, out_b, out_s);
   }
   if ((e = launch_end(L, "sym_write_rev")) != cudaSuccess) return e;
-  if ((e = launch_begin(L, "sym_write")) != cudaSuccess) return e;
-  k_sym_write<<<grid_of((uint64_t)R.n_genes * 32, 256, 152u * 16u), 256, 0, s>>>(R, stored, tiecnt, row_ptr, out_b,
-                                                                                 out_s);
-  if ((e = launch_end(L, "sym_write")) != cudaSuccess) return e;
+  if (!whole) {
+    if ((e = launch_begin(L, "sym_write")) != cudaSuccess) return e;
+    k_sym_write<<<grid_of((uint64_t)R.n_genes * 32, 256, 152u * 16u), 256, 0, s>>>(R, stored, ties, row_ptr, out_b,
+                                                                                   out_s);
+    if ((e = launch_end(L, "sym_write")) != cudaSuccess) return e;
+  }
   if (R.n_ties == 0) return cudaSuccess;
   if ((e = launch_begin(L, "sym_put_ties")) != cudaSuccess) return e;
   k_sym_put_ties<<<grid_of(R.n_ties, 256, 152u * 16u), 256, 0, s>>>(R, tie_ok, stored, row_ptr, tie_fill, out_b,
                                                                       out_s);
   if ((e = launch_end(L, "sym_put_ties")) != cudaSuccess) return e;
   if ((e = launch_begin(L, "sym_sort_ties")) != cudaSuccess) return e;
-  k_sym_sort_ties<<<grid_of(R.n_genes, 256, 152u * 16u), 256, 0, s>>>(R.n_genes, stored, tiecnt, row_ptr, out_b,
-                                                                        out_s);
+  k_sym_sort_ties<<<grid_of(std::min<unsigned long long>(R.n_ties, R.n_genes) * 32, 256, 152u * 8u), 256, 0, s>>>(
+      R, stored, tiecnt, row_ptr, out_b, out_s);
   return launch_end(L, "sym_sort_ties");
 }
 

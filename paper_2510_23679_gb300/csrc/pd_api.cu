@@ -57,6 +57,8 @@ cudaError_t launch_end(Launcher* L, const char* name) {
   return cudaSuccess;
 }
 
+DevErr* launch_err(Launcher* L) { return L->ctx->d_err; }
+
 }  // namespace pdg
 
 // ------------------------------------------------------------------ internal accessors
@@ -277,7 +279,8 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
 
   // ---- genome offsets on the host (small; checked before any kernel reads them,
   // except on the non-segmented path with device offsets, where the checks
-  // come after the dictionary pass and before the first kernel that uses them)
+  // come with the first synchronisation and before the first kernel that relies
+  // on them)
   std::vector<int32_t> hgn(n_genomes + 1);
   const bool gp_dev = is_device_ptr(gene_ptr), gn_dev = is_device_ptr(genome_ptr);
   const bool early_genomes = !gn_dev || genome_seg;
@@ -341,11 +344,10 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   const bool copy_res = n_res > 0 && !is_device_ptr(residues);
   Carve ct;
   // zeroed words first: [0] windows, [1..4] postings and ids (so far, before the slice), [5] join, [6] longest
-  // list, [7] records of the slice; then the order's counts
+  // list; then the order's counts
   const size_t o_words = ct.add(8 * sizeof(unsigned long long)),
                o_ocount = ct.add(sizeof(uint32_t) * (2 * pdg::kOrderBuckets + 1)), zeroed = ct.bytes,
                o_minhash = ct.add(sizeof(uint32_t) * n_genes), o_cursor = ct.add(sizeof(uint32_t) * n_genes),
-               o_start = ct.add(sizeof(unsigned long long) * pdg::kDigitStarts),
                o_scan = ct.add(pdg::scan_temp_bytes(std::max<uint64_t>((uint64_t)n_genes + 1, pdg::kOrderBuckets)) + 64),
                o_gene_ptr = ct.add(gp_dev ? 0 : sizeof(int64_t) * (n_genes + 1)),
                o_code_base = ct.add(genome_seg ? sizeof(unsigned long long) * n_genomes : 0),
@@ -367,17 +369,15 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
     gp_devp = piece<int64_t>(tmp1, o_gene_ptr);
   }
   CK(cudaMemsetAsync(words, 0, zeroed, c->stream));
-  CK(cudaMemsetAsync(minhash, 0xFF, sizeof(uint32_t) * std::max<uint32_t>(n_genes, 1), c->stream));
   CK(cudaMemcpyAsync(d_genome_ptr, genome_ptr, sizeof(int32_t) * (n_genomes + 1), cudaMemcpyDefault, c->stream));
 
   // ---- offsets and letters checked, window offsets, genes' genomes
   if (n_genes)
-    CK(pdg::run_gene_windows(L, gp_devp, n_genes, n_res, gene_src ? 0 : 1, k, d_La, c->d_err, c->stream));
+    CK(pdg::run_gene_windows(L, gp_devp, n_genes, n_res, gene_src ? 0 : 1, k, d_genome_ptr, n_genomes, d_La,
+                             d_gene_genome, d_ginfo, minhash, c->d_err, c->stream));
   CK(pdg::scan_u32_total(L, d_La, n_genes, d_win_off, words, scan_tmp, c->stream));
   if (n_genes)
     CK(pdg::run_check_letters(L, res_dev, n_res, gp_devp, gene_src, n_genes, alphabet, c->d_err, c->stream));
-  if (early_genomes)
-    CK(pdg::run_gene_info(L, d_genome_ptr, n_genomes, d_La, d_gene_genome, d_ginfo, c->stream));
   unsigned long long* d_code_base = nullptr;
   if (genome_seg) {
     d_code_base = piece<unsigned long long>(tmp1, o_code_base);
@@ -391,10 +391,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   if (st != PD_OK) return st;
   const uint64_t W = hb[0];
   if (W > 0xFFFFFFF0ull) return fail(c, PD_ERR_ARG, "more than 2^32 k-mer windows in the dataset");
-  if (!early_genomes) {
-    if ((st = check_genomes()) != PD_OK) return st;
-    CK(pdg::run_gene_info(L, d_genome_ptr, n_genomes, d_La, d_gene_genome, d_ginfo, c->stream));
-  }
+  if (!early_genomes && (st = check_genomes()) != PD_OK) return st;
   P->h_genome_ptr = hgn;
 
   // ---- vectors, postings, and one record buffer that ends up holding the
@@ -408,9 +405,11 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   uint32_t *d_post = piece<uint32_t>(P->windows, o_post), *d_post_ptr = piece<uint32_t>(P->windows, o_lists);
   uint32_t* d_code_lo = d_post_ptr + (W + 1);
   uint8_t* d_code_hi = wide_codes ? piece<uint8_t>(P->windows, o_code_hi) : nullptr;
+  uint32_t* cursor = piece<uint32_t>(tmp1, o_cursor);
   if (W == 0) {
     CK(cudaMemsetAsync(d_post_ptr, 0, sizeof(uint32_t), c->stream));
-    if (n_genes) CK(cudaMemsetAsync(d_mv_n, 0, sizeof(uint32_t) * n_genes, c->stream));
+    if (n_genes)
+      CK(cudaMemcpyAsync(cursor, d_win_off, sizeof(uint32_t) * n_genes, cudaMemcpyDeviceToDevice, c->stream));
   } else {
     const pdg::SortScratch X = pdg::sort_scratch(K, W);
     const uint32_t n_dtiles = pdg::dedupe_tiles(W);
@@ -423,22 +422,22 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
     uint32_t *tile_e = piece<uint32_t>(tmp2, o_tile_e), *tile_id = piece<uint32_t>(tmp2, o_tile_id);
     pdg::WindowSource S{res_dev, gp_devp, gene_src, d_win_off, piece<uint32_t>(tmp2, o_tile_gene), d_gene_genome,
                         d_code_base, k, alphabet, W};
-    CK(pdg::run_tile_genes(L, d_win_off, n_genes, W, piece<uint32_t>(tmp2, o_tile_gene), c->stream));
     // two record buffers, one of which ends up holding lists and codes
     unsigned long long *rec = piece<unsigned long long>(tmp2, o_rec), *other = (unsigned long long*)d_post_ptr;
     const bool odd = K.passes & 1u;
-    unsigned long long* start = piece<unsigned long long>(tmp1, o_start);
-    uint32_t* cursor = piece<uint32_t>(tmp1, o_cursor);
-    CK(cudaMemcpyAsync(cursor, d_win_off, sizeof(uint32_t) * n_genes, cudaMemcpyDeviceToDevice, c->stream));
+    CK(pdg::run_tile_genes(L, d_win_off, n_genes, W, piece<uint32_t>(tmp2, o_tile_gene), cursor, c->stream));
     Buf slice_rec;
     for (K.slice = 0; K.slice < K.n_slices; ++K.slice) {
       CK(cudaMemsetAsync(scratch, 0, X.bytes, c->stream));
-      CK(pdg::run_code_hist(L, S, K, scratch, X, start, words + 7, K.slice ? nullptr : minhash, c->stream));
+      CK(pdg::run_code_hist(L, S, K, scratch, X, K.slice ? nullptr : minhash, c->stream));
       uint64_t n = W;
       if (K.n_slices > 1) {
-        CK(cudaMemcpyAsync(hb, words + 7, sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+        std::vector<uint32_t> hist(pdg::kSortBins);  // of the first pass: the slice's records
+        CK(cudaMemcpyAsync(hist.data(), scratch + X.hist, sizeof(uint32_t) * hist.size(), cudaMemcpyDeviceToHost,
+                           c->stream));
         CK(cudaStreamSynchronize(c->stream));
-        n = hb[0];
+        n = 0;
+        for (uint32_t x : hist) n += x;
         if (n == 0) continue;
         // the memory above holds what the slices before left: records of their own
         ALLOC(slice_rec, 2 * sizeof(unsigned long long) * n);
@@ -446,21 +445,19 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
         other = rec + n;
       }
       unsigned long long* sorted = nullptr;
-      CK(pdg::run_sort(L, S, K, n, scratch, X, start, odd ? rec : other, odd ? other : rec, &sorted, c->d_err,
-                       c->stream));
+      CK(pdg::run_sort(L, S, K, n, scratch, X, odd ? rec : other, odd ? other : rec, &sorted, c->d_err, c->stream));
       CK(pdg::run_dedupe(L, sorted, n, K, scratch, X, cnt_bits, cnt_cap, words + 1, d_post, d_post_ptr, d_code_lo,
                          d_code_hi, tile_e, tile_id, c->d_err, c->stream));
       CK(pdg::run_lists(L, sorted, n, K, tile_e, tile_id, d_post, d_post_ptr, d_code_lo, d_code_hi, cnt_bits, cnt_cap,
                         d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5, c->stream));
     }
     if (K.n_slices > 1) CK(cudaStreamSynchronize(c->stream));  // the last slice's records end here
-    CK(pdg::run_vector_lengths(L, cursor, d_win_off, n_genes, d_mv_n, c->stream));
   }
 
   // ---- all-pairs query order: min-hash buckets
   if (n_genes)
-    CK(pdg::run_order(L, minhash, d_La, n_genes, length_buckets, piece<uint32_t>(tmp1, o_ocount), d_order, scan_tmp,
-                      c->stream));
+    CK(pdg::run_order(L, minhash, d_La, n_genes, length_buckets, cursor, d_win_off, d_mv_n,
+                      piece<uint32_t>(tmp1, o_ocount), d_order, scan_tmp, c->stream));
   CK(cudaMemcpyAsync(hb, words, 7 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
   st = check_dev_err(c);  // synchronizes; temporaries are released after this
   if (st != PD_OK) return st;
@@ -689,23 +686,26 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
   else
     cap = (uint64_t)nq * 4 + 4096;
   if (emit_all) cap = (uint64_t)nq * 64 + 4096;
-  Buf counters, def0, def1, def2;
-  ALLOC(counters, 5 * sizeof(unsigned long long));
-  ALLOC(def0, sizeof(uint32_t) * std::max<uint32_t>(nq, 1));
+  // counters: [0] hits, [1] postings walked, [2], [3] deferred by tiers 1 and 2, [4] deferred by the warp tier and
+  // its ticket, [5] ties of the symmetric form; then the lists of deferred queries
+  constexpr size_t kCounters = 6;
+  Carve ct;
+  const size_t o_cnt = ct.add(kCounters * sizeof(unsigned long long)), o_def0 = ct.add(sizeof(uint32_t) * nq),
+               o_def1 = ct.add(sizeof(uint32_t) * nq), o_def2 = ct.add(sizeof(uint32_t) * nq);
+  Buf tmp;
+  ALLOC(tmp, ct.bytes);
   ALLOC(H->row_off, sizeof(unsigned long long) * std::max<uint32_t>(n_rows, 1));
   ALLOC(H->row_len, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1));
-  ALLOC(def1, sizeof(uint32_t) * std::max<uint32_t>(nq, 1));
-  ALLOC(def2, sizeof(uint32_t) * std::max<uint32_t>(nq, 1));
+  unsigned long long* cnt = piece<unsigned long long>(tmp, o_cnt);
   for (int attempt = 0; attempt < 3; ++attempt) {
     ALLOC(H->out_b, sizeof(uint32_t) * cap);
     ALLOC(H->out_s, sizeof(uint32_t) * cap);
-    CK(cudaMemsetAsync(counters.p, 0, 5 * sizeof(unsigned long long), c->stream));
-    CK(cudaMemsetAsync(H->row_len.p, 0, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1), c->stream));
-    if (Q.symbest) {  // a rerun starts the reverse maxima and their tie list afresh
+    CK(cudaMemsetAsync(cnt, 0, kCounters * sizeof(unsigned long long), c->stream));
+    // rows that no query writes (all-pairs rows are the dataset's genes)
+    if (Q.all_pairs && (nq != n_rows || Q.n_shards))
+      CK(cudaMemsetAsync(H->row_len.p, 0, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1), c->stream));
+    if (Q.symbest)  // a rerun starts the reverse maxima and their tie list afresh
       CK(cudaMemsetAsync(Q.symbest, 0, sizeof(unsigned long long) * v.n_genes * v.n_genomes, c->stream));
-      CK(cudaMemsetAsync(Q.tie_count, 0, sizeof(unsigned long long), c->stream));
-    }
-    unsigned long long* cnt = counters.as<unsigned long long>();
     pdg::HitsOut O;
     O.out_b = H->out_b.as<uint32_t>();
     O.out_s = H->out_s.as<uint32_t>();
@@ -716,16 +716,17 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
     O.n_def2 = (uint32_t*)(cnt + 3);
     O.n_def0 = (uint32_t*)(cnt + 4);
     O.ticket = O.n_def0 + 1;
-    O.def0 = def0.as<uint32_t>();
+    O.def0 = piece<uint32_t>(tmp, o_def0);
     O.row_off = H->row_off.as<unsigned long long>();
     O.row_len = H->row_len.as<uint32_t>();
-    O.def1 = def1.as<uint32_t>();
-    O.def2 = def2.as<uint32_t>();
+    O.def1 = piece<uint32_t>(tmp, o_def1);
+    O.def2 = piece<uint32_t>(tmp, o_def2);
     pdg::QuerySet Qw = Q;  // the context's walk unless the call chose one
     if (Qw.walk == PD_WALK_AUTO) Qw.walk = c->walk;
+    Qw.tie_count = cnt + 5;
     CK(pdg::run_summin_tiers(L, v, Qw, O, c->d_err, emit_all, c->stream));
-    unsigned long long h[4];
-    CK(cudaMemcpyAsync(h, counters.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    unsigned long long* h = c->h_build;  // pinned
+    CK(cudaMemcpyAsync(h, cnt, kCounters * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
     pd_status st = check_dev_err(c);
     if (st != PD_OK) return st;
     const uint32_t n_def1 = (uint32_t)h[2], n_def2 = (uint32_t)h[3];
@@ -750,14 +751,15 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
       B.vals = bv.as<uint32_t>();
       B.used = bu.as<uint32_t>();
       B.out = bo.as<unsigned long long>();
-      CK(pdg::run_summin_global(L, v, Q, O, B, n_ctas, c->d_err, emit_all, c->stream));
-      CK(cudaMemcpyAsync(h, counters.p, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+      CK(pdg::run_summin_global(L, v, Qw, O, B, n_ctas, c->d_err, emit_all, c->stream));
+      CK(cudaMemcpyAsync(h, cnt, kCounters * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
       st = check_dev_err(c);  // synchronizes (scratch lifetime)
       if (st != PD_OK) return st;
     }
     if (h[0] <= cap) {
       H->n_hits = h[0];
       H->walked = h[1];
+      H->n_ties = h[5];
       H->n_deferred = n_def1;
       H->n_rows = n_rows;
       return PD_OK;
@@ -893,9 +895,8 @@ static pd_status sym_hits_impl(pd_ctx* c, const pd_profiles* P, pd_hits* H) {
   const uint32_t G = v.n_genes, NG = v.n_genomes;
   const unsigned long long sym_bytes = 8ull * G * NG;
   unsigned long long tie_cap = std::max<unsigned long long>(G, 1ull << 16);
-  Buf symbest, ties, tcount;
+  Buf symbest, ties;
   ALLOC(symbest, sym_bytes);
-  ALLOC(tcount, sizeof(unsigned long long));
   for (int attempt = 0; attempt < 3; ++attempt) {
     ALLOC(ties, 2 * sizeof(unsigned long long) * tie_cap);
     pdg::QuerySet Q{};  // run_hits clears the maxima and the tie count before each launch
@@ -907,72 +908,70 @@ static pd_status sym_hits_impl(pd_ctx* c, const pd_profiles* P, pd_hits* H) {
     Q.n_queries = G;
     Q.symbest = symbest.as<unsigned long long>();
     Q.tie_rec = ties.as<unsigned long long>();
-    Q.tie_count = tcount.as<unsigned long long>();
     Q.tie_cap = tie_cap;
     pd_hits F;
     F.ctx = c;
     F.all_pairs = 1;
     pd_status st = run_hits(c, P, Q, false, &F);  // forward rows (genomes after each query's own)
     if (st != PD_OK) return st;
-    unsigned long long n_ties = 0;
-    CK(cudaMemcpyAsync(&n_ties, tcount.p, sizeof(n_ties), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    const unsigned long long n_ties = F.n_ties;
     if (n_ties > tie_cap) {  // more exact ties than the list held: run again with room for all
       tie_cap = n_ties + 4096;
       continue;
     }
     // a query handed to the next tier after its Best Hit passes records its
     // ties twice: a set keeps the first record of each pair
-    Buf tie_set;
-    const unsigned long long set_slots = pdg::next_pow2((uint32_t)std::min<unsigned long long>(
-        std::max<unsigned long long>(2 * n_ties, 2), 1ull << 31));
-    ALLOC(tie_set, sizeof(unsigned long long) * set_slots);
-    CK(cudaMemsetAsync(tie_set.p, 0xFF, sizeof(unsigned long long) * set_slots, c->stream));
+    const unsigned long long set_slots =
+        n_ties ? pdg::next_pow2((uint32_t)std::min<unsigned long long>(std::max<unsigned long long>(2 * n_ties, 2),
+                                                                     1ull << 31))
+               : 0;
+    Carve ct;
+    const size_t o_tiecnt = ct.add(sizeof(uint32_t) * G), o_fill = ct.add(sizeof(uint32_t) * G), o_listed = ct.add(sizeof(uint32_t)), zeroed = ct.bytes,
+                 o_set = ct.add(sizeof(unsigned long long) * set_slots), o_stored = ct.add(sizeof(uint32_t) * G),
+                 o_ok = ct.add(n_ties), o_tgene = ct.add(sizeof(uint32_t) * std::min<unsigned long long>(n_ties, G)),
+                 o_bcnt = ct.add(sizeof(uint32_t) * G),
+                 o_bstart = ct.add(sizeof(uint32_t) * ((size_t)G + 1)),
+                 o_scan = ct.add(pdg::scan_temp_bytes((uint64_t)G + 1) + 64), o_flag = ct.add(F.n_hits);
+    Buf tmp, row_ptr, total;
+    ALLOC(tmp, ct.bytes);
+    ALLOC(total, sizeof(uint32_t) * G);
+    ALLOC(row_ptr, sizeof(unsigned long long) * ((size_t)G + 1));
+    uint32_t *tiecnt = piece<uint32_t>(tmp, o_tiecnt), *stored = piece<uint32_t>(tmp, o_stored),
+             *bstart = piece<uint32_t>(tmp, o_bstart);
+    uint8_t *tie_ok = piece<uint8_t>(tmp, o_ok), *flag = piece<uint8_t>(tmp, o_flag);
+    void* scan_tmp = piece<void>(tmp, o_scan);
     pdg::SymRows R{G, NG, v.gene_genome, v.La, symbest.as<unsigned long long>(), ties.as<unsigned long long>(),
-                   n_ties, tie_set.as<unsigned long long>(), set_slots - 1, F.row_off.as<unsigned long long>(),
-                   F.row_len.as<uint32_t>(), F.out_b.as<uint32_t>(), F.out_s.as<uint32_t>()};
-    Buf stored, tiecnt, tie_ok, total, row_ptr, tmp, tie_fill;
-    const size_t G1 = std::max<uint32_t>(G, 1);
-    ALLOC(stored, sizeof(uint32_t) * G1);
-    ALLOC(tiecnt, sizeof(uint32_t) * G1);
-    ALLOC(tie_fill, sizeof(uint32_t) * G1);
-    ALLOC(tie_ok, std::max<unsigned long long>(n_ties, 1));
-    ALLOC(total, sizeof(uint32_t) * G1);
-    ALLOC(row_ptr, sizeof(unsigned long long) * (G + 1));
-    ALLOC(tmp, pdg::scan_temp_bytes(G + 1) + 64);
-    CK(cudaMemsetAsync(tiecnt.p, 0, sizeof(uint32_t) * G1, c->stream));
-    CK(cudaMemsetAsync(tie_fill.p, 0, sizeof(uint32_t) * G1, c->stream));
-    CK(pdg::run_sym_count(L, R, stored.as<uint32_t>(), tiecnt.as<uint32_t>(), tie_ok.as<uint8_t>(),
-                          total.as<uint32_t>(), c->stream));
-    CK(pdg::scan_u32_to_u64(L, total.as<uint32_t>(), G, row_ptr.as<unsigned long long>(), tmp.p, c->stream));
-    unsigned long long n = 0;
-    CK(cudaMemcpyAsync(&n, row_ptr.as<unsigned long long>() + G, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
+                   n_ties, piece<unsigned long long>(tmp, o_set), set_slots ? set_slots - 1 : 0,
+                   piece<uint32_t>(tmp, o_listed), piece<uint32_t>(tmp, o_tgene), F.row_off.as<unsigned long long>(), F.row_len.as<uint32_t>(), F.out_b.as<uint32_t>(),
+                   F.out_s.as<uint32_t>()};
+    if (n_ties) {
+      CK(cudaMemsetAsync(tiecnt, 0, zeroed, c->stream));
+      CK(cudaMemsetAsync(R.tie_set, 0xFF, sizeof(unsigned long long) * set_slots, c->stream));
+    }
+    CK(pdg::run_sym_count(L, R, stored, tiecnt, tie_ok, total.as<uint32_t>(), c->stream));
+    CK(pdg::scan_u32_to_u64(L, total.as<uint32_t>(), G, row_ptr.as<unsigned long long>(), scan_tmp, c->stream));
+    // BBH while the reverse maxima are at hand
+    CK(pdg::run_sym_bbh_count(L, R, flag, piece<uint32_t>(tmp, o_bcnt), bstart, scan_tmp, c->stream));
+    unsigned long long* h = c->h_build;  // pinned: the row total, the BBH total
+    CK(cudaMemcpyAsync(h, row_ptr.as<unsigned long long>() + G, sizeof(*h), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(h + 1, bstart + G, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
+    const unsigned long long n = h[0];
+    const uint32_t n_bbh = *(const uint32_t*)(h + 1);
     ALLOC(H->out_b, sizeof(uint32_t) * std::max<unsigned long long>(n, 1));
     ALLOC(H->out_s, sizeof(uint32_t) * std::max<unsigned long long>(n, 1));
-    CK(pdg::run_sym_write(L, R, stored.as<uint32_t>(), tiecnt.as<uint32_t>(), tie_ok.as<uint8_t>(),
-                          row_ptr.as<unsigned long long>(), tie_fill.as<uint32_t>(), H->out_b.as<uint32_t>(),
-                          H->out_s.as<uint32_t>(), c->stream));
-    // BBH while the reverse maxima are at hand
-    Buf flag, bcnt, bstart;
-    ALLOC(flag, std::max<unsigned long long>(F.out_b.n / sizeof(uint32_t), 1));
-    ALLOC(bcnt, sizeof(uint32_t) * G1);
-    ALLOC(bstart, sizeof(uint32_t) * (G + 1));
-    CK(pdg::run_sym_bbh_count(L, R, flag.as<uint8_t>(), bcnt.as<uint32_t>(), bstart.as<uint32_t>(), tmp.p,
-                              c->stream));
-    uint32_t n_bbh = 0;
-    CK(cudaMemcpyAsync(&n_bbh, bstart.as<uint32_t>() + G, sizeof(n_bbh), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    ALLOC(H->bbh_a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
-    ALLOC(H->bbh_b, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
+    CK(pdg::run_sym_write(L, R, stored, tiecnt, tie_ok, row_ptr.as<unsigned long long>(), piece<uint32_t>(tmp, o_fill),
+                          H->out_b.as<uint32_t>(), H->out_s.as<uint32_t>(), c->stream));
+    H->bbh = std::make_shared<pd_bbh_set>();
+    H->bbh->ctx = c;
+    H->bbh->n = n_bbh;
+    ALLOC(H->bbh->a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
+    ALLOC(H->bbh->b, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
     if (n_bbh)
-      CK(pdg::run_sym_bbh_write(L, R, flag.as<uint8_t>(), bstart.as<uint32_t>(), H->bbh_a.as<int32_t>(),
-                                H->bbh_b.as<int32_t>(), c->stream));
+      CK(pdg::run_sym_bbh_write(L, R, flag, bstart, H->bbh->a.as<int32_t>(), H->bbh->b.as<int32_t>(), c->stream));
     st = check_dev_err(c);  // synchronizes: the forward rows and the tables end here
     if (st != PD_OK) return st;
-    H->has_bbh = true;
     H->csr = true;
-    H->n_bbh = n_bbh;
     H->row_off = std::move(row_ptr);
     H->row_len = std::move(total);
     H->n_rows = G;
@@ -1273,17 +1272,21 @@ PD_API pd_status pd_bbh_all(pd_ctx* c, const pd_profiles* P, const pd_hits* H, p
   if (!H->all_pairs || H->paralog) return fail(c, PD_ERR_ARG, "pd_bbh_all needs the result of pd_best_hits_all");
   try {
     CK(cudaSetDevice(c->device));
-    if (H->has_bbh) {  // found with the rows (the symmetric form)
+    if (H->bbh) {  // found with the rows (the symmetric form)
       std::unique_ptr<pd_bbh_set> S(new pd_bbh_set());
       S->ctx = c;
-      S->n = H->n_bbh;
-      ALLOC(S->a, sizeof(int32_t) * std::max<uint64_t>(H->n_bbh, 1));
-      ALLOC(S->b, sizeof(int32_t) * std::max<uint64_t>(H->n_bbh, 1));
-      if (H->n_bbh) {
-        CK(cudaMemcpyAsync(S->a.p, H->bbh_a.p, sizeof(int32_t) * H->n_bbh, cudaMemcpyDeviceToDevice, c->stream));
-        CK(cudaMemcpyAsync(S->b.p, H->bbh_b.p, sizeof(int32_t) * H->n_bbh, cudaMemcpyDeviceToDevice, c->stream));
+      S->n = H->bbh->n;
+      if (c == H->ctx) {  // one context: the handles share the pairs
+        S->shared = H->bbh;
+      } else {
+        ALLOC(S->a, sizeof(int32_t) * std::max<uint64_t>(S->n, 1));
+        ALLOC(S->b, sizeof(int32_t) * std::max<uint64_t>(S->n, 1));
+        if (S->n) {
+          CK(cudaMemcpyAsync(S->a.p, H->bbh->a.p, sizeof(int32_t) * S->n, cudaMemcpyDeviceToDevice, c->stream));
+          CK(cudaMemcpyAsync(S->b.p, H->bbh->b.p, sizeof(int32_t) * S->n, cudaMemcpyDeviceToDevice, c->stream));
+        }
+        CK(cudaStreamSynchronize(c->stream));
       }
-      CK(cudaStreamSynchronize(c->stream));
       *out = S.release();
       return PD_OK;
     }
@@ -1466,8 +1469,8 @@ PD_API pd_status pd_bbh_copy(pd_ctx* c, const pd_bbh_set* S, int32_t* a, int32_t
   try {
     if (n_pairs) *n_pairs = S->n;
     pd_status st;
-    if ((st = copy_out(c, a, S->a.p, sizeof(int32_t) * S->n)) != PD_OK) return st;
-    if ((st = copy_out(c, b, S->b.p, sizeof(int32_t) * S->n)) != PD_OK) return st;
+    if ((st = copy_out(c, a, S->first(), sizeof(int32_t) * S->n)) != PD_OK) return st;
+    if ((st = copy_out(c, b, S->second(), sizeof(int32_t) * S->n)) != PD_OK) return st;
     CK(cudaStreamSynchronize(c->stream));
     return PD_OK;
   } catch (...) {

@@ -240,19 +240,21 @@ struct pd_hits {
   uint64_t n_hits = 0, walked = 0;
   uint32_t n_deferred = 0;
   Buf row_off, row_len, out_b, out_s;
+  uint64_t n_ties = 0;  // exact ties of reverse maxima (a launch of the symmetric form)
   // the symmetric all-pairs form finds the BBH pairs with the rows, and its
   // rows are already one CSR: row_off holds n_rows + 1 offsets into
   // out_b / out_s, in row order
-  bool has_bbh = false;
+  std::shared_ptr<struct pd_bbh_set> bbh;
   bool csr = false;
-  uint64_t n_bbh = 0;
-  Buf bbh_a, bbh_b;
 };
 
 struct pd_bbh_set {
   pd_ctx* ctx = nullptr;
   uint64_t n = 0;
   Buf a, b;
+  std::shared_ptr<pd_bbh_set> shared;  // the pairs, if another handle found them
+  const int32_t* first() const { return (shared ? shared->a : a).as<int32_t>(); }
+  const int32_t* second() const { return (shared ? shared->b : b).as<int32_t>(); }
 };
 
 

@@ -179,6 +179,84 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
   return r;
 }
 
+// ---------------------------------------------------------------- look-back
+// Running sums over tiles that one launch computes in any order (decoupled
+// look-back: Merrill and Garland, "Single-pass Parallel Prefix Scan with
+// Decoupled Look-back", 2016).  A status word holds two flag bits above a
+// tile's sum alone or of all tiles up to it, written and read whole.  Tiles are
+// numbered by a ticket, so every tile waited for is already running; a wait
+// that runs out is reported by the caller (PD_ERR_INTERNAL).
+template <typename T>
+struct Status {
+  static constexpr T kAggregate = (T)1 << (sizeof(T) * 8 - 2);
+  static constexpr T kInclusive = (T)2 << (sizeof(T) * 8 - 2);
+  static constexpr T kValue = kAggregate - 1;
+};
+constexpr uint32_t kMaxPolls = 1u << 21;
+
+// Sum over the tiles before `tile` of one column of statuses (status[t *
+// stride]), walked back until an inclusive sum; four predecessors are read at
+// a time.  False if a wait ran out.
+template <typename T>
+__device__ __forceinline__ bool look_back(const volatile T* status, uint32_t tile, uint32_t stride, T* sum,
+                                          const DevErr* err) {
+  T s = 0;
+  uint32_t polls = 0;
+  int64_t t = (int64_t)tile - 1;
+  while (t >= 0) {
+    T v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = t - j >= 0 ? status[(uint64_t)(t - j) * stride] : (T)0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (v[j] & Status<T>::kInclusive) {
+        *sum = s + (v[j] & Status<T>::kValue);
+        return true;
+      }
+      if (!(v[j] & Status<T>::kAggregate)) break;
+      s += v[j] & Status<T>::kValue;
+      --t;
+    }
+    if (++polls > 64u) {
+      __nanosleep(100);
+      if (polls > kMaxPolls || ((polls & 255u) == 0 && *(volatile const int*)&err->code)) return false;
+    }
+  }
+  *sum = s;
+  return true;
+}
+
+// The same for one column by a whole warp, 32 predecessors at a time.
+__device__ __forceinline__ bool look_back_warp(const volatile unsigned long long* status, uint32_t tile, unsigned long long* sum, const DevErr* err) {
+  using S = Status<unsigned long long>;
+  const uint32_t lane = threadIdx.x & 31u;
+  unsigned long long s = 0;
+  uint32_t polls = 0;
+  for (int64_t t = (int64_t)tile - 1; t >= 0;) {
+    const int64_t mine = t - lane;
+    const unsigned long long v = mine >= 0 ? status[mine] : S::kInclusive;
+    const uint32_t inc = __ballot_sync(0xffffffffu, (v & S::kInclusive) != 0ull);
+    const uint32_t set = __ballot_sync(0xffffffffu, (v & (S::kInclusive | S::kAggregate)) != 0ull);
+    // the lanes up to the first inclusive sum, or up to the first one missing
+    const uint32_t n = inc ? (uint32_t)__ffs((int)inc) : 32u;
+    const uint32_t ready = set == 0xffffffffu ? 32u : (uint32_t)__ffs((int)~set) - 1u;
+    const uint32_t take = min(n, ready);
+    unsigned long long x = lane < take ? v & S::kValue : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    s += x;
+    t -= take;
+    if (inc && n <= ready) break;
+    if (take < 32u && ++polls > 64u) {
+      __nanosleep(100);
+      const bool failed = (polls & 255u) == 0 && *(volatile const int*)&err->code;
+      if (polls > kMaxPolls || __any_sync(0xffffffffu, failed)) return false;
+    }
+  }
+  *sum = s;
+  return true;
+}
+
 // Exact ratio order: s1/d1 > s2/d2 by 64-bit cross-multiplication.
 __host__ __device__ __forceinline__ bool ratio_greater(uint32_t s1, uint32_t d1, uint32_t s2, uint32_t d2) {
   return (uint64_t)s1 * (uint64_t)d2 > (uint64_t)s2 * (uint64_t)d1;
@@ -324,6 +402,7 @@ struct TierIO {
 struct Launcher;  // opaque: pd_ctx side (timing + launch counting)
 cudaError_t launch_begin(Launcher* L, const char* name);
 cudaError_t launch_end(Launcher* L, const char* name);
+DevErr* launch_err(Launcher* L);  // the context's device error block
 
 // scans (k_scan.cu)
 size_t scan_temp_bytes(uint64_t n);
@@ -340,12 +419,14 @@ cudaError_t scan_u32_total(Launcher* L, const uint32_t* in, uint64_t n, uint32_t
                            unsigned long long* total, void* temp, cudaStream_t s);
 
 // profiles and index of a dataset (k_index.cu)
-// Gene offsets -> window counts on the device.  Checks every gene (offsets
-// from 0, non-decreasing, ending at n_res unless check_end is 0; at most
-// PD_MAX_WINDOWS windows), recording PD_ERR_ARG / PD_ERR_GENE_TOO_LONG with
-// the gene as detail (such a gene gets La 0).
+// Gene offsets -> window counts and genomes on the device, min-hashes cleared
+// (all ones).  Checks every gene (offsets from 0, non-decreasing, ending at
+// n_res unless check_end is 0; at most PD_MAX_WINDOWS windows), recording
+// PD_ERR_ARG / PD_ERR_GENE_TOO_LONG with the gene as detail (such a gene gets La
+// 0).  genome_ptr need not have been checked yet.
 cudaError_t run_gene_windows(Launcher* L, const int64_t* gene_ptr, uint32_t n_genes, uint64_t n_res, int check_end,
-                             int k, uint32_t* La, DevErr* err, cudaStream_t s);
+                             int k, const int32_t* genome_ptr, uint32_t n_genomes, uint32_t* La, uint16_t* gene_genome,
+                             uint32_t* ginfo, uint32_t* minhash, DevErr* err, cudaStream_t s);
 // PD_ERR_ALPHABET (detail: the position) for a byte outside the alphabet: all
 // n_res bytes, or with gene_src the genes' bytes.
 cudaError_t run_check_letters(Launcher* L, const uint8_t* res, uint64_t n_res, const int64_t* gene_ptr,
@@ -379,19 +460,19 @@ struct SortScratch {
 SortScratch sort_scratch(const SortKey& K, uint64_t n);
 uint32_t sort_tiles(uint64_t n);    // tiles of the sort (tile_gene holds one more entry)
 uint32_t dedupe_tiles(uint64_t n);  // tiles of the dedupe pass (tile_e and tile_id hold one more entry)
-constexpr size_t kDigitStarts = (size_t)kMaxSortPasses * 512;
+constexpr uint32_t kSortBins = 512;  // words of one pass's digit counts
+// Also copies win_off to cursor.
 cudaError_t run_tile_genes(Launcher* L, const uint32_t* win_off, uint32_t n_genes, uint64_t n_windows,
-                           uint32_t* tile_gene, cudaStream_t s);
-// Digit starts of every pass, the records of the slice (*total) and, if not
-// null, the min-hashes (set to all ones before).
+                           uint32_t* tile_gene, uint32_t* cursor, cudaStream_t s);
+// Digit counts of every pass (into the scratch, at hist) and, if not null, the
+// min-hashes (set to all ones before).
 cudaError_t run_code_hist(Launcher* L, const WindowSource& S, const SortKey& K, uint8_t* scratch, const SortScratch& X,
-                          unsigned long long* digit_start, unsigned long long* total, uint32_t* minhash,
-                          cudaStream_t s);
+                          uint32_t* minhash, cudaStream_t s);
 // The slice's n records sorted by code, equal codes by gene: in a after an odd
 // number of passes, else in b.
 cudaError_t run_sort(Launcher* L, const WindowSource& S, const SortKey& K, uint64_t n, uint8_t* scratch,
-                     const SortScratch& X, const unsigned long long* digit_start, unsigned long long* a,
-                     unsigned long long* b, unsigned long long** sorted, DevErr* err, cudaStream_t s);
+                     const SortScratch& X, unsigned long long* a, unsigned long long* b, unsigned long long** sorted,
+                     DevErr* err, cudaStream_t s);
 // Sorted records -> post, post_ptr, code_lo / code_hi and the postings and ids
 // before each tile; totals: [4] words, the postings and ids so far first.
 cudaError_t run_dedupe(Launcher* L, const unsigned long long* rec, uint64_t n, const SortKey& K, uint8_t* scratch,
@@ -407,8 +488,6 @@ cudaError_t run_lists(Launcher* L, const unsigned long long* rec, uint64_t n, co
                       const uint8_t* code_hi, uint32_t cnt_bits, uint32_t cnt_cap, const int32_t* genome_ptr,
                       uint32_t n_genomes, uint32_t n_genes, uint32_t* cursor, uint4* mv, uint32_t* max_list,
                       unsigned long long* join, cudaStream_t s);
-cudaError_t run_vector_lengths(Launcher* L, const uint32_t* cursor, const uint32_t* win_off, uint32_t n_genes,
-                               uint32_t* mv_n, cudaStream_t s);
 
 // profiles (k_profiles.cu)
 // The bits of all codes of an index in a zeroed dictionary.
@@ -430,12 +509,12 @@ cudaError_t run_mv_build(Launcher* L, const uint8_t* res, const int64_t* gene_pt
                          uint32_t n_genes, int k, const uint32_t* dict, const MvOut& M, const uint32_t* mid_genes, uint32_t n_mid, const uint32_t* long_genes,
                          uint32_t n_long, unsigned long long* long_scratch, const unsigned long long* long_scratch_off,
                          cudaStream_t s);
+// Query order, and the lengths of the vectors (what their cursors passed).
 // count must hold 2 * kOrderBuckets + 1 words (zeroed counts, then their prefix sum).
 constexpr uint32_t kOrderBuckets = 65536;
 cudaError_t run_order(Launcher* L, const uint32_t* minhash, const uint32_t* La, uint32_t n_genes, int length_buckets,
-                      uint32_t* count, uint32_t* order, void* scan_tmp, cudaStream_t s);
-cudaError_t run_gene_info(Launcher* L, const int32_t* genome_ptr, uint32_t n_genomes, const uint32_t* La,
-                          uint16_t* gene_genome, uint32_t* ginfo, cudaStream_t s);
+                      const uint32_t* cursor, const uint32_t* win_off, uint32_t* mv_n, uint32_t* count,
+                      uint32_t* order, void* scan_tmp, cudaStream_t s);
 cudaError_t run_export_codes(Launcher* L, const ProfilesView& P, unsigned long long* codes, cudaStream_t s);
 // Distinct k-mers per gene (n zeroed before).
 cudaError_t run_export_mv_count(Launcher* L, const ProfilesView& P, uint32_t* n, cudaStream_t s);
@@ -467,13 +546,16 @@ struct SymRows {
   unsigned long long n_ties;
   unsigned long long* tie_set;        // [tie_set_mask + 1] all-ones: the pairs already counted
   unsigned long long tie_set_mask;
+  uint32_t* n_tie_genes;              // genes with valid ties (zero at first) ...
+  uint32_t* tie_gene;                 // ... and which: room for min(n_ties, n_genes)
   const unsigned long long* fwd_off;  // forward rows of the launch
   const uint32_t* fwd_len;
   const uint32_t* fwd_b;
   const uint32_t* fwd_s;
 };
 // Per gene: stored maxima (stored), valid ties (tiecnt, must start at zero;
-// tie_ok flags each tie) and the row length (total).
+// tie_ok flags each tie; neither is used without ties) and the row length
+// (total).
 cudaError_t run_sym_count(Launcher* L, const SymRows& R, uint32_t* stored, uint32_t* tiecnt, uint8_t* tie_ok,
                           uint32_t* total, cudaStream_t s);
 // Rows written at row_ptr (exclusive scan of total); tie_fill must start at zero.
