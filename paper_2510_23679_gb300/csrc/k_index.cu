@@ -303,31 +303,36 @@ __device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, const uint32_t
 
 // Stable counting step of one tile.  xr: the thread's records, striped within
 // the warp's run of 32 * kItems (item r of lane l is position r * 32 + l).
-// Ranks within the warp come from the lanes holding the same digit (the AND
-// over the digit's bits of each bit's ballot or its complement).
+// Ranks within the warp come from the lanes holding the same digit: each lane
+// sets its bit in the digit's word of a table of the warp's (in the staging
+// memory, not in use yet).  Finding them with one ballot per digit bit took
+// four instructions a bit and kept the ALU the busiest pipe (1.65 ms a pass
+// against 1.35 at 264 M records).
 template <int kBits, typename T>
 __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid_mask, uint32_t shift, T* status,
                                                u64* __restrict__ out, PassShared<kBits>& sh, u64* stage, DevErr* err) {
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   constexpr uint32_t bins = 1u << kBits, dmask = bins - 1u;
   constexpr int kOwn = (int)((bins + kThreads - 1) / kThreads);  // digits kOwn * t .. of thread t
+  static_assert((size_t)kWarps * bins * 4 <= (size_t)kTile * 8, "the match table fits the staging memory");
   const uint32_t below = (1u << lane) - 1u;
+  uint32_t* match = (uint32_t*)stage + warp * bins;
+  for (uint32_t d = lane; d < bins; d += 32) match[d] = 0;
+  __syncwarp();
   uint32_t rk[(kItems + 1) / 2];  // two 16-bit ranks each
 #pragma unroll
   for (int r = 0; r < kItems; ++r) {
     const bool valid = (valid_mask >> r) & 1u;
     const uint32_t d = (uint32_t)(xr[r] >> shift) & dmask;
-    uint32_t peers = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < kBits; ++b) {
-      const bool bit = (d >> b) & 1u;
-      const uint32_t bal = __ballot_sync(0xffffffffu, bit);
-      peers &= bit ? bal : ~bal;
-    }
-    uint16_t* c = &sh.wcnt[warp][d];
-    const uint32_t base = *c, before = (uint32_t)__popc(peers & below);
+    if (valid) atomicOr(&match[d], 1u << lane);
     __syncwarp();
-    if (valid && before == 0) *c = (uint16_t)(base + (uint32_t)__popc(peers));
+    const uint32_t peers = *(volatile uint32_t*)&match[d], base = sh.wcnt[warp][d];
+    const uint32_t before = (uint32_t)__popc(peers & below);
+    __syncwarp();
+    if (valid && before == 0) {
+      sh.wcnt[warp][d] = (uint16_t)(base + (uint32_t)__popc(peers));
+      match[d] = 0;
+    }
     __syncwarp();
     if (r & 1) rk[r / 2] |= (base + before) << 16; else rk[r / 2] = base + before;
   }
@@ -448,8 +453,13 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
 
 // ---------------------------------------------------------------- dedupe
 // Tiles of sorted records, striped within each warp like the sort's.
-constexpr int kDThreads = 512, kDWarps = kDThreads / 32, kDItems = 8;
+constexpr int kDThreads = 512, kDWarps = kDThreads / 32, kDItems = 16;
 constexpr uint32_t kDTile = kDThreads * kDItems;
+// ... and of postings: those of half a tile of records (longer tiles wait less
+// for one another, shorter ones leave room for more blocks of the lists pass).
+constexpr int kLItems = 8;
+constexpr uint32_t kLTile = kDThreads * kLItems, kHalves = kDTile / kLTile;
+static_assert(kHalves == 2 && kDWarps % 2 == 0, "a list tile is half the warps of a dedupe tile");
 
 // First record after i (in [lo, n)) whose key differs from `key`; records
 // before lo are equal to it.  Runs are short, so the search gallops first.
@@ -470,10 +480,10 @@ __device__ __forceinline__ uint64_t run_end(const u64* __restrict__ rec, uint64_
 
 // Sorted records of one slice -> postings, posting-list starts and codes.
 // A posting is the first record of a run of equal ones, its count the length
-// of the run.  tile_e / tile_id: postings and ids before each tile (and, at
-// n_tiles, in all); totals[0], totals[1]: postings and ids so far, read and
+// of the run.  tile_e / tile_id: postings and ids before each half tile (and,
+// after the last, in all); totals[0], totals[1]: postings and ids so far, read and
 // advanced by each slice.
-__global__ void __launch_bounds__(kDThreads, 3)
+__global__ void __launch_bounds__(kDThreads, 2)
     k_dedupe(const u64* __restrict__ rec, uint64_t n, SortKey K, uint32_t n_tiles, uint32_t cnt_bits, uint32_t cnt_cap,
              u64* status_e, u64* status_id, uint32_t* ticket, u64* totals, uint32_t* __restrict__ post,
              uint32_t* __restrict__ post_ptr, uint32_t* __restrict__ code_lo, uint8_t* __restrict__ code_hi, uint32_t* __restrict__ tile_e, uint32_t* __restrict__ tile_id,
@@ -570,12 +580,14 @@ __global__ void __launch_bounds__(kDThreads, 3)
   if (s_failed) return;
   const uint32_t e0 = (uint32_t)s_base[0], id0 = (uint32_t)s_base[1];
   if (threadIdx.x == 0) {
-    tile_e[tile] = e0;
-    tile_id[tile] = id0;
+    for (uint32_t half = 0; half < kHalves; ++half) {
+      tile_e[kHalves * tile + half] = e0 + s_we[half * (kDWarps / 2)];
+      tile_id[kHalves * tile + half] = id0 + s_wi[half * (kDWarps / 2)];
+    }
     if (tile + 1u == n_tiles) {
       const uint32_t e1 = e0 + s_we[kDWarps], id1 = id0 + s_wi[kDWarps];
-      tile_e[n_tiles] = e1;
-      tile_id[n_tiles] = id1;
+      tile_e[kHalves * n_tiles] = e1;
+      tile_id[kHalves * n_tiles] = id1;
       post_ptr[id1] = e1;
       totals[0] = e1;
       totals[1] = id1;
@@ -611,8 +623,8 @@ __global__ void __launch_bounds__(kDThreads, 3)
 //   x = list start, y = count, z = list length | (another posting of the
 //   gene's genome) << 31, w = offset in the list of the first posting past the
 //   gene's genome,
-// goes to the next free place of the gene's vector (cursor).  Tiles are the
-// dedupe's; blocks are persistent, so that the table that gives a gene's
+// goes to the next free place of the gene's vector (cursor).  Tiles are halves
+// of the dedupe's; blocks are persistent, so that the table that gives a gene's
 // genome is built once per block: a gene's genome lies between those of the
 // table's entries around it.  Runs of one genome are marked in a bit mask of the
 // tile, whose next set bit gives w.  Also the longest list and the sum of
@@ -645,10 +657,10 @@ __global__ void __launch_bounds__(kDThreads, 3)
             const uint32_t* __restrict__ post_ptr, uint32_t cnt_bits, uint32_t cnt_cap,
             const int32_t* __restrict__ genome_ptr, uint32_t n_genomes, uint32_t n_genes, uint32_t table_bits,
             uint32_t* cursor, uint4* __restrict__ mv, uint32_t* max_list, u64* join) {
-  __shared__ uint32_t start[kDTile + 2];
-  __shared__ uint32_t is_head[kDTile / 32], run_head[kDTile / 32];
-  __shared__ uint16_t genome[kDTile];
-  __shared__ uint32_t before[kDTile / 32];  // list heads before each word
+  __shared__ uint32_t start[kLTile + 2];
+  __shared__ uint32_t is_head[kLTile / 32], run_head[kLTile / 32];
+  __shared__ uint16_t genome[kLTile];
+  __shared__ uint32_t before[kLTile / 32];  // list heads before each word
   __shared__ uint16_t table[kGenomeTable + 1];
   extern __shared__ int32_t gend[];  // first gene past each genome
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -673,7 +685,7 @@ __global__ void __launch_bounds__(kDThreads, 3)
     const uint32_t id0 = tile_id[tile], id1 = tile_id[tile + 1];
     const uint32_t n = e1 - e0, n_heads = id1 - id0;
     __syncthreads();  // the table is built; the last tile's shared arrays are done with
-    for (uint32_t i = threadIdx.x; i < kDTile / 32; i += kDThreads) is_head[i] = 0;
+    for (uint32_t i = threadIdx.x; i < kLTile / 32; i += kDThreads) is_head[i] = 0;
     __syncthreads();
     // start[l]: list l of the tile; list 0 is the one begun before it (if any)
     for (uint32_t l = threadIdx.x; l < n_heads + 2u; l += kDThreads) {
@@ -686,16 +698,16 @@ __global__ void __launch_bounds__(kDThreads, 3)
         squares += len * len;
       }
     }
-    uint32_t pv[kDItems];
+    uint32_t pv[kLItems];
 #pragma unroll
-    for (int r = 0; r < kDItems; ++r) {
+    for (int r = 0; r < kLItems; ++r) {
       const uint32_t i = (uint32_t)r * kDThreads + threadIdx.x;
       pv[r] = i < n ? post[e0 + i] : 0u;
     }
     __syncthreads();
     if (warp == 0) {
       uint32_t carry = 0;
-      for (uint32_t w0 = 0; w0 < kDTile / 32; w0 += 32) {
+      for (uint32_t w0 = 0; w0 < kLTile / 32; w0 += 32) {
         const uint32_t c = __popc(is_head[w0 + lane]);
         const uint32_t inc = warp_inclusive_scan(c);
         before[w0 + lane] = carry + inc - c;
@@ -709,7 +721,7 @@ __global__ void __launch_bounds__(kDThreads, 3)
     // genomes of the postings of lists of two and more
     uint32_t kept = 0;
 #pragma unroll
-    for (int r = 0; r < kDItems; ++r) {
+    for (int r = 0; r < kLItems; ++r) {
       const uint32_t i = (uint32_t)r * kDThreads + threadIdx.x;
       if (i < n) {
         const uint32_t l = list_of(i);
@@ -721,7 +733,7 @@ __global__ void __launch_bounds__(kDThreads, 3)
     }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kDItems; ++r) {
+    for (int r = 0; r < kLItems; ++r) {
       const uint32_t i = (uint32_t)r * kDThreads + threadIdx.x;
       bool f = false;
       if (i < n) {
@@ -733,12 +745,12 @@ __global__ void __launch_bounds__(kDThreads, 3)
       if (lane == 0) run_head[(r * kDThreads + warp * 32u) >> 5] = m;
     }
     __syncthreads();
-    uint32_t at[kDItems];  // all places first: the atomics are in flight together
+    uint32_t at[kLItems];  // all places first: the atomics are in flight together
 #pragma unroll
-    for (int r = 0; r < kDItems; ++r)
+    for (int r = 0; r < kLItems; ++r)
       if ((kept >> r) & 1u) at[r] = atomicAdd(&cursor[pv[r] >> cnt_bits], 1u);
 #pragma unroll
-    for (int r = 0; r < kDItems; ++r) {
+    for (int r = 0; r < kLItems; ++r) {
       if (!((kept >> r) & 1u)) continue;
       const uint32_t i = (uint32_t)r * kDThreads + threadIdx.x, l = list_of(i);
       const uint32_t s = start[l], t = start[l + 1];
@@ -755,8 +767,8 @@ __global__ void __launch_bounds__(kDThreads, 3)
       uint32_t c = pv[r] & ((1u << cnt_bits) - 1u);
       if (c >= cnt_cap) {
         const u64 code = code_at(code_lo, code_hi, id0 + l - 1u) & ((1ull << K.code_bits) - 1ull);
-        const uint64_t t0 = (uint64_t)tile * kDTile;
-        c = exact_count(rec, t0 + i, min(n_rec, t0 + kDTile), n_rec, (code << K.gene_bits) | (pv[r] >> cnt_bits));
+        const uint64_t t0 = (uint64_t)tile * kLTile;
+        c = exact_count(rec, t0 + i, min(n_rec, t0 + kLTile), n_rec, (code << K.gene_bits) | (pv[r] >> cnt_bits));
       }
       mv[at[r]] = make_uint4(s, c, (t - s) | (more ? 0x80000000u : 0u), next - s);
     }
@@ -859,7 +871,8 @@ SortKey sort_key(uint64_t n_codes, uint32_t gene_bits) {
 }
 
 uint32_t sort_tiles(uint64_t n) { return (uint32_t)((n + kTile - 1) / kTile); }
-uint32_t dedupe_tiles(uint64_t n) { return (uint32_t)((n + kDTile - 1) / kDTile); }
+static uint32_t dedupe_tiles(uint64_t n) { return (uint32_t)((n + kDTile - 1) / kDTile); }
+uint32_t list_tiles(uint64_t n) { return kHalves * dedupe_tiles(n); }
 // Zeroed scratch of one slice: tickets, digit counts, look-back statuses.
 SortScratch sort_scratch(const SortKey& K, uint64_t n) {
   SortScratch x{};
@@ -957,7 +970,7 @@ cudaError_t run_lists(Launcher* L, const u64* rec, uint64_t n, const SortKey& K,
                       const uint8_t* code_hi, uint32_t cnt_bits, uint32_t cnt_cap, const int32_t* genome_ptr,
                       uint32_t n_genomes, uint32_t n_genes, uint32_t* cursor, uint4* mv, uint32_t* max_list, u64* join,
                       cudaStream_t s) {
-  const uint32_t nt = dedupe_tiles(n);
+  const uint32_t nt = list_tiles(n);
   uint32_t table_bits = 0;
   while (((n_genes - 1) >> table_bits) >= kGenomeTable) ++table_bits;
   const size_t smem = sizeof(int32_t) * n_genomes;

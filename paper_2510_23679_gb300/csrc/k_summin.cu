@@ -218,11 +218,11 @@ __device__ __forceinline__ void best_update(unsigned long long* slot, uint32_t s
 // that equals the stored maximum is listed as a tie (b << 32 | a, s).  Ties of
 // a maximum later beaten stay in the list and are dropped when the rows are
 // assembled.
-__device__ __forceinline__ void sym_update(const QuerySet& Q, unsigned long long* slot, uint32_t b, uint32_t a,
-                                           uint32_t s, uint32_t den) {
+// `old`: the stored word, read by the caller.
+__device__ __forceinline__ void sym_update(const QuerySet& Q, unsigned long long* slot, unsigned long long old,
+                                           uint32_t b, uint32_t a, uint32_t s, uint32_t den) {
   const unsigned long long mine =
       ((unsigned long long)s << 48) | ((unsigned long long)den << 31) | (unsigned long long)a;
-  unsigned long long old = *((volatile unsigned long long*)slot);
   while (true) {
     if (old != 0ull) {
       const uint32_t os = (uint32_t)(old >> 48), od = (uint32_t)(old >> 31) & 0x1FFFFu;
@@ -633,7 +633,10 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
         const uint32_t den = La_a + (gi & 0xFFFFu) - s;
         best_update(&best[Q.all_pairs ? (gi >> 16) : 0u], s, den);
         if (Q.colbest) best_update(&Q.colbest[(size_t)b * Q.col_stride + col], s, den);
-        if (Q.symbest) sym_update(Q, &Q.symbest[(size_t)col * P.n_genes + b], b, a, s, den);
+        if (Q.symbest) {
+          unsigned long long* slot = &Q.symbest[(size_t)col * P.n_genes + b];
+          sym_update(Q, slot, *(volatile unsigned long long*)slot, b, a, s, den);
+        }
       }
       __syncthreads();
       for (uint32_t u = tid; u < n_occ; u += kThreads) {
@@ -750,6 +753,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
 // A query that lists more than kWUsed slots, or whose vector is longer than
 // kWEntries, goes to the next tier.
 constexpr uint32_t kWSlots = 1024, kWUsed = 832, kWEntries = 2048, kWPend = 160, kWRing = 64;
+constexpr uint32_t kWBatch = 2;
 constexpr int kWThreads = 128, kWWarps = kWThreads / 32;
 // Target genomes up to which the warp tier runs (10 bytes each per warp).
 constexpr uint32_t kWMaxGenomes = 512;
@@ -763,7 +767,7 @@ __host__ __device__ constexpr size_t warp_tier_bytes(uint32_t n_best) {
 
 template <int kGroup>
 __global__ void __launch_bounds__(kWThreads, 6)
-    k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best) {
+    k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best, uint32_t max_entries) {
   extern __shared__ __align__(16) unsigned char smem[];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   unsigned char* mine = smem + (size_t)warp * warp_tier_bytes(n_best);
@@ -799,7 +803,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
     const uint32_t m0 = (ext ? P.q_win_off : P.win_off)[q.a], E = (ext ? P.q_mv_n : P.mv_n)[q.a];
     const uint32_t La_a = (ext ? P.q_La : P.La)[q.a];
     // a packed slot holds s <= La_a
-    bool overflow = E > kWEntries || La_a >= cmask;
+    bool overflow = E > max_entries || La_a >= cmask;
     uint32_t n_used = 0;
     // Adds the postings put aside (words gene | min of the counts) in [from, to).
     auto flush = [&](uint32_t from, uint32_t to) {
@@ -959,25 +963,58 @@ __global__ void __launch_bounds__(kWThreads, 6)
     auto is_target = [&](uint32_t b) {
       return !(Q.all_pairs && ((b >= q.own0 && b < q.own1) || b >= q.tend)) && b != q.self;
     };
-    for (uint32_t u = lane; u < n_used; u += 32) {
-      const uint32_t k = tab[used[u]], b = k >> P.cnt_bits, s = k & cmask;
-      if (!is_target(b)) continue;
-      const uint32_t gi = P.ginfo[b], den = La_a + (gi & 0xFFFFu) - s;
-      if (!wanted(q, gi >> 16)) continue;
-      if (Q.symbest) sym_update(Q, &Q.symbest[(size_t)q.col * P.n_genes + b], b, q.a, s, den);
-      if (Q.colbest) best_update(&Q.colbest[(size_t)b * Q.col_stride + q.col], s, den);
-      best_update(&best[Q.all_pairs ? (gi >> 16) : 0u], s, den);
+    // kWBatch candidates a lane at a time, their gene words (and reverse
+    // maxima) in flight together
+    for (uint32_t u0 = lane; u0 < n_used; u0 += 32u * kWBatch) {
+      uint32_t k[kWBatch], gi[kWBatch];
+      unsigned long long old[kWBatch];
+      bool live[kWBatch];
+#pragma unroll
+      for (uint32_t j = 0; j < kWBatch; ++j) {
+        const uint32_t u = u0 + 32u * j;
+        k[j] = u < n_used ? tab[used[u]] : 0u;
+        live[j] = u < n_used && is_target(k[j] >> P.cnt_bits);
+        gi[j] = live[j] ? P.ginfo[k[j] >> P.cnt_bits] : 0u;
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < kWBatch; ++j) {
+        live[j] = live[j] && wanted(q, gi[j] >> 16);
+        old[j] = 0ull;
+        if (Q.symbest && live[j])
+          old[j] = *(volatile unsigned long long*)&Q.symbest[(size_t)q.col * P.n_genes + (k[j] >> P.cnt_bits)];
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < kWBatch; ++j) {
+        if (!live[j]) continue;
+        const uint32_t b = k[j] >> P.cnt_bits, s = k[j] & cmask, den = La_a + (gi[j] & 0xFFFFu) - s;
+        if (Q.symbest) sym_update(Q, &Q.symbest[(size_t)q.col * P.n_genes + b], old[j], b, q.a, s, den);
+        if (Q.colbest) best_update(&Q.colbest[(size_t)b * Q.col_stride + q.col], s, den);
+        best_update(&best[Q.all_pairs ? (gi[j] >> 16) : 0u], s, den);
+      }
     }
     __syncwarp();
-    for (uint32_t u = lane; u < n_used; u += 32) {
-      const uint32_t h = used[u], k = tab[h], b = k >> P.cnt_bits, s = k & cmask;
-      if (!is_target(b)) continue;
-      const uint32_t gi = P.ginfo[b], g = Q.all_pairs ? (gi >> 16) : 0u;
-      const unsigned long long bv = best[g];
-      if (wanted(q, gi >> 16) && ratio_equal(s, La_a + (gi & 0xFFFFu) - s, (uint32_t)(bv >> 32), (uint32_t)bv)) {
-        // 16-bit counts, two to a word
-        atomicAdd((uint32_t*)((uintptr_t)&hcnt[g] & ~(uintptr_t)3), ((uintptr_t)&hcnt[g] & 2u) ? 0x10000u : 1u);
-        used[u] = (uint16_t)(h | kWHit);
+    for (uint32_t u0 = lane; u0 < n_used; u0 += 32u * kWBatch) {
+      uint32_t h[kWBatch], k[kWBatch], gi[kWBatch];
+      bool live[kWBatch];
+#pragma unroll
+      for (uint32_t j = 0; j < kWBatch; ++j) {
+        const uint32_t u = u0 + 32u * j;
+        h[j] = u < n_used ? used[u] : 0u;
+        k[j] = tab[h[j]];
+        live[j] = u < n_used && is_target(k[j] >> P.cnt_bits);
+        gi[j] = live[j] ? P.ginfo[k[j] >> P.cnt_bits] : 0u;
+      }
+#pragma unroll
+      for (uint32_t j = 0; j < kWBatch; ++j) {
+        if (!live[j]) continue;
+        const uint32_t s = k[j] & cmask, g = Q.all_pairs ? (gi[j] >> 16) : 0u;
+        const unsigned long long bv = best[g];
+        if (wanted(q, gi[j] >> 16) &&
+            ratio_equal(s, La_a + (gi[j] & 0xFFFFu) - s, (uint32_t)(bv >> 32), (uint32_t)bv)) {
+          // 16-bit counts, two to a word
+          atomicAdd((uint32_t*)((uintptr_t)&hcnt[g] & ~(uintptr_t)3), ((uintptr_t)&hcnt[g] & 2u) ? 0x10000u : 1u);
+          used[u0 + 32u * j] = (uint16_t)(h[j] | kWHit);
+        }
       }
     }
     __syncwarp();
@@ -1213,7 +1250,7 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
                                                                    (uint32_t)n_sm * std::max(per_sm, 1)));
     TierIO t0{nullptr, nullptr, O.def0, O.n_def0};
     if ((e = launch_begin(L, "summin_warp")) != cudaSuccess) return e;
-    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best);
+    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best, kWEntries);
     if ((e = launch_end(L, "summin_warp")) != cudaSuccess) return e;
     t1.in_list = O.def0;
     t1.in_count = O.n_def0;

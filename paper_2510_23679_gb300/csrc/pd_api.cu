@@ -412,10 +412,10 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
       CK(cudaMemcpyAsync(cursor, d_win_off, sizeof(uint32_t) * n_genes, cudaMemcpyDeviceToDevice, c->stream));
   } else {
     const pdg::SortScratch X = pdg::sort_scratch(K, W);
-    const uint32_t n_dtiles = pdg::dedupe_tiles(W);
+    const uint32_t n_ltiles = pdg::list_tiles(W);
     Carve cs;
     const size_t o_tile_gene = cs.add(sizeof(uint32_t) * (pdg::sort_tiles(W) + 1)),
-                 o_tile_e = cs.add(sizeof(uint32_t) * (n_dtiles + 1)), o_tile_id = cs.add(sizeof(uint32_t) * (n_dtiles + 1)),
+                 o_tile_e = cs.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)), o_tile_id = cs.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)),
                  o_scratch = cs.add(X.bytes), o_rec = cs.add(sizeof(unsigned long long) * W);
     ALLOC(tmp2, cs.bytes);
     uint8_t* scratch = piece<uint8_t>(tmp2, o_scratch);

@@ -459,7 +459,7 @@ struct SortScratch {
 };
 SortScratch sort_scratch(const SortKey& K, uint64_t n);
 uint32_t sort_tiles(uint64_t n);    // tiles of the sort (tile_gene holds one more entry)
-uint32_t dedupe_tiles(uint64_t n);  // tiles of the dedupe pass (tile_e and tile_id hold one more entry)
+uint32_t list_tiles(uint64_t n);    // tiles of the lists pass (tile_e and tile_id hold one more entry)
 constexpr uint32_t kSortBins = 512;  // words of one pass's digit counts
 // Also copies win_off to cursor.
 cudaError_t run_tile_genes(Launcher* L, const uint32_t* win_off, uint32_t n_genes, uint64_t n_windows,
