@@ -206,14 +206,17 @@ void pd_profiles_free(pd_profiles* prof);
  * target genome because global ids are contiguous per genome, and ascending. */
 pd_status pd_best_hits_all(pd_ctx* ctx, const pd_profiles* prof, pd_hits** out);
 
-/* How pd_best_hits_all covers the genome pairs (no counterpart in the paper;
- * the results are identical either way).  enable != 0 (the default): the
- * similarity is symmetric (Eq. (5)), so each unordered genome pair is walked
- * from one side -- a query gene walks only the genomes after its own, emits
- * its Best Hits there and keeps, for every target, the best ratio over the
- * query's genome (the reverse direction, the column maximum of Algorithm 3);
- * used while genes x genomes x 8 bytes stay within 4 GiB.  enable == 0: every
- * query walks every other genome.  Errors: PD_ERR_ARG (null context). */
+/* How pd_best_hits_all, pd_bbh_pairs and pd_bbh_batch cover the genome pairs
+ * (no counterpart in the paper; the results are identical either way).
+ * enable != 0 (the default): the similarity is symmetric (Eq. (5)), so each
+ * unordered genome pair is walked from one side -- a query gene walks only the
+ * genomes after its own, emits its Best Hits there and keeps, for every
+ * target, the best ratio over the query's genome (the reverse direction, the
+ * column maximum of Algorithm 3); used while genes x genomes x 8 bytes stay
+ * within 4 GiB (a batch needs 8 bytes a gene), and for listed pairs and
+ * batches where the postings saved are worth the table of maxima.
+ * enable == 0: every query walks all of its targets.  Errors: PD_ERR_ARG
+ * (null context). */
 pd_status pd_ctx_set_symmetric(pd_ctx* ctx, int enable);
 
 /* Posting walk of the sum-min kernel (no counterpart in the paper; results

@@ -260,7 +260,7 @@ __device__ __forceinline__ bool wanted(const Query& q, uint32_t genome) {
   return !q.mask || ((q.mask[genome >> 5] >> (genome & 31u)) & 1u);
 }
 
-// False if the query is another shard's.
+// False if there is nothing to do for the query: another shard's, or a gene that is a target only.
 __device__ __forceinline__ bool load_query(uint32_t qi, const ProfilesView& P, const QuerySet& Q, Query* q) {
   q->own0 = q->own1 = q->t0 = q->t1 = q->col = 0;
   q->tend = q->self = kEmpty;
@@ -276,11 +276,12 @@ __device__ __forceinline__ bool load_query(uint32_t qi, const ProfilesView& P, c
       q->col = x;
     } else {
       const uint32_t gg = P.gene_genome[a];
+      if (Q.two_genomes && (gg & 1u)) return false;  // no genome after its own: a target only
       q->own0 = (uint32_t)P.genome_ptr[gg];
       q->own1 = (uint32_t)P.genome_ptr[gg + 1];
       if (Q.tgt_end) q->tend = Q.tgt_end[gg];
       if (Q.tgt_mask) q->mask = Q.tgt_mask + (size_t)gg * Q.mask_words;
-      q->col = gg - Q.col_genome0;
+      q->col = Q.two_genomes ? 0u : gg - Q.col_genome0;
     }
     return true;
   }
@@ -393,7 +394,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
   unsigned long long* out = tb.out;
   const uint32_t mask = tb.cap - 1u;
   Query q;
-  if (!load_query(qi, P, Q, &q)) return;  // another shard's query (uniform over the block)
+  if (!load_query(qi, P, Q, &q)) return;  // not a query (uniform over the block)
   const uint32_t a = q.a, row = q.row, own0 = q.own0, own1 = q.own1, tend = q.tend, col = q.col, self = q.self;
   // one target range that fits the table: direct slots instead of hashing
   if (!Q.all_pairs && q.t1 > q.t0 && q.t1 - q.t0 <= tb.cap) acc.dense_lo = q.t0;

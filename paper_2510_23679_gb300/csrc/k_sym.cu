@@ -13,6 +13,9 @@
 // (the stored maxima and the ties that equal them, ascending) followed by its
 // forward Best Hits in the genomes after its own -- ascending overall, since
 // genes are numbered genome by genome.
+//
+// Listed pairs take the same form with a mask of target genomes, and a batch,
+// whose segments are two genomes each, with one maximum a gene.
 #include <algorithm>
 
 #include "pd_internal.cuh"
@@ -26,13 +29,21 @@ __device__ __forceinline__ void unpack(unsigned long long w, uint32_t* s, uint32
   *a = (uint32_t)w & 0x7FFFFFFFu;
 }
 
+// Maxima a gene may have, and the one that gene a's genome keeps.
+__device__ __forceinline__ uint32_t n_columns(const SymRows& R, uint32_t b) {
+  return R.two_genomes ? 1u : R.gene_genome[b];
+}
+__device__ __forceinline__ size_t column_of(const SymRows& R, uint32_t a) {
+  return R.two_genomes ? 0u : R.gene_genome[a];
+}
+
 // One thread per gene: stored maxima of the genomes before its own (the
 // maxima are genome-major, so neighbouring threads read neighbouring words),
 // and the length of its row (tiecnt null: no ties).
 __global__ void __launch_bounds__(256) k_sym_count(SymRows R, const uint32_t* __restrict__ tiecnt,
                                                    uint32_t* __restrict__ stored, uint32_t* __restrict__ total) {
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < R.n_genes; b += gridDim.x * blockDim.x) {
-    const uint32_t gb = R.gene_genome[b];
+    const uint32_t gb = n_columns(R, b);
     uint32_t n = 0;
     for (uint32_t g = 0; g < gb; ++g) n += R.symbest[(size_t)g * R.n_genes + b] != 0ull ? 1u : 0u;
     stored[b] = n;
@@ -64,7 +75,7 @@ __global__ void k_sym_ties(SymRows R, uint32_t* __restrict__ tiecnt, uint8_t* __
        t += (unsigned long long)gridDim.x * blockDim.x) {
     const unsigned long long r = R.tie_rec[2 * t];
     const uint32_t b = (uint32_t)(r >> 32), a = (uint32_t)r, s = (uint32_t)R.tie_rec[2 * t + 1];
-    const unsigned long long w = R.symbest[(size_t)R.gene_genome[a] * R.n_genes + b];
+    const unsigned long long w = R.symbest[column_of(R, a) * R.n_genes + b];
     uint32_t ms, md, ma;
     unpack(w, &ms, &md, &ma);
     const bool ok = w != 0ull && ma != a && ratio_equal(s, R.La[a] + R.La[b] - s, ms, md) &&
@@ -79,7 +90,7 @@ __global__ void __launch_bounds__(256)
     k_sym_write_rev(SymRows R, const unsigned long long* __restrict__ row_ptr, uint32_t* __restrict__ out_b,
                     uint32_t* __restrict__ out_s) {
   for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < R.n_genes; b += gridDim.x * blockDim.x) {
-    const uint32_t gb = R.gene_genome[b];
+    const uint32_t gb = n_columns(R, b);
     unsigned long long at = row_ptr[b];
     for (uint32_t g = 0; g < gb; ++g) {
       const unsigned long long w = R.symbest[(size_t)g * R.n_genes + b];
@@ -111,12 +122,12 @@ __global__ void __launch_bounds__(256)
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
   for (uint32_t b0 = blockIdx.x * 32u; b0 < R.n_genes; b0 += gridDim.x * 32u) {
     const uint32_t nb = min(32u, R.n_genes - b0);
-    const uint32_t gmax = R.gene_genome[b0 + nb - 1];
+    const uint32_t gmax = n_columns(R, b0 + nb - 1);
     for (uint32_t g = warp; g < gmax; g += n_warps)
       tile[g * 33u + lane] = lane < nb ? R.symbest[(size_t)g * R.n_genes + b0 + lane] : 0ull;
     __syncthreads();
     for (uint32_t j = warp; j < nb; j += n_warps) {
-      const uint32_t b = b0 + j, gb = R.gene_genome[b];
+      const uint32_t b = b0 + j, gb = n_columns(R, b);
       unsigned long long at = row_ptr[b];
       for (uint32_t g0 = 0; g0 < gb; g0 += 32) {
         const uint32_t g = g0 + lane;
@@ -253,13 +264,14 @@ __global__ void __launch_bounds__(256) k_sym_bbh_count(SymRows R, uint8_t* __res
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   for (uint32_t a = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; a < R.n_genes; a += warps) {
-    const uint32_t ga = R.gene_genome[a], La = R.La[a];
+    const uint32_t La = R.La[a];
+    const size_t col = column_of(R, a);
     const unsigned long long fo = R.fwd_off[a];
     const uint32_t fl = R.fwd_len[a];
     uint32_t n = 0;
     for (uint32_t e = lane; e < fl; e += 32) {
       const uint32_t b = R.fwd_b[fo + e], sv = R.fwd_s[fo + e];
-      const unsigned long long w = R.symbest[(size_t)ga * R.n_genes + b];
+      const unsigned long long w = R.symbest[col * R.n_genes + b];
       const bool f = ratio_equal(sv, La + R.La[b] - sv, (uint32_t)(w >> 48), (uint32_t)(w >> 31) & 0x1FFFFu);
       flag[fo + e] = f ? 1 : 0;
       n += f ? 1u : 0u;

@@ -702,10 +702,11 @@ static pd_status run_hits_on(pd_ctx* c, const pdg::ProfilesView& v, const pdg::Q
     ALLOC(H->out_s, sizeof(uint32_t) * cap);
     CK(cudaMemsetAsync(cnt, 0, kCounters * sizeof(unsigned long long), c->stream));
     // rows that no query writes (all-pairs rows are the dataset's genes)
-    if (Q.all_pairs && (nq != n_rows || Q.n_shards))
+    if (Q.all_pairs && (nq != n_rows || Q.n_shards || Q.two_genomes))
       CK(cudaMemsetAsync(H->row_len.p, 0, sizeof(uint32_t) * std::max<uint32_t>(n_rows, 1), c->stream));
     if (Q.symbest)  // a rerun starts the reverse maxima and their tie list afresh
-      CK(cudaMemsetAsync(Q.symbest, 0, sizeof(unsigned long long) * v.n_genes * v.n_genomes, c->stream));
+      CK(cudaMemsetAsync(Q.symbest, 0, sizeof(unsigned long long) * v.n_genes * (Q.two_genomes ? 1 : v.n_genomes),
+                         c->stream));
     pdg::HitsOut O;
     O.out_b = H->out_b.as<uint32_t>();
     O.out_s = H->out_s.as<uint32_t>();
@@ -883,36 +884,28 @@ static pd_status hits_pair_impl(pd_ctx* c, const pd_profiles* P, uint32_t gi, ui
   return run_hits(c, P, Q, emit_all, H);
 }
 
-// Largest reverse-maximum table (genes x genomes x 8 B) of the symmetric form.
-constexpr unsigned long long kSymMaxBytes = 4ull << 30;
-
 // The symmetric all-pairs form (k_sym.cu): each unordered genome pair is
 // walked from one side; the launch emits the forward Best Hits and keeps the
 // reverse maxima, and the rows are assembled from both.
-static pd_status sym_hits_impl(pd_ctx* c, const pd_profiles* P, pd_hits* H) {
+pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& queries, bool want_bbh, pd_hits* H,
+                        uint32_t genomes_per_query) {
   const pdg::ProfilesView& v = P->view;
   pdg::Launcher* L = &c->L;
-  const uint32_t G = v.n_genes, NG = v.n_genomes;
+  const uint32_t G = v.n_genes, NG = queries.two_genomes ? 1 : v.n_genomes;
   const unsigned long long sym_bytes = 8ull * G * NG;
   unsigned long long tie_cap = std::max<unsigned long long>(G, 1ull << 16);
   Buf symbest, ties;
   ALLOC(symbest, sym_bytes);
   for (int attempt = 0; attempt < 3; ++attempt) {
     ALLOC(ties, 2 * sizeof(unsigned long long) * tie_cap);
-    pdg::QuerySet Q{};  // run_hits clears the maxima and the tie count before each launch
-    Q.all_pairs = 1;
-    // queries in gene order, i.e. genome by genome: the reverse maxima of the
-    // query genome in flight (its slice of the genome-major array) stay in L2
-    Q.order = nullptr;
-    Q.q0 = 0;
-    Q.n_queries = G;
+    pdg::QuerySet Q = queries;  // run_hits clears the maxima and the tie count before each launch
     Q.symbest = symbest.as<unsigned long long>();
     Q.tie_rec = ties.as<unsigned long long>();
     Q.tie_cap = tie_cap;
     pd_hits F;
     F.ctx = c;
     F.all_pairs = 1;
-    pd_status st = run_hits(c, P, Q, false, &F);  // forward rows (genomes after each query's own)
+    pd_status st = run_hits(c, P, Q, false, &F, genomes_per_query);  // forward rows (genomes after each query's own)
     if (st != PD_OK) return st;
     const unsigned long long n_ties = F.n_ties;
     if (n_ties > tie_cap) {  // more exact ties than the list held: run again with room for all
@@ -940,7 +933,7 @@ static pd_status sym_hits_impl(pd_ctx* c, const pd_profiles* P, pd_hits* H) {
              *bstart = piece<uint32_t>(tmp, o_bstart);
     uint8_t *tie_ok = piece<uint8_t>(tmp, o_ok), *flag = piece<uint8_t>(tmp, o_flag);
     void* scan_tmp = piece<void>(tmp, o_scan);
-    pdg::SymRows R{G, NG, v.gene_genome, v.La, symbest.as<unsigned long long>(), ties.as<unsigned long long>(),
+    pdg::SymRows R{G, NG, v.gene_genome, v.La, queries.two_genomes, symbest.as<unsigned long long>(), ties.as<unsigned long long>(),
                    n_ties, piece<unsigned long long>(tmp, o_set), set_slots ? set_slots - 1 : 0,
                    piece<uint32_t>(tmp, o_listed), piece<uint32_t>(tmp, o_tgene), F.row_off.as<unsigned long long>(), F.row_len.as<uint32_t>(), F.out_b.as<uint32_t>(),
                    F.out_s.as<uint32_t>()};
@@ -951,22 +944,24 @@ static pd_status sym_hits_impl(pd_ctx* c, const pd_profiles* P, pd_hits* H) {
     CK(pdg::run_sym_count(L, R, stored, tiecnt, tie_ok, total.as<uint32_t>(), c->stream));
     CK(pdg::scan_u32_to_u64(L, total.as<uint32_t>(), G, row_ptr.as<unsigned long long>(), scan_tmp, c->stream));
     // BBH while the reverse maxima are at hand
-    CK(pdg::run_sym_bbh_count(L, R, flag, piece<uint32_t>(tmp, o_bcnt), bstart, scan_tmp, c->stream));
+    if (want_bbh) CK(pdg::run_sym_bbh_count(L, R, flag, piece<uint32_t>(tmp, o_bcnt), bstart, scan_tmp, c->stream));
     unsigned long long* h = c->h_build;  // pinned: the row total, the BBH total
     CK(cudaMemcpyAsync(h, row_ptr.as<unsigned long long>() + G, sizeof(*h), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(h + 1, bstart + G, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
+    if (want_bbh) CK(cudaMemcpyAsync(h + 1, bstart + G, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     const unsigned long long n = h[0];
-    const uint32_t n_bbh = *(const uint32_t*)(h + 1);
+    const uint32_t n_bbh = want_bbh ? *(const uint32_t*)(h + 1) : 0u;
     ALLOC(H->out_b, sizeof(uint32_t) * std::max<unsigned long long>(n, 1));
     ALLOC(H->out_s, sizeof(uint32_t) * std::max<unsigned long long>(n, 1));
     CK(pdg::run_sym_write(L, R, stored, tiecnt, tie_ok, row_ptr.as<unsigned long long>(), piece<uint32_t>(tmp, o_fill),
                           H->out_b.as<uint32_t>(), H->out_s.as<uint32_t>(), c->stream));
-    H->bbh = std::make_shared<pd_bbh_set>();
-    H->bbh->ctx = c;
-    H->bbh->n = n_bbh;
-    ALLOC(H->bbh->a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
-    ALLOC(H->bbh->b, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
+    if (want_bbh) {
+      H->bbh = std::make_shared<pd_bbh_set>();
+      H->bbh->ctx = c;
+      H->bbh->n = n_bbh;
+      ALLOC(H->bbh->a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
+      ALLOC(H->bbh->b, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
+    }
     if (n_bbh)
       CK(pdg::run_sym_bbh_write(L, R, flag, bstart, H->bbh->a.as<int32_t>(), H->bbh->b.as<int32_t>(), c->stream));
     st = check_dev_err(c);  // synchronizes: the forward rows and the tables end here
@@ -994,7 +989,12 @@ PD_API pd_status pd_best_hits_all(pd_ctx* c, const pd_profiles* P, pd_hits** out
     H->all_pairs = 1;
     const uint32_t G = P->view.n_genes, NG = P->view.n_genomes;
     if (c->symmetric && G > 0 && NG >= 2 && 8ull * G * NG <= kSymMaxBytes) {
-      pd_status st = sym_hits_impl(c, P, H.get());
+      pdg::QuerySet Q{};
+      Q.all_pairs = 1;
+      // queries in gene order, i.e. genome by genome: the reverse maxima of the
+      // query genome in flight (its slice of the genome-major array) stay in L2
+      Q.n_queries = G;
+      pd_status st = sym_hits(c, P, Q, true, H.get());
       if (st != PD_OK) return st;
       *out = H.release();
       return PD_OK;

@@ -140,8 +140,14 @@ struct ChunkOut {
   std::vector<ChunkJob> jobs;
   Buf d_jobs;
   pd_hits hits;
-  pd_bbh_set bbh;
+  std::shared_ptr<pd_bbh_set> bbh;
 };
+
+// Postings of a chunk from which its jobs are walked from one side: the
+// launches that make the second genomes' rows take some 50 us (4 jobs x 1200
+// genes 0.93 against 0.90 ms, 16 jobs x 1600 1.85 against 2.16, 32 jobs x 6500
+// 10.0 against 12.0).
+constexpr uint64_t kSymMinJoin = 12ull << 20;
 
 pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const int64_t* gene_ptr, uint32_t n_genes,
                      const int32_t* genome_ptr, uint32_t n_genomes, const uint32_t* jobs, const int32_t* job_k,
@@ -277,18 +283,27 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
     Q.walk = tuning ? tuning->walk : PD_WALK_AUTO;
     C->hits.ctx = c;
     C->hits.all_pairs = 1;
-    if ((st = run_hits(c, P.get(), Q, false, &C->hits, 1)) != PD_OK) return st;
+    if (c->symmetric && P->view.n_join >= kSymMinJoin) {
+      // each job walked from its first genome, the second's rows from the
+      // maxima its genes have met
+      Q.two_genomes = 1;
+      if ((st = sym_hits(c, P.get(), Q, true, &C->hits, 1)) != PD_OK) return st;
+      C->bbh = C->hits.bbh;
+    } else {
+      if ((st = run_hits(c, P.get(), Q, false, &C->hits, 1)) != PD_OK) return st;
+      pdg::BbhRows R{};
+      R.all_pairs = 1;
+      R.n_rows = C->hits.n_rows;
+      R.gene_genome = P->view.gene_genome;
+      R.genome_ptr = P->view.genome_ptr;
+      R.row_off = C->hits.row_off.as<unsigned long long>();
+      R.row_len = C->hits.row_len.as<uint32_t>();
+      R.hit_b = C->hits.out_b.as<uint32_t>();
+      C->bbh = std::make_shared<pd_bbh_set>();
+      if ((st = bbh_impl(c, R, C->hits.out_b.n / sizeof(uint32_t), 0, 0, C->bbh.get())) != PD_OK) return st;
+    }
     walked += C->hits.walked;
     n_hits_total += C->hits.n_hits;
-    pdg::BbhRows R{};
-    R.all_pairs = 1;
-    R.n_rows = C->hits.n_rows;
-    R.gene_genome = P->view.gene_genome;
-    R.genome_ptr = P->view.genome_ptr;
-    R.row_off = C->hits.row_off.as<unsigned long long>();
-    R.row_len = C->hits.row_len.as<uint32_t>();
-    R.hit_b = C->hits.out_b.as<uint32_t>();
-    if ((st = bbh_impl(c, R, C->hits.out_b.n / sizeof(uint32_t), 0, 0, &C->bbh)) != PD_OK) return st;
 
     for (uint32_t x = 0; x < cj.size(); ++x) {
       ChunkJob J{};
@@ -308,7 +323,7 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
                                       C->d_jobs.as<ChunkJob>(), nj, C->hits.row_len.as<uint32_t>(),
                                       row_len.as<uint32_t>())));
     PD_KLAUNCH("batch_bbh_runs", (k_bbh_runs<<<grid_of(nj, 128, 152u * 4u), 128, 0, c->stream>>>(
-                                      C->d_jobs.as<ChunkJob>(), nj, C->bbh.a.as<int32_t>(), (uint32_t)C->bbh.n,
+                                      C->d_jobs.as<ChunkJob>(), nj, C->bbh->a.as<int32_t>(), (uint32_t)C->bbh->n,
                                       job_cnt.as<uint32_t>())));
     CK(cudaStreamSynchronize(c->stream));  // host staging vectors and the source offsets are released next
     chunks.push_back(std::move(C));
@@ -338,7 +353,7 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
                    C->hits.row_len.as<uint32_t>(), C->hits.out_b.as<uint32_t>(), C->hits.out_s.as<uint32_t>(),
                    B->row_ptr.as<unsigned long long>(), B->cols.as<int32_t>(), B->s.as<uint32_t>())));
     PD_KLAUNCH("batch_bbh_fill", (k_bbh_fill<<<grid_of(nj, 1, 152u * 16u), 256, 0, c->stream>>>(
-                                      C->d_jobs.as<ChunkJob>(), nj, C->bbh.a.as<int32_t>(), C->bbh.b.as<int32_t>(),
+                                      C->d_jobs.as<ChunkJob>(), nj, C->bbh->a.as<int32_t>(), C->bbh->b.as<int32_t>(),
                                       B->job_ptr.as<unsigned long long>(), B->a.as<int32_t>(),
                                       B->b.as<int32_t>())));
   }
@@ -498,6 +513,12 @@ __global__ void k_pairs_job_ptr(const PairJob* __restrict__ jobs, uint32_t n_job
 // (its genome's range searched in every list): 843 M postings for 180 k genes
 // take 5.0 ms, 1.8 M listed queries on the same dataset 20.9 ms.
 constexpr uint64_t kPostingsPerQuery = 2000;
+// Postings that have to be saved by walking pairs from one side (300 pairs of
+// 60 genomes x 3000 genes 4.8 against 7.9 ms, 1500 pairs 7.3 against 10.1) for
+// each word of the table of maxima: a word is cleared, counted and read again (24 bytes,
+// 3.5 ps at the copy rate), a posting takes 6 to 8 ps.  Below kSymMinSaved the
+// launches that make rows of the maxima cost more than the walk saves.
+constexpr uint64_t kPostingsPerMaximum = 2, kSymMinSaved = 8ull << 20;
 
 pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint32_t n_jobs, pd_batch** out) {
   if (n_jobs && !jobs) return fail(c, PD_ERR_ARG, "null jobs");
@@ -531,45 +552,64 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   // its own is paired with, and the jobs' rows are slices of theirs.
   const uint32_t words = (n_genomes + 31) / 32;
   std::vector<uint32_t> mask((size_t)n_genomes * words, 0);
-  uint64_t n_named = 0, n_directed = 0;  // genes of the genomes named; rows of the distinct ordered pairs
-  std::vector<GenomeSpan> spans;
+  std::vector<uint32_t> last(n_genomes, 0);  // past the last partner of each genome
+  uint64_t n_named = 0, n_directed = 0;      // genes of the genomes named; rows of the distinct ordered pairs
   for (uint32_t j = 0; j < n_jobs; ++j)
     for (int way = 0; way < 2; ++way) {
       const uint32_t a = jobs[2 * j + way], b = jobs[2 * j + 1 - way];
       uint32_t& w = mask[(size_t)a * words + b / 32];
       if (!((w >> (b & 31)) & 1u)) n_directed += (uint64_t)(gp[a + 1] - gp[a]);
       w |= 1u << (b & 31);
+      last[a] = std::max(last[a], b + 1);
     }
+  // Symmetric: each pair is walked from its first genome only (the part of a
+  // list after the gene's own genome), the other direction comes from the
+  // maxima met.
+  uint64_t ahead = 0;  // genes after those of the queries of the symmetric form, summed
   for (uint32_t g = 0; g < n_genomes; ++g) {
-    bool any = false;
-    for (uint32_t w = 0; w < words; ++w) any = any || mask[(size_t)g * words + w] != 0;
-    const uint32_t n = (uint32_t)(gp[g + 1] - gp[g]);
-    if (!any || n == 0) continue;
-    spans.push_back(GenomeSpan{(uint32_t)gp[g], n, (uint32_t)n_named});
-    n_named += n;
+    const uint64_t n = (uint64_t)(gp[g + 1] - gp[g]);
+    if (last[g]) n_named += n;
+    if (last[g] <= g) continue;
+    ahead += n * (uint64_t)(gp[n_genomes] - gp[g + 1]);
   }
-  const uint64_t walk = P->view.n_genes ? P->view.n_join / P->view.n_genes : 0;  // postings of one gene's walk
+  const uint64_t G = P->view.n_genes;
+  const uint64_t walk = G ? P->view.n_join / G : 0;  // postings of one gene's walk
   const bool grouped = n_q && kPostingsPerQuery * n_q >= n_named * walk;
+  const bool symmetric = grouped && c->symmetric && 8ull * G * n_genomes <= kSymMaxBytes &&
+                         (n_named - (double)ahead / G) * walk >= kSymMinSaved + kPostingsPerMaximum * (double)G * n_genomes;
   pd_hits H;
   H.ctx = c;
   pdg::QuerySet Q{};
   pd_status st = PD_OK;
   if (grouped) {
-    const uint32_t n_named32 = (uint32_t)n_named;
-    ALLOC(d_spans, sizeof(GenomeSpan) * spans.size());
     ALLOC(d_mask, sizeof(uint32_t) * mask.size());
     ALLOC(d_qg, sizeof(uint32_t) * n_named);
-    CK(cudaMemcpyAsync(d_spans.p, spans.data(), sizeof(GenomeSpan) * spans.size(), cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemcpyAsync(d_mask.p, mask.data(), sizeof(uint32_t) * mask.size(), cudaMemcpyHostToDevice, c->stream));
-    PD_KLAUNCH("pairs_genes", (k_span_genes<<<grid_of(spans.size(), 1, 152u * 8u), 256, 0, c->stream>>>(
-                                  d_spans.as<GenomeSpan>(), (uint32_t)spans.size(), d_qg.as<uint32_t>())));
     Q.all_pairs = 1;
     Q.order = d_qg.as<uint32_t>();
-    Q.n_queries = n_named32;
     Q.tgt_mask = d_mask.as<uint32_t>();
     Q.mask_words = words;
     H.all_pairs = 1;
-    st = run_hits(c, P, Q, false, &H, (uint32_t)((n_directed + n_named - 1) / n_named));
+    std::vector<GenomeSpan> spans;
+    for (bool sym = symmetric;; sym = false) {
+      spans.clear();
+      uint32_t n_listed = 0;
+      for (uint32_t g = 0; g < n_genomes; ++g) {
+        const uint32_t n = (uint32_t)(gp[g + 1] - gp[g]);
+        if (last[g] <= (sym ? g : 0u) || n == 0) continue;
+        spans.push_back(GenomeSpan{(uint32_t)gp[g], n, n_listed});
+        n_listed += n;
+      }
+      ALLOC(d_spans, sizeof(GenomeSpan) * std::max<size_t>(spans.size(), 1));
+      CK(cudaMemcpyAsync(d_spans.p, spans.data(), sizeof(GenomeSpan) * spans.size(), cudaMemcpyHostToDevice, c->stream));
+      PD_KLAUNCH("pairs_genes", (k_span_genes<<<grid_of(spans.size(), 1, 152u * 8u), 256, 0, c->stream>>>(
+                                    d_spans.as<GenomeSpan>(), (uint32_t)spans.size(), d_qg.as<uint32_t>())));
+      Q.n_queries = n_listed;
+      const uint64_t n_dir = sym ? n_directed / 2 : n_directed;  // rows that the launch emits
+      const uint32_t per_query = (uint32_t)((n_dir + n_listed) / std::max<uint32_t>(n_listed, 1));
+      st = sym ? sym_hits(c, P, Q, false, &H, per_query) : run_hits(c, P, Q, false, &H, per_query);
+      if (st != PD_ERR_OOM || !sym) break;  // no room for the maxima: the plain form needs none
+    }
     if (st != PD_OK) return st;
     ALLOC(d_off, sizeof(unsigned long long) * n_q);
     ALLOC(d_len, sizeof(uint32_t) * n_q);

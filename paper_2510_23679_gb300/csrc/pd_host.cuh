@@ -53,7 +53,7 @@ struct pd_ctx {
   std::string err;
   uint64_t launches = 0;
   bool timing = false;
-  bool symmetric = true;  // pd_best_hits_all walks each genome pair from one side (pd_ctx_set_symmetric)
+  bool symmetric = true;  // each genome pair is walked from one side (pd_ctx_set_symmetric)
   uint32_t walk = PD_WALK_AUTO;  // posting walk of the sum-min kernel (pd_ctx_set_walk)
   std::string timing_filter;  // empty: time every kernel; else only launches of this name
   std::vector<PendingTiming> pending;
@@ -295,6 +295,14 @@ pd_status build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res
 // query can hit; it only sizes the first output allocation.
 pd_status run_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool emit_all, pd_hits* H,
                    uint32_t genomes_per_query = 0);
+// Best Hit rows of every gene by the symmetric form, for the queries of Q (an
+// all-pairs set; its target mask, if any, must be symmetric, and its queries
+// all genes with a target in a later genome), with their BBH pairs if asked
+// for.  genomes_per_query as above.
+pd_status sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool want_bbh, pd_hits* H,
+                   uint32_t genomes_per_query = 0);
+// Largest reverse-maximum table (genes x genomes x 8 B) of the symmetric form.
+constexpr unsigned long long kSymMaxBytes = 4ull << 30;
 // Mutual Best Hits of the rows R into S.
 pd_status bbh_impl(pd_ctx* c, const pdg::BbhRows& R, uint64_t n_hit_slots, uint32_t a_base, uint32_t b_base,
                    pd_bbh_set* S);

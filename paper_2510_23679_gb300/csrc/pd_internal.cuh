@@ -317,8 +317,11 @@ struct QuerySet {
   // genome at symbest[genome(a) * n_genes + b] -- the reverse-direction
   // maximum, packed s << 48 | den << 31 | a -- and lists exact ties of that
   // maximum as the pair of words (b << 32 | a, s) in tie_rec (tie_cap pairs;
-  // the count keeps counting past it).
+  // the count keeps counting past it).  two_genomes: every segment of the
+  // dataset is two genomes, an even one and the next; the genes of the even
+  // ones are the queries, and a gene has one maximum, at symbest[b].
   unsigned long long* symbest;
+  int two_genomes;
   unsigned long long* tie_rec;
   unsigned long long* tie_count;
   unsigned long long tie_cap;
@@ -541,6 +544,7 @@ struct SymRows {
   uint32_t n_genes, n_genomes;
   const uint16_t* gene_genome;
   const uint32_t* La;
+  int two_genomes;                    // one maximum a gene (see QuerySet)
   const unsigned long long* symbest;  // [n_genomes * n_genes], genome-major: b over genome g at g * n_genes + b
   const unsigned long long* tie_rec;  // [2 * n_ties]: (b << 32 | a), s
   unsigned long long n_ties;
