@@ -423,7 +423,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
     // per-posting range tests.  `e` is the query's chunk entry of the k-mer.
     auto accumulate = [&](uint32_t p, uint32_t ca, uint32_t e) {
       uint32_t cb = p & cnt_mask;
-      if (cb == P.cnt_cap && ca > cb) cb = mv_count_of(P, p >> P.cnt_bits, q_mv[m0 + c0 + e].x);
+      if (cb == P.cnt_cap && (kFilter || ca > cb)) cb = mv_count_of(P, p >> P.cnt_bits, q_mv[m0 + c0 + e].x);
       const uint32_t key = kPacked ? (p & ~cnt_mask) : (p >> P.cnt_bits);
       if (!acc.add(mask, key, min(ca, cb), ca, cb)) sh->overflow = 1;
     };

@@ -50,3 +50,18 @@ def test_targets(targets):
             if r == best:
                 row.append((b, s))
         assert list(zip(got[1][got[0][a]:got[0][a + 1]].tolist(), got[2][got[0][a]:got[0][a + 1]].tolist())) == row
+
+
+def test_counts_that_do_not_fit_a_posting():
+    """The directional sums hold the target's own multiplicity, also where it
+    does not fit a posting (14 bits among 140 000 genes): A x 10000 against A x
+    65535, all of whose windows are shared, passes tau = 9/10 both ways."""
+    ctx = pd.pd_ctx_create(0)
+    ds = synth.from_strings([[b"A" * 10000, b"A" * 65535], [b"A" * 65535, b"A" * 9000 + b"C" * 30000],
+                             [b"D" * 9] * 140000])
+    prof = pd.pd_build_profiles(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, 1)
+    assert pd.pd_profiles_get_info(prof).count_bits == 14
+    ptr, col, s = pd.pd_hits_copy(ctx, pd.pd_best_hits_filtered(ctx, prof, 0, 1, (0, 1), (9, 10)))
+    assert (ptr.tolist(), col.tolist(), s.tolist()) == ([0, 1, 2], [0, 0], [10000, 65535])
+    ptr, col, s = pd.pd_hits_copy(ctx, pd.pd_best_hits_filtered(ctx, prof, 0, 1, (0, 1), (1, 5)))
+    assert (ptr.tolist(), col.tolist(), s.tolist()) == ([0, 1, 2], [1, 0], [9000, 65535])
