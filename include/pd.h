@@ -206,8 +206,9 @@ void pd_profiles_free(pd_profiles* prof);
  * target genome because global ids are contiguous per genome, and ascending. */
 pd_status pd_best_hits_all(pd_ctx* ctx, const pd_profiles* prof, pd_hits** out);
 
-/* How pd_best_hits_all, pd_bbh_pairs and pd_bbh_batch cover the genome pairs
- * (no counterpart in the paper; the results are identical either way).
+/* How pd_best_hits_all, pd_best_hits_all_filtered, pd_bbh_pairs and
+ * pd_bbh_batch cover the genome pairs (no counterpart in the paper; the
+ * results are identical either way).
  * enable != 0 (the default): the similarity is symmetric (Eq. (5)), so each
  * unordered genome pair is walked from one side -- a query gene walks only the
  * genomes after its own, emits its Best Hits there and keeps, for every

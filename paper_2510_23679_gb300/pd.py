@@ -303,9 +303,9 @@ def pd_ctx_set_timing(ctx: Ctx, enable: bool) -> None:
 
 
 def pd_ctx_set_symmetric(ctx: Ctx, enable: bool) -> None:
-    """Each genome pair of pd_best_hits_all, pd_bbh_pairs and pd_bbh_batch is
-    walked from one side (True, the default) or every target from every query
-    (False); same results."""
+    """Each genome pair of pd_best_hits_all (filtered or not), pd_bbh_pairs and
+    pd_bbh_batch is walked from one side (True, the default) or every target
+    from every query (False); same results."""
     _check(ctx, _lib.pd_ctx_set_symmetric(ctx.handle, 1 if enable else 0), "pd_ctx_set_symmetric")
 
 

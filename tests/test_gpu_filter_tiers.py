@@ -65,3 +65,25 @@ def test_counts_that_do_not_fit_a_posting():
     assert (ptr.tolist(), col.tolist(), s.tolist()) == ([0, 1, 2], [0, 0], [10000, 65535])
     ptr, col, s = pd.pd_hits_copy(ctx, pd.pd_best_hits_filtered(ctx, prof, 0, 1, (0, 1), (1, 5)))
     assert (ptr.tolist(), col.tolist(), s.tolist()) == ([0, 1, 2], [1, 0], [9000, 65535])
+
+
+@pytest.mark.parametrize("theta,tau", [((0, 1), (0, 1)), ((3, 4), (0, 1)), ((0, 1), (1, 2)), ((4, 5), (2, 5))])
+@pytest.mark.parametrize("genomes,letters,k", [(2, b"AC", 3), (9, b"ACD", 3), (64, synth.ALPHABET, 2)])
+def test_walked_from_one_side(genomes, letters, k, theta, tau):
+    """All pairs walked from one side give the rows and BBH pairs of the form
+    that walks both, on data full of exact ties and with genomes without genes."""
+    ctx = pd.pd_ctx_create(0)
+    rng = np.random.default_rng(genomes)
+    lets = np.frombuffer(letters, np.uint8)
+    genes = [[lets[rng.integers(0, len(lets), int(rng.integers(1, 40)))].tobytes()
+              for _ in range(0 if g == 1 and genomes > 2 else int(rng.integers(20, 90)))] for g in range(genomes)]
+    ds = synth.from_strings(genes)
+    prof = pd.pd_build_profiles(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, k)
+    out = []
+    for symmetric in (True, False):
+        pd.pd_ctx_set_symmetric(ctx, symmetric)
+        hits = pd.pd_best_hits_all_filtered(ctx, prof, theta, tau)
+        out.append([*pd.pd_hits_copy(ctx, hits), pd.pd_bbh_copy(ctx, pd.pd_bbh_all(ctx, prof, hits))])
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
+    assert len(out[0][1])
