@@ -383,16 +383,26 @@ constexpr uint32_t kWarpWalkMinAvg = 16;
 constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
 // The warp tier pays when there are queries for several per resident warp
 // (3648 of them: with one genome pair's 3000 queries the launch takes 0.17
-// against 0.11 ms, with 4800 0.12 against 0.09), and either a query meets few
-// targets (lists of fewer than 8 postings on average, or one target range:
-// 39k queries of 23 genomes 0.33 against 0.50 ms, paralogs of 180k genes 1.0
-// against 1.8) or its lists are long and the index far larger than L2 (200
-// genomes x 4000 genes: 26 against 27 ms).  Between them (50 x 3000) a query
-// meets several hundred chance targets, more of which overflow the warp's
-// table, and the block tier is the faster one (3.2 against 3.4 ms); so do
-// queries from outside the dataset, whose lists are whole (16k queries of a
-// served tick 0.25 ms more).
+// against 0.11 ms, with 4800 0.12 against 0.09), and for queries that meet few
+// targets: those of one target range (paralogs of 180k genes 1.0 against 1.8
+// ms), of short lists (39k queries of 23 genomes 0.30 against 0.45), and in
+// the symmetric form those of few postings.  Where lists are long a query's
+// vector length and the genes after its genome tell how many postings it will
+// walk, and the ones of more than kWMaxPostings leave the warp tier at once,
+// with a table that would have overflowed or a walk that a block does faster:
+// both tiers' time, ms, warp tier for no / the short / every query:
+//   50 genomes x 3000 genes 3.08 / 2.82 / 3.25, 30 x 2000 0.89 / 0.68,
+//   100 x 4000 7.70 / 7.23, 200 x 4000 25.7 / 24.2 / 24.8
+// (1500 postings: 2.98 at 50 x 3000; 4000: 3.03).  Without the symmetric form
+// whole lists are walked and the warp tier takes short lists or, of an index
+// far larger than L2, long ones; queries from outside the dataset stay with
+// the blocks (16k queries of a served tick 0.25 ms more).
 constexpr uint32_t kWarpTierMinQueries = 16384, kWarpTierMaxAvg = 8;
+constexpr float kWMaxPostings = 2500.f;
+// Average list length from which two lanes rather than one share a list in the
+// warp tier of the symmetric form (100 x 4000 7.23 against 7.94 ms, 50 x 3000,
+// with lists of 12, 2.91 against 2.82; 60 x 3000, of 14, 3.57 against 3.48).
+constexpr uint32_t kWPairMinAvg = 15;
 // Target genomes from which a query's Best Hits are ranked through per-genome
 // positions rather than pairwise.
 constexpr uint32_t kRankByGenomeMin = 64;
@@ -803,7 +813,8 @@ __host__ __device__ constexpr size_t warp_tier_bytes(uint32_t n_best) {
 
 template <int kGroup, int kForm>
 __global__ void __launch_bounds__(kWThreads, 6)
-    k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best, uint32_t max_entries) {
+    k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best,
+                  float per_entry) {
   extern __shared__ __align__(16) unsigned char smem[];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   unsigned char* mine = smem + (size_t)warp * warp_tier_bytes(n_best);
@@ -838,7 +849,9 @@ __global__ void __launch_bounds__(kWThreads, 6)
     const uint32_t m0 = P.win_off[q.a], E = P.mv_n[q.a];
     const uint32_t La_a = P.La[q.a];
     // a packed slot holds s <= La_a
-    bool overflow = E > max_entries || La_a >= cmask;
+    bool overflow = E > kWEntries || La_a >= cmask;
+    // too many postings to be expected (per_entry: of an entry, per gene after the query's genome)
+    if (kForm == kSymmetricForm && (float)E * per_entry * (float)(P.n_genes - q.own1) > kWMaxPostings) overflow = true;
     uint32_t n_used = 0;
     // Adds the postings put aside (words gene | min of the counts) in [from, to).
     auto flush = [&](uint32_t from, uint32_t to) {
@@ -1287,12 +1300,14 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   // Where one warp per query pays (see kWarpTier*); tier 1 takes what it defers.
   const bool long_lists = P.n_join >= (uint64_t)kWarpWalkMinAvg * P.n_entries &&
                           P.n_entries * 4ull >= kWarpWalkMinIndexBytes;
-  const bool short_rows = !Q.all_pairs || P.n_join < (uint64_t)kWarpTierMaxAvg * P.n_entries;
+  const bool short_lists = P.n_join < (uint64_t)kWarpTierMaxAvg * P.n_entries;
   if (!emit_all && !P.q_win_off && !Q.colbest && !Q.tgt_end && Q.walk == PD_WALK_AUTO && n_best <= kWMaxGenomes &&
-      Q.n_queries >= kWarpTierMinQueries && (long_lists || short_rows)) {
-    auto kernel = Q.symbest     ? (long_lists ? k_summin_warp<2, kSymmetricForm> : k_summin_warp<1, kSymmetricForm>)
-                  : Q.all_pairs ? (long_lists ? k_summin_warp<2, kAllPairsForm> : k_summin_warp<1, kAllPairsForm>)
-                                : (long_lists ? k_summin_warp<2, kRangeForm> : k_summin_warp<1, kRangeForm>);
+      Q.n_queries >= kWarpTierMinQueries && (long_lists || short_lists || !Q.all_pairs || Q.symbest)) {
+    const bool two = Q.symbest ? P.n_join >= (uint64_t)kWPairMinAvg * P.n_entries : long_lists;
+    auto kernel = Q.symbest     ? (two ? k_summin_warp<2, kSymmetricForm> : k_summin_warp<1, kSymmetricForm>)
+                  : Q.all_pairs ? (two ? k_summin_warp<2, kAllPairsForm> : k_summin_warp<1, kAllPairsForm>)
+                                : (two ? k_summin_warp<2, kRangeForm> : k_summin_warp<1, kRangeForm>);
+    const float per_entry = short_lists ? 0.f : (float)P.n_join / ((float)P.n_entries * (float)P.n_genes);
     const size_t smem = kWWarps * warp_tier_bytes(n_best);
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
       return e;
@@ -1304,7 +1319,7 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
                                                                    (uint32_t)n_sm * std::max(per_sm, 1)));
     TierIO t0{nullptr, nullptr, O.def0, O.n_def0};
     if ((e = launch_begin(L, "summin_warp")) != cudaSuccess) return e;
-    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best, kWEntries);
+    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best, per_entry);
     if ((e = launch_end(L, "summin_warp")) != cudaSuccess) return e;
     t1.in_list = O.def0;
     t1.in_count = O.n_def0;

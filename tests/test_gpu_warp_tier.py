@@ -99,3 +99,15 @@ def test_saturated_counts(ctx):
     prof = pd.pd_build_profiles(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, 5)
     assert pd.pd_profiles_get_info(prof).count_bits == 14
     all_forms(ctx, prof)
+
+
+def test_split_by_expected_postings(ctx):
+    """Lists of more than 8 postings on average: the queries of the first
+    genomes and of long genes go to the blocks, the others to the warps."""
+    for genomes, genes in ((24, 700), (70, 250)):
+        ds = synth.workload("pan50x3000", n_genomes=genomes, genes_per_genome=("fixed", genes), n_families=genes // 2,
+                            seed=genomes)
+        prof = pd.pd_build_profiles(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, 5)
+        info = pd.pd_profiles_get_info(prof)
+        assert info.n_genes >= 16384 and info.n_join >= 8 * info.n_entries
+        all_forms(ctx, prof)
