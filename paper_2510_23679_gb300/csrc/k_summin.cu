@@ -1205,11 +1205,14 @@ constexpr int kT1Threads = 256, kT1MinBlocks = 6;
 // to tier 2.  Past kT1CompactGenomes target genomes the per-genome maxima (12
 // bytes each) no longer leave room for that; the middle layout lists at most
 // 2048 occupied slots and 384 hits and stays within 164 KB up to
-// kT1MidGenomes genomes; past that the full layout (4096 slots listed, 512
-// hits) takes the 196 KB carveout.
+// kT1MidGenomes genomes.  Past that the full layout (4096 slots listed, 512
+// hits) takes the blocks that fit 164 KB, five at first: as many as fit the SM
+// would leave 28 KB of L1, which the walk's loads overrun (300 genomes x 600
+// genes 19.9 against 10.5 ms, 500 x 400 22.6 against 11.5).
 constexpr uint32_t kT1Cap = 4096, kT1OutEmit = 3072;
 constexpr uint32_t kT1Out = 448, kT1Used = 3072;          // compact layout
 constexpr uint32_t kT1OutFull = 512, kT1UsedFull = 4096;  // full layout
+constexpr uint32_t kT1FullCarveout = 164;
 constexpr uint32_t kT1UsedMid = 2048, kT1OutMid = 384;    // middle layout
 constexpr int kT2Threads = 1024;
 constexpr uint32_t kT2Cap = 16384, kT2Out = 2048, kT2OutEmit = 4096;
@@ -1232,10 +1235,13 @@ static_assert(T1F::bytes(PD_MAX_GENOMES) <= 227 * 1024, "tier 1 shared memory");
 static_assert(T2::bytes(PD_MAX_GENOMES) <= 227 * 1024, "tier 2 shared memory");
 static_assert(T2E::bytes(1) <= 227 * 1024, "tier 2 (emit-all, one target genome) shared memory");
 // Filtered queries (Eqs. (6)-(7)): packed 4096-slot table, the two directional
-// sums in one more word a slot (five blocks per SM: 60 k queries of 30 genomes
-// 1.7 ms, against 2.1 for the split table's two blocks); what does not fit goes
-// to a split table of as many slots, then straight to the global tier.
-constexpr int kF1MinBlocks = 5;
+// sums in one more word a slot; what does not fit goes to a split table of as
+// many slots, then straight to the global tier.  Four blocks in a 196 KB
+// carveout, which leaves 60 KB of L1 for the walk: 60 k queries of 30 genomes
+// 1.02 ms, five blocks with 28 KB of L1 1.13, three with 92 KB 1.22 (a split
+// table's two blocks, walking from both sides, 2.1 against 1.7 of the packed).
+constexpr int kF1MinBlocks = 4;
+constexpr uint32_t kF1Carveout = 196;
 constexpr uint32_t kF1Cap = 4096, kF1Used = 2560, kF1Out = 448;
 using TF1 = SmemTier<256, kF1Cap, kF1Out, true, true, kF1Used>;
 static_assert(TF1::bytes(PD_MAX_GENOMES) <= 227 * 1024, "filtered tier shared memory");
@@ -1244,14 +1250,20 @@ constexpr uint32_t kFCap = 4096, kFOut = 512;
 using TF = SmemTier<kFThreads, kFCap, kFOut, false, true>;
 static_assert(TF::bytes(PD_MAX_GENOMES) <= 227 * 1024, "filtered tier shared memory");
 
+// carveout (KB, 0: what the resident blocks take): shared memory of an SM to
+// stay within, the rest being L1.
 template <typename K>
 cudaError_t launch_smem(K kernel, Launcher* L, const char* name, int threads, size_t smem, uint32_t max_grid,
                         const ProfilesView& P, const QuerySet& Q, const HitsOut& O, const TierIO& T, DevErr* err,
-                        cudaStream_t s) {
+                        cudaStream_t s, uint32_t carveout = 0) {
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  if (carveout && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                            (int)(carveout * 100 / 228))) != cudaSuccess)
+    return e;
   int per_sm = 1, dev = 0, n_sm = 152;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+  if (carveout) per_sm = std::min<int>(per_sm, (int)(carveout * 1024u / (smem + 1024u + sizeof(Scalars))));
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   const uint32_t grid = std::max<uint32_t>(1, std::min<uint32_t>(max_grid, (uint32_t)n_sm * std::max(per_sm, 1)));
@@ -1272,7 +1284,7 @@ cudaError_t launch_t1(Launcher* L, uint32_t n_best, const ProfilesView& P, const
     return launch_smem(k_summin_smem<t, b, kT1Cap, kT1OutMid, true, false, false, kT1UsedMid, kWarpWalk, kForm>, L,
                        "summin_bh", t, T1M::bytes(n_best), Q.n_queries, P, Q, O, T, err, s);
   return launch_smem(k_summin_smem<t, b, kT1Cap, kT1OutFull, true, false, false, kT1UsedFull, kWarpWalk, kForm>, L,
-                     "summin_bh", t, T1F::bytes(n_best), Q.n_queries, P, Q, O, T, err, s);
+                     "summin_bh", t, T1F::bytes(n_best), Q.n_queries, P, Q, O, T, err, s, kT1FullCarveout);
 }
 
 }  // namespace
@@ -1287,9 +1299,9 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
     const cudaError_t e1 =
         Q.symbest ? launch_smem(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used, false,
                                               kSymmetricForm>,
-                                L, "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s)
+                                L, "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout)
                   : launch_smem(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used>, L,
-                                "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s);
+                                "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout);
     if (e1 != cudaSuccess) return e1;
     return launch_smem(k_summin_smem<kFThreads, kFMinBlocks, kFCap, kFOut, false, false, true>, L, "summin_bh_f",
                        kFThreads, TF::bytes(n_best), Q.n_queries, P, Q, O, tf, err, s);
