@@ -151,6 +151,15 @@ def captured_counter(kernel_src, summary, key="dram_bytes_per_launch"):
     return int(m_val.group(1))
 
 
+SUMMIN_TIERS = ("summin_warp", "summin_bh", "summin_bh_t2", "summin_bh_t3")
+
+
+def summin_ms(pd, ctx):
+    """Device ms of the sum-min tiers since the last timing reset (one call of
+    the Best Hits launches each tier once)."""
+    return sum(pd.pd_ctx_kernel_time(ctx, name)[0] for name in SUMMIN_TIERS)
+
+
 def alphabet_of(name):
     return 4 if synth.WORKLOADS.get(name, {}).get("alphabet") == "nt" else 20
 
@@ -605,7 +614,6 @@ def run_sharded(args):
         step(res_d, gp_d, gn_d)
     torch.cuda.synchronize()
     pd.pd_ctx_reset_timing(ctx)
-    pd.pd_ctx_set_timing_filter(ctx, "summin_bh")
     pd.pd_ctx_set_timing(ctx, True)
     launches0 = pd.pd_ctx_launch_count(ctx)
     times = []
@@ -622,7 +630,7 @@ def run_sharded(args):
             times.append(e0.elapsed_time(e1))
     dist.barrier()
     gpu_launches = pd.pd_ctx_launch_count(ctx) - launches0
-    k_ms, k_n = pd.pd_ctx_kernel_time(ctx, "summin_bh")
+    k_avg = summin_ms(pd, ctx) / max(1, args.steps)
     pd.pd_ctx_set_timing(ctx, False)
     ms_local = sum(times) / len(times)
     ms = max_over_ranks(ms_local, world)
@@ -634,7 +642,6 @@ def run_sharded(args):
     shard_hits = pd.pd_hits_get_info(pd.pd_best_hits_shard(ctx, prof, rank, world))
     alg = (pinfo.n_entries * 14 + pinfo.n_genes * 12) / world + shard_hits.postings_walked * 4 + \
         shard_hits.n_hits * 8
-    k_avg = k_ms / max(1, k_n)
     peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6800.0)) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
     clocks = clk.summary()
@@ -646,7 +653,7 @@ def run_sharded(args):
                 "config": config_of(ds, args.workload, k, L2_NOTE, parallelism_of(world, "shard")),
                 "genome_pairs_per_s": ds.n_genomes * (ds.n_genomes - 1) // 2 / (ms / 1e3), "step_ms": times,
                 "roofline": {"bound": "hbm", "achieved": alg / (k_avg / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
-                             "frac": alg / (k_avg / 1e3) / 1e9 / peak, "traffic": None, "kernel": "summin_bh",
+                             "frac": alg / (k_avg / 1e3) / 1e9 / peak, "traffic": None, "kernel": "sum-min tiers",
                              "kernel_ms": k_avg, "alg_bytes": alg, "scope": "rank 0's shard"},
                 "e2e": None, "gpu_launches": gpu_launches, "cpu_baseline": None, "clocks": clocks,
                 "stats": {"best_hits": pd.pd_hits_get_info(hits).n_hits, "bbh_pairs": pd.pd_bbh_count(bbh)}}
@@ -703,11 +710,8 @@ def main():
             import torch.distributed as dist
             dist.barrier()
 
-    # ---- device-resident timed region (per-launch events on the dominant
-    # kernel only, so the other launches run without event records)
-    pd.pd_ctx_reset_timing(ctx)
-    pd.pd_ctx_set_timing_filter(ctx, "summin_bh")
-    pd.pd_ctx_set_timing(ctx, True)
+    # ---- device-resident timed region (no per-launch events: the kernels' own
+    # times are taken in the phase breakdown below)
     launches0 = pd.pd_ctx_launch_count(ctx)
     ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(args.steps)]
     barrier()
@@ -723,9 +727,6 @@ def main():
     barrier()
     gpu_launches = pd.pd_ctx_launch_count(ctx) - launches0
     step_ms = [a.elapsed_time(b) for a, b in ev]
-    k_ms, k_n = pd.pd_ctx_kernel_time(ctx, "summin_bh")
-    pd.pd_ctx_set_timing(ctx, False)
-    pd.pd_ctx_set_timing_filter(ctx, None)
     ms_local = sum(step_ms) / len(step_ms)
     pairs = ds.logical_pairs()
     value = whole_job_rate(pairs, ms_local / 1e3, world)
@@ -737,12 +738,10 @@ def main():
     hinfo = pd.pd_hits_get_info(hits)
     n_bbh = pd.pd_bbh_count(bbh)
 
-    # ---- roofline of the dominant kernel (sum-min + Best Hits), algorithmic bytes per launch
+    # ---- roofline of the dominant kernels (the sum-min + Best Hit tiers), algorithmic bytes per step
     E = pinfo.n_entries
     J = hinfo.postings_walked
     alg_bytes = E * 6 + E * 8 + J * 4 + hinfo.n_hits * 8 + pinfo.n_genes * 12
-    k_avg_ms = k_ms / max(1, k_n)
-    achieved = alg_bytes / (k_avg_ms / 1e3) / 1e9
     peaks = {}
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
@@ -765,23 +764,31 @@ def main():
         return out, e0.elapsed_time(e1), kms, kn
 
     ph = {"build": [], "best_hits": [], "bbh": []}
+    tiers = []
     pd.pd_ctx_set_timing(ctx, True)
     for i in range(3):
         flush.fill_(i)
         torch.cuda.synchronize()
         p_, *t_b = timed_phase(lambda: pd.pd_build_profiles_alphabet(ctx, res_d, gp_d, gn_d, alpha, k))
         h_, *t_h = timed_phase(lambda: pd.pd_best_hits_all(ctx, p_))
+        tiers.append(summin_ms(pd, ctx))
         _, *t_x = timed_phase(lambda: pd.pd_bbh_all(ctx, p_, h_))
         for name, t in (("build", t_b), ("best_hits", t_h), ("bbh", t_x)):
             ph[name].append(t)
     pd.pd_ctx_set_timing(ctx, False)
     phases = {name: {"ms": statistics.median(t[0] for t in v), "kernel_ms": statistics.median(t[1] for t in v),
                      "launches": int(v[0][2])} for name, v in ph.items()}
-    # encoder (profiles + inverted index) roofline: algorithmic bytes of one build
+    k_avg_ms = statistics.median(tiers)
+    achieved = alg_bytes / (k_avg_ms / 1e3) / 1e9
+    # encoder (profiles + inverted index) roofline: algorithmic bytes of one
+    # build.  Residues read for the check, the digit counts and the first sort
+    # pass; 8-byte records written by it, read and written by each later pass
+    # and read by the dedupe pass; the index (4 bytes a posting, list starts
+    # and codes) written, and read once for the vectors, whose entries (those
+    # of k-mers that several genes hold, not counted here) come on top.
     W, D = pinfo.n_windows, pinfo.n_distinct
-    passes = (max(1, int(D).bit_length()) + 8) // 9
-    enc_bytes = (2 * ds.n_residues + E * 6 + pinfo.n_genes * 4 + W * 8 + passes * W * 16
-                 + W * 8 + E * 4 + D * 4 + E * 12)
+    passes = ((alpha ** k - 1).bit_length() + 8) // 9
+    enc_bytes = 3 * ds.n_residues + W * 8 + (passes - 1) * W * 16 + W * 8 + 2 * (E * 4 + D * 4) + D * (4 if alpha ** k <= 1 << 32 else 8)
     enc_ms = phases["build"]["kernel_ms"]
     encoder = {"bound": "hbm", "alg_bytes": int(enc_bytes), "kernel_ms": enc_ms,
                "achieved": enc_bytes / (enc_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
@@ -869,19 +876,19 @@ def main():
                "sample": f"genome pairs {done} of the same workload ({npairs} gene pairs, {dt:.1f} s, "
                          f"profiles of both genomes included), oracle threads={cores}"}
 
-    # the pipe that bounds the sum-min kernel: L1TEX data-pipe wavefronts
-    # (shared-memory accumulator + posting loads; ncu counts one launch) per
-    # second of the live kernel time, against one wavefront per cycle per SM
+    # a pipe that the sum-min tiers load: L1TEX data-pipe wavefronts
+    # (shared-memory accumulators + posting loads; ncu, all tiers of one step)
+    # per second of the live kernel time, against one wavefront per cycle per SM
     # at the SM clock sampled during the timed region
     clocks = clk.summary()
-    wavefronts = captured_counter("paper_2510_23679_gb300/csrc/k_summin.cu", f"summin_bh_{args.workload}.md",
+    wavefronts = captured_counter("paper_2510_23679_gb300/csrc/k_summin.cu", f"summin_{args.workload}.md",
                                   "l1tex_wavefronts_per_launch")
     l1tex = None
     if wavefronts and clocks.get("sm_mhz"):
         n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
         l1_peak = n_sm * clocks["sm_mhz"] * 1e6 / 1e9
         l1_achieved = wavefronts / (k_avg_ms / 1e3) / 1e9
-        l1tex = {"bound": "l1tex", "kernel": "summin_bh", "achieved": l1_achieved, "peak": l1_peak,
+        l1tex = {"bound": "l1tex", "kernel": "sum-min tiers", "achieved": l1_achieved, "peak": l1_peak,
                  "unit": "G wavefronts/s", "frac": l1_achieved / l1_peak, "wavefronts": wavefronts,
                  "peak_source": f"{n_sm} SMs x 1 wavefront/cycle x {clocks['sm_mhz']:.0f} MHz"}
 
@@ -897,8 +904,8 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
                          "traffic": captured_counter("paper_2510_23679_gb300/csrc/k_summin.cu",
-                                                     f"summin_bh_{args.workload}.md"),
-                         "kernel": "summin_bh",
+                                                     f"summin_{args.workload}.md"),
+                         "kernel": "sum-min tiers",
                          "kernel_ms": k_avg_ms, "alg_bytes": alg_bytes, "peak_source": peak_src},
             "e2e": e2e,
             "served": served,

@@ -32,10 +32,14 @@
 // (Adinets and Merrill, "Onesweep", 2022).  A wait that runs out raises
 // PD_ERR_INTERNAL and its tile writes nothing.
 //
-// Measured at 200 genomes x 4000 genes, k = 7 (264 M windows): 17.5 ms for the
+// Measured at 200 genomes x 4000 genes, k = 7 (264 M windows): 15.1 ms for the
 // whole build against 23.4 ms for a dictionary of all codes (marked and looked
 // up at random, 183 MB), hash tables per gene and a gather of every vector
-// entry's list; 2.9 against 3.3 ms at 50 x 3000, k = 6.
+// entry's list; 2.6 against 3.3 ms at 50 x 3000, k = 6.  Of the 15.1: windows
+// counted 0.9, four sort passes 6.9 (each moves 4.2 GB in 1.6, 40% of the copy
+// rate: bound by the latency of its phases at two blocks per SM), dedupe 1.8,
+// lists 5.4 (an atomic and a 16-byte store at random for each of 130 M
+// entries: bound by the rate of scattered requests to L2).
 #include <algorithm>
 #include <type_traits>
 

@@ -34,11 +34,13 @@
 // query's genome in global memory (the reverse-direction maximum needed for
 // the mutual check of Eq. (9)).
 // The similarity matrix S_ij is never materialised: only pairs sharing a
-// k-mer are touched.  A query whose insertions probe too far (a nearly full
-// table), or whose Best Hit list does not fit, is deferred to the next tier:
-// 4096 slots in shared memory (256 threads) -> 16384 slots in shared memory
-// (1024 threads, one block per SM) -> a global-memory table sized for every
-// possible target.  Results are exact and independent of the tier.
+// k-mer are touched.  Where queries are many, one warp each takes those that
+// meet few targets (the warp tier below); blocks take the others.  A query
+// whose insertions probe too far (a nearly full table), or whose Best Hit list
+// does not fit, is deferred to the next tier: 4096 slots in shared memory (256
+// threads) -> 16384 slots in shared memory (1024 threads, one block per SM) ->
+// a global-memory table sized for every possible target.  Results are exact
+// and independent of the tier.
 #include <algorithm>
 
 #include "pd_internal.cuh"
@@ -385,15 +387,16 @@ constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
 // (3648 of them: with one genome pair's 3000 queries the launch takes 0.17
 // against 0.11 ms, with 4800 0.12 against 0.09), and for queries that meet few
 // targets: those of one target range (paralogs of 180k genes 1.0 against 1.8
-// ms), of short lists (39k queries of 23 genomes 0.30 against 0.45), and in
+// ms), of short lists (39k queries of 23 genomes 0.33 against 0.50), and in
 // the symmetric form those of few postings.  Where lists are long a query's
 // vector length and the genes after its genome tell how many postings it will
 // walk, and the ones of more than kWMaxPostings leave the warp tier at once,
 // with a table that would have overflowed or a walk that a block does faster:
 // both tiers' time, ms, warp tier for no / the short / every query:
-//   50 genomes x 3000 genes 3.08 / 2.82 / 3.25, 30 x 2000 0.89 / 0.68,
-//   100 x 4000 7.70 / 7.23, 200 x 4000 25.7 / 24.2 / 24.8
-// (1500 postings: 2.98 at 50 x 3000; 4000: 3.03).  Without the symmetric form
+//   50 genomes x 3000 genes 3.08 / 2.82 / 3.25, 30 x 2000 0.89 / 0.68 / -,
+//   100 x 4000 7.70 / 7.23 / -, 200 x 4000 - / 24.2 / 24.8
+// (1500 postings instead: 2.98 at 50 x 3000, 25.2 at 200 x 4000; 4000: 3.03
+// and 24.4).  Without the symmetric form
 // whole lists are walked and the warp tier takes short lists or, of an index
 // far larger than L2, long ones; queries from outside the dataset stay with
 // the blocks (16k queries of a served tick 0.25 ms more).

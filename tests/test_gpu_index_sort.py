@@ -63,9 +63,9 @@ def dataset(rng, lengths, letters, genomes):
     return synth.from_strings([genes[a:b] for a, b in zip([0] + cuts, cuts + [len(genes)])])
 
 
-# window totals one below, at and one above the tiles of the sort (7680) and
-# of the pass over the sorted records (4096), and several of each
-@pytest.mark.parametrize("total", [1, 31, 4095, 4096, 4097, 7679, 7680, 7681, 15360, 15361, 40961])
+# window totals one below, at and one above the tiles of the sort (7680), of
+# the pass over the sorted records (8192) and its halves, and several of each
+@pytest.mark.parametrize("total", [1, 31, 4095, 4096, 4097, 7679, 7680, 7681, 8191, 8192, 8193, 15360, 15361, 40961])
 @pytest.mark.parametrize("letters,k", [(b"AC", 1), (b"ACD", 3), (synth.ALPHABET, 2), (synth.ALPHABET, 8)])
 def test_window_totals(ctx, total, letters, k):
     rng = np.random.default_rng(total * 100 + k)
