@@ -209,7 +209,7 @@ __device__ __forceinline__ void tile_windows(const WindowSource& S, const uint8_
     const uint32_t c = lut[*s++];
     code = code * a + c;
     recent = (recent << bits) | c;
-    emit(i, code + base, g);
+    emit(i, (code << S.code_shift) + base, g);
     code -= (Code)(uint32_t)(recent >> drop) * lead_w;
     recent &= keep;
   }
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kThreads)
       if (all || ((u64)code >> K.code_bits) == K.slice) {
 #pragma unroll
         for (uint32_t p = 0; p < kPasses; ++p)
-          atomicAdd(&cnt[p * kMaxBins + ((uint32_t)(code >> (p * K.width)) & (p + 1 < kPasses ? dmask : K.last_mask))],
+          atomicAdd(&cnt[p * kMaxBins + ((uint32_t)(code >> (K.skip + p * K.width)) & (p + 1 < kPasses ? dmask : K.last_mask))],
                     1u);
       }
     });
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
     valid |= xr[r] != ~0ull ? 1u << r : 0u;
   }
   __syncthreads();
-  rank_and_write<kBits, T>(xr, valid, K.gene_bits, status, out, sh, stage, err);
+  rank_and_write<kBits, T>(xr, valid, K.gene_bits + K.skip, status, out, sh, stage, err);
 }
 
 template <int kBits, typename T>
@@ -803,7 +803,7 @@ unsigned grid_for(uint64_t items, unsigned per_block, unsigned cap) {
 
 // Digit bits of pass p: at least 5 (the bits past the key's are zero).
 uint32_t pass_bits(const SortKey& K, uint32_t p) {
-  return std::max<uint32_t>(5u, p + 1 < K.passes ? K.width : K.code_bits - (K.passes - 1) * K.width);
+  return std::max<uint32_t>(5u, p + 1 < K.passes ? K.width : K.code_bits - K.skip - (K.passes - 1) * K.width);
 }
 
 // Calls f with the digit bits as a compile-time constant.
@@ -825,7 +825,7 @@ cudaError_t sort_passes(Launcher* L, const WindowSource& S, const SortKey& K, ui
   uint32_t* ticket = (uint32_t*)(scratch + X.tickets);
   u64 *src = a, *dst = a;
   for (uint32_t p = 0; p < K.passes; ++p) {
-    const uint32_t shift = K.gene_bits + p * K.width;
+    const uint32_t shift = K.gene_bits + K.skip + p * K.width;
     T* status = (T*)(scratch + X.pass[p]);
     const uint32_t* hist = (const uint32_t*)(scratch + X.hist) + p * kMaxBins;
     const cudaError_t e = with_bits(pass_bits(K, p), [&](auto w) -> cudaError_t {
@@ -857,7 +857,7 @@ cudaError_t sort_passes(Launcher* L, const WindowSource& S, const SortKey& K, ui
 
 }  // namespace
 
-SortKey sort_key(uint64_t n_codes, uint32_t gene_bits) {
+SortKey sort_key(uint64_t n_codes, uint32_t gene_bits, uint32_t skip) {
   SortKey K{};
   uint32_t bits = 1;
   while (bits < 63 && ((n_codes - 1) >> bits) != 0) ++bits;
@@ -868,9 +868,11 @@ SortKey sort_key(uint64_t n_codes, uint32_t gene_bits) {
   K.total_bits = bits;
   K.code_bits = std::min(bits, most);
   K.n_slices = bits > most ? 1u << (bits - most) : 1u;
-  K.passes = (K.code_bits + 8) / 9;
-  K.width = (K.code_bits + K.passes - 1) / K.passes;
-  K.last_mask = (1u << (K.code_bits - (K.passes - 1) * K.width)) - 1u;
+  K.skip = skip;
+  const uint32_t sorted = K.code_bits - skip;
+  K.passes = (sorted + 8) / 9;
+  K.width = (sorted + K.passes - 1) / K.passes;
+  K.last_mask = (1u << (sorted - (K.passes - 1) * K.width)) - 1u;
   return K;
 }
 

@@ -263,7 +263,7 @@ static constexpr uint64_t kMaxDictCodes = (uint64_t)32 << 30;
 pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const int64_t* gene_ptr,
                                      uint32_t n_genes, const int32_t* genome_ptr, uint32_t n_genomes, int k,
                                      const uint32_t* genome_seg, pd_profiles** out, const int64_t* gene_src,
-                                     int alphabet, int length_buckets) {
+                                     int alphabet, int length_buckets, bool code_order) {
   PhaseRange range_("pd: profiles");
   if (alphabet != PD_ALPHABET_AMINO && alphabet != PD_ALPHABET_NUCLEOTIDE)
     return fail(c, PD_ERR_ARG, "alphabet must be 20 (amino acids) or 4 (nucleotides)");
@@ -327,7 +327,18 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   const uint32_t gene_bits = bits_for(n_genes);
   const uint32_t cnt_bits = 32 - gene_bits;
   const uint32_t cnt_cap = std::min<uint32_t>((1u << cnt_bits) - 1u, 65535u);
-  pdg::SortKey K = pdg::sort_key(n_seg * n_codes, gene_bits);
+  // Segments that may stand below the k-mer in the code need no sorting: the
+  // windows are made in gene order, which is theirs (a pass fewer for 16 jobs
+  // at k = 6, 32 genome pairs at k = 5 and 6 10.0 -> 9.6 ms).
+  uint32_t seg_bits = 0, kmer_bits = 1;
+  while ((n_seg - 1) >> seg_bits) ++seg_bits;
+  while (kmer_bits < 63 && ((n_codes - 1) >> kmer_bits)) ++kmer_bits;
+  const bool below = genome_seg && !code_order && kmer_bits + seg_bits + gene_bits <= 64;
+  if (!below) seg_bits = 0;
+  const uint64_t all_codes = below ? n_codes << seg_bits : n_seg * n_codes;
+  if (below)
+    for (uint32_t i = 0; i < n_genomes; ++i) code_base[i] = genome_seg[i];
+  pdg::SortKey K = pdg::sort_key(all_codes, gene_bits, seg_bits);
 
   // ---- per-gene arrays, inputs on the device
   Carve cg;
@@ -396,7 +407,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
 
   // ---- vectors, postings, and one record buffer that ends up holding the
   // posting-list starts and the codes (at most one of each per window)
-  const bool wide_codes = n_seg * n_codes > (1ull << 32);
+  const bool wide_codes = all_codes > (1ull << 32);
   Carve cw;
   const size_t o_mv = cw.add(sizeof(uint4) * W), o_post = cw.add(sizeof(uint32_t) * W),
                o_lists = cw.add(2 * sizeof(uint32_t) * (W + 1)), o_code_hi = cw.add(wide_codes ? W : 0);
@@ -421,7 +432,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
     uint8_t* scratch = piece<uint8_t>(tmp2, o_scratch);
     uint32_t *tile_e = piece<uint32_t>(tmp2, o_tile_e), *tile_id = piece<uint32_t>(tmp2, o_tile_id);
     pdg::WindowSource S{res_dev, gp_devp, gene_src, d_win_off, piece<uint32_t>(tmp2, o_tile_gene), d_gene_genome,
-                        d_code_base, k, alphabet, W};
+                        d_code_base, k, alphabet, W, seg_bits};
     // two record buffers, one of which ends up holding lists and codes
     unsigned long long *rec = piece<unsigned long long>(tmp2, o_rec), *other = (unsigned long long*)d_post_ptr;
     const bool odd = K.passes & 1u;

@@ -286,10 +286,13 @@ pd_status run_hits_view(pd_ctx* c, const pdg::ProfilesView& v, const pdg::QueryS
 // segment its own k-mer namespace.  gene_src (device, per gene, or null):
 // gene g starts at residues + gene_src[g] instead of residues + gene_ptr[g];
 // gene_ptr then gives only the lengths, and residues must be a device pointer.
+// code_order: lists in order of segment, then code; without it (genome_seg
+// must not decrease) in any order that suits the build.
 pd_status build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const int64_t* gene_ptr,
                               uint32_t n_genes, const int32_t* genome_ptr, uint32_t n_genomes, int k,
                               const uint32_t* genome_seg, pd_profiles** out, const int64_t* gene_src = nullptr,
-                              int alphabet = PD_ALPHABET_AMINO, int length_buckets = 1);
+                              int alphabet = PD_ALPHABET_AMINO, int length_buckets = 1,
+                              bool code_order = true);
 // Sum-min + Best Hits of the query set Q into H (all tiers, output sized
 // exactly).  genomes_per_query (0 = n_genomes - 1) bounds the genomes one
 // query can hit; it only sizes the first output allocation.

@@ -442,19 +442,24 @@ struct WindowSource {
   const uint32_t* win_off;
   const uint32_t* tile_gene;   // gene of the first window of each sort tile
   const uint16_t* gene_genome;
-  const unsigned long long* genome_code_base;  // per genome: segment * 20^k, or null (one segment)
+  const unsigned long long* genome_code_base;  // per genome, or null (one segment): see code_shift
   int k, alpha;
   uint64_t n_windows;
+  // a window's code: (its k-mer's << code_shift) + the base of its genome's
+  // segment, which is segment * 20^k, or with a shift the segment
+  uint32_t code_shift;
 };
 // A sort record: code << gene_bits | gene.  Codes that do not fit beside the
 // gene are sorted in slices of equal high bits (code >> code_bits == slice).
 constexpr uint32_t kMaxSortPasses = 4;
 struct SortKey {
   uint32_t gene_bits, total_bits, code_bits, n_slices;  // total_bits: of a whole code
-  uint32_t passes, width, last_mask;  // digits: width bits each, the last one's mask
+  // digits above the lowest `skip` bits of the code (which the order of the
+  // genes sorts): width bits each, the last one's mask
+  uint32_t skip, passes, width, last_mask;
   unsigned long long slice;
 };
-SortKey sort_key(uint64_t n_codes, uint32_t gene_bits);
+SortKey sort_key(uint64_t n_codes, uint32_t gene_bits, uint32_t skip);
 // Byte offsets into the zeroed scratch of one slice.
 struct SortScratch {
   size_t tickets, hist, dedupe, pass[kMaxSortPasses], bytes;
