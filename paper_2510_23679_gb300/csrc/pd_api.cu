@@ -1350,9 +1350,12 @@ PD_API pd_status pd_best_hits_all_filtered(pd_ctx* c, const pd_profiles* P, cons
     // side (30 genomes x 2000 genes 1.45 against 1.87 ms; 60 x 3000, where half
     // the targets also fit the packed table, 10.7 against 30.5)
     const uint32_t G = P->view.n_genes, NG = P->view.n_genomes;
-    if (c->symmetric && G > 0 && NG >= 2 && 8ull * G * NG <= kSymMaxBytes) {
-      st = sym_hits(c, P, Q, true, H.get());
-    } else {
+    const bool symmetric = c->symmetric && G > 0 && NG >= 2 && 8ull * G * NG <= kSymMaxBytes;
+    if (symmetric) st = sym_hits(c, P, Q, true, H.get());
+    if (!symmetric || st == PD_ERR_OOM) {  // the plain form needs no room for the maxima
+      H.reset(new pd_hits());
+      H->ctx = c;
+      H->all_pairs = 1;
       Q.order = P->view.order;
       st = run_hits(c, P, Q, false, H.get());
     }

@@ -283,13 +283,21 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
     Q.walk = tuning ? tuning->walk : PD_WALK_AUTO;
     C->hits.ctx = c;
     C->hits.all_pairs = 1;
-    if (c->symmetric && P->view.n_join >= kSymMinJoin) {
+    bool symmetric = c->symmetric && P->view.n_join >= kSymMinJoin;
+    if (symmetric) {
       // each job walked from its first genome, the second's rows from the
       // maxima its genes have met
       Q.two_genomes = 1;
-      if ((st = sym_hits(c, P.get(), Q, true, &C->hits, 1)) != PD_OK) return st;
+      st = sym_hits(c, P.get(), Q, true, &C->hits, 1);
+      if (st != PD_OK && st != PD_ERR_OOM) return st;
+      symmetric = st == PD_OK;
       C->bbh = C->hits.bbh;
-    } else {
+    }
+    if (!symmetric) {  // or no room for the maxima
+      Q.two_genomes = 0;
+      C->hits = pd_hits();
+      C->hits.ctx = c;
+      C->hits.all_pairs = 1;
       if ((st = run_hits(c, P.get(), Q, false, &C->hits, 1)) != PD_OK) return st;
       pdg::BbhRows R{};
       R.all_pairs = 1;

@@ -87,3 +87,52 @@ def test_batched_jobs(ctx, query_order):
     got = both(ctx, lambda: pd.pd_bbh_batch(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, jobs, ks,
                                             query_order=query_order))
     check_oracle(ds, got, jobs[0], 3, 0, 0)
+
+
+class Refuse:
+    def __init__(self):
+        self.calls = self.at = 0
+
+    def on_alloc(self, nbytes):
+        self.calls += 1
+        return self.calls != self.at
+
+
+@pytest.mark.parametrize("form", ["pairs", "batch", "filtered"])
+def test_no_room_for_the_maxima(form):
+    """Each allocation of a call refused in turn: the call reports it, or finds
+    room for the form that walks both sides and gives the same result."""
+    refuse = Refuse()
+    ctx = pd.pd_ctx_create(0, on_alloc=refuse.on_alloc)
+    rng = np.random.default_rng(3)
+    ds = dataset(rng, [150] * 12 + [0], b"ACD", 50)
+    if form == "batch":
+        ds = dataset(rng, [900, 900, 0], b"ACD", 60)
+    prof = pd.pd_build_profiles(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, 3)
+    pairs = np.array([(a, b) for a in range(12) for b in range(a)], np.uint32)
+
+    def call():
+        if form == "filtered":
+            hits = pd.pd_best_hits_all_filtered(ctx, prof, (1, 2), (1, 4))
+            return [*pd.pd_hits_copy(ctx, hits), pd.pd_bbh_copy(ctx, pd.pd_bbh_all(ctx, prof, hits))]
+        if form == "pairs":
+            b = pd.pd_bbh_pairs(ctx, prof, pairs)
+        else:
+            b = pd.pd_bbh_batch(ctx, ds.residues, ds.gene_ptr, ds.genome_ptr, np.array([[0, 1]], np.uint32),
+                                np.array([3], np.int32))
+        return [*pd.pd_batch_copy_hits(ctx, b), *pd.pd_batch_copy_bbh(ctx, b)]
+
+    refuse.calls = 0
+    want, total, found_room = call(), refuse.calls, 0
+    for at in range(1, total + 1):
+        refuse.calls, refuse.at = 0, at
+        try:
+            got = call()
+        except pd.PdError as err:
+            assert err.status == 5
+            continue
+        found_room += 1
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
+    assert found_room
+    refuse.at = 0
+    assert all(np.array_equal(x, y) for x, y in zip(call(), want))
