@@ -634,6 +634,8 @@ __global__ void __launch_bounds__(kDThreads, 2)
 // tile, whose next set bit gives w.  Also the longest list and the sum of
 // squared lengths.
 constexpr uint32_t kGenomeTable = 2048;
+static_assert((kLTile + 2) * 4 + 3 * kLTile / 8 + kLTile * 2 + (kGenomeTable + 2) * 2 + PD_MAX_GENOMES * 4 <= 48 * 1024,
+              "the lists pass fits the shared memory that every launch may use");
 
 __device__ __forceinline__ uint32_t lower_bound_gene(const uint32_t* __restrict__ post, uint32_t lo, uint32_t hi,
                                                      uint32_t cnt_bits, uint32_t gene) {
@@ -979,9 +981,7 @@ cudaError_t run_lists(Launcher* L, const u64* rec, uint64_t n, const SortKey& K,
   const uint32_t nt = list_tiles(n);
   uint32_t table_bits = 0;
   while (((n_genes - 1) >> table_bits) >= kGenomeTable) ++table_bits;
-  const size_t smem = sizeof(int32_t) * n_genomes;
-  cudaError_t e = cudaFuncSetAttribute(k_lists, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  const size_t smem = sizeof(int32_t) * n_genomes;  // at most 16 KB: beside the static arrays no attribute is needed
   PD_LAUNCH(L, "lists", k_lists<<<std::min(nt, 152u * 3u), kDThreads, smem, s>>>(
                             tile_e, tile_id, nt, rec, n, K, code_lo, code_hi, post, post_ptr, cnt_bits, cnt_cap,
                             genome_ptr, n_genomes, n_genes, table_bits, cursor, mv, max_list, join));

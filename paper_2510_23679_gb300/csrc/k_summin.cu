@@ -1253,13 +1253,19 @@ constexpr uint32_t kFCap = 4096, kFOut = 512;
 using TF = SmemTier<kFThreads, kFCap, kFOut, false, true>;
 static_assert(TF::bytes(PD_MAX_GENOMES) <= 227 * 1024, "filtered tier shared memory");
 
-// carveout (KB, 0: what the resident blocks take): shared memory of an SM to
-// stay within, the rest being L1.
-template <typename K>
-cudaError_t launch_smem(K kernel, Launcher* L, const char* name, int threads, size_t smem, uint32_t max_grid,
+// Tier: the kernel's SmemTier; n_best: target genomes of the launch, at most
+// kMaxBest.  A function's attributes are shared by every context and host
+// thread, so the limit set is always the kernel's largest: another thread's
+// launch between the two calls then finds room for its own size.  carveout (KB,
+// 0: what the resident blocks take): shared memory of an SM to stay within,
+// the rest being L1.
+template <typename Tier, uint32_t kMaxBest = PD_MAX_GENOMES, typename K>
+cudaError_t launch_smem(K kernel, Launcher* L, const char* name, int threads, uint32_t n_best, uint32_t max_grid,
                         const ProfilesView& P, const QuerySet& Q, const HitsOut& O, const TierIO& T, DevErr* err,
                         cudaStream_t s, uint32_t carveout = 0) {
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const size_t smem = Tier::bytes(n_best);
+  cudaError_t e =
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tier::bytes(kMaxBest));
   if (e != cudaSuccess) return e;
   if (carveout && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                             (int)(carveout * 100 / 228))) != cudaSuccess)
@@ -1281,13 +1287,13 @@ cudaError_t launch_t1(Launcher* L, uint32_t n_best, const ProfilesView& P, const
                       const TierIO& T, DevErr* err, cudaStream_t s) {
   constexpr int t = kT1Threads, b = kT1MinBlocks;
   if (n_best <= kT1CompactGenomes)
-    return launch_smem(k_summin_smem<t, b, kT1Cap, kT1Out, true, false, false, kT1Used, kWarpWalk, kForm>, L, "summin_bh",
-                       t, T1::bytes(n_best), Q.n_queries, P, Q, O, T, err, s);
+    return launch_smem<T1, kT1CompactGenomes>(k_summin_smem<t, b, kT1Cap, kT1Out, true, false, false, kT1Used, kWarpWalk, kForm>, L, "summin_bh",
+                       t, n_best, Q.n_queries, P, Q, O, T, err, s);
   if (n_best <= kT1MidGenomes)
-    return launch_smem(k_summin_smem<t, b, kT1Cap, kT1OutMid, true, false, false, kT1UsedMid, kWarpWalk, kForm>, L,
-                       "summin_bh", t, T1M::bytes(n_best), Q.n_queries, P, Q, O, T, err, s);
-  return launch_smem(k_summin_smem<t, b, kT1Cap, kT1OutFull, true, false, false, kT1UsedFull, kWarpWalk, kForm>, L,
-                     "summin_bh", t, T1F::bytes(n_best), Q.n_queries, P, Q, O, T, err, s, kT1FullCarveout);
+    return launch_smem<T1M, kT1MidGenomes>(k_summin_smem<t, b, kT1Cap, kT1OutMid, true, false, false, kT1UsedMid, kWarpWalk, kForm>, L,
+                       "summin_bh", t, n_best, Q.n_queries, P, Q, O, T, err, s);
+  return launch_smem<T1F>(k_summin_smem<t, b, kT1Cap, kT1OutFull, true, false, false, kT1UsedFull, kWarpWalk, kForm>, L,
+                     "summin_bh", t, n_best, Q.n_queries, P, Q, O, T, err, s, kT1FullCarveout);
 }
 
 }  // namespace
@@ -1300,14 +1306,14 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
     if (emit_all) return cudaErrorInvalidValue;
     TierIO tf1{nullptr, nullptr, O.def0, O.n_def0}, tf{O.def0, O.n_def0, O.def2, O.n_def2};
     const cudaError_t e1 =
-        Q.symbest ? launch_smem(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used, false,
+        Q.symbest ? launch_smem<TF1>(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used, false,
                                               kSymmetricForm>,
-                                L, "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout)
-                  : launch_smem(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used>, L,
-                                "summin_bh_f1", 256, TF1::bytes(n_best), Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout);
+                                L, "summin_bh_f1", 256, n_best, Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout)
+                  : launch_smem<TF1>(k_summin_smem<256, kF1MinBlocks, kF1Cap, kF1Out, true, false, true, kF1Used>, L,
+                                "summin_bh_f1", 256, n_best, Q.n_queries, P, Q, O, tf1, err, s, kF1Carveout);
     if (e1 != cudaSuccess) return e1;
-    return launch_smem(k_summin_smem<kFThreads, kFMinBlocks, kFCap, kFOut, false, false, true>, L, "summin_bh_f",
-                       kFThreads, TF::bytes(n_best), Q.n_queries, P, Q, O, tf, err, s);
+    return launch_smem<TF>(k_summin_smem<kFThreads, kFMinBlocks, kFCap, kFOut, false, false, true>, L, "summin_bh_f",
+                       kFThreads, n_best, Q.n_queries, P, Q, O, tf, err, s);
   }
   TierIO t1{nullptr, nullptr, O.def1, O.n_def1};
   TierIO t2{O.def1, O.n_def1, O.def2, O.n_def2};
@@ -1324,7 +1330,8 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
                                 : (two ? k_summin_warp<2, kRangeForm> : k_summin_warp<1, kRangeForm>);
     const float per_entry = short_lists ? 0.f : (float)P.n_join / ((float)P.n_entries * (float)P.n_genes);
     const size_t smem = kWWarps * warp_tier_bytes(n_best);
-    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(kWWarps * warp_tier_bytes(kWMaxGenomes)))) != cudaSuccess)
       return e;
     int per_sm = 1, dev = 0, n_sm = 152;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kWThreads, smem);
@@ -1341,8 +1348,8 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   }
   // tier 1: several resident blocks per SM, each looping over queries
   if (emit_all)
-    e = launch_smem(k_summin_smem<kT1Threads, kT1MinBlocks, kT1Cap, kT1OutEmit, true, true, false, kT1Used>, L, "summin_pairs",
-                    kT1Threads, T1E::bytes(n_best), Q.n_queries, P, Q, O, t1, err, s);
+    e = launch_smem<T1E, 1>(k_summin_smem<kT1Threads, kT1MinBlocks, kT1Cap, kT1OutEmit, true, true, false, kT1Used>, L, "summin_pairs",
+                    kT1Threads, n_best, Q.n_queries, P, Q, O, t1, err, s);
   else {
     // merge-path walk, or the warp-cooperative one for long lists
     const bool merge = Q.walk == PD_WALK_MERGE ||
@@ -1357,11 +1364,11 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
   if (e != cudaSuccess) return e;
   // tier 2: one 1024-thread block per SM over the deferred queries (exits at once if none)
   if (emit_all)
-    e = launch_smem(k_summin_smem<kT2Threads, 1, kT2Cap, kT2OutEmit, false, true>, L, "summin_pairs_t2", kT2Threads,
-                    T2E::bytes(n_best), Q.n_queries, P, Q, O, t2, err, s);
+    e = launch_smem<T2E, 1>(k_summin_smem<kT2Threads, 1, kT2Cap, kT2OutEmit, false, true>, L, "summin_pairs_t2", kT2Threads,
+                    n_best, Q.n_queries, P, Q, O, t2, err, s);
   else
-    e = launch_smem(k_summin_smem<kT2Threads, 1, kT2Cap, kT2Out, false, false>, L, "summin_bh_t2", kT2Threads,
-                    T2::bytes(n_best), Q.n_queries, P, Q, O, t2, err, s);
+    e = launch_smem<T2>(k_summin_smem<kT2Threads, 1, kT2Cap, kT2Out, false, false>, L, "summin_bh_t2", kT2Threads,
+                    n_best, Q.n_queries, P, Q, O, t2, err, s);
   return e;
 }
 
@@ -1372,21 +1379,22 @@ size_t summin_global_smem_bytes(uint32_t n_genomes) {
 cudaError_t run_summin_global(Launcher* L, const ProfilesView& P, const QuerySet& Q, const HitsOut& O,
                               const BigScratch& B, uint32_t n_ctas, DevErr* err, bool emit_all, cudaStream_t s) {
   const size_t smem = summin_global_smem_bytes(Q.all_pairs ? P.n_genomes : 1u);
+  const int most = (int)summin_global_smem_bytes(PD_MAX_GENOMES);
   TierIO t3{O.def2, O.n_def2, nullptr, nullptr};
   const char* name = Q.filter ? "summin_bh_f_t3" : (emit_all ? "summin_pairs_t3" : "summin_bh_t3");
   cudaError_t e;
   if (Q.filter) {
     if (emit_all || !B.vpa || !B.vpb) return cudaErrorInvalidValue;
-    e = cudaFuncSetAttribute(k_summin_global<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_summin_global<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     if ((e = launch_begin(L, name)) != cudaSuccess) return e;
     k_summin_global<false, true><<<n_ctas, 256, smem, s>>>(P, Q, O, t3, B, err);
     return launch_end(L, name);
   }
   if (emit_all)
-    e = cudaFuncSetAttribute(k_summin_global<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_summin_global<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   else
-    e = cudaFuncSetAttribute(k_summin_global<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_summin_global<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   if (e != cudaSuccess) return e;
   if ((e = launch_begin(L, name)) != cudaSuccess) return e;
   if (emit_all)

@@ -337,8 +337,9 @@ cudaError_t run_sym_write(Launcher* L, const SymRows& R, const uint32_t* stored,
   if ((e = launch_begin(L, "sym_write_rev")) != cudaSuccess) return e;
   if (R.n_genomes <= kRevTileGenomes) {
     const size_t smem = (size_t)R.n_genomes * 33u * sizeof(unsigned long long);
-    if ((e = cudaFuncSetAttribute(k_sym_write_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-        cudaSuccess)
+    // the largest, whatever this launch takes: the attribute is every thread's
+    if ((e = cudaFuncSetAttribute(k_sym_write_tile, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)(kRevTileGenomes * 33u * sizeof(unsigned long long)))) != cudaSuccess)
       return e;
     k_sym_write_tile<<<grid_of((uint64_t)R.n_genes, 32, 152u * 8u), 256, smem, s>>>(R, ties, row_ptr, whole, out_b,
                                                                                     out_s);
