@@ -30,7 +30,8 @@
 // Each sort pass reads and writes every record once: a tile's digit counts
 // are combined with those of the tiles before it by decoupled look-back
 // (Adinets and Merrill, "Onesweep", 2022).  A wait that runs out raises
-// PD_ERR_INTERNAL and its tile writes nothing.
+// PD_ERR_INTERNAL and its tile writes nothing; the blocks and passes that start
+// after it write nothing either, since what they would read was not written.
 //
 // Measured at 200 genomes x 4000 genes, k = 7 (264 M windows): 15.1 ms for the
 // whole build against 23.4 ms for a dictionary of all codes (marked and looked
@@ -282,16 +283,19 @@ struct PassShared {
   int failed;
 };
 
-// Takes a tile.  The first one also scans the digit counts into gbase (the
-// digits' starts), so that the running sums over the tiles are output positions.
+// Takes a tile, unless something failed before (false).  The first one also
+// scans the digit counts into gbase (the digits' starts), so that the running
+// sums over the tiles are output positions.
 template <int kBits>
-__device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, const uint32_t* __restrict__ hist, uint32_t* ticket) {
+__device__ __forceinline__ bool begin_tile(PassShared<kBits>& sh, const uint32_t* __restrict__ hist, uint32_t* ticket,
+                                           const DevErr* err) {
   for (uint32_t x = threadIdx.x; x < (kWarps << kBits) / 2; x += kThreads) ((uint32_t*)&sh.wcnt[0][0])[x] = 0;
   if (threadIdx.x == 0) {
-    sh.tile = atomicAdd(ticket, 1u);
-    sh.failed = 0;
+    sh.failed = failed(err);
+    if (!sh.failed) sh.tile = atomicAdd(ticket, 1u);
   }
   __syncthreads();
+  if (sh.failed) return false;
   if (sh.tile == 0) {
     uint32_t carry = 0;
     for (uint32_t d0 = 0; d0 < (1u << kBits); d0 += kThreads) {
@@ -303,6 +307,7 @@ __device__ __forceinline__ void begin_tile(PassShared<kBits>& sh, const uint32_t
     }
     __syncthreads();
   }
+  return true;
 }
 
 // Stable counting step of one tile.  xr: the thread's records, striped within
@@ -413,7 +418,7 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
   __shared__ PassShared<kBits> sh;
   __shared__ uint8_t lut[256];
   init_code_table(lut, S.alpha);
-  begin_tile<kBits>(sh, hist, ticket);
+  if (!begin_tile<kBits>(sh, hist, ticket, err)) return;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint32_t at = threadIdx.x * kItems;
   // the all-ones word is no record: the gene field never holds all ones
@@ -441,7 +446,7 @@ __global__ void __launch_bounds__(kThreads, kSortBlocks)
                    T* status, uint32_t* ticket, u64* __restrict__ out, DevErr* err) {
   extern __shared__ u64 stage[];
   __shared__ PassShared<kBits> sh;
-  begin_tile<kBits>(sh, hist, ticket);
+  if (!begin_tile<kBits>(sh, hist, ticket, err)) return;
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   const uint64_t t0 = (uint64_t)sh.tile * kTile + warp * 32u * kItems;
   u64 xr[kItems];
@@ -498,10 +503,11 @@ __global__ void __launch_bounds__(kDThreads, 2)
   __shared__ uint32_t head[kDTile + 1];  // tile position of each posting's first record
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
-    s_tile = atomicAdd(ticket, 1u);
-    s_failed = 0;
+    s_failed = failed(err);
+    if (!s_failed) s_tile = atomicAdd(ticket, 1u);
   }
   __syncthreads();
+  if (s_failed) return;
   const uint32_t tile = s_tile;
   const uint64_t t0 = (uint64_t)tile * kDTile;
   const uint32_t p0 = warp * 32u * kDItems + lane;
@@ -662,7 +668,8 @@ __global__ void __launch_bounds__(kDThreads, 3)
             const uint8_t* __restrict__ code_hi, const uint32_t* __restrict__ post,
             const uint32_t* __restrict__ post_ptr, uint32_t cnt_bits, uint32_t cnt_cap,
             const int32_t* __restrict__ genome_ptr, uint32_t n_genomes, uint32_t n_genes, uint32_t table_bits,
-            uint32_t* cursor, uint4* __restrict__ mv, uint32_t* max_list, u64* join) {
+            uint32_t* cursor, uint4* __restrict__ mv, uint32_t* max_list, u64* join, const DevErr* err) {
+  if (failed(err)) return;  // the same in every thread: nothing is reported from here
   __shared__ uint32_t start[kLTile + 2];
   __shared__ uint32_t is_head[kLTile / 32], run_head[kLTile / 32];
   __shared__ uint16_t genome[kLTile];
@@ -977,14 +984,14 @@ cudaError_t run_lists(Launcher* L, const u64* rec, uint64_t n, const SortKey& K,
                       const uint32_t* tile_id, const uint32_t* post, const uint32_t* post_ptr, const uint32_t* code_lo,
                       const uint8_t* code_hi, uint32_t cnt_bits, uint32_t cnt_cap, const int32_t* genome_ptr,
                       uint32_t n_genomes, uint32_t n_genes, uint32_t* cursor, uint4* mv, uint32_t* max_list, u64* join,
-                      cudaStream_t s) {
+                      const DevErr* err, cudaStream_t s) {
   const uint32_t nt = list_tiles(n);
   uint32_t table_bits = 0;
   while (((n_genes - 1) >> table_bits) >= kGenomeTable) ++table_bits;
   const size_t smem = sizeof(int32_t) * n_genomes;  // at most 16 KB: beside the static arrays no attribute is needed
   PD_LAUNCH(L, "lists", k_lists<<<std::min(nt, 152u * 3u), kDThreads, smem, s>>>(
                             tile_e, tile_id, nt, rec, n, K, code_lo, code_hi, post, post_ptr, cnt_bits, cnt_cap,
-                            genome_ptr, n_genomes, n_genes, table_bits, cursor, mv, max_list, join));
+                            genome_ptr, n_genomes, n_genes, table_bits, cursor, mv, max_list, join, err));
   return cudaSuccess;
 }
 

@@ -161,6 +161,16 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
   O.row_len = row_len;
   O.def1 = def1;
   O.def2 = def2;
+  // device-side errors (the pinned mirror belongs to the context); synchronizes
+  auto device_errors = [&]() -> pd_status {
+    cudaError_t copied = cudaMemcpyAsync(cv.h_err, cv.d_err, sizeof(DevErr), cudaMemcpyDeviceToHost, st);
+    if (copied == cudaSuccess) copied = cudaStreamSynchronize(st);
+    if (copied != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(copied));
+    const int code = cv.h_err->code;
+    if (code == 0) return PD_OK;
+    cudaMemsetAsync(cv.d_err, 0, sizeof(DevErr), st);
+    return ctx_fail(ctx, (pd_status)code, "pd_best_hits_noalloc: device reported an error");
+  };
   unsigned long long h[4] = {0, 0, 0, 0};
   if ((e = cudaMemsetAsync(counters, 0, 5 * sizeof(unsigned long long), st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
   if ((e = cudaMemsetAsync(row_len, 0, sizeof(uint32_t) * rows, st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
@@ -178,15 +188,8 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
           (e = cudaStreamSynchronize(st)) != cudaSuccess)
         return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
     }
-    // device-side errors (the pinned mirror belongs to the context)
-    if ((e = cudaMemcpyAsync(cv.h_err, cv.d_err, sizeof(DevErr), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-      return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
-    if (cv.h_err->code != 0) {
-      const int code = cv.h_err->code;
-      cudaMemsetAsync(cv.d_err, 0, sizeof(DevErr), st);
-      return ctx_fail(ctx, (pd_status)code, "pd_best_hits_noalloc: device reported an error");
-    }
+    const pd_status found = device_errors();
+    if (found != PD_OK) return found;
   }
   const uint64_t total = h[0];
   if (n_hits) *n_hits = total;
@@ -203,8 +206,7 @@ pd_status noalloc_impl(pd_ctx* ctx, const pd_profiles* prof, uint32_t gi, uint32
                              s, st)) != cudaSuccess)
       return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
   }
-  if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return ctx_fail(ctx, PD_ERR_CUDA, cudaGetErrorString(e));
-  return PD_OK;
+  return device_errors();  // of the scan; a failed one's offsets stay below the true ones, inside cols and s
 }
 
 }  // namespace

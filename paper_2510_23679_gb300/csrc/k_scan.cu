@@ -80,7 +80,8 @@ __global__ void __launch_bounds__(kThreads)
         if (lane == 0) st[0] = S::kInclusive | all;
       } else {
         if (lane == 0) st[tile] = S::kAggregate | all;
-        if (!look_back_warp(st, tile, &before, err)) {  // reported; offsets stay in range
+        // reported; the offsets from here on, and the total, are then too small
+        if (!look_back_warp(st, tile, &before, err)) {
           if (lane == 0) raise_error(err, PD_ERR_INTERNAL, tile);
           before = 0;
         }

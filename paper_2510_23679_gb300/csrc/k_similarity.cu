@@ -61,7 +61,9 @@ constexpr int kAhead = 4;  // the second gene's entries loaded ahead, per lane
 
 __global__ void __launch_bounds__(kThreads)
     k_pair_similarity(pdg::ProfilesView P, const uint32_t* __restrict__ a, const uint32_t* __restrict__ b, uint32_t n,
-                      const uint32_t* __restrict__ order, uint32_t* __restrict__ s_out, uint32_t* __restrict__ den_out) {
+                      const uint32_t* __restrict__ order, uint32_t* __restrict__ s_out, uint32_t* __restrict__ den_out,
+                      const pdg::DevErr* err) {
+  if (pdg::failed(err)) return;  // the scan of the places: the order is not whole
   __shared__ uint32_t keys[kWarps][kSlots];
   __shared__ uint16_t cnts[kWarps][kSlots];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
@@ -190,7 +192,8 @@ pd_status summin_list_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* a, c
     CK(pdg::launch_end(L, "pair_order"));
     CK(pdg::launch_begin(L, "pair_similarity"));
     k_pair_similarity<<<grid_of(m, 32 * kWarps, 152u * 32u), kThreads, 0, c->stream>>>(
-        v, pa + p0, pb + p0, m, order.as<uint32_t>(), ps ? ps + p0 : nullptr, pden ? pden + p0 : nullptr);
+        v, pa + p0, pb + p0, m, order.as<uint32_t>(), ps ? ps + p0 : nullptr, pden ? pden + p0 : nullptr,
+        c->d_err);
     CK(pdg::launch_end(L, "pair_similarity"));
   }
   if (ps != s) CK(cudaMemcpyAsync(s, ps, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost, c->stream));

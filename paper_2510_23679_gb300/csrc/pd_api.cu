@@ -460,7 +460,8 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
       CK(pdg::run_dedupe(L, sorted, n, K, scratch, X, cnt_bits, cnt_cap, words + 1, d_post, d_post_ptr, d_code_lo,
                          d_code_hi, tile_e, tile_id, c->d_err, c->stream));
       CK(pdg::run_lists(L, sorted, n, K, tile_e, tile_id, d_post, d_post_ptr, d_code_lo, d_code_hi, cnt_bits, cnt_cap,
-                        d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5, c->stream));
+                        d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5, c->d_err,
+                        c->stream));
     }
     if (K.n_slices > 1) CK(cudaStreamSynchronize(c->stream));  // the last slice's records end here
   }
@@ -604,7 +605,8 @@ PD_API pd_status pd_profiles_copy_mv(pd_ctx* c, const pd_profiles* P, int64_t* m
       // per-gene power-of-two scratch for the sort by code
       std::vector<uint32_t> n(v.n_genes);
       CK(cudaMemcpyAsync(n.data(), n_of.p, sizeof(uint32_t) * v.n_genes, cudaMemcpyDeviceToHost, c->stream));
-      CK(cudaStreamSynchronize(c->stream));
+      const pd_status scanned = check_dev_err(c);  // synchronizes
+      if (scanned != PD_OK) return scanned;
       std::vector<unsigned long long> off(v.n_genes + 1, 0);
       for (uint32_t g = 0; g < v.n_genes; ++g) off[g + 1] = off[g] + (n[g] ? pdg::next_pow2(n[g]) : 0);
       ALLOC(pad_off, sizeof(unsigned long long) * (v.n_genes + 1));
@@ -626,8 +628,7 @@ PD_API pd_status pd_profiles_copy_mv(pd_ctx* c, const pd_profiles* P, int64_t* m
     if ((st = copy_out(c, codes, d_codes.p, sizeof(uint64_t) * v.n_entries)) != PD_OK) return st;
     if ((st = copy_out(c, counts, d_counts.p, sizeof(uint32_t) * v.n_entries)) != PD_OK) return st;
     if ((st = copy_out(c, La, v.La, sizeof(uint32_t) * v.n_genes)) != PD_OK) return st;
-    CK(cudaStreamSynchronize(c->stream));
-    return PD_OK;
+    return check_dev_err(c);  // synchronizes
   } catch (...) {
     return fail(c, PD_ERR_INTERNAL, "exception in pd_profiles_copy_mv");
   }
@@ -792,7 +793,8 @@ pd_status pdh::build_dictionary(pd_ctx* c, pd_profiles* P) {
     CK(pdg::run_dict_mark(&c->L, v.code_lo, v.code_hi, v.n_distinct, P->dict.as<uint32_t>(), c->stream));
   uint32_t* total = (uint32_t*)((unsigned char*)tmp.p + pdg::scan_temp_bytes(n_dict));
   CK(pdg::scan_dict_blocks(&c->L, P->dict.as<uint32_t>(), n_dict, total, tmp.p, c->stream));
-  CK(cudaStreamSynchronize(c->stream));  // the scan's scratch ends here
+  const pd_status st = check_dev_err(c);  // synchronizes: the scan's scratch ends here
+  if (st != PD_OK) return st;
   v.dict = P->dict.as<uint32_t>();
   v.n_dict_blocks = n_dict;
   P->info.device_bytes += P->dict.n;
@@ -959,7 +961,7 @@ pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& qu
     unsigned long long* h = c->h_build;  // pinned: the row total, the BBH total
     CK(cudaMemcpyAsync(h, row_ptr.as<unsigned long long>() + G, sizeof(*h), cudaMemcpyDeviceToHost, c->stream));
     if (want_bbh) CK(cudaMemcpyAsync(h + 1, bstart + G, sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
+    if ((st = check_dev_err(c)) != PD_OK) return st;  // synchronizes
     const unsigned long long n = h[0];
     const uint32_t n_bbh = want_bbh ? *(const uint32_t*)(h + 1) : 0u;
     ALLOC(H->out_b, sizeof(uint32_t) * std::max<unsigned long long>(n, 1));
@@ -1206,9 +1208,11 @@ static pd_status hits_to_csr(pd_ctx* c, const pd_hits* H, uint32_t n_rows, uint3
   ALLOC(tmp, pdg::scan_temp_bytes(n_rows + 1) + 64);
   CK(pdg::scan_u32_to_u64(L, H->row_len.as<uint32_t>(), n_rows, row_ptr.as<unsigned long long>(), tmp.p,
                           c->stream));
-  unsigned long long n = 0;
-  CK(cudaMemcpyAsync(&n, row_ptr.as<unsigned long long>() + n_rows, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  CK(cudaMemcpyAsync(c->h_build, row_ptr.as<unsigned long long>() + n_rows, sizeof(*c->h_build),
+                     cudaMemcpyDeviceToHost, c->stream));
+  const pd_status st = check_dev_err(c);  // synchronizes
+  if (st != PD_OK) return st;
+  const uint64_t n = c->h_build[0];
   ALLOC(cols, sizeof(int32_t) * std::max<uint64_t>(n, 1));
   ALLOC(s, sizeof(uint32_t) * std::max<uint64_t>(n, 1));
   if (n_rows)
@@ -1262,9 +1266,11 @@ pd_status pdh::bbh_impl(pd_ctx* c, const pdg::BbhRows& R, uint64_t n_hit_slots, 
   ALLOC(tmp, pdg::scan_temp_bytes(R.n_rows + 1) + 64);
   if (R.n_rows) CK(pdg::run_bbh_count(L, R, flags.as<uint8_t>(), row_cnt.as<uint32_t>(), c->stream));
   CK(pdg::scan_u32(L, row_cnt.as<uint32_t>(), R.n_rows, row_start.as<uint32_t>(), tmp.p, c->stream));
-  uint32_t n = 0;
-  CK(cudaMemcpyAsync(&n, row_start.as<uint32_t>() + R.n_rows, sizeof(n), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  CK(cudaMemcpyAsync(c->h_build, row_start.as<uint32_t>() + R.n_rows, sizeof(uint32_t), cudaMemcpyDeviceToHost,
+                     c->stream));
+  const pd_status st = check_dev_err(c);  // synchronizes
+  if (st != PD_OK) return st;
+  const uint32_t n = *(const uint32_t*)c->h_build;
   S->ctx = c;
   S->n = n;
   ALLOC(S->a, sizeof(int32_t) * std::max<uint32_t>(n, 1));

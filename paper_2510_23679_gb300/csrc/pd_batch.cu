@@ -347,7 +347,8 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
                      cudaMemcpyDeviceToHost, c->stream));
   CK(cudaMemcpyAsync(&tot[1], B->job_ptr.as<unsigned long long>() + n_jobs, sizeof(unsigned long long),
                      cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  const pd_status scanned = check_dev_err(c);  // synchronizes
+  if (scanned != PD_OK) return scanned;
   if (tot[0] != n_hits_total) return fail(c, PD_ERR_INTERNAL, "batch Best Hit count mismatch");
   ALLOC(B->cols, sizeof(int32_t) * std::max<unsigned long long>(tot[0], 1));
   ALLOC(B->s, sizeof(uint32_t) * std::max<unsigned long long>(tot[0], 1));
@@ -660,7 +661,7 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   CK(cudaMemcpyAsync(&n_hits, Bt->row_ptr.as<unsigned long long>() + n_q, sizeof(n_hits), cudaMemcpyDeviceToHost,
                      c->stream));
   CK(cudaMemcpyAsync(&n_bbh, start.as<uint32_t>() + n_q, sizeof(n_bbh), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  if ((st = check_dev_err(c)) != PD_OK) return st;  // synchronizes
   ALLOC(Bt->cols, sizeof(int32_t) * std::max<unsigned long long>(n_hits, 1));
   ALLOC(Bt->s, sizeof(uint32_t) * std::max<unsigned long long>(n_hits, 1));
   ALLOC(Bt->a, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));

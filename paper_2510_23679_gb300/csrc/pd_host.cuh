@@ -62,7 +62,7 @@ struct pd_ctx {
   pdg::Launcher L{nullptr};
   pdg::DevErr* d_err = nullptr;  // device error block
   pdg::DevErr* h_err = nullptr;  // pinned host mirror
-  // pinned host words the profile build reads back after its dictionary pass
+  // pinned host words: sizes and counters read back in the middle of a call
   unsigned long long* h_build = nullptr;  // [8]
   int32_t* h_genome_ptr = nullptr;        // [PD_MAX_GENOMES + 1]
   cudaMemPool_t pool = nullptr;  // without hooks: allocate from this pool (null: the device's default pool)

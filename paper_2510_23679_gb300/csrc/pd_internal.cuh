@@ -104,6 +104,9 @@ struct DevErr {
 __device__ __forceinline__ void raise_error(DevErr* e, int code, unsigned long long detail) {
   if (atomicCAS(&e->code, 0, code) == 0) e->detail = detail;
 }
+// Has a kernel before this one (or a block of this one) failed?  Passes that
+// index with what an earlier pass should have written look first.
+__device__ __forceinline__ bool failed(const DevErr* e) { return *(volatile const int*)&e->code != 0; }
 
 // ---------------------------------------------------------------- helpers
 __host__ __device__ __forceinline__ uint32_t next_pow2(uint32_t x) {
@@ -185,14 +188,27 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* w
 // Decoupled Look-back", 2016).  A status word holds two flag bits above a
 // tile's sum alone or of all tiles up to it, written and read whole.  Tiles are
 // numbered by a ticket, so every tile waited for is already running; a wait
-// that runs out is reported by the caller (PD_ERR_INTERNAL).
+// that runs out is reported by the caller (PD_ERR_INTERNAL), its tile writes
+// nothing or offsets too small, and nothing may index with the pass's output
+// before the error block has been looked at.
 template <typename T>
 struct Status {
   static constexpr T kAggregate = (T)1 << (sizeof(T) * 8 - 2);
   static constexpr T kInclusive = (T)2 << (sizeof(T) * 8 - 2);
   static constexpr T kValue = kAggregate - 1;
 };
-constexpr uint32_t kMaxPolls = 1u << 21;
+#ifndef PD_MAX_POLLS
+#define PD_MAX_POLLS (1u << 21)  // some 0.3 s; a build for a test sets it so that waits run out
+#endif
+constexpr uint32_t kMaxPolls = PD_MAX_POLLS;
+
+// Counts a poll that found nothing; false when the wait is given up.
+__device__ __forceinline__ bool poll_again(uint32_t* polls, const DevErr* err) {
+  if (++*polls > kMaxPolls) return false;
+  if (*polls <= 64u) return true;
+  __nanosleep(100);
+  return (*polls & 255u) != 0 || !failed(err);
+}
 
 // Sum over the tiles before `tile` of one column of statuses (status[t *
 // stride]), walked back until an inclusive sum; four predecessors are read at
@@ -204,6 +220,7 @@ __device__ __forceinline__ bool look_back(const volatile T* status, uint32_t til
   uint32_t polls = 0;
   int64_t t = (int64_t)tile - 1;
   while (t >= 0) {
+    const int64_t t0 = t;
     T v[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) v[j] = t - j >= 0 ? status[(uint64_t)(t - j) * stride] : (T)0;
@@ -217,10 +234,7 @@ __device__ __forceinline__ bool look_back(const volatile T* status, uint32_t til
       s += v[j] & Status<T>::kValue;
       --t;
     }
-    if (++polls > 64u) {
-      __nanosleep(100);
-      if (polls > kMaxPolls || ((polls & 255u) == 0 && *(volatile const int*)&err->code)) return false;
-    }
+    if (t == t0 && !poll_again(&polls, err)) return false;
   }
   *sum = s;
   return true;
@@ -247,11 +261,7 @@ __device__ __forceinline__ bool look_back_warp(const volatile unsigned long long
     s += x;
     t -= take;
     if (inc && n <= ready) break;
-    if (take < 32u && ++polls > 64u) {
-      __nanosleep(100);
-      const bool failed = (polls & 255u) == 0 && *(volatile const int*)&err->code;
-      if (polls > kMaxPolls || __any_sync(0xffffffffu, failed)) return false;
-    }
+    if (take < 32u && __any_sync(0xffffffffu, !poll_again(&polls, err))) return false;
   }
   *sum = s;
   return true;
@@ -407,7 +417,9 @@ cudaError_t launch_begin(Launcher* L, const char* name);
 cudaError_t launch_end(Launcher* L, const char* name);
 DevErr* launch_err(Launcher* L);  // the context's device error block
 
-// scans (k_scan.cu)
+// scans (k_scan.cu).  One that fails (see k_scan.cu) reports it in the error
+// block and leaves offsets, and a total, that may be too small: the block is
+// read (check_dev_err) before the total sizes anything.
 size_t scan_temp_bytes(uint64_t n);
 // Rank bases of the dictionary: word 0 of each of the n_blocks blocks gets
 // the set bits of the blocks before it; *total gets the number of codes.
@@ -495,7 +507,7 @@ cudaError_t run_lists(Launcher* L, const unsigned long long* rec, uint64_t n, co
                       const uint32_t* tile_id, const uint32_t* post, const uint32_t* post_ptr, const uint32_t* code_lo,
                       const uint8_t* code_hi, uint32_t cnt_bits, uint32_t cnt_cap, const int32_t* genome_ptr,
                       uint32_t n_genomes, uint32_t n_genes, uint32_t* cursor, uint4* mv, uint32_t* max_list,
-                      unsigned long long* join, cudaStream_t s);
+                      unsigned long long* join, const DevErr* err, cudaStream_t s);
 
 // profiles (k_profiles.cu)
 // The bits of all codes of an index in a zeroed dictionary.

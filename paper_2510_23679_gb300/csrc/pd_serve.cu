@@ -467,7 +467,7 @@ pd_status answer_level(pd_index* I, const Level& L, const uint8_t* tick_res, con
   unsigned long long n_hits = 0;
   CK(cudaMemcpyAsync(&n_hits, row_ptr.as<unsigned long long>() + n_q, sizeof(n_hits), cudaMemcpyDeviceToHost,
                      c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  if ((st = check_dev_err(c)) != PD_OK) return st;  // synchronizes
   ALLOC(cols, sizeof(int32_t) * std::max<unsigned long long>(n_hits, 1));
   ALLOC(sv, sizeof(uint32_t) * std::max<unsigned long long>(n_hits, 1));
   CK(pdg::run_gather_rows(&c->L, n_q, H.row_off.as<unsigned long long>(), H.row_len.as<uint32_t>(),
@@ -484,7 +484,7 @@ pd_status answer_level(pd_index* I, const Level& L, const uint8_t* tick_res, con
   CK(pdg::scan_u32(&c->L, cnt.as<uint32_t>(), n_q, start.as<uint32_t>(), tmp.p, c->stream));
   uint32_t n_bbh = 0;
   CK(cudaMemcpyAsync(&n_bbh, start.as<uint32_t>() + n_q, sizeof(n_bbh), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
+  if ((st = check_dev_err(c)) != PD_OK) return st;  // synchronizes
   ALLOC(pa, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
   ALLOC(pb, sizeof(int32_t) * std::max<uint32_t>(n_bbh, 1));
   if (n_bbh)
