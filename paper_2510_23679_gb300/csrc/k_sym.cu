@@ -194,7 +194,7 @@ __global__ void k_sym_put_ties(SymRows R, const uint8_t* __restrict__ tie_ok, co
 // maxima are ascending already, so an entry's place is its index among them
 // plus the ties below it, a tie's the stored below it (bisection) plus the ties
 // below it.  The part is read before it is written, at most kTieLanes entries a
-// lane; a longer part falls back to an insertion sort by one lane.
+// lane; longer parts are left to k_sym_sort_long.
 constexpr uint32_t kTieLanes = 16;
 __global__ void __launch_bounds__(256)
     k_sym_sort_ties(SymRows R, const uint32_t* __restrict__ stored, const uint32_t* __restrict__ tiecnt,
@@ -237,20 +237,77 @@ __global__ void __launch_bounds__(256)
           kb[at[j]] = x[j];
           ks[at[j]] = y[j];
         }
-    } else if (lane == 0) {
-      for (uint32_t i = 1; i < n; ++i) {
-        const uint32_t x = kb[i], y = ks[i];
-        uint32_t j = i;
-        while (j > 0 && kb[j - 1] > x) {
-          kb[j] = kb[j - 1];
-          ks[j] = ks[j - 1];
-          --j;
-        }
-        kb[j] = x;
-        ks[j] = y;
-      }
     }
     __syncwarp();
+  }
+}
+
+// One block per gene whose reverse part is longer than a warp takes: a bitonic
+// network in the form whose exchanges all put the smaller entry at the lower
+// place, so that the entries missing to a power of two need not exist.  In
+// shared memory up to kLongShared entries, else in place (2000 genomes x 20
+// genes, rows of 1000: 1.7 ms, where an insertion sort by one lane took 580).
+constexpr uint32_t kLongShared = 4096;
+__global__ void __launch_bounds__(256)
+    k_sym_sort_long(SymRows R, const uint32_t* __restrict__ stored, const uint32_t* __restrict__ tiecnt,
+                    const unsigned long long* __restrict__ row_ptr, uint32_t* __restrict__ out_b,
+                    uint32_t* __restrict__ out_s) {
+  __shared__ unsigned long long sh[kLongShared];
+  __shared__ uint32_t longs;  // of the 32 genes, those with long rows
+  const uint32_t n_listed = *R.n_tie_genes;
+  auto network = [&](uint32_t n, auto exchange) {
+    for (uint32_t size = 2; size / 2 < n; size <<= 1)
+      for (uint32_t stride = size / 2; stride > 0; stride >>= 1) {
+        for (uint32_t i = threadIdx.x;; i += blockDim.x) {
+          const uint32_t lo = 2 * i - (i & (stride - 1));
+          if (lo >= n) break;
+          const uint32_t hi = stride == size / 2 ? lo ^ (size - 1) : lo + stride;
+          if (hi < n) exchange(lo, hi);
+        }
+        __syncthreads();
+      }
+  };
+  // few genes' rows are long: a block looks at 32 at a time
+  for (uint32_t x0 = blockIdx.x * 32u; x0 < n_listed; x0 += gridDim.x * 32u) {
+    if (threadIdx.x < 32u) {
+      const uint32_t x = x0 + threadIdx.x, b = x < n_listed ? R.tie_gene[x] : 0u;
+      const uint32_t m = __ballot_sync(0xffffffffu, x < n_listed && stored[b] + tiecnt[b] > 32u * kTieLanes);
+      if (threadIdx.x == 0) longs = m;
+    }
+    __syncthreads();
+    for (uint32_t left = longs; left; left &= left - 1u) {
+      const uint32_t b = R.tie_gene[x0 + (uint32_t)__ffs((int)left) - 1u], n = stored[b] + tiecnt[b];
+      uint32_t* kb = out_b + row_ptr[b];
+      uint32_t* ks = out_s + row_ptr[b];
+      if (n > kLongShared) {
+        network(n, [&](uint32_t lo, uint32_t hi) {
+          const uint32_t p = kb[lo], q = kb[hi];
+          if (p > q) {
+            const uint32_t s = ks[lo];
+            kb[lo] = q;
+            kb[hi] = p;
+            ks[lo] = ks[hi];
+            ks[hi] = s;
+          }
+        });
+        continue;
+      }
+      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) sh[i] = (unsigned long long)kb[i] << 32 | ks[i];
+      __syncthreads();
+      network(n, [&](uint32_t lo, uint32_t hi) {
+        const unsigned long long p = sh[lo], q = sh[hi];
+        if (p > q) {
+          sh[lo] = q;
+          sh[hi] = p;
+        }
+      });
+      for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        kb[i] = (uint32_t)(sh[i] >> 32);
+        ks[i] = (uint32_t)sh[i];
+      }
+      __syncthreads();
+    }
+    __syncthreads();
   }
 }
 
@@ -361,7 +418,13 @@ cudaError_t run_sym_write(Launcher* L, const SymRows& R, const uint32_t* stored,
   if ((e = launch_begin(L, "sym_sort_ties")) != cudaSuccess) return e;
   k_sym_sort_ties<<<grid_of(std::min<unsigned long long>(R.n_ties, R.n_genes) * 32, 256, 152u * 8u), 256, 0, s>>>(
       R, stored, tiecnt, row_ptr, out_b, out_s);
-  return launch_end(L, "sym_sort_ties");
+  if ((e = launch_end(L, "sym_sort_ties")) != cudaSuccess) return e;
+  // a gene's reverse part holds a maximum for each other genome, and ties
+  if (R.n_genomes + R.n_ties <= 32u * kTieLanes) return cudaSuccess;
+  if ((e = launch_begin(L, "sym_sort_long")) != cudaSuccess) return e;
+  k_sym_sort_long<<<grid_of(std::min<unsigned long long>(R.n_ties, R.n_genes), 32, 152u * 6u), 256, 0, s>>>(
+      R, stored, tiecnt, row_ptr, out_b, out_s);
+  return launch_end(L, "sym_sort_long");
 }
 
 cudaError_t run_sym_bbh_count(Launcher* L, const SymRows& R, uint8_t* flag, uint32_t* cnt, uint32_t* start,

@@ -901,7 +901,8 @@ static pd_status hits_pair_impl(pd_ctx* c, const pd_profiles* P, uint32_t gi, ui
 // walked from one side; the launch emits the forward Best Hits and keeps the
 // reverse maxima, and the rows are assembled from both.
 pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& queries, bool want_bbh, pd_hits* H,
-                        uint32_t genomes_per_query) {
+                        bool* too_many, uint32_t genomes_per_query) {
+  *too_many = false;
   const pdg::ProfilesView& v = P->view;
   pdg::Launcher* L = &c->L;
   const uint32_t G = v.n_genes, NG = queries.two_genomes ? 1 : v.n_genomes;
@@ -921,16 +922,19 @@ pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& qu
     pd_status st = run_hits(c, P, Q, false, &F, genomes_per_query);  // forward rows (genomes after each query's own)
     if (st != PD_OK) return st;
     const unsigned long long n_ties = F.n_ties;
-    if (n_ties > tie_cap) {  // more exact ties than the list held: run again with room for all
-      tie_cap = n_ties + 4096;
+    if (n_ties > tie_cap) {
+      // More exact ties than the list held: run again with room for them.  A
+      // tie with a maximum that is beaten later is listed too, so the number
+      // depends on the order the queries run in; with 4096 to spare one run in
+      // four at 800 genomes x 40 short genes found no room in three attempts.
+      tie_cap = n_ties + n_ties / 4 + 4096;
       continue;
     }
+    if (n_ties > kSymMaxTies) break;
     // a query handed to the next tier after its Best Hit passes records its
     // ties twice: a set keeps the first record of each pair
     const unsigned long long set_slots =
-        n_ties ? pdg::next_pow2((uint32_t)std::min<unsigned long long>(std::max<unsigned long long>(2 * n_ties, 2),
-                                                                     1ull << 31))
-               : 0;
+        n_ties ? pdg::next_pow2((uint32_t)std::max<unsigned long long>(2 * n_ties, 2)) : 0;
     Carve ct;
     const size_t o_tiecnt = ct.add(sizeof(uint32_t) * G), o_fill = ct.add(sizeof(uint32_t) * G), o_listed = ct.add(sizeof(uint32_t)), zeroed = ct.bytes,
                  o_set = ct.add(sizeof(unsigned long long) * set_slots), o_stored = ct.add(sizeof(uint32_t) * G),
@@ -988,6 +992,7 @@ pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& qu
     H->n_deferred = F.n_deferred;
     return PD_OK;
   }
+  *too_many = true;
   return fail(c, PD_ERR_INTERNAL, "symmetric Best Hits: the tie list did not converge");
 }
 
@@ -1007,10 +1012,16 @@ PD_API pd_status pd_best_hits_all(pd_ctx* c, const pd_profiles* P, pd_hits** out
       // queries in gene order, i.e. genome by genome: the reverse maxima of the
       // query genome in flight (its slice of the genome-major array) stay in L2
       Q.n_queries = G;
-      pd_status st = sym_hits(c, P, Q, true, H.get());
-      if (st != PD_OK) return st;
-      *out = H.release();
-      return PD_OK;
+      bool too_many;
+      pd_status st = sym_hits(c, P, Q, true, H.get(), &too_many);
+      if (st != PD_OK && !too_many) return st;
+      if (st == PD_OK) {
+        *out = H.release();
+        return PD_OK;
+      }
+      H.reset(new pd_hits());
+      H->ctx = c;
+      H->all_pairs = 1;
     }
     pdg::QuerySet Q{};
     Q.all_pairs = 1;
@@ -1352,13 +1363,15 @@ PD_API pd_status pd_best_hits_all_filtered(pd_ctx* c, const pd_profiles* P, cons
     Q.n_queries = P->view.n_genes;
     pd_status st = set_filter(c, f, &Q);
     if (st != PD_OK) return st;
-    // both filters treat (a, b) and (b, a) alike, so pairs are walked from one
-    // side (30 genomes x 2000 genes 1.45 against 1.87 ms; 60 x 3000, where half
-    // the targets also fit the packed table, 10.7 against 30.5)
+    // both filters treat (a, b) and (b, a) alike, so pairs can be walked from one
+    // side (60 genomes x 3000 genes, where half the targets also fit the packed
+    // table, 10.7 against 30.5 ms)
     const uint32_t G = P->view.n_genes, NG = P->view.n_genomes;
-    const bool symmetric = c->symmetric && G > 0 && NG >= 2 && 8ull * G * NG <= kSymMaxBytes;
-    if (symmetric) st = sym_hits(c, P, Q, true, H.get());
-    if (!symmetric || st == PD_ERR_OOM) {  // the plain form needs no room for the maxima
+    const bool symmetric =
+        c->symmetric && G > 0 && NG >= 2 && sym_pays((double)P->view.n_join / 2, (double)G * NG);
+    bool too_many = false;
+    if (symmetric) st = sym_hits(c, P, Q, true, H.get(), &too_many);
+    if (!symmetric || st == PD_ERR_OOM || too_many) {  // the plain form needs no room for maxima and ties
       H.reset(new pd_hits());
       H->ctx = c;
       H->all_pairs = 1;

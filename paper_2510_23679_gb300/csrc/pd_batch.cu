@@ -288,12 +288,13 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
       // each job walked from its first genome, the second's rows from the
       // maxima its genes have met
       Q.two_genomes = 1;
-      st = sym_hits(c, P.get(), Q, true, &C->hits, 1);
-      if (st != PD_OK && st != PD_ERR_OOM) return st;
+      bool too_many;
+      st = sym_hits(c, P.get(), Q, true, &C->hits, &too_many, 1);
+      if (st != PD_OK && st != PD_ERR_OOM && !too_many) return st;
       symmetric = st == PD_OK;
       C->bbh = C->hits.bbh;
     }
-    if (!symmetric) {  // or no room for the maxima
+    if (!symmetric) {  // or no room for the maxima or their ties
       Q.two_genomes = 0;
       C->hits = pd_hits();
       C->hits.ctx = c;
@@ -522,13 +523,6 @@ __global__ void k_pairs_job_ptr(const PairJob* __restrict__ jobs, uint32_t n_job
 // (its genome's range searched in every list): 843 M postings for 180 k genes
 // take 5.0 ms, 1.8 M listed queries on the same dataset 20.9 ms.
 constexpr uint64_t kPostingsPerQuery = 2000;
-// Postings that have to be saved by walking pairs from one side (300 pairs of
-// 60 genomes x 3000 genes 4.8 against 7.9 ms, 1500 pairs 7.3 against 10.1) for
-// each word of the table of maxima: a word is cleared, counted and read again (24 bytes,
-// 3.5 ps at the copy rate), a posting takes 6 to 8 ps.  Below kSymMinSaved the
-// launches that make rows of the maxima cost more than the walk saves.
-constexpr uint64_t kPostingsPerMaximum = 2, kSymMinSaved = 8ull << 20;
-
 pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint32_t n_jobs, pd_batch** out) {
   if (n_jobs && !jobs) return fail(c, PD_ERR_ARG, "null jobs");
   if (n_jobs && is_device_ptr(jobs)) return fail(c, PD_ERR_ARG, "jobs must be a host array");
@@ -584,8 +578,8 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   const uint64_t G = P->view.n_genes;
   const uint64_t walk = G ? P->view.n_join / G : 0;  // postings of one gene's walk
   const bool grouped = n_q && kPostingsPerQuery * n_q >= n_named * walk;
-  const bool symmetric = grouped && c->symmetric && 8ull * G * n_genomes <= kSymMaxBytes &&
-                         (n_named - (double)ahead / G) * walk >= kSymMinSaved + kPostingsPerMaximum * (double)G * n_genomes;
+  const bool symmetric = grouped && c->symmetric &&
+                         sym_pays((n_named - (double)ahead / G) * walk, (double)G * n_genomes);
   pd_hits H;
   H.ctx = c;
   pdg::QuerySet Q{};
@@ -616,8 +610,9 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
       Q.n_queries = n_listed;
       const uint64_t n_dir = sym ? n_directed / 2 : n_directed;  // rows that the launch emits
       const uint32_t per_query = (uint32_t)((n_dir + n_listed) / std::max<uint32_t>(n_listed, 1));
-      st = sym ? sym_hits(c, P, Q, false, &H, per_query) : run_hits(c, P, Q, false, &H, per_query);
-      if (st != PD_ERR_OOM || !sym) break;  // no room for the maxima: the plain form needs none
+      bool too_many = false;
+      st = sym ? sym_hits(c, P, Q, false, &H, &too_many, per_query) : run_hits(c, P, Q, false, &H, per_query);
+      if (!sym || (st != PD_ERR_OOM && !too_many)) break;  // no room for maxima or ties: the plain form needs none
     }
     if (st != PD_OK) return st;
     ALLOC(d_off, sizeof(unsigned long long) * n_q);

@@ -301,11 +301,30 @@ pd_status run_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool
 // Best Hit rows of every gene by the symmetric form, for the queries of Q (an
 // all-pairs set; its target mask, if any, must be symmetric, and its queries
 // all genes with a target in a later genome), with their BBH pairs if asked
-// for.  genomes_per_query as above.
+// for.  genomes_per_query as above.  The list of exact ties has no bound known
+// beforehand, and their number changes a little from run to run: if no list
+// held them all, *too_many is set (with a status other than PD_OK) and the
+// caller takes the plain form, which lists none.
 pd_status sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool want_bbh, pd_hits* H,
-                   uint32_t genomes_per_query = 0);
+                   bool* too_many, uint32_t genomes_per_query = 0);
 // Largest reverse-maximum table (genes x genomes x 8 B) of the symmetric form.
 constexpr unsigned long long kSymMaxBytes = 4ull << 30;
+// ... and most exact ties (the set of those counted has twice as many places,
+// a power of two in 32 bits).
+constexpr unsigned long long kSymMaxTies = 1ull << 30;
+// Where both forms serve a call: is walking each pair from one side worth a
+// table of `words` maxima, given the postings it saves?  A word is cleared,
+// counted and read again (24 bytes, 3.5 ps at the copy rate), a posting takes 6
+// to 8 ps: two postings a word.  Below 8 M saved the launches that make rows of
+// the maxima cost more than the walk saves.  300 pairs of 60 genomes x 3000
+// genes 4.8 against 7.9 ms, 1500 pairs 7.3 against 10.1; filtered, all pairs
+// (saved, words): 4 x 250 (0.3 M, 4 k) 0.174 against 0.123 ms, 20 x 500 (7 M, 0.2 M)
+// 0.30 against 0.27, 20 x 1000 (15 M, 0.4 M) 0.44 against 0.46, 30 x 2000 (70 M,
+// 1.8 M) 1.22 against 1.56, 2000 x 20 short genes full of ties (50 M, 80 M) 610
+// against 347.
+inline bool sym_pays(double saved, double words) {
+  return words * 8.0 <= (double)kSymMaxBytes && saved >= (double)(8ull << 20) + 2.0 * words;
+}
 // Mutual Best Hits of the rows R into S.
 pd_status bbh_impl(pd_ctx* c, const pdg::BbhRows& R, uint64_t n_hit_slots, uint32_t a_base, uint32_t b_base,
                    pd_bbh_set* S);
