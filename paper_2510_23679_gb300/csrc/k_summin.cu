@@ -60,7 +60,6 @@ struct Scalars {
 // mean a nearly full table; the query then moves to a larger tier, so the
 // bound never changes a result, only where it is computed.
 constexpr uint32_t kMaxProbe = 64;
-
 // Two table layouts share the code below.
 //   packed (tier 1): one word per slot, (b << cnt_bits) | s.  A posting is
 //     packed the same way, so the walk keys the table with the posting's own
@@ -299,6 +298,7 @@ __device__ __forceinline__ bool load_query(uint32_t qi, const ProfilesView& P, c
       if (Q.two_genomes && (gg & 1u)) return false;  // no genome after its own: a target only
       q->own0 = (uint32_t)P.genome_ptr[gg];
       q->own1 = (uint32_t)P.genome_ptr[gg + 1];
+      if (Q.two_genomes) q->tend = (uint32_t)P.genome_ptr[gg + 2];
       if (kForm == kAnyForm && Q.tgt_end) q->tend = Q.tgt_end[gg];
       if (Q.tgt_mask) q->mask = Q.tgt_mask + (size_t)gg * Q.mask_words;
       q->col = Q.two_genomes ? 0u : gg - Q.col_genome0;
@@ -396,12 +396,17 @@ constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
 //   50 genomes x 3000 genes 3.08 / 2.82 / 3.25, 30 x 2000 0.89 / 0.68 / -,
 //   100 x 4000 7.70 / 7.23 / -, 200 x 4000 - / 24.2 / 24.8
 // (1500 postings instead: 2.98 at 50 x 3000, 25.2 at 200 x 4000; 4000: 3.03
-// and 24.4).  Without the symmetric form
+// and 24.4).  Queries of one target range are judged by the range's share of
+// the dataset and leave at kWMaxRangePostings, since where lists are long most
+// of their postings are another gene's (whole calls, ms, no limit / 2500 / 1250:
+// three pairs of 3 genomes x 30000 genes, k = 5, 20.4 / 18.2 / 16.6; paralogs of
+// 4 x 6000, k = 4, 9.9 / 6.6 / 6.6, of 20 x 9000, k = 5, 5.4 / 5.4 / 4.7).
+// Without the symmetric form
 // whole lists are walked and the warp tier takes short lists or, of an index
 // far larger than L2, long ones; queries from outside the dataset stay with
 // the blocks (16k queries of a served tick 0.25 ms more).
 constexpr uint32_t kWarpTierMinQueries = 16384, kWarpTierMaxAvg = 8;
-constexpr float kWMaxPostings = 2500.f;
+constexpr float kWMaxPostings = 2500.f, kWMaxRangePostings = 1250.f;
 // Average list length from which two lanes rather than one share a list in the
 // warp tier of the symmetric form (100 x 4000 7.23 against 7.94 ms, 50 x 3000,
 // with lists of 12, 2.91 against 2.82; 60 x 3000, of 14, 3.57 against 3.48).
@@ -827,7 +832,7 @@ __host__ __device__ constexpr size_t warp_tier_bytes(uint32_t n_best) {
 template <int kGroup, int kForm>
 __global__ void __launch_bounds__(kWThreads, 6)
     k_summin_warp(ProfilesView P, QuerySet Q, HitsOut O, TierIO T, uint32_t* ticket, uint32_t n_best,
-                  float per_entry) {
+                  float avg_list) {
   extern __shared__ __align__(16) unsigned char smem[];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
   unsigned char* mine = smem + (size_t)warp * warp_tier_bytes(n_best);
@@ -863,8 +868,18 @@ __global__ void __launch_bounds__(kWThreads, 6)
     const uint32_t La_a = P.La[q.a];
     // a packed slot holds s <= La_a
     bool overflow = E > kWEntries || La_a >= cmask;
-    // too many postings to be expected (per_entry: of an entry, per gene after the query's genome)
-    if (kForm == kSymmetricForm && (float)E * per_entry * (float)(P.n_genes - q.own1) > kWMaxPostings) overflow = true;
+    // too many postings to be expected: of each list (avg_list; 0: not looked at)
+    // the share of its genes that the query walks -- of the dataset's, or in a
+    // batch, where a list holds the genes of one job, of the job's
+    if (kForm != kAllPairsForm && avg_list > 0.f) {
+      uint32_t walk = q.t1 - q.t0, of = P.n_genes;
+      if (kForm == kSymmetricForm) {
+        walk = (Q.two_genomes ? q.tend : P.n_genes) - q.own1;
+        if (Q.two_genomes) of = q.tend - q.own0;
+      }
+      const float most = kForm == kRangeForm ? kWMaxRangePostings : kWMaxPostings;
+      if ((float)E * avg_list * (float)walk > most * (float)of) overflow = true;
+    }
     uint32_t n_used = 0;
     // Adds the postings put aside (words gene | min of the counts) in [from, to).
     auto flush = [&](uint32_t from, uint32_t to) {
@@ -1338,7 +1353,7 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
     auto kernel = Q.symbest     ? (two ? k_summin_warp<2, kSymmetricForm> : k_summin_warp<1, kSymmetricForm>)
                   : Q.all_pairs ? (two ? k_summin_warp<2, kAllPairsForm> : k_summin_warp<1, kAllPairsForm>)
                                 : (two ? k_summin_warp<2, kRangeForm> : k_summin_warp<1, kRangeForm>);
-    const float per_entry = short_lists ? 0.f : (float)P.n_join / ((float)P.n_entries * (float)P.n_genes);
+    const float avg_list = short_lists ? 0.f : (float)P.n_join / (float)P.n_entries;
     const size_t smem = kWWarps * warp_tier_bytes(n_best);
     if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)(kWWarps * warp_tier_bytes(kWMaxGenomes)))) != cudaSuccess)
@@ -1351,7 +1366,7 @@ cudaError_t run_summin_tiers(Launcher* L, const ProfilesView& P, const QuerySet&
                                                                    (uint32_t)n_sm * std::max(per_sm, 1)));
     TierIO t0{nullptr, nullptr, O.def0, O.n_def0};
     if ((e = launch_begin(L, "summin_warp")) != cudaSuccess) return e;
-    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best, per_entry);
+    kernel<<<grid, kWThreads, smem, s>>>(P, Q, O, t0, O.ticket, n_best, avg_list);
     if ((e = launch_end(L, "summin_warp")) != cudaSuccess) return e;
     t1.in_list = O.def0;
     t1.in_count = O.n_def0;

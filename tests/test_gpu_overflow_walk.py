@@ -1,5 +1,6 @@
 """Queries that meet far more targets than a tier's table holds: their walk ends
-where the table is full.  Results equal those of the other forms; the times are
+where the table is full, and queries expected to overflow the warp tier are not
+walked there first.  Results equal those of the other forms; the times are
 compared with those of launches of the same run."""
 import numpy as np
 import pytest
@@ -58,3 +59,20 @@ def test_full_tables_end_the_walk(ctx):
     pd.pd_ctx_set_symmetric(ctx, True)
     for got in results[1:]:
         assert all(np.array_equal(x, y) for x, y in zip(got, results[0]))
+
+
+def test_heavy_queries_pass_by_the_warp_tier(ctx):
+    """Paralogs, listed pairs and batched jobs of many postings a query take no
+    longer than with the block tiers alone."""
+    data = dataset(4, 6000, 300, 2)
+    prof = pd.pd_build_profiles(ctx, *data, 4)
+    pairs = np.array([[0, 1], [2, 3]], np.uint32)
+    calls = (lambda: pd.pd_hits_copy(ctx, pd.pd_paralog_hits(ctx, prof)),
+             lambda: pd.pd_batch_copy_hits(ctx, pd.pd_bbh_pairs(ctx, prof, pairs)),
+             lambda: pd.pd_batch_copy_hits(ctx, pd.pd_bbh_batch(ctx, *data, pairs, np.array([4, 4], np.int32))))
+    for call in calls:
+        got, want = call(), forced(ctx, pd.PD_WALK_MERGE, call)
+        assert all(np.array_equal(x, y) for x, y in zip(got, want))
+        ours, = kernel_ms(ctx, call)
+        blocks, = forced(ctx, pd.PD_WALK_MERGE, lambda: kernel_ms(ctx, call))
+        assert ours < 1.2 * blocks, (ours, blocks)
