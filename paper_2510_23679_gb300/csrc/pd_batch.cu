@@ -470,6 +470,19 @@ __global__ void k_pairs_bbh(const PairJob* __restrict__ jobs, uint32_t n_jobs, u
   }
 }
 
+// Target genomes of each genome (bits of the words from mask[genome * words],
+// zeroed), from the genes of the jobs; a pair with an empty genome has no rows.
+__global__ void k_pairs_mask(const PairJob* __restrict__ jobs, uint32_t n_jobs,
+                             const uint16_t* __restrict__ gene_genome, uint32_t words, uint32_t* __restrict__ mask) {
+  for (uint32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < n_jobs; j += gridDim.x * blockDim.x) {
+    const PairJob J = jobs[j];
+    if (J.nA == 0 || J.nB == 0) continue;
+    const uint32_t a = gene_genome[J.A0], b = gene_genome[J.B0];
+    atomicOr(&mask[(size_t)a * words + b / 32], 1u << (b & 31u));
+    atomicOr(&mask[(size_t)b * words + a / 32], 1u << (a & 31u));
+  }
+}
+
 // Query genes and their target ranges, row by row (listed form).
 __global__ void k_pairs_queries(const PairJob* __restrict__ jobs, uint32_t n_jobs, uint32_t n_rows,
                                 uint32_t* __restrict__ gene, uint32_t* __restrict__ t0, uint32_t* __restrict__ t1) {
@@ -554,15 +567,11 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   // queries are then the genes of the genomes named, each against the genomes
   // its own is paired with, and the jobs' rows are slices of theirs.
   const uint32_t words = (n_genomes + 31) / 32;
-  std::vector<uint32_t> mask((size_t)n_genomes * words, 0);
   std::vector<uint32_t> last(n_genomes, 0);  // past the last partner of each genome
-  uint64_t n_named = 0, n_directed = 0;      // genes of the genomes named; rows of the distinct ordered pairs
+  uint64_t n_named = 0;                      // genes of the genomes named
   for (uint32_t j = 0; j < n_jobs; ++j)
     for (int way = 0; way < 2; ++way) {
       const uint32_t a = jobs[2 * j + way], b = jobs[2 * j + 1 - way];
-      uint32_t& w = mask[(size_t)a * words + b / 32];
-      if (!((w >> (b & 31)) & 1u)) n_directed += (uint64_t)(gp[a + 1] - gp[a]);
-      w |= 1u << (b & 31);
       last[a] = std::max(last[a], b + 1);
     }
   // Symmetric: each pair is walked from its first genome only (the part of a
@@ -585,9 +594,14 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
   pdg::QuerySet Q{};
   pd_status st = PD_OK;
   if (grouped) {
-    ALLOC(d_mask, sizeof(uint32_t) * mask.size());
+    // the mask is made on the device (2 MB at 4096 genomes, which a call of one
+    // pair cleared and copied on the host: 0.21 against 0.19 ms)
+    const size_t mask_bytes = sizeof(uint32_t) * n_genomes * (size_t)words;
+    ALLOC(d_mask, mask_bytes);
     ALLOC(d_qg, sizeof(uint32_t) * n_named);
-    CK(cudaMemcpyAsync(d_mask.p, mask.data(), sizeof(uint32_t) * mask.size(), cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemsetAsync(d_mask.p, 0, mask_bytes, c->stream));
+    PD_KLAUNCH("pairs_mask", (k_pairs_mask<<<grid_of(n_jobs, 256, 152u * 8u), 256, 0, c->stream>>>(
+                                 d_jobs.as<PairJob>(), n_jobs, P->view.gene_genome, words, d_mask.as<uint32_t>())));
     Q.all_pairs = 1;
     Q.order = d_qg.as<uint32_t>();
     Q.tgt_mask = d_mask.as<uint32_t>();
@@ -608,8 +622,9 @@ pd_status pairs_impl(pd_ctx* c, const pd_profiles* P, const uint32_t* jobs, uint
       PD_KLAUNCH("pairs_genes", (k_span_genes<<<grid_of(spans.size(), 1, 152u * 8u), 256, 0, c->stream>>>(
                                     d_spans.as<GenomeSpan>(), (uint32_t)spans.size(), d_qg.as<uint32_t>())));
       Q.n_queries = n_listed;
-      const uint64_t n_dir = sym ? n_directed / 2 : n_directed;  // rows that the launch emits
-      const uint32_t per_query = (uint32_t)((n_dir + n_listed) / std::max<uint32_t>(n_listed, 1));
+      const uint64_t n_dir = sym ? n_q / 2 : n_q;  // rows that the launch emits, if no pair is listed twice
+      const uint32_t per_query = std::min<uint32_t>(
+          (uint32_t)((n_dir + n_listed) / std::max<uint32_t>(n_listed, 1)), std::max<uint32_t>(n_genomes - 1, 1));
       bool too_many = false;
       st = sym ? sym_hits(c, P, Q, false, &H, &too_many, per_query) : run_hits(c, P, Q, false, &H, per_query);
       if (!sym || (st != PD_ERR_OOM && !too_many)) break;  // no room for maxima or ties: the plain form needs none
