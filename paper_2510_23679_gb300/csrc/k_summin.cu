@@ -856,7 +856,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
   const uint32_t* __restrict__ post = P.post;
   static_assert(kWSlots == 2u << 9, "512 buckets of two slots");
   auto home = [](uint32_t key) { return ((key * 0x9E3779B1u) >> 22) & ~1u; };
-  unsigned long long walked = 0;
+  unsigned long long walked = 0;  // postings of the queries kept (another tier counts the others')
   for (;;) {
     uint32_t qi = 0;
     if (lane == 0) qi = atomicAdd(ticket, 1u);
@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
       const float most = kForm == kRangeForm ? kWMaxRangePostings : kWMaxPostings;
       if ((float)E * avg_list * (float)walk > most * (float)of) overflow = true;
     }
-    uint32_t n_used = 0;
+    uint32_t n_used = 0, n_walked = 0;
     // Adds the postings put aside (words gene | min of the counts) in [from, to).
     auto flush = [&](uint32_t from, uint32_t to) {
       uint32_t claimed = kEmpty;
@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
         ring_ce[x] = nv.y | (c0 + lane) << 16;
       }
       staged += (uint32_t)__popc(some);
-      walked += len;
+      n_walked += len;
       c0 += 32u;
       if (c0 + lane < E) nv = q_mv[m0 + c0 + lane];
       __syncwarp();
@@ -1030,6 +1030,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
       __syncwarp();
       continue;
     }
+    walked += n_walked;
     // ---- per target genome: the maximum ratio, then the entries at it
     for (uint32_t j = lane; j <= n_best; j += 32) {
       if (j < n_best) best[j] = 0ull;
