@@ -225,15 +225,6 @@ __device__ __forceinline__ void init_code_table(uint8_t* lut, int alpha) {
   __syncthreads();
 }
 
-__device__ __forceinline__ uint32_t mix32(uint32_t x) {
-  x ^= x >> 16;
-  x *= 0x7feb352du;
-  x ^= x >> 15;
-  x *= 0x846ca68bu;
-  x ^= x >> 16;
-  return x;
-}
-
 // Digit counts of every pass (hist[pass * kMaxBins + digit]) over the windows
 // of this slice, and the genes' min-hashes (minimum of a hash of the codes).
 // Bound by the shared-memory atomics (one per window and pass).

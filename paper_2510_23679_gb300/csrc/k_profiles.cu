@@ -26,15 +26,6 @@ constexpr int kMvLongThreads = 1024;
 constexpr uint32_t kMvSmallCap = 2048;  // table slots of the shared-memory multiplicity-vector build
 constexpr uint32_t kMvMidCap = 16384;   // ... of its 1024-thread variant (one block per SM)
 
-__device__ __forceinline__ uint32_t mix32(uint32_t x) {
-  x ^= x >> 16;
-  x *= 0x7feb352du;
-  x ^= x >> 15;
-  x *= 0x846ca68bu;
-  x ^= x >> 16;
-  return x;
-}
-
 // ------------------------------------------------------------ dictionary
 __global__ void k_dict_mark(const uint32_t* __restrict__ code_lo, const uint8_t* __restrict__ code_hi, uint64_t n,
                             uint32_t* __restrict__ dict) {
@@ -186,16 +177,6 @@ __global__ void k_export_codes(const uint32_t* __restrict__ code_lo, const uint8
                                unsigned long long* __restrict__ codes) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
     codes[i] = code_at(code_lo, code_hi, i);
-}
-
-// Exact count of the k-mer whose list starts at `start` in gene g (its
-// multiplicity vector is unordered, and holds every count that does not fit
-// the posting).
-__device__ __forceinline__ uint32_t mv_count_of(const ProfilesView& P, uint32_t g, uint32_t start) {
-  const uint32_t off = P.win_off[g], n = P.mv_n[g];
-  for (uint32_t e = 0; e < n; ++e)
-    if (P.mv[off + e].x == start) return P.mv[off + e].y;
-  return 0u;
 }
 
 // Export of the multiplicity vectors (inspection hook), transposed from the

@@ -120,6 +120,15 @@ __host__ __device__ __forceinline__ uint32_t next_pow2(uint32_t x) {
   return x + 1;
 }
 
+__device__ __forceinline__ uint32_t mix32(uint32_t x) {
+  x ^= x >> 16;
+  x *= 0x7feb352du;
+  x ^= x >> 15;
+  x *= 0x846ca68bu;
+  x ^= x >> 16;
+  return x;
+}
+
 // Letter -> 0..alpha-1, 255 otherwise; built per block.  alpha 20: amino
 // acids in ACDEFGHIKLMNPQRSTVWY order; alpha 4: nucleotides in ACGT order.
 __device__ __forceinline__ void init_letter_table(uint8_t* lut, int alpha) {
@@ -305,6 +314,17 @@ struct ProfilesView {
   const uint4* q_mv;
   const uint32_t* q_La;
 };
+
+// Exact multiplicity in gene g of the k-mer whose posting list starts at
+// `start`, for a saturated packed count.  A multiplicity vector is unordered
+// (and holds every count that does not fit its posting), so this is a linear
+// scan (rare: only counts at the cap of the packed field come here).
+__device__ __forceinline__ uint32_t mv_count_of(const ProfilesView& P, uint32_t g, uint32_t start) {
+  const uint32_t off = P.win_off[g], n = P.mv_n[g];
+  for (uint32_t e = 0; e < n; ++e)
+    if (P.mv[off + e].x == start) return P.mv[off + e].y;
+  return 0u;
+}
 
 // Target selection of one sum-min launch.
 //   all_pairs = 1: query index x is gene order[x] (or q0 + x without an order)
