@@ -153,14 +153,14 @@ __device__ __forceinline__ uint32_t order_bucket(uint32_t minhash, uint32_t La, 
   return (lb << 14) | (h >> 18);
 }
 
-// Also the length of every gene's vector: what its cursor passed.
+// Also (cursor not null) the length of every gene's vector: what its cursor passed.
 __global__ void k_order_count(const uint32_t* __restrict__ minhash, const uint32_t* __restrict__ La, uint32_t n_genes,
                               int length_buckets, const uint32_t* __restrict__ cursor,
                               const uint32_t* __restrict__ win_off, uint32_t* __restrict__ mv_n,
                               uint32_t* __restrict__ count) {
   for (uint32_t g = blockIdx.x * blockDim.x + threadIdx.x; g < n_genes; g += gridDim.x * blockDim.x) {
     atomicAdd(&count[order_bucket(minhash[g], La[g], length_buckets)], 1u);
-    mv_n[g] = cursor[g] - win_off[g];
+    if (cursor) mv_n[g] = cursor[g] - win_off[g];
   }
 }
 

@@ -105,14 +105,14 @@ __global__ void __launch_bounds__(kThreads)
     const uint32_t n_here = min(per, n - chunk * per);
     const uint32_t i = lane < n_here ? order[chunk * per + lane] : 0u;  // lane j holds pair j
     const uint32_t ga = lane < n_here ? a[i] : pdg::kEmpty, gb = lane < n_here ? b[i] : 0u;
-    const uint32_t b0 = lane < n_here ? P.win_off[gb] : 0u, bn = lane < n_here ? P.mv_n[gb] : 0u;
+    const uint32_t b0 = lane < n_here ? P.mv_off[gb] : 0u, bn = lane < n_here ? P.mv_n[gb] : 0u;
     uint32_t s = 0;
     bool left = false;
     for (uint32_t j0 = 0; j0 < n_here;) {
       const uint32_t g = __shfl_sync(0xffffffffu, ga, j0);
       const uint32_t run = __ballot_sync(0xffffffffu, ga == g);  // the pairs of this gene, j0 first
       const uint32_t j1 = j0 + (uint32_t)__popc(run);
-      const uint32_t m0 = P.win_off[g], na = P.mv_n[g];
+      const uint32_t m0 = P.mv_off[g], na = P.mv_n[g];
       if (na > kWarpEntries) {
         if (ga == g) {
           longs[atomicAdd(n_longs, 1u)] = i;
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kLongThreads, 2)
   const uint32_t n = *n_longs, lane = threadIdx.x & 31u;
   for (uint32_t x = blockIdx.x; x < n; x += gridDim.x) {
     const uint32_t i = longs[x], ga = a[i], gb = b[i];
-    const uint4 *va = P.mv + P.win_off[ga], *vb = P.mv + P.win_off[gb];
+    const uint4 *va = P.mv + P.mv_off[ga], *vb = P.mv + P.mv_off[gb];
     const uint32_t na = P.mv_n[ga], nb = P.mv_n[gb];
     uint32_t sum = 0;
     if (threadIdx.x == 0) total = 0;

@@ -437,7 +437,7 @@ __device__ __forceinline__ void process_query(uint32_t qi, const ProfilesView& P
   // the query's own vector (its dataset's, or the external query arrays)
   const bool ext = kForm == kAnyForm && P.q_win_off != nullptr;
   const uint4* __restrict__ q_mv = ext ? P.q_mv : P.mv;
-  const uint32_t m0 = (ext ? P.q_win_off : P.win_off)[a], E = (ext ? P.q_mv_n : P.mv_n)[a];
+  const uint32_t m0 = (ext ? P.q_win_off : P.mv_off)[a], E = (ext ? P.q_mv_n : P.mv_n)[a];
   const uint32_t La_a = (ext ? P.q_La : P.La)[a];
   const uint32_t cnt_mask = (1u << P.cnt_bits) - 1u;
   const uint32_t tid = threadIdx.x;
@@ -854,7 +854,7 @@ __global__ void __launch_bounds__(kWThreads, 6)
     if (qi >= Q.n_queries) break;
     Query q;
     if (!load_query<kForm>(qi, P, Q, &q)) continue;
-    const uint32_t m0 = P.win_off[q.a], E = P.mv_n[q.a];
+    const uint32_t m0 = P.mv_off[q.a], E = P.mv_n[q.a];
     const uint32_t La_a = P.La[q.a];
     // a packed slot holds s <= La_a
     bool overflow = E > kWEntries || La_a >= cmask;

@@ -116,6 +116,7 @@ PD_API pd_status pd_ctx_create(int device, void* cuda_stream, pd_alloc_fn alloc,
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_err, sizeof(DevErr));
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_build, 8 * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_genome_ptr, sizeof(int32_t) * (PD_MAX_GENOMES + 1));
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->sizes, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMemset(c->d_err, 0, sizeof(DevErr));
   if (e == cudaSuccess && !alloc) {
     // Without hooks the context allocates from a pool of its own that keeps
@@ -137,6 +138,7 @@ PD_API pd_status pd_ctx_create(int device, void* cuda_stream, pd_alloc_fn alloc,
     if (c->h_err) cudaFreeHost(c->h_err);
     if (c->h_build) cudaFreeHost(c->h_build);
     if (c->h_genome_ptr) cudaFreeHost(c->h_genome_ptr);
+    if (c->sizes) cudaEventDestroy(c->sizes);
     if (c->own_pool) cudaMemPoolDestroy(c->pool);
     delete c;
     return PD_ERR_CUDA;
@@ -157,6 +159,7 @@ PD_API void pd_ctx_destroy(pd_ctx* c) {
   cudaFreeHost(c->h_err);
   cudaFreeHost(c->h_build);
   cudaFreeHost(c->h_genome_ptr);
+  cudaEventDestroy(c->sizes);
   // allocations still held by handles keep the pool alive until they are freed
   if (c->own_pool) cudaMemPoolDestroy(c->pool);
   delete c;
@@ -260,10 +263,17 @@ PD_API int pd_choose_k(uint64_t total, int alphabet) {
 // bit each, 4 GiB of bits (4.6 GiB of rank blocks).
 static constexpr uint64_t kMaxDictCodes = (uint64_t)32 << 30;
 
+// Windows of a dataset up to which its index and vectors stay in arrays of a
+// window's size, 28 bytes a window where 17 to 20 are used (the build by
+// dictionary kept 18 to 22): at most 0.1 GB more than before, where making them
+// fit takes 20 to 100 us, 4 to 8% of a whole run (4 genomes x 250 genes 401 and 426
+// us, 8 x 600 nucleotide 672 and 732, 23 x 1700 1.70 and 1.80 ms).
+static constexpr uint64_t kFewWindows = 16ull << 20;
+
 pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const int64_t* gene_ptr,
                                      uint32_t n_genes, const int32_t* genome_ptr, uint32_t n_genomes, int k,
                                      const uint32_t* genome_seg, pd_profiles** out, const int64_t* gene_src,
-                                     int alphabet, int length_buckets, bool code_order) {
+                                     int alphabet, int length_buckets, ProfileUse use) {
   PhaseRange range_("pd: profiles");
   if (alphabet != PD_ALPHABET_AMINO && alphabet != PD_ALPHABET_NUCLEOTIDE)
     return fail(c, PD_ERR_ARG, "alphabet must be 20 (amino acids) or 4 (nucleotides)");
@@ -333,7 +343,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   uint32_t seg_bits = 0, kmer_bits = 1;
   while ((n_seg - 1) >> seg_bits) ++seg_bits;
   while (kmer_bits < 63 && ((n_codes - 1) >> kmer_bits)) ++kmer_bits;
-  const bool below = genome_seg && !code_order && kmer_bits + seg_bits + gene_bits <= 64;
+  const bool below = genome_seg && use == ProfileUse::kCall && kmer_bits + seg_bits + gene_bits <= 64;
   if (!below) seg_bits = 0;
   const uint64_t all_codes = below ? n_codes << seg_bits : n_seg * n_codes;
   if (below)
@@ -343,30 +353,33 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   // ---- per-gene arrays, inputs on the device
   Carve cg;
   const size_t o_genome_ptr = cg.add(sizeof(int32_t) * (n_genomes + 1)), o_La = cg.add(sizeof(uint32_t) * n_genes),
-               o_win_off = cg.add(sizeof(uint32_t) * (n_genes + 1)), o_mv_n = cg.add(sizeof(uint32_t) * n_genes),
+               o_mv_off = cg.add(sizeof(uint32_t) * (n_genes + 1)), o_mv_n = cg.add(sizeof(uint32_t) * n_genes),
                o_gene_genome = cg.add(sizeof(uint16_t) * n_genes), o_ginfo = cg.add(sizeof(uint32_t) * n_genes),
                o_order = cg.add(sizeof(uint32_t) * n_genes);
   ALLOC(P->genes, cg.bytes);
   int32_t* d_genome_ptr = piece<int32_t>(P->genes, o_genome_ptr);
-  uint32_t *d_La = piece<uint32_t>(P->genes, o_La), *d_win_off = piece<uint32_t>(P->genes, o_win_off),
+  uint32_t *d_La = piece<uint32_t>(P->genes, o_La), *d_mv_off = piece<uint32_t>(P->genes, o_mv_off),
            *d_mv_n = piece<uint32_t>(P->genes, o_mv_n), *d_ginfo = piece<uint32_t>(P->genes, o_ginfo),
            *d_order = piece<uint32_t>(P->genes, o_order);
   uint16_t* d_gene_genome = piece<uint16_t>(P->genes, o_gene_genome);
   const bool copy_res = n_res > 0 && !is_device_ptr(residues);
   Carve ct;
   // zeroed words first: [0] windows, [1..4] postings and ids (so far, before the slice), [5] join, [6] longest
-  // list; then the order's counts
+  // list, [7] vector entries; then the order's counts
   const size_t o_words = ct.add(8 * sizeof(unsigned long long)),
                o_ocount = ct.add(sizeof(uint32_t) * (2 * pdg::kOrderBuckets + 1)), zeroed = ct.bytes,
-               o_minhash = ct.add(sizeof(uint32_t) * n_genes), o_cursor = ct.add(sizeof(uint32_t) * n_genes),
+               o_minhash = ct.add(sizeof(uint32_t) * n_genes),
+               o_cursor = ct.add(sizeof(uint32_t) * n_genes),
+               o_win_off = ct.add(sizeof(uint32_t) * ((size_t)n_genes + 1)),
                o_scan = ct.add(pdg::scan_temp_bytes(std::max<uint64_t>((uint64_t)n_genes + 1, pdg::kOrderBuckets)) + 64),
                o_gene_ptr = ct.add(gp_dev ? 0 : sizeof(int64_t) * (n_genes + 1)),
                o_code_base = ct.add(genome_seg ? sizeof(unsigned long long) * n_genomes : 0),
                o_res = ct.add(copy_res ? n_res : 0);
-  Buf tmp1, tmp2;
+  Buf tmp1;
   ALLOC(tmp1, ct.bytes);
   unsigned long long* words = piece<unsigned long long>(tmp1, o_words);
-  uint32_t* minhash = piece<uint32_t>(tmp1, o_minhash);
+  uint32_t *minhash = piece<uint32_t>(tmp1, o_minhash), *d_win_off = piece<uint32_t>(tmp1, o_win_off),
+           *cursor = piece<uint32_t>(tmp1, o_cursor);
   void* scan_tmp = piece<void>(tmp1, o_scan);
   const uint8_t* res_dev = residues;
   const int64_t* gp_devp = gene_ptr;
@@ -385,7 +398,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   // ---- offsets and letters checked, window offsets, genes' genomes
   if (n_genes)
     CK(pdg::run_gene_windows(L, gp_devp, n_genes, n_res, gene_src ? 0 : 1, k, d_genome_ptr, n_genomes, d_La,
-                             d_gene_genome, d_ginfo, minhash, c->d_err, c->stream));
+                             d_gene_genome, d_ginfo, minhash, d_mv_n, c->d_err, c->stream));
   CK(pdg::scan_u32_total(L, d_La, n_genes, d_win_off, words, scan_tmp, c->stream));
   if (n_genes)
     CK(pdg::run_check_letters(L, res_dev, n_res, gp_devp, gene_src, n_genes, alphabet, c->d_err, c->stream));
@@ -405,44 +418,56 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   if (!early_genomes && (st = check_genomes()) != PD_OK) return st;
   P->h_genome_ptr = hgn;
 
-  // ---- vectors, postings, and one record buffer that ends up holding the
-  // posting-list starts and the codes (at most one of each per window)
-  const bool wide_codes = all_codes > (1ull << 32);
-  Carve cw;
-  const size_t o_mv = cw.add(sizeof(uint4) * W), o_post = cw.add(sizeof(uint32_t) * W),
-               o_lists = cw.add(2 * sizeof(uint32_t) * (W + 1)), o_code_hi = cw.add(wide_codes ? W : 0);
-  ALLOC(P->windows, cw.bytes);
-  uint4* d_mv = piece<uint4>(P->windows, o_mv);
-  uint32_t *d_post = piece<uint32_t>(P->windows, o_post), *d_post_ptr = piece<uint32_t>(P->windows, o_lists);
-  uint32_t* d_code_lo = d_post_ptr + (W + 1);
-  uint8_t* d_code_hi = wide_codes ? piece<uint8_t>(P->windows, o_code_hi) : nullptr;
-  uint32_t* cursor = piece<uint32_t>(tmp1, o_cursor);
+  // ---- index and vectors.  The sort's second buffer ends up holding list starts
+  // and codes (at most one of each a window), and arrays of a window's size hold
+  // the rest; or, once the windows are sorted and it is known how much there is of
+  // everything, memory of that size is taken, list starts and codes are copied to
+  // it and the vectors made there (200 genomes x 4000 genes: 4.8 GB in 16.2 ms, 7.5
+  // in 15.4 in arrays of a window's size, 5.5 by dictionary; 50 x 3000 0.97 GB in
+  // 2.86 ms, 1.40 in 2.71).  Records sorted in slices leave no choice.
+  const bool wide_codes = all_codes > (1ull << 32), sliced = K.n_slices > 1,
+             fit = !sliced && (use == ProfileUse::kBudget || (use == ProfileUse::kKept && W > kFewWindows));
+  const pdg::SortScratch X = pdg::sort_scratch(K, W);
+  const uint32_t n_ltiles = pdg::list_tiles(W);
+  Carve c2, c3;
+  const size_t o_rec = c2.add(sliced ? 0 : sizeof(unsigned long long) * W),
+               o_tile_gene = c2.add(sizeof(uint32_t) * (pdg::sort_tiles(W) + 1)),
+               o_tile_e = c2.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)),
+               o_tile_id = c2.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)), o_scratch = c2.add(X.bytes);
+  const size_t o_ptr = c3.add(sizeof(uint32_t) * (W + 1)), o_code = c3.add(sizeof(uint32_t) * W),
+               o_code_hi = c3.add(wide_codes ? W : 0), o_post = c3.add(fit ? 0 : sizeof(uint32_t) * W),
+               o_mv = c3.add(fit ? 0 : sizeof(uint4) * W);
+  Buf tmp2, whole, slice_rec;
+  ALLOC(whole, c3.bytes);
+  ALLOC(tmp2, c2.bytes);
+  if (fit) ALLOC(P->postings, sizeof(uint32_t) * W);
+  uint32_t *d_post_ptr = piece<uint32_t>(whole, o_ptr), *d_code_lo = piece<uint32_t>(whole, o_code);
+  uint8_t* d_code_hi = wide_codes ? piece<uint8_t>(whole, o_code_hi) : nullptr;
+  uint32_t* d_post = fit ? P->postings.as<uint32_t>() : piece<uint32_t>(whole, o_post);
+  uint4* d_mv = fit ? nullptr : piece<uint4>(whole, o_mv);
+  uint8_t* scratch = piece<uint8_t>(tmp2, o_scratch);
+  uint32_t *tile_e = piece<uint32_t>(tmp2, o_tile_e), *tile_id = piece<uint32_t>(tmp2, o_tile_id);
+  // the sort ends in the first of the two record buffers
+  unsigned long long *sorted = nullptr, *rec = piece<unsigned long long>(tmp2, o_rec), *other = whole.as<unsigned long long>();
+  pdg::WindowSource S{res_dev, gp_devp, gene_src, d_win_off, piece<uint32_t>(tmp2, o_tile_gene), d_gene_genome,
+                      d_code_base, k, alphabet, W, seg_bits};
+  uint64_t n = W;  // records of the slice
+  auto lists = [&] {
+    return pdg::run_lists(L, sorted, n, K, tile_e, tile_id, d_post, d_post_ptr, d_code_lo, d_code_hi, cnt_bits,
+                          cnt_cap, d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5,
+                          c->d_err, c->stream);
+  };
   if (W == 0) {
     CK(cudaMemsetAsync(d_post_ptr, 0, sizeof(uint32_t), c->stream));
     if (n_genes)
       CK(cudaMemcpyAsync(cursor, d_win_off, sizeof(uint32_t) * n_genes, cudaMemcpyDeviceToDevice, c->stream));
   } else {
-    const pdg::SortScratch X = pdg::sort_scratch(K, W);
-    const uint32_t n_ltiles = pdg::list_tiles(W);
-    Carve cs;
-    const size_t o_tile_gene = cs.add(sizeof(uint32_t) * (pdg::sort_tiles(W) + 1)),
-                 o_tile_e = cs.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)), o_tile_id = cs.add(sizeof(uint32_t) * ((size_t)n_ltiles + 1)),
-                 o_scratch = cs.add(X.bytes), o_rec = cs.add(sizeof(unsigned long long) * W);
-    ALLOC(tmp2, cs.bytes);
-    uint8_t* scratch = piece<uint8_t>(tmp2, o_scratch);
-    uint32_t *tile_e = piece<uint32_t>(tmp2, o_tile_e), *tile_id = piece<uint32_t>(tmp2, o_tile_id);
-    pdg::WindowSource S{res_dev, gp_devp, gene_src, d_win_off, piece<uint32_t>(tmp2, o_tile_gene), d_gene_genome,
-                        d_code_base, k, alphabet, W, seg_bits};
-    // two record buffers, one of which ends up holding lists and codes
-    unsigned long long *rec = piece<unsigned long long>(tmp2, o_rec), *other = (unsigned long long*)d_post_ptr;
     const bool odd = K.passes & 1u;
     CK(pdg::run_tile_genes(L, d_win_off, n_genes, W, piece<uint32_t>(tmp2, o_tile_gene), cursor, c->stream));
-    Buf slice_rec;
     for (K.slice = 0; K.slice < K.n_slices; ++K.slice) {
       CK(cudaMemsetAsync(scratch, 0, X.bytes, c->stream));
       CK(pdg::run_code_hist(L, S, K, scratch, X, K.slice ? nullptr : minhash, c->stream));
-      uint64_t n = W;
-      if (K.n_slices > 1) {
+      if (sliced) {
         std::vector<uint32_t> hist(pdg::kSortBins);  // of the first pass: the slice's records
         CK(cudaMemcpyAsync(hist.data(), scratch + X.hist, sizeof(uint32_t) * hist.size(), cudaMemcpyDeviceToHost,
                            c->stream));
@@ -455,25 +480,71 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
         rec = slice_rec.as<unsigned long long>();
         other = rec + n;
       }
-      unsigned long long* sorted = nullptr;
       CK(pdg::run_sort(L, S, K, n, scratch, X, odd ? rec : other, odd ? other : rec, &sorted, c->d_err, c->stream));
       CK(pdg::run_dedupe(L, sorted, n, K, scratch, X, cnt_bits, cnt_cap, words + 1, d_post, d_post_ptr, d_code_lo,
-                         d_code_hi, tile_e, tile_id, c->d_err, c->stream));
-      CK(pdg::run_lists(L, sorted, n, K, tile_e, tile_id, d_post, d_post_ptr, d_code_lo, d_code_hi, cnt_bits, cnt_cap,
-                        d_genome_ptr, n_genomes, n_genes, cursor, d_mv, (uint32_t*)(words + 6), words + 5, c->d_err,
-                        c->stream));
+                         d_code_hi, tile_e, tile_id, fit ? d_mv_n : nullptr, c->d_err, c->stream));
+      if (!fit) CK(lists());
     }
-    if (K.n_slices > 1) CK(cudaStreamSynchronize(c->stream));  // the last slice's records end here
+    K.slice = 0;
   }
-
-  // ---- all-pairs query order: min-hash buckets
-  if (n_genes)
-    CK(pdg::run_order(L, minhash, d_La, n_genes, length_buckets, cursor, d_win_off, d_mv_n,
-                      piece<uint32_t>(tmp1, o_ocount), d_order, scan_tmp, c->stream));
+  // all-pairs query order: min-hash buckets (and the lengths of vectors that are made)
+  auto order = [&]() -> cudaError_t {
+    return n_genes ? pdg::run_order(L, minhash, d_La, n_genes, length_buckets, fit ? nullptr : cursor, d_win_off,
+                                    d_mv_n, piece<uint32_t>(tmp1, o_ocount), d_order, scan_tmp, c->stream)
+                   : cudaSuccess;
+  };
+  if (!fit) {
+    CK(order());
+    CK(cudaMemcpyAsync(d_mv_off, d_win_off, sizeof(uint32_t) * ((size_t)n_genes + 1), cudaMemcpyDeviceToDevice,
+                       c->stream));
+  } else {
+    CK(pdg::scan_u32_total(L, d_mv_n, n_genes, d_mv_off, words + 7, scan_tmp, c->stream));
+    CK(cudaMemcpyAsync(hb, words, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(DevErr), cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaEventRecord(c->sizes, c->stream));
+    CK(order());  // while the host waits for the sizes and finds room
+    CK(cudaEventSynchronize(c->sizes));
+    if (c->h_err->code != 0) return check_dev_err(c);
+    const uint64_t D = hb[2], n_mv = hb[7];
+    // Where most k-mers are shared the vectors would be the most that the call
+    // holds at a time: the second record buffer is given back before they are made.
+    const bool tight = n_mv * 4 > W * 3;
+    // the codes of profiles with a budget end where their dictionary is made
+    const bool drop_codes = use == ProfileUse::kBudget;
+    Carve ci, cc;
+    Carve& of_codes = drop_codes ? cc : ci;
+    const size_t i_code = of_codes.add(sizeof(uint32_t) * D), i_code_hi = of_codes.add(wide_codes ? D : 0),
+                 i_ptr = ci.add(sizeof(uint32_t) * (D + 1)), i_mv = ci.add(tight ? 0 : sizeof(uint4) * n_mv);
+    if (!P->index.alloc(c, ci.bytes) || (drop_codes && !P->codes.alloc(c, cc.bytes))) {
+      cudaStreamSynchronize(c->stream);  // the order's kernels still use memory of the call
+      return fail(c, PD_ERR_OOM, "device allocation of the index failed");
+    }
+    pdg::PackList moved;
+    auto move = [&](auto* from, const Buf& to, size_t at, uint64_t count) {
+      moved.add(piece<void>(to, at), from, sizeof(*from) * count);
+      return (decltype(from))piece<void>(to, at);
+    };
+    const Buf& codes = drop_codes ? P->codes : P->index;
+    d_post_ptr = move(d_post_ptr, P->index, i_ptr, D + 1);
+    d_code_lo = move(d_code_lo, codes, i_code, D);
+    if (wide_codes) d_code_hi = move(d_code_hi, codes, i_code_hi, D);
+    moved.add(cursor, d_mv_off, sizeof(uint32_t) * n_genes);
+    CK(pdg::run_pack(L, moved, c->stream));
+    d_mv = piece<uint4>(P->index, i_mv);
+    if (tight) {
+      CK(cudaStreamSynchronize(c->stream));
+      whole.release();
+      ALLOC(P->vectors, sizeof(uint4) * n_mv);
+      d_mv = P->vectors.as<uint4>();
+    }
+    if (W) CK(lists());
+  }
   CK(cudaMemcpyAsync(hb, words, 7 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, c->stream));
   st = check_dev_err(c);  // synchronizes; temporaries are released after this
   if (st != PD_OK) return st;
-  const uint64_t E = hb[1], D = hb[2], n_join = hb[5];
+  if (!fit) P->index = std::move(whole);
+  const uint64_t E = hb[1], D = hb[2];
+  const uint64_t n_join = hb[5];
   const uint32_t max_posting = (uint32_t)hb[6];
 
   pdg::ProfilesView& v = P->view;
@@ -487,7 +558,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   v.cnt_cap = cnt_cap;
   v.max_posting = max_posting;
   v.n_join = n_join;
-  v.win_off = d_win_off;
+  v.mv_off = d_mv_off;
   v.mv_n = d_mv_n;
   v.mv = d_mv;
   v.La = d_La;
@@ -510,7 +581,7 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
   in.n_join = n_join;
   in.count_bits = cnt_bits;
   in.alphabet = alphabet;
-  in.device_bytes = P->genes.n + P->windows.n;
+  in.device_bytes = P->genes.n + P->index.n + P->postings.n + P->vectors.n + P->codes.n;
   *out = guard.release();
   return PD_OK;
 }
@@ -798,6 +869,12 @@ pd_status pdh::build_dictionary(pd_ctx* c, pd_profiles* P) {
   v.dict = P->dict.as<uint32_t>();
   v.n_dict_blocks = n_dict;
   P->info.device_bytes += P->dict.n;
+  if (P->codes.p) {  // the dictionary gives a k-mer's id; nobody asks for an id's code
+    P->info.device_bytes -= P->codes.n;
+    P->codes.release();
+    v.code_lo = nullptr;
+    v.code_hi = nullptr;
+  }
   return PD_OK;
 }
 

@@ -270,7 +270,7 @@ pd_status batch_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const i
     const int length_buckets = (tuning && tuning->query_order == 1) ? 0 : 1;
     pd_status st = build_profiles_impl(c, res_dev, (uint64_t)cg.back(), cg.data(), chunk_genes, cgn.data(),
                                        (uint32_t)genomes.size(), k, seg.data(), &Praw, d_src.as<int64_t>(),
-                                       PD_ALPHABET_AMINO, length_buckets, false);
+                                       PD_ALPHABET_AMINO, length_buckets, ProfileUse::kCall);
     if (st != PD_OK) return st;
     std::unique_ptr<pd_profiles> P(Praw);
 

@@ -65,6 +65,7 @@ struct pd_ctx {
   // pinned host words: sizes and counters read back in the middle of a call
   unsigned long long* h_build = nullptr;  // [8]
   int32_t* h_genome_ptr = nullptr;        // [PD_MAX_GENOMES + 1]
+  cudaEvent_t sizes = nullptr;  // the sizes of a build have arrived in h_build
   cudaMemPool_t pool = nullptr;  // without hooks: allocate from this pool (null: the device's default pool)
   bool own_pool = false;         // the pool was created by (and is destroyed with) this context
   uint64_t pool_bytes = 0;       // bytes currently allocated through this context (pool allocations only)
@@ -226,7 +227,9 @@ struct pd_profiles {
   pdg::ProfilesView view{};
   pd_profiles_info info{};
   Buf genes;    // per-gene and per-genome arrays
-  Buf windows;  // vectors, postings, posting-list starts and codes
+  // list starts and codes, vectors, postings: all in the first, or in their own
+  Buf index, postings, vectors;
+  Buf codes;    // the codes, of profiles that drop them for a dictionary
   Buf dict;     // dictionary, when outside queries need it
   std::vector<int32_t> h_genome_ptr;
 };
@@ -282,17 +285,22 @@ pdg::ProfilesView external_view(const pd_profiles* P, const QueryProfiles& Qp);
 pd_status run_hits_view(pd_ctx* c, const pdg::ProfilesView& v, const pdg::QuerySet& Q, pd_hits* H,
                         uint32_t genomes_per_query);
 
+// What profiles are built for.  kCall: one call, which drops them again: lists in
+// any order (genome_seg must not decrease) and arrays of a window's size.  kKept:
+// lists in order of segment, then code, and of many windows arrays of the size
+// that is needed.  kBudget: arrays of the size that is needed, always, and no
+// codes once build_dictionary has been called.
+enum class ProfileUse { kCall, kKept, kBudget };
 // Profiles of a dataset; genome_seg (host, per genome, or null) gives each
 // segment its own k-mer namespace.  gene_src (device, per gene, or null):
 // gene g starts at residues + gene_src[g] instead of residues + gene_ptr[g];
 // gene_ptr then gives only the lengths, and residues must be a device pointer.
-// code_order: lists in order of segment, then code; without it (genome_seg
-// must not decrease) in any order that suits the build.
+// use: what the profiles are for (see ProfileUse).
 pd_status build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t n_res, const int64_t* gene_ptr,
                               uint32_t n_genes, const int32_t* genome_ptr, uint32_t n_genomes, int k,
                               const uint32_t* genome_seg, pd_profiles** out, const int64_t* gene_src = nullptr,
                               int alphabet = PD_ALPHABET_AMINO, int length_buckets = 1,
-                              bool code_order = true);
+                              ProfileUse use = ProfileUse::kKept);
 // Sum-min + Best Hits of the query set Q into H (all tiers, output sized
 // exactly).  genomes_per_query (0 = n_genomes - 1) bounds the genomes one
 // query can hit; it only sizes the first output allocation.

@@ -4,7 +4,6 @@
 // pd_build_profiles and read by every later call):
 //
 //   gene g (global id, 0..G-1) has La[g] = max(0, |g|-k+1) k-mer windows.
-//   win_off[G+1]   uint32  exclusive prefix of La: window range of each gene.
 //   post_ptr[D+1]  uint32  inverted index: postings of id w (k-mers numbered by
 //   post[E]        uint32  ascending code) are post[post_ptr[w] .. post_ptr[w+1]),
 //                          ascending by gene, each packed as (gene << cnt_bits)
@@ -14,8 +13,10 @@
 //   code_lo[D]     uint32  code of each id (with code_hi[D], its bits above 32,
 //                          when the codes need more).
 //   mv_n[G]        uint32  k-mers of the gene that another gene has too.
-//   mv[W]          uint4   the gene's multiplicity vector (Algorithm 1) over
-//                          those k-mers, at win_off[g] .. +mv_n[g] (the entries
+//   mv_off[G+1]    uint32  their exclusive prefix (the prefix of La in a dataset
+//                          of few windows, see build_profiles_impl).
+//   mv[]           uint4   the gene's multiplicity vector (Algorithm 1) over
+//                          those k-mers, at mv_off[g] .. +mv_n[g] (the entries
 //                          of one gene are unordered).  x: start of the k-mer's
 //                          posting list; y: its multiplicity in the gene; z: the
 //                          list's length, with the top bit set if it holds
@@ -291,9 +292,9 @@ struct ProfilesView {
   uint64_t n_windows, n_distinct, n_entries;
   uint32_t cnt_bits, cnt_cap, max_posting;
   uint64_t n_join;              // postings the all-against-all walk visits (sum over entries of list length)
-  const uint32_t* win_off;      // [G+1] window range of each gene
-  const uint32_t* mv_n;         // [G]   entries of each gene's vector
-  const uint4* mv;              // [W]   multiplicity vectors
+  const uint32_t* mv_off;       // [G+1] place of each gene's vector
+  const uint32_t* mv_n;         // [G]   its entries
+  const uint4* mv;              // multiplicity vectors
   const uint32_t* La;           // [G]   windows per gene
   const uint16_t* gene_genome;  // [G]   genome of each gene
   const uint32_t* ginfo;        // [G]   La | genome << 16
@@ -320,7 +321,7 @@ struct ProfilesView {
 // (and holds every count that does not fit its posting), so this is a linear
 // scan (rare: only counts at the cap of the packed field come here).
 __device__ __forceinline__ uint32_t mv_count_of(const ProfilesView& P, uint32_t g, uint32_t start) {
-  const uint32_t off = P.win_off[g], n = P.mv_n[g];
+  const uint32_t off = P.mv_off[g], n = P.mv_n[g];
   for (uint32_t e = 0; e < n; ++e)
     if (P.mv[off + e].x == start) return P.mv[off + e].y;
   return 0u;
@@ -455,13 +456,13 @@ cudaError_t scan_u32_total(Launcher* L, const uint32_t* in, uint64_t n, uint32_t
 
 // profiles and index of a dataset (k_index.cu)
 // Gene offsets -> window counts and genomes on the device, min-hashes cleared
-// (all ones).  Checks every gene (offsets from 0, non-decreasing, ending at
+// (all ones) and vector entries too (zero).  Checks every gene (offsets from 0, non-decreasing, ending at
 // n_res unless check_end is 0; at most PD_MAX_WINDOWS windows), recording
 // PD_ERR_ARG / PD_ERR_GENE_TOO_LONG with the gene as detail (such a gene gets La
 // 0).  genome_ptr need not have been checked yet.
 cudaError_t run_gene_windows(Launcher* L, const int64_t* gene_ptr, uint32_t n_genes, uint64_t n_res, int check_end,
                              int k, const int32_t* genome_ptr, uint32_t n_genomes, uint32_t* La, uint16_t* gene_genome,
-                             uint32_t* ginfo, uint32_t* minhash, DevErr* err, cudaStream_t s);
+                             uint32_t* ginfo, uint32_t* minhash, uint32_t* mv_n, DevErr* err, cudaStream_t s);
 // PD_ERR_ALPHABET (detail: the position) for a byte outside the alphabet: all
 // n_res bytes, or with gene_src the genes' bytes.
 cudaError_t run_check_letters(Launcher* L, const uint8_t* res, uint64_t n_res, const int64_t* gene_ptr,
@@ -514,13 +515,28 @@ cudaError_t run_sort(Launcher* L, const WindowSource& S, const SortKey& K, uint6
                      const SortScratch& X, unsigned long long* a, unsigned long long* b, unsigned long long** sorted,
                      DevErr* err, cudaStream_t s);
 // Sorted records -> post, post_ptr, code_lo / code_hi and the postings and ids
-// before each tile; totals: [4] words, the postings and ids so far first.
+// before each tile; totals: [4] words, the postings and ids so far first.  mv_n,
+// if not null: the vector entries of each gene, counted on.
 cudaError_t run_dedupe(Launcher* L, const unsigned long long* rec, uint64_t n, const SortKey& K, uint8_t* scratch,
                        const SortScratch& X, uint32_t cnt_bits, uint32_t cnt_cap, unsigned long long* totals,
                        uint32_t* post, uint32_t* post_ptr, uint32_t* code_lo, uint8_t* code_hi, uint32_t* tile_e,
-                       uint32_t* tile_id, DevErr* err, cudaStream_t s);
+                       uint32_t* tile_id, uint32_t* mv_n, DevErr* err, cudaStream_t s);
+// Copies of a few arrays in one launch, all 16-byte aligned and padded to that.
+struct PackList {
+  static constexpr int kMost = 4;
+  const void* from[kMost] = {};
+  void* to[kMost] = {};
+  uint64_t bytes[kMost] = {};
+  int n = 0;
+  void add(void* dst, const void* src, uint64_t size) {
+    from[n] = src;
+    to[n] = dst;
+    bytes[n++] = size;
+  }
+};
+cudaError_t run_pack(Launcher* L, const PackList& list, cudaStream_t s);
 // Vector entries of the slice's postings; cursor: the next free place of each
-// gene's vector (its first window before the first slice).  The longest list
+// gene's vector (its first place before the first slice).  The longest list
 // and the sum of squared list lengths (the postings an all-against-all walk
 // visits) are added to *max_list and *join.
 cudaError_t run_lists(Launcher* L, const unsigned long long* rec, uint64_t n, const SortKey& K, const uint32_t* tile_e,
@@ -549,8 +565,9 @@ cudaError_t run_mv_build(Launcher* L, const uint8_t* res, const int64_t* gene_pt
                          uint32_t n_genes, int k, const uint32_t* dict, const MvOut& M, const uint32_t* mid_genes, uint32_t n_mid, const uint32_t* long_genes,
                          uint32_t n_long, unsigned long long* long_scratch, const unsigned long long* long_scratch_off,
                          cudaStream_t s);
-// Query order, and the lengths of the vectors (what their cursors passed).
-// count must hold 2 * kOrderBuckets + 1 words (zeroed counts, then their prefix sum).
+// Query order, and with a cursor the lengths of the vectors (what it passed of
+// each).  count must hold 2 * kOrderBuckets + 1 words (zeroed counts, then their
+// prefix sum).
 constexpr uint32_t kOrderBuckets = 65536;
 cudaError_t run_order(Launcher* L, const uint32_t* minhash, const uint32_t* La, uint32_t n_genes, int length_buckets,
                       const uint32_t* cursor, const uint32_t* win_off, uint32_t* mv_n, uint32_t* count,

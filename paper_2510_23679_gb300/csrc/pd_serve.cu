@@ -287,7 +287,7 @@ pd_status build_level_on(pd_ctx* c, int k, const uint8_t* res, const std::vector
   for (auto& x : gn) x -= (int32_t)L->gene0;
   pd_profiles* P = nullptr;
   pd_status st = build_profiles_impl(c, res + r0, (uint64_t)gp.back(), gp.data(), L->gene1 - L->gene0, gn.data(),
-                                     g1 - g0, k, nullptr, &P);
+                                     g1 - g0, k, nullptr, &P, nullptr, PD_ALPHABET_AMINO, 1, ProfileUse::kBudget);
   if (st != PD_OK) return st;
   L->P.reset(P);
   st = build_dictionary(c, P);
