@@ -160,6 +160,29 @@ def summin_ms(pd, ctx):
     return sum(pd.pd_ctx_kernel_time(ctx, name)[0] for name in SUMMIN_TIERS)
 
 
+def shared_entries(pd, ctx, prof, dev):
+    """Vector entries of the profiles: (gene, k-mer) pairs whose k-mer another gene has too."""
+    import torch
+    lists = torch.empty(pd.pd_profiles_get_info(prof).n_distinct + 1, dtype=torch.int64, device=dev)
+    if pd.load().pd_profiles_copy_index(ctx.handle, prof.handle, lists.data_ptr(), None, None, None):
+        raise RuntimeError(pd.pd_last_error(ctx))
+    size = lists.diff()
+    return int(size[size > 1].sum())
+
+
+def forward_hits(pd, ctx, hits, ds, dev):
+    """Best Hits in genomes after the query's own: what the walk from one side emits."""
+    import torch
+    n = pd.pd_hits_get_info(hits).n_hits
+    row_ptr = torch.empty(ds.n_genes + 1, dtype=torch.int64, device=dev)
+    cols, s = (torch.empty(max(n, 1), dtype=torch.int32, device=dev) for _ in range(2))
+    pd.pd_hits_copy(ctx, hits, row_ptr, cols, s)
+    ends = torch.from_numpy(ds.genome_ptr[1:].astype("int32")).to(dev)
+    genome = torch.bucketize(torch.arange(ds.n_genes, dtype=torch.int32, device=dev), ends, right=True)
+    past = ends[genome]  # first gene after each gene's genome
+    return int((cols[:n] >= torch.repeat_interleave(past, row_ptr.diff())).sum())
+
+
 def alphabet_of(name):
     return 4 if synth.WORKLOADS.get(name, {}).get("alphabet") == "nt" else 20
 
@@ -636,12 +659,12 @@ def run_sharded(args):
     ms = max_over_ranks(ms_local, world)
     pairs = ds.logical_pairs()
     # roofline of this rank's shard: its postings walked and hits, and its
-    # share (1/world) of the vector, row and gene bytes
+    # share (1/world) of the vectors and of the row and gene words
     prof, hits, bbh = keep
     pinfo = pd.pd_profiles_get_info(prof)
     shard_hits = pd.pd_hits_get_info(pd.pd_best_hits_shard(ctx, prof, rank, world))
-    alg = (pinfo.n_entries * 14 + pinfo.n_genes * 12) / world + shard_hits.postings_walked * 4 + \
-        shard_hits.n_hits * 8
+    alg = (shared_entries(pd, ctx, prof, dev) * 16 + pinfo.n_genes * 12) / world + \
+        shard_hits.postings_walked * 4 + shard_hits.n_hits * 8
     peak = float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))).get("hbm_gbs", 6800.0)) \
         if os.path.exists(os.path.join(ROOT, "MEASURED_PEAKS.json")) else 6800.0
     clocks = clk.summary()
@@ -738,10 +761,15 @@ def main():
     hinfo = pd.pd_hits_get_info(hits)
     n_bbh = pd.pd_bbh_count(bbh)
 
-    # ---- roofline of the dominant kernels (the sum-min + Best Hit tiers), algorithmic bytes per step
+    # ---- roofline of the dominant kernels (the sum-min + Best Hit tiers),
+    # algorithmic bytes per step: vector entries, postings walked, the hits that
+    # the tiers emit (those of the later genomes; the rows' other part is assembled
+    # by other kernels), row and gene words
     E = pinfo.n_entries
     J = hinfo.postings_walked
-    alg_bytes = E * 6 + E * 8 + J * 4 + hinfo.n_hits * 8 + pinfo.n_genes * 12
+    n_vector = shared_entries(pd, ctx, prof, dev)
+    n_forward = forward_hits(pd, ctx, hits, ds, dev)
+    alg_bytes = n_vector * 16 + J * 4 + n_forward * 8 + pinfo.n_genes * 12
     peaks = {}
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
@@ -784,11 +812,10 @@ def main():
     # build.  Residues read for the check, the digit counts and the first sort
     # pass; 8-byte records written by it, read and written by each later pass
     # and read by the dedupe pass; the index (4 bytes a posting, list starts
-    # and codes) written, and read once for the vectors, whose entries (those
-    # of k-mers that several genes hold, not counted here) come on top.
+    # and codes) written, and read once for the vectors; their entries written.
     W, D = pinfo.n_windows, pinfo.n_distinct
     passes = ((alpha ** k - 1).bit_length() + 8) // 9
-    enc_bytes = 3 * ds.n_residues + W * 8 + (passes - 1) * W * 16 + W * 8 + 2 * (E * 4 + D * 4) + D * (4 if alpha ** k <= 1 << 32 else 8)
+    enc_bytes = 3 * ds.n_residues + W * 8 + (passes - 1) * W * 16 + W * 8 + 2 * (E * 4 + D * 4) + D * (4 if alpha ** k <= 1 << 32 else 8) + n_vector * 16
     enc_ms = phases["build"]["kernel_ms"]
     encoder = {"bound": "hbm", "alg_bytes": int(enc_bytes), "kernel_ms": enc_ms,
                "achieved": enc_bytes / (enc_ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
@@ -796,7 +823,7 @@ def main():
 
     # ---- the pair form of Eq. (5) (pd_summin_list: the two vectors joined on
     # their k-mers) on this step's BBH pairs, once
-    merge_form = None
+    pair_form = None
     if n_bbh:
         a_d, b_d = torch.empty(n_bbh, dtype=torch.int32, device=dev), torch.empty(n_bbh, dtype=torch.int32, device=dev)
         pd.pd_bbh_copy(ctx, bbh, a_d, b_d)
@@ -808,8 +835,8 @@ def main():
             e1.record(stream)
             torch.cuda.synchronize()
         m_ms = e0.elapsed_time(e1)
-        merge_form = {"pairs": n_bbh, "ms": m_ms, "pairs_per_s": n_bbh / (m_ms / 1e3),
-                      "what": "sum-min and sum-max of every BBH pair of the step by joining the two multiplicity vectors"}
+        pair_form = {"pairs": n_bbh, "ms": m_ms, "pairs_per_s": n_bbh / (m_ms / 1e3),
+                     "what": "sum-min and sum-max of every BBH pair of the step by joining the two multiplicity vectors"}
         del a_d, b_d, s_d, den_d
 
     # ---- end to end through the C ABI from pinned host buffers: inputs
@@ -876,22 +903,7 @@ def main():
                "sample": f"genome pairs {done} of the same workload ({npairs} gene pairs, {dt:.1f} s, "
                          f"profiles of both genomes included), oracle threads={cores}"}
 
-    # a pipe that the sum-min tiers load: L1TEX data-pipe wavefronts
-    # (shared-memory accumulators + posting loads; ncu, all tiers of one step)
-    # per second of the live kernel time, against one wavefront per cycle per SM
-    # at the SM clock sampled during the timed region
     clocks = clk.summary()
-    wavefronts = captured_counter("paper_2510_23679_gb300/csrc/k_summin.cu", f"summin_{args.workload}.md",
-                                  "l1tex_wavefronts_per_launch")
-    l1tex = None
-    if wavefronts and clocks.get("sm_mhz"):
-        n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
-        l1_peak = n_sm * clocks["sm_mhz"] * 1e6 / 1e9
-        l1_achieved = wavefronts / (k_avg_ms / 1e3) / 1e9
-        l1tex = {"bound": "l1tex", "kernel": "sum-min tiers", "achieved": l1_achieved, "peak": l1_peak,
-                 "unit": "G wavefronts/s", "frac": l1_achieved / l1_peak, "wavefronts": wavefronts,
-                 "peak_source": f"{n_sm} SMs x 1 wavefront/cycle x {clocks['sm_mhz']:.0f} MHz"}
-
     if rank == 0:
         line = {
             "metric": "gene-pair GJ evals/s", "value": value, "unit": "gene-pairs/s", "n_gpus": world,
@@ -909,14 +921,14 @@ def main():
                          "kernel_ms": k_avg_ms, "alg_bytes": alg_bytes, "peak_source": peak_src},
             "e2e": e2e,
             "served": served,
-            "merge_form": merge_form,
+            "pair_form": pair_form,
             "phases": phases,
             "encoder_roofline": encoder,
-            "l1tex_roofline": l1tex,
             "gpu_launches": gpu_launches,
             "cpu_baseline": cpu,
             "clocks": clocks,
-            "stats": {"n_distinct_kmers": pinfo.n_distinct, "mv_entries": E, "postings_walked": J,
+            "stats": {"n_distinct_kmers": pinfo.n_distinct, "postings": E, "vector_entries": n_vector,
+                      "forward_hits": n_forward, "postings_walked": J,
                       "best_hits": hinfo.n_hits, "bbh_pairs": n_bbh, "deferred_queries": hinfo.n_deferred,
                       "max_posting": pinfo.max_posting, "profile_bytes": pinfo.device_bytes},
         }

@@ -61,7 +61,8 @@ typedef enum {
 /* Alphabets ("nucleotide or amino acid", Basic notions). */
 #define PD_ALPHABET_AMINO 20      /* ACDEFGHIKLMNPQRSTVWY */
 #define PD_ALPHABET_NUCLEOTIDE 4  /* ACGT */
-/* Largest k: the k-mer dictionary is a bitmap over all |alphabet|^k codes. */
+/* Largest k: 20^8 and 4^16 codes take 35 and 33 bits of a record that is sorted
+ * with the gene beside the code. */
 #define PD_MAX_K 8
 #define PD_MAX_K_NUCLEOTIDE 16
 /* Largest number of windows (|g| - k + 1) of one gene: counts are 16-bit. */
@@ -119,8 +120,8 @@ int pd_choose_k(uint64_t total_residues, int alphabet);
 
 /* Build the k-mer profiles of a dataset ("Multiplicity vector building
  * phase", Algorithm 1; steps: residue mapping, rolling base-20 k-mer codes,
- * dictionary of distinct codes -> dense ids, per-gene sorted (id, count)
- * vectors, and the inverted index id -> (gene, count) postings).
+ * distinct codes -> dense ids by a sort of all windows, the inverted index id ->
+ * (gene, count) postings, and per-gene (k-mer, count) vectors).
  *   residues   n_res bytes, all genes concatenated, letters ACDEFGHIKLMNPQRSTVWY
  *   gene_ptr   n_genes+1 int64: gene g is residues[gene_ptr[g] .. gene_ptr[g+1])
  *              (gene_ptr[0] = 0, non-decreasing, gene_ptr[n_genes] = n_res)
@@ -147,14 +148,13 @@ pd_status pd_build_profiles_alphabet(pd_ctx* ctx, const uint8_t* residues, uint6
 
 /* pd_build_profiles over several independent problems at once.  genome_seg
  * (HOST array, n_genomes entries, each < n_genomes) assigns every genome to a
- * segment; k-mers of different segments are different dictionary entries
+ * segment; k-mers of different segments are different k-mers
  * (the segment is part of the k-mer's identity), so genes of different
  * segments share no k-mer, have sum-min 0 and are never candidates (reading
  * of "minimum overlap" under Eq. (8)).  Best Hits and BBH of a segmented
  * profile set therefore equal those of each segment profiled alone.  Codes
  * returned by pd_profiles_copy_mv / _copy_index are segment * 20^k + code.
- * Extra error: PD_ERR_BUDGET when (max segment + 1) * 20^k bits exceed the
- * 4 GiB dictionary bitmap limit. */
+ * Extra error: PD_ERR_BUDGET when (max segment + 1) * 20^k exceeds 2^35 codes. */
 pd_status pd_build_profiles_segmented(pd_ctx* ctx, const uint8_t* residues, uint64_t n_res,
                                       const int64_t* gene_ptr, uint32_t n_genes, const int32_t* genome_ptr,
                                       uint32_t n_genomes, const uint32_t* genome_seg, int k,
@@ -164,7 +164,7 @@ typedef struct {
   int k;
   uint32_t n_genes, n_genomes;
   uint64_t n_windows;   /* sum of La over genes */
-  uint64_t n_distinct;  /* distinct k-mers of the dataset (dictionary size D) */
+  uint64_t n_distinct;  /* distinct k-mers of the dataset (D) */
   uint64_t n_entries;   /* sum over genes of distinct k-mers (MV entries = postings) */
   uint32_t max_posting; /* longest posting list */
   uint32_t count_bits;  /* bits of the count field in a packed posting */
@@ -384,9 +384,9 @@ typedef struct pd_batch pd_batch;
  * jobs.  Zero fields take the defaults. */
 typedef struct {
   uint64_t max_chunk_windows; /* k-mer windows profiled together (default 2^29) */
-  uint32_t max_chunk_jobs;    /* jobs per chunk (default: as many as the 256 MiB
-                                 chunk dictionary bitmap holds at the job's k,
-                                 at most PD_MAX_GENOMES / 2) */
+  uint32_t max_chunk_jobs;    /* jobs per chunk (default: as many as keep jobs *
+                                 20^k within 2^31, at least one and at most
+                                 PD_MAX_GENOMES / 2) */
   uint32_t query_order;       /* sum-min work queue: 0 = length buckets (longest
                                  first), min-hash inside a bucket; 1 = min-hash only */
   uint32_t walk;              /* posting walk of the sum-min kernel (PD_WALK_*) */
@@ -411,7 +411,7 @@ typedef struct {
  *   job_k      HOST array of n_jobs k values, each in 1..PD_MAX_K
  *   tuning     NULL for the defaults
  * Jobs with the same k are profiled together in chunks (segmented profiles:
- * one dictionary namespace per job), so one launch sequence serves a whole
+ * one k-mer namespace per job), so one launch sequence serves a whole
  * chunk.  Each job's result equals pd_bbh / pd_best_hits on a dataset of its
  * two genomes alone.  Errors as pd_build_profiles, plus PD_ERR_ARG for bad job
  * entries.  *out receives a device-resident handle. */
@@ -430,7 +430,7 @@ pd_status pd_bbh_pairs(pd_ctx* ctx, const pd_profiles* prof, const uint32_t* job
                        pd_batch** out);
 pd_status pd_batch_get_info(const pd_batch* batch, pd_batch_info* info);
 /* Autotuner of pd_bbh_batch: runs the first n_sample jobs (0 = min(n_jobs,
- * 100)) once with each candidate tuning (jobs per chunk 8 / 32 / dictionary
+ * 100)) once with each candidate tuning (jobs per chunk 8 / 32 / the
  * default, windows per chunk 2^28 / 2^29, both query orders, the automatic
  * walk; then the fastest of these with each explicit posting walk), timed
  * with CUDA events on the context's stream after one warm-up, and writes the

@@ -33,14 +33,15 @@
 // PD_ERR_INTERNAL and its tile writes nothing; the blocks and passes that start
 // after it write nothing either, since what they would read was not written.
 //
-// Measured at 200 genomes x 4000 genes, k = 7 (264 M windows): 15.1 ms for the
+// Measured at 200 genomes x 4000 genes, k = 7 (266 M windows): 16.2 ms for the
 // whole build against 23.4 ms for a dictionary of all codes (marked and looked
 // up at random, 183 MB), hash tables per gene and a gather of every vector
-// entry's list; 2.6 against 3.3 ms at 50 x 3000, k = 6.  Of the 15.1: windows
+// entry's list; 2.9 against 3.3 ms at 50 x 3000, k = 6.  Of the 16.2: windows
 // counted 0.9, four sort passes 6.9 (each moves 4.2 GB in 1.6, 40% of the copy
-// rate: bound by the latency of its phases at two blocks per SM), dedupe 1.8,
-// lists 5.4 (an atomic and a 16-byte store at random for each of 130 M
-// entries: bound by the rate of scattered requests to L2).
+// rate: bound by the latency of its phases at two blocks per SM), dedupe 2.2 (1.8
+// without the counts of the vectors), list starts and codes copied 0.3, lists 5.4
+// (an atomic and a 16-byte store at random for each of 130 M entries: bound by
+// the rate of scattered requests to L2).
 #include <algorithm>
 #include <type_traits>
 
@@ -308,8 +309,8 @@ __device__ __forceinline__ bool begin_tile(PassShared<kBits>& sh, const uint32_t
 // Ranks within the warp come from the lanes holding the same digit: each lane
 // sets its bit in the digit's word of a table of the warp's (in the staging
 // memory, not in use yet).  Finding them with one ballot per digit bit took
-// four instructions a bit and kept the ALU the busiest pipe (1.65 ms a pass
-// against 1.35 at 264 M records).
+// four instructions a bit and kept the ALU the busiest pipe (266 M records, the
+// whole run of 200 genomes x 4000 genes 46.0 ms against 44.7; 1.6 a pass now).
 template <int kBits, typename T>
 __device__ __forceinline__ void rank_and_write(u64 (&xr)[kItems], uint32_t valid_mask, uint32_t shift, T* status,
                                                u64* __restrict__ out, PassShared<kBits>& sh, u64* stage, DevErr* err) {

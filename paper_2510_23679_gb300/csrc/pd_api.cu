@@ -259,9 +259,10 @@ PD_API int pd_choose_k(uint64_t total, int alphabet) {
 }
 
 // ------------------------------------------------------------------ profiles
-// Most codes a segmented dataset's dictionary may cover (segments x 20^k): one
-// bit each, 4 GiB of bits (4.6 GiB of rank blocks).
-static constexpr uint64_t kMaxDictCodes = (uint64_t)32 << 30;
+// Most codes of a segmented dataset (segments x 20^k): 35 bits, which four sort
+// passes of 9 bits and the 40 bits that are kept of a code hold also where the
+// segment stands below the k-mer.
+static constexpr uint64_t kMaxCodes = (uint64_t)32 << 30;
 
 // Windows of a dataset up to which its index and vectors stay in arrays of a
 // window's size, 28 bytes a window where 17 to 20 are used (the build by
@@ -327,9 +328,9 @@ pd_status pdh::build_profiles_impl(pd_ctx* c, const uint8_t* residues, uint64_t 
       n_seg = std::max<uint64_t>(n_seg, (uint64_t)genome_seg[i] + 1);
       code_base[i] = (unsigned long long)genome_seg[i] * n_codes;
     }
-    if (n_seg * n_codes > kMaxDictCodes)
-      return fail(c, PD_ERR_BUDGET, "segments x 20^k exceed the dictionary limit (" +
-                                        std::to_string(kMaxDictCodes >> 30) + " Gi codes)");
+    if (n_seg * n_codes > kMaxCodes)
+      return fail(c, PD_ERR_BUDGET, "segments x 20^k exceed the limit of " +
+                                        std::to_string(kMaxCodes >> 30) + " Gi codes");
   }
   pdg::Launcher* L = &c->L;
   // gene field wide enough to keep the all-ones id unused (see the packed

@@ -261,7 +261,7 @@ struct pd_bbh_set {
 };
 
 
-// Genes profiled against another dataset's dictionary (external queries):
+// Genes profiled against another dataset's index (external queries):
 // their vectors hold only k-mers that dataset contains, with posting ranges
 // into its index, while La counts every window.
 struct QueryProfiles {
