@@ -989,7 +989,9 @@ pd_status pdh::sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& qu
   Buf symbest, ties;
   ALLOC(symbest, sym_bytes);
   for (int attempt = 0; attempt < 3; ++attempt) {
+    *too_many = attempt > 0;  // no room for a longer list: the plain form needs none
     ALLOC(ties, 2 * sizeof(unsigned long long) * tie_cap);
+    *too_many = false;
     pdg::QuerySet Q = queries;  // run_hits clears the maxima and the tie count before each launch
     Q.symbest = symbest.as<unsigned long long>();
     Q.tie_rec = ties.as<unsigned long long>();

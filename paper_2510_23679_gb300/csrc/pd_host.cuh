@@ -311,7 +311,7 @@ pd_status run_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool
 // all genes with a target in a later genome), with their BBH pairs if asked
 // for.  genomes_per_query as above.  The list of exact ties has no bound known
 // beforehand, and their number changes a little from run to run: if no list
-// held them all, *too_many is set (with a status other than PD_OK) and the
+// held them all, or there is no room for a longer one, *too_many is set (with a status other than PD_OK) and the
 // caller takes the plain form, which lists none.
 pd_status sym_hits(pd_ctx* c, const pd_profiles* P, const pdg::QuerySet& Q, bool want_bbh, pd_hits* H,
                    bool* too_many, uint32_t genomes_per_query = 0);

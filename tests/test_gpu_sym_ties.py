@@ -67,6 +67,25 @@ def test_number_of_ties_varies(ctx):
         equal_to_plain(ctx, prof, call, repeats=8)
 
 
+def test_no_room_for_a_longer_list_of_ties():
+    """The plain form, which lists no ties, answers instead."""
+    refused = []
+
+    def on_alloc(nbytes):
+        if nbytes > 300 << 20:  # the longer list; the maxima take 205 MB, rows 153
+            refused.append(nbytes)
+        return nbytes <= 300 << 20
+
+    ctx = pd.pd_ctx_create(0, on_alloc=on_alloc)
+    genomes, genes, length = 800, 40, 60
+    n = genomes * genes
+    residues = LETTERS[np.random.default_rng(1).integers(0, 20, n * length)]
+    prof = pd.pd_build_profiles(ctx, residues, np.arange(n + 1, dtype=np.int64) * length,
+                                np.arange(genomes + 1, dtype=np.int32) * genes, 3)
+    equal_to_plain(ctx, prof, unfiltered)
+    assert len(refused) == 1
+
+
 @pytest.mark.parametrize("theta,tau", [((0, 1), (0, 1)), ((3, 4), (0, 1)), ((0, 1), (1, 2)), ((4, 5), (2, 5))])
 @pytest.mark.parametrize("genomes,genes", [(2, 1500), (9, 400), (64, 120)])
 def test_filtered_of_many_postings(ctx, genomes, genes, theta, tau):
