@@ -372,10 +372,11 @@ constexpr uint32_t kWarpWalkMinAvg = 16;
 // taken: below a few L2 sizes the merge-path walk's runs of postings keep
 // hitting the sectors they have already brought in.
 constexpr uint64_t kWarpWalkMinIndexBytes = 512ull << 20;
-// The warp tier pays when there are queries for several per resident warp
-// (3648 of them: with one genome pair's 3000 queries the launch takes 0.17
-// against 0.11 ms, with 4800 0.12 against 0.09), and for queries that meet few
-// targets: those of one target range (paralogs of 180k genes 1.0 against 1.8
+// The warp tier pays when there are queries for several per resident warp (3648
+// of them; whole calls, ms, blocks alone / warp tier too: 8 genomes x 1000 genes
+// 0.28 / 0.36, 8 x 1500 0.27 / 0.26, 10 x 1600 0.31 / 0.28, 20 x 1000 0.41 / 0.32;
+// of batched jobs, where half of the genes are queries, sum-min alone, 8000 genes
+// 0.12 / 0.15, 16000 0.16 / 0.15), and for queries that meet few targets: those of one target range (paralogs of 180k genes 1.0 against 1.8
 // ms), of short lists (39k queries of 23 genomes 0.33 against 0.50), and in
 // the symmetric form those of few postings.  Where lists are long a query's
 // vector length and the genes after its genome tell how many postings it will
