@@ -214,8 +214,9 @@ pd_status pd_best_hits_all(pd_ctx* ctx, const pd_profiles* prof, pd_hits** out);
  * genomes after its own, emits its Best Hits there and keeps, for every
  * target, the best ratio over the query's genome (the reverse direction, the
  * column maximum of Algorithm 3); used while genes x genomes x 8 bytes stay
- * within 4 GiB (a batch needs 8 bytes a gene), and for listed pairs and
- * batches where the postings saved are worth the table of maxima.
+ * within 4 GiB (a batch needs 8 bytes a gene) and at most 2^30 exact ties are
+ * met, and for filtered calls, listed pairs and batches where the postings saved
+ * are worth the table of maxima.
  * enable == 0: every query walks all of its targets.  Errors: PD_ERR_ARG
  * (null context). */
 pd_status pd_ctx_set_symmetric(pd_ctx* ctx, int enable);
